@@ -92,7 +92,8 @@ template <int NT> struct Shape {
     // small-row form of the narrow shape: "scores of buffer b read" and "P buffer b consumed"
     static constexpr int BAR_SREAD = BAR_ALLDONE + NT;         // + buffer
     static constexpr int BAR_PFREE = BAR_SREAD + 2;            // + buffer
-    static constexpr int NUM_BARS = BAR_PFREE + 2;
+    static constexpr int BAR_DRAIN = BAR_PFREE + 2;            // + MMA warp: its MMAs retired, after a wait gave up
+    static constexpr int NUM_BARS = BAR_DRAIN + 2;
     static_assert(NUM_BARS <= MAX_BARS, "barrier area");
     // TMEM columns: the NT output accumulators, then two score buffers per query tile
     static constexpr uint32_t TM_COLS = 256 * NT;
@@ -258,6 +259,8 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                     mbar_init(bar(C::BAR_PFREE + sb), 1);
                 }
         }
+        mbar_init(bar(C::BAR_DRAIN), 1);
+        mbar_init(bar(C::BAR_DRAIN + 1), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
         prefetch_map(&tm.k); prefetch_map(&tm.v); prefetch_map(&tm.q);
@@ -332,14 +335,24 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     // The ring holds K and V tiles in the order the MMAs consume them: K0, K1, V0, K2, V1, ...,
     // K(n-1), V(n-2), V(n-1) (the product P.V of a tile is issued after the scores of the next
     // one), so that slots are freed in the order they were filled and a V tile does not sit
-    // in the ring while its softmax is still to come.  Item j lives in slot j % NSLOT.
+    // in the ring while its softmax is still to come.  Item j lives in slot j % NSLOT, except in the
+    // small-row form: there two warps consume the tiles, each waiting for its own kind only, so a
+    // slot holds tiles of one kind (K tile t in slot t % 3, V tile t in slot 3 + t % 2).  With
+    // mixed slots a warp skips the phases of the other's tiles, and a parity wait that is two
+    // phases ahead of its barrier succeeds at once: the QK^T warp could take a slot whose V tile
+    // had not even landed.
     auto item_of_k = [&](int t) { return t == 0 ? 0 : 2 * t - 1; };
     auto item_of_v = [&](int t) { return min(2 * t + 2, 2 * n_tiles - 1); };
+    auto v_item = [&](int j) { return j == 2 * n_tiles - 1 || (j > 0 && (j & 1) == 0); };
+    auto tile_of = [&](int j) { return v_item(j) ? (j == 2 * n_tiles - 1 ? n_tiles - 1 : j / 2 - 1) : (j + 1) / 2; };
+    static_assert(!SM || NSLOT == 5, "three K slots, two V slots");
+    auto slot_of = [&](int j) { return !SM ? j % NSLOT : (v_item(j) ? 3 + tile_of(j) % 2 : tile_of(j) % 3); };
+    auto use_of = [&](int j) { return !SM ? j / NSLOT : (v_item(j) ? tile_of(j) / 2 : tile_of(j) / 3); };
     const uint64_t stream_policy = policy_evict_first();
     auto issue_item = [&](int j) {
-        const int slot = j % NSLOT;
-        const bool is_v = j == 2 * n_tiles - 1 || (j > 0 && (j & 1) == 0);
-        const int t = is_v ? (j == 2 * n_tiles - 1 ? n_tiles - 1 : j / 2 - 1) : (j + 1) / 2;
+        const int slot = slot_of(j);
+        const bool is_v = v_item(j);
+        const int t = tile_of(j);
         const uint32_t dst = sbase + OFF_RING + slot * SLOT_BYTES;
         const uint32_t fb = bar(BAR_FULL + slot);
         mbar_expect_tx(fb, SLOT_BYTES);
@@ -464,6 +477,14 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                 }
                 const float m_new = fmaxf(m_run, mx * sc);
                 const bool need = m_new > m_run + RESCALE_THRESHOLD;   // also the first finite maximum
+                if constexpr (SM) {
+                    // the product of tile t - 2 has read P buffer sb (and with it BAR_PVDONE is at
+                    // most one phase behind tile t - 1, which is what a parity wait can tell)
+                    if (t >= 2) {
+                        ok = mbar_wait_warp(bar(C::BAR_PFREE + sb), ((t >> 1) - 1) & 1, abort_flag);
+                        if (!ok) break;
+                    }
+                }
                 if (__any_sync(0xffffffffu, need)) {
                     const float alpha = need ? ex2(m_run - m_new) : 1.f;
                     if (need) { m_run = m_new; l_run *= alpha; }
@@ -519,12 +540,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                 }
                 l_run += (acc0.x + acc0.y) + (acc1.x + acc1.y);
                 if constexpr (SM) {
-                    // P row r into shared memory buffer sb ([64 rows][64 keys] bf16, 128-byte swizzle),
-                    // once the product of tile t - 2 has read that buffer
-                    if (t >= 2) {
-                        ok = mbar_wait_warp(bar(C::BAR_PFREE + sb), ((t >> 1) - 1) & 1, abort_flag);
-                        if (!ok) break;
-                    }
+                    // P row r into shared memory buffer sb ([64 rows][64 keys] bf16, 128-byte swizzle)
                     unsigned char *prow = smem + OFF_Q + (sb ? 3 : 1) * (QSUB_BYTES / 2) + r * 128;
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
@@ -634,15 +650,17 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             bool ok = true;
             const int n_items = 2 * n_tiles;
             while (produced < n_items && ok) {
-                const int slot = produced % NSLOT, use = produced / NSLOT;
+                const int slot = slot_of(produced), use = use_of(produced);
                 if (use > 0) ok = mbar_wait(bar(BAR_EMPTY + slot), (use - 1) & 1, abort_flag);
                 if (ok) { issue_item(produced); ++produced; }
             }
             if (*abort_flag) {
                 // give the copies that were armed a bounded time to land before smem is released
-                for (int j = max(0, produced - NSLOT); j < produced; ++j) {   // latest use of each slot
+                uint32_t seen = 0;
+                for (int j = produced - 1; j >= 0 && seen != (1u << NSLOT) - 1; --j) {   // latest use of each slot
                     int dummy = 0;
-                    mbar_wait(bar(BAR_FULL + j % NSLOT), (j / NSLOT) & 1, &dummy);
+                    if (!(seen >> slot_of(j) & 1)) mbar_wait(bar(BAR_FULL + slot_of(j)), use_of(j) & 1, &dummy);
+                    seen |= 1u << slot_of(j);
                 }
                 int dummy = 0;
                 mbar_wait(bar(BAR_QFULL), 0, &dummy);
@@ -655,8 +673,8 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
         constexpr uint32_t IDESC_PV = make_idesc(HD, 1);      // A = P (TMEM), B = V tile (MN-major)
         const uint32_t q_addr = sbase + OFF_Q + ti * 2 * QSUB_BYTES;
         auto issue_qk = [&](int t) -> bool {
-            const int j = item_of_k(t), slot = j % NSLOT;
-            if (!mbar_wait_warp(bar(BAR_FULL + slot), (j / NSLOT) & 1, abort_flag)) return false;
+            const int j = item_of_k(t), slot = slot_of(j);
+            if (!mbar_wait_warp(bar(BAR_FULL + slot), use_of(j) & 1, abort_flag)) return false;
             tc_fence_after();
             if (lane == 0) {
                 const uint32_t k_addr = sbase + OFF_RING + slot * SLOT_BYTES;
@@ -674,8 +692,8 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             return true;
         };
         auto issue_pv = [&](int t) -> bool {
-            const int j = item_of_v(t), slot = j % NSLOT;
-            if (!mbar_wait_warp(bar(BAR_FULL + slot), (j / NSLOT) & 1, abort_flag)) return false;
+            const int j = item_of_v(t), slot = slot_of(j);
+            if (!mbar_wait_warp(bar(BAR_FULL + slot), use_of(j) & 1, abort_flag)) return false;
             // Only the 16-key groups that hold keys are multiplied (an instruction costs its issuing
             // thread the same whatever its size): the block's own tile is K keys wide, a ragged
             // prefix tile ends at the prefix.  In the last group, V rows past the keys may hold
@@ -744,7 +762,15 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             }
         }
         // every MMA of this warp must have retired before TMEM is freed
-        if (ok) mbar_wait_warp(bar(C::BAR_ALLDONE + ti), 0, abort_flag);
+        if (ok) ok = mbar_wait_warp(bar(C::BAR_ALLDONE + ti), 0, abort_flag);
+        if (!ok) {
+            // a wait gave up: this warp's MMAs in flight still read shared memory and write TMEM
+            const int drain = C::BAR_DRAIN + warp - C::MMA_WARP;
+            if (lane == 0) umma_commit(bar(drain));
+            __syncwarp();
+            int dummy = 0;
+            mbar_wait_warp(bar(drain), 0, &dummy);
+        }
         tc_fence_before();
     }
 

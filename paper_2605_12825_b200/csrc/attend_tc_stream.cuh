@@ -33,8 +33,8 @@
 // unit, at most 128 batch entries (their lengths are ranked in shared memory).
 
 constexpr int STREAM_MAX_B = 128;
-// extra barriers of the persistent kernel, behind those of Shape<1>
-constexpr int SBAR_QFREE = Shape<1>::NUM_BARS, SBAR_OFREE = SBAR_QFREE + 1, SBAR_NUM = SBAR_OFREE + 1;
+// two more barriers of the persistent kernel, in the place of two that only the small-row form has
+constexpr int SBAR_QFREE = Shape<1>::BAR_SREAD, SBAR_OFREE = SBAR_QFREE + 1, SBAR_NUM = Shape<1>::NUM_BARS;
 static_assert(SBAR_NUM <= 24, "the barrier area's last 128 bytes hold the ranking");
 // Two CTAs per SM leave 640 bytes beside Shape<1>'s map: the ranked sequences go into the unused
 // end of the barrier area, the flag into the spare words next to the TMEM address, the tile
@@ -149,6 +149,7 @@ attend_tc_stream_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, c
         }
         mbar_init(bar(BAR_PVDONE), 1);
         mbar_init(bar(BAR_ALLDONE), 1);
+        mbar_init(bar(C::BAR_DRAIN), 1);
         mbar_init(bar(SBAR_QFREE), 1);
         mbar_init(bar(SBAR_OFREE), n_act);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -531,7 +532,13 @@ attend_tc_stream_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, c
             ++pcidx;
         }
         // every MMA must have retired before TMEM is freed
-        if (ok && pcidx > 0) mbar_wait_warp(bar(BAR_ALLDONE), (pcidx - 1) & 1, abort_flag);
+        if (ok && pcidx > 0) ok = mbar_wait_warp(bar(BAR_ALLDONE), (pcidx - 1) & 1, abort_flag);
+        if (!ok) {                            // a wait gave up: the MMAs in flight end before TMEM is freed
+            if (lane == 0) umma_commit(bar(C::BAR_DRAIN));
+            __syncwarp();
+            int dummy = 0;
+            mbar_wait_warp(bar(C::BAR_DRAIN), 0, &dummy);
+        }
         tc_fence_before();
     }
 
