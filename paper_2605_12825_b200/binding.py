@@ -1,4 +1,5 @@
-"""Thin ctypes binding of liborthrus.so (argument marshalling only).
+"""Thin binding of liborthrus.so (argument marshalling only): the hot calls through a small native
+module, everything else through ctypes.
 
 Every function has the name of the C entry point it calls; tensors are torch CUDA
 tensors whose device pointers are handed over unchanged.  torch is used for device
@@ -118,6 +119,17 @@ _lib = None
 _lib = _load()
 
 
+# after torch and liborthrus.so, whose symbols it uses
+from . import _native  # noqa: E402
+
+
+def _raise(code: int, where: str) -> None:
+    raise OrthrusError(code, where)
+
+
+_native.set_raiser(_raise)
+
+
 def lib() -> ctypes.CDLL:
     return _lib
 
@@ -128,10 +140,6 @@ def dtype_code(dt: torch.dtype) -> int:
     if dt == torch.float32:
         return FP32
     raise TypeError(f"unsupported dtype {dt}")
-
-
-def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
-    return None if t is None else t.data_ptr()
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
@@ -171,16 +179,12 @@ def new_workspace(nbytes: int, device="cuda") -> torch.Tensor:
 
 def orthrus_diffusion_block_attend(layer: Layer, q_diff, k_diff_blk, v_diff_blk, out, workspace,
                                    stream=None) -> None:
-    _check(_lib.orthrus_diffusion_block_attend(
-        ctypes.byref(layer), _ptr(q_diff), _ptr(k_diff_blk), _ptr(v_diff_blk), _ptr(out),
-        _ptr(workspace), workspace.numel(), _stream(stream)), "orthrus_diffusion_block_attend")
+    _native.diffusion_block_attend(layer, q_diff, k_diff_blk, v_diff_blk, out, workspace, stream)
 
 
 def orthrus_ar_verify_attend(layer: Layer, q_ar, k_ar_blk, v_ar_blk, out, workspace,
                              stream=None) -> None:
-    _check(_lib.orthrus_ar_verify_attend(
-        ctypes.byref(layer), _ptr(q_ar), _ptr(k_ar_blk), _ptr(v_ar_blk), _ptr(out),
-        _ptr(workspace), workspace.numel(), _stream(stream)), "orthrus_ar_verify_attend")
+    _native.ar_verify_attend(layer, q_ar, k_ar_blk, v_ar_blk, out, workspace, stream)
 
 
 def orthrus_multi_block_workspace_bytes(layer: Layer, n_blocks: int) -> int:
@@ -191,9 +195,7 @@ def orthrus_multi_block_attend(layer: Layer, anchors, q_diff, k_diff_blk, v_diff
                                stream=None) -> None:
     """Diffusion-view attention under the multi-block mask of Eq. 6; anchors int32 [S][n_blocks],
     q_diff / out [S][n_blocks][K][Hq][d], block K/V [S][n_blocks][K][Hkv][d]."""
-    _check(_lib.orthrus_multi_block_attend(
-        ctypes.byref(layer), anchors.shape[1], _ptr(anchors), _ptr(q_diff), _ptr(k_diff_blk), _ptr(v_diff_blk),
-        _ptr(out), _ptr(workspace), workspace.numel(), _stream(stream)), "orthrus_multi_block_attend")
+    _native.multi_block_attend(layer, anchors, q_diff, k_diff_blk, v_diff_blk, out, workspace, stream)
 
 
 def orthrus_consensus_workspace_bytes(batch: int, block: int, vocab: int) -> int:
@@ -202,11 +204,7 @@ def orthrus_consensus_workspace_bytes(batch: int, block: int, vocab: int) -> int
 
 def orthrus_consensus_accept(ar_logits, draft, n_commit, committed, ar_argmax, next_anchor,
                              workspace, stream=None) -> None:
-    B, K, V = ar_logits.shape
-    _check(_lib.orthrus_consensus_accept(
-        _ptr(ar_logits), dtype_code(ar_logits.dtype), _ptr(draft), B, K, V, _ptr(n_commit),
-        _ptr(committed), _ptr(ar_argmax), _ptr(next_anchor), _ptr(workspace), workspace.numel(),
-        _stream(stream)), "orthrus_consensus_accept")
+    _native.consensus_accept(ar_logits, draft, n_commit, committed, ar_argmax, next_anchor, workspace, stream)
 
 
 def orthrus_consensus_sample_workspace_bytes(batch: int, block: int, vocab: int) -> int:
@@ -216,15 +214,8 @@ def orthrus_consensus_sample_workspace_bytes(batch: int, block: int, vocab: int)
 def orthrus_consensus_sample(ar_logits, diff_logits, draft, u_accept, u_resample, temperature: float,
                              n_commit, committed, next_anchor, workspace, stream=None) -> None:
     """Sampled consensus for T > 0; u_accept / u_resample are float32 [B][K] device tensors."""
-    B, K, V = ar_logits.shape
-    if diff_logits.shape != ar_logits.shape or diff_logits.dtype != ar_logits.dtype:
-        raise TypeError("the two logit tensors must agree in shape and dtype")
-    if u_accept.dtype != torch.float32 or u_resample.dtype != torch.float32:
-        raise TypeError("the uniforms must be float32")
-    _check(_lib.orthrus_consensus_sample(
-        _ptr(ar_logits), _ptr(diff_logits), dtype_code(ar_logits.dtype), _ptr(draft), _ptr(u_accept),
-        _ptr(u_resample), float(temperature), B, K, V, _ptr(n_commit), _ptr(committed), _ptr(next_anchor),
-        _ptr(workspace), workspace.numel(), _stream(stream)), "orthrus_consensus_sample")
+    _native.consensus_sample(ar_logits, diff_logits, draft, u_accept, u_resample, temperature, n_commit,
+                             committed, next_anchor, workspace, stream)
 
 
 STATIC_CONSENSUS_SCRATCH_BYTES = 65536
@@ -236,11 +227,7 @@ def orthrus_consensus_accept_static(ar_logits, draft, n_commit, committed, ar_ar
     device memory.  The scratch is a fixed array inside the library, shared by all calls
     on a device (calls that overlap on the GPU race on it).  Problems that need more than
     STATIC_CONSENSUS_SCRATCH_BYTES of scratch raise OrthrusError (workspace too small)."""
-    B, K, V = ar_logits.shape
-    _check(_lib.orthrus_consensus_accept_static(
-        _ptr(ar_logits), dtype_code(ar_logits.dtype), _ptr(draft), B, K, V, _ptr(n_commit),
-        _ptr(committed), _ptr(ar_argmax), _ptr(next_anchor), _stream(stream)),
-        "orthrus_consensus_accept_static")
+    _native.consensus_accept_static(ar_logits, draft, n_commit, committed, ar_argmax, next_anchor, stream)
 
 
 def orthrus_lm_head_consensus_workspace_bytes(batch: int, block: int, vocab: int) -> int:
@@ -251,57 +238,36 @@ def orthrus_lm_head_consensus(hidden, lm_head, draft, n_commit, committed, ar_ar
                               workspace, stream=None) -> None:
     """Greedy consensus from the last hidden states [B][K][H] and the LM head [V][H] (bf16);
     the logits are never materialised."""
-    B, K, H = hidden.shape
-    V = lm_head.shape[0]
-    _check(_lib.orthrus_lm_head_consensus(
-        _ptr(hidden), _ptr(lm_head), dtype_code(hidden.dtype), H, _ptr(draft), B, K, V, _ptr(n_commit),
-        _ptr(committed), _ptr(ar_argmax), _ptr(next_anchor), _ptr(workspace), workspace.numel(),
-        _stream(stream)), "orthrus_lm_head_consensus")
+    _native.lm_head_consensus(hidden, lm_head, draft, n_commit, committed, ar_argmax, next_anchor, workspace,
+                              stream)
 
 
 def orthrus_kv_append(layer: Layer, k_ar_blk, v_ar_blk, n_commit, update_len: bool = True,
                       workspace=None, stream=None) -> None:
-    _check(_lib.orthrus_kv_append(
-        ctypes.byref(layer), _ptr(k_ar_blk), _ptr(v_ar_blk), _ptr(n_commit),
-        1 if update_len else 0, _ptr(workspace), 0 if workspace is None else workspace.numel(),
-        _stream(stream)), "orthrus_kv_append")
+    _native.kv_append(layer, k_ar_blk, v_ar_blk, n_commit, update_len, workspace, stream)
 
 
 def orthrus_kv_append_layers(layers, k_ar_blks, v_ar_blks, n_commit, update_len: bool = True,
                              workspace=None, stream=None) -> None:
     """`layers`: sequence of Layer; `k_ar_blks` / `v_ar_blks`: one tensor per layer."""
-    n = len(layers)
-    arr = (Layer * n)(*layers)
-    kp = (ctypes.c_void_p * n)(*[t.data_ptr() for t in k_ar_blks])
-    vp = (ctypes.c_void_p * n)(*[t.data_ptr() for t in v_ar_blks])
-    _check(_lib.orthrus_kv_append_layers(
-        arr, n, kp, vp, _ptr(n_commit), 1 if update_len else 0, _ptr(workspace),
-        0 if workspace is None else workspace.numel(), _stream(stream)), "orthrus_kv_append_layers")
-
-
-def _ws_args(workspace):
-    return _ptr(workspace), 0 if workspace is None else workspace.numel()
+    _native.kv_append_layers(layers, k_ar_blks, v_ar_blks, n_commit, update_len, workspace, stream)
 
 
 def orthrus_block_kv_write(layer: Layer, k_blk, v_blk, workspace=None, stream=None) -> None:
     """All K block rows go behind the prefix (cache rows [P_b, P_b + K)); lengths unchanged."""
-    _check(_lib.orthrus_block_kv_write(ctypes.byref(layer), _ptr(k_blk), _ptr(v_blk), *_ws_args(workspace),
-                                       _stream(stream)), "orthrus_block_kv_write")
+    _native.block_kv_write(layer, k_blk, v_blk, workspace, stream)
 
 
 def orthrus_commit_len(layer: Layer, n_commit, workspace=None, stream=None) -> None:
     """cache_len += n_commit for the layer's length array."""
-    _check(_lib.orthrus_commit_len(ctypes.byref(layer), _ptr(n_commit), *_ws_args(workspace), _stream(stream)),
-           "orthrus_commit_len")
+    _native.commit_len(layer, n_commit, workspace, stream)
 
 
 def orthrus_rope_block_kv_write(layer: Layer, q, k_blk, v_blk, rope_theta: float, q_out, workspace=None,
                                 stream=None) -> None:
     """Rotary embedding of the block's queries (to q_out) and keys, keys and values written to
     cache rows [P_b, P_b + K)."""
-    _check(_lib.orthrus_rope_block_kv_write(ctypes.byref(layer), _ptr(q), _ptr(k_blk), _ptr(v_blk),
-                                            float(rope_theta), _ptr(q_out), *_ws_args(workspace), _stream(stream)),
-           "orthrus_rope_block_kv_write")
+    _native.rope_block_kv_write(layer, q, k_blk, v_blk, rope_theta, q_out, workspace, stream)
 
 
 def orthrus_read_status(workspace, stream=None) -> int:

@@ -1,4 +1,5 @@
-"""Builds liborthrus.so (sm_100a) in-tree with nvcc.  Usable without a GPU."""
+"""Builds liborthrus.so (sm_100a) with nvcc and the native argument marshalling with g++, in-tree.
+Usable without a GPU."""
 from __future__ import annotations
 
 import glob
@@ -10,6 +11,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liborthrus.so")
+NATIVE_SRC = os.path.join(CSRC, "native_binding.cpp")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -17,6 +20,44 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
 
 def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def stale_native() -> bool:
+    if not os.path.exists(NATIVE):
+        return True
+    t = os.path.getmtime(NATIVE)
+    return any(os.path.getmtime(f) > t for f in [NATIVE_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h")))
+
+
+def start_native():
+    """Starts the compilation of the native argument marshalling (it needs torch's and Python's
+    headers and links against torch and liborthrus.so); finish_native() links it."""
+    import sysconfig
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    obj = os.path.join(HERE, "_build", "native_binding.o")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-w",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", inc,
+           "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"],
+           "-isystem", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"),
+           "-c", NATIVE_SRC, "-o", obj]
+    return obj, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+
+
+def finish_native(started) -> None:
+    import torch
+    obj, pr = started
+    out = pr.communicate()[0].decode()
+    if pr.returncode != 0:
+        sys.stderr.write(out)
+        raise RuntimeError("compiling native_binding.cpp failed")
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, "-L", HERE, "-l:liborthrus.so",
+                    "-Wl,-rpath,$ORIGIN", "-L", os.path.join(os.path.dirname(torch.__file__), "lib"),
+                    "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
+    os.replace(tmp, NATIVE)
 
 
 def stale() -> bool:
@@ -29,10 +70,17 @@ def stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not stale():
-        return LIB
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
+    native = start_native() if force or stale_native() else None
+    if force or stale():
+        build_lib(objdir, verbose)
+    if native:
+        finish_native(native)
+    return LIB
+
+
+def build_lib(objdir: str, verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     inc = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
     procs = []
@@ -57,7 +105,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.run([nvcc, "-shared", "-o", tmp, *objs, "-gencode",
                     "arch=compute_100a,code=sm_100a"], check=True)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":
