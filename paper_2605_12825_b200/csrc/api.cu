@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <unistd.h>
 #include "common.cuh"
 
 namespace orthrus {
@@ -34,12 +35,35 @@ static int current_path()
     return v;
 }
 
-static int env_int(const char *name, int dflt)
+// The tuning variables of the environment, read at every call that plans (a test changes them
+// between calls).  One walk over the environment, which hardly ever holds any of them, instead of a
+// search per variable: half a dozen searches were a tenth of a call's host time.
+struct Knobs {
+    int splits = 0, min_chunk_tiles = 2, target_ctas = 0;     // 0: not forced / the default
+    bool no_early_launch = false, stream = false, pack = true;
+};
+static Knobs read_knobs()
 {
-    const char *s = getenv(name);
-    if (!s || !*s) return dflt;
-    const int v = atoi(s);
-    return v > 0 ? v : dflt;
+    Knobs k;
+    for (char **e = environ; e && *e; ++e) {
+        const char *s = *e;
+        if (s[0] != 'O' || strncmp(s, "ORTHRUS_", 8) != 0) continue;
+        s += 8;
+        const char *eq = strchr(s, '=');
+        if (!eq || !eq[1]) continue;
+        const size_t n = (size_t)(eq - s);
+        const char *val = eq + 1;
+        auto is = [&](const char *name) { return strlen(name) == n && !strncmp(s, name, n); };
+        auto positive = [&](int &x) { const int v = atoi(val); if (v > 0) x = v; };
+        int on = 0;
+        if (is("SPLITS")) positive(k.splits);
+        else if (is("MIN_CHUNK_TILES")) positive(k.min_chunk_tiles);
+        else if (is("TARGET_CTAS")) positive(k.target_ctas);
+        else if (is("NO_EARLY_LAUNCH")) { positive(on); k.no_early_launch = on > 0; }
+        else if (is("TC_SCHEDULE")) k.stream = !strcmp(val, "stream");
+        else if (is("MULTI_BLOCK_PACK")) k.pack = val[0] != '0';
+    }
+    return k;
 }
 
 }  // namespace orthrus
@@ -115,20 +139,17 @@ static bool tc_usable(const orthrus_layer_t *L)
 // ORTHRUS_TC_SCHEDULE=stream (read at every call) selects the persistent kernel, which cuts the
 // work by tiles instead of by units, for the shapes it serves; it was measured slower than the
 // cluster kernel and is a measurement knob.  A forced split count keeps the cluster kernel.
-static bool tc_use_stream(const orthrus_layer_t *L)
+static bool tc_use_stream(const orthrus_layer_t *L, const Knobs &kn)
 {
-    if (!tc_usable(L)) return false;
-    const int G = L->n_q_heads / L->n_kv_heads;
-    if (!tc_stream_shape(L->batch, G, L->block) || env_int("ORTHRUS_SPLITS", 0) > 0) return false;
-    const char *e = getenv("ORTHRUS_TC_SCHEDULE");
-    return e && !strcmp(e, "stream");
+    return kn.stream && kn.splits == 0 && tc_usable(L) &&
+           tc_stream_shape(L->batch, L->n_q_heads / L->n_kv_heads, L->block);
 }
 static int tc_stream_ctas() { return tc_ctas_per_sm(1) * num_sms(); }
 
-static Plan make_plan(const orthrus_layer_t *L, bool tc)
+static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 {
     const int max_len = max_len_of(L);
-    const int forced = env_int("ORTHRUS_SPLITS", 0);
+    const int forced = kn.splits;
     Plan pl;
     if (tc) {
         // The splits of a unit are the CTAs of one thread-block cluster (<= 16).  Few units:
@@ -143,8 +164,7 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc)
         if (forced > 0) {
             S = forced;
         } else if (units * 2 <= slots) {
-            const int min_tiles = env_int("ORTHRUS_MIN_CHUNK_TILES", 2);
-            while (S < 16 && units * S * 2 <= slots && tiles / (S * 2) >= min_tiles) S *= 2;
+            while (S < 16 && units * S * 2 <= slots && tiles / (S * 2) >= kn.min_chunk_tiles) S *= 2;
         } else {
             // (a lone CTA streams slower than an SM's share of HBM, so the longest unit is
             //  still split; many small CTAs would spend their time starting and merging)
@@ -162,8 +182,8 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc)
     const int granule = 128;
     const int units = L->batch * L->n_kv_heads;
     const int tiles = max_len > 0 ? (max_len + granule - 1) / granule : 1;
-    const int target = env_int("ORTHRUS_TARGET_CTAS", 2 * num_sms());
-    const int min_chunk_tiles = env_int("ORTHRUS_MIN_CHUNK_TILES", 2);
+    const int target = kn.target_ctas > 0 ? kn.target_ctas : 2 * num_sms();
+    const int min_chunk_tiles = kn.min_chunk_tiles;
     int splits = (target + units - 1) / units;
     if (forced > 0) splits = forced;
     int max_splits = forced > 0 ? tiles : tiles / min_chunk_tiles;
@@ -210,8 +230,9 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
         return ORTHRUS_ERR_INVALID_ARG;
     const int want = current_path();
     const bool tc = (want == PATH_AUTO || want == PATH_TCGEN05) && tc_usable(L);
-    const bool stream_k = tc && tc_use_stream(L);
-    Plan pl = make_plan(L, tc);
+    const Knobs kn = read_knobs();
+    const bool stream_k = tc && tc_use_stream(L, kn);
+    Plan pl = make_plan(L, tc, kn);
     if (stream_k) pl.n_splits = 1;
     size_t ml_off = 0;
     const size_t need = kHeaderBytes + (stream_k ? tc_stream_workspace_bytes(L->batch, L->n_kv_heads, tc_stream_ctas())
@@ -233,13 +254,15 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     const float scale = L->softmax_scale > 0.f ? L->softmax_scale : 1.f / sqrtf((float)p.d);
     p.scale_log2 = scale * 1.4426950408889634f;
 
+    int flags = (int)(L->flags & (ORTHRUS_LAYER_CACHE_QUIESCENT | ORTHRUS_LAYER_NO_EARLY_LAUNCH));
+    if (kn.no_early_launch) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
+    p.early = !(flags & ORTHRUS_LAYER_NO_EARLY_LAUNCH);
+
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     bool merge_kernel = pl.n_splits > 1;
     if (tc) {
         t_last_path = "tcgen05";
-        int flags = (int)(L->flags & (ORTHRUS_LAYER_CACHE_QUIESCENT | ORTHRUS_LAYER_NO_EARLY_LAUNCH));
-        if (env_int("ORTHRUS_NO_EARLY_LAUNCH", 0)) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
         if (stream_k) e = launch_attend_tc_stream(p, tc_stream_ctas(), base + kHeaderBytes, flags, cs);
         else e = launch_attend_tc(p, flags, cs);
         merge_kernel = false;
@@ -268,11 +291,12 @@ size_t orthrus_attend_workspace_bytes(const orthrus_layer_t *layer)
 {
     if (check_layer(layer) != ORTHRUS_OK) return 0;
     // enough for whichever kernel path a later call resolves to
-    size_t need = partial_bytes(layer, make_plan(layer, false), nullptr, false);
+    const Knobs kn = read_knobs();
+    size_t need = partial_bytes(layer, make_plan(layer, false, kn), nullptr, false);
     if (tc_usable(layer)) {
-        const size_t n2 = partial_bytes(layer, make_plan(layer, true), nullptr, true);
+        const size_t n2 = partial_bytes(layer, make_plan(layer, true, kn), nullptr, true);
         if (n2 > need) need = n2;
-        if (tc_use_stream(layer)) {
+        if (tc_use_stream(layer, kn)) {
             const size_t n3 = tc_stream_workspace_bytes(layer->batch, layer->n_kv_heads, tc_stream_ctas());
             if (n3 > need) need = n3;
         }
@@ -318,15 +342,14 @@ static bool multi_block_layer(const orthrus_layer_t *layer, int32_t n_blocks, co
 // The packed form of Eq. 6 (tcgen05 path): the blocks of a sequence share 128-row query tiles, so
 // the prefix is streamed once per tile instead of once per block.  Taken when at least two blocks
 // fit one tile; ORTHRUS_MULTI_BLOCK_PACK=0 keeps the one-unit-per-block form (a measurement knob).
-static bool multi_block_packed(const orthrus_layer_t *layer, int32_t n_blocks)
+static bool multi_block_packed(const orthrus_layer_t *layer, int32_t n_blocks, const Knobs &kn)
 {
     if (n_blocks < 2 || check_layer(layer) != ORTHRUS_OK || !tc_usable(layer)) return false;
     const int want = current_path();
     if (want != PATH_AUTO && want != PATH_TCGEN05) return false;
     if (2 * (layer->n_q_heads / layer->n_kv_heads) * layer->block > 128) return false;
     if ((long long)n_blocks * layer->block > (1 << 20)) return false;
-    const char *e = getenv("ORTHRUS_MULTI_BLOCK_PACK");
-    return !(e && e[0] == '0');
+    return kn.pack;
 }
 
 // the descriptor the packed form plans with: one "block" of n_blocks * K positions per sequence
@@ -341,14 +364,14 @@ static orthrus_layer_t packed_layer(const orthrus_layer_t *layer, int32_t n_bloc
 
 static orthrus_status_t attend_packed(const orthrus_layer_t *layer, int32_t n_blocks, const int32_t *anchors,
                                       const void *q, const void *k_blk, const void *v_blk, void *out,
-                                      void *ws, size_t ws_bytes, void *stream)
+                                      void *ws, size_t ws_bytes, void *stream, const Knobs &kn)
 {
     if (!q || !k_blk || !v_blk || !out || !ws || !layer->k_cache || !layer->v_cache) return ORTHRUS_ERR_INVALID_ARG;
     if (!aligned16(q) || !aligned16(k_blk) || !aligned16(v_blk) || !aligned16(out) || !aligned16(ws) ||
         !aligned16(layer->k_cache) || !aligned16(layer->v_cache) || (reinterpret_cast<uintptr_t>(anchors) & 3))
         return ORTHRUS_ERR_INVALID_ARG;
     const orthrus_layer_t L = packed_layer(layer, n_blocks);
-    const Plan pl = make_plan(&L, true);
+    const Plan pl = make_plan(&L, true, kn);
     size_t ml_off = 0;
     if (ws_bytes < kHeaderBytes + partial_bytes(&L, pl, &ml_off, true)) return ORTHRUS_ERR_WORKSPACE;
 
@@ -367,7 +390,8 @@ static orthrus_status_t attend_packed(const orthrus_layer_t *layer, int32_t n_bl
     p.scale_log2 = scale * 1.4426950408889634f;
     t_last_path = "tcgen05";
     int flags = (int)(layer->flags & (ORTHRUS_LAYER_CACHE_QUIESCENT | ORTHRUS_LAYER_NO_EARLY_LAUNCH));
-    if (env_int("ORTHRUS_NO_EARLY_LAUNCH", 0)) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
+    if (kn.no_early_launch) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
+    p.early = !(flags & ORTHRUS_LAYER_NO_EARLY_LAUNCH);
     return launch_attend_tc_packed(p, flags, static_cast<cudaStream_t>(stream)) == cudaSuccess
                ? ORTHRUS_OK : ORTHRUS_ERR_CUDA;
 }
@@ -381,7 +405,7 @@ size_t orthrus_multi_block_workspace_bytes(const orthrus_layer_t *layer, int32_t
     if (need && check_layer(layer) == ORTHRUS_OK && tc_usable(layer) && n_blocks >= 2 &&
         (long long)n_blocks * layer->block <= (1 << 20)) {
         const orthrus_layer_t Lp = packed_layer(layer, n_blocks);
-        const size_t n2 = kHeaderBytes + partial_bytes(&Lp, make_plan(&Lp, true), nullptr, true);
+        const size_t n2 = kHeaderBytes + partial_bytes(&Lp, make_plan(&Lp, true, read_knobs()), nullptr, true);
         if (n2 > need) need = n2;
     }
     return need;
@@ -394,9 +418,10 @@ orthrus_status_t orthrus_multi_block_attend(const orthrus_layer_t *layer, int32_
     orthrus_layer_t L;
     if (!anchors || !multi_block_layer(layer, n_blocks, anchors, &L)) return ORTHRUS_ERR_INVALID_ARG;
     if (layer->flags & ORTHRUS_LAYER_BLOCK_IN_CACHE) return ORTHRUS_ERR_INVALID_ARG;
-    if (multi_block_packed(layer, n_blocks))
+    const Knobs kn = read_knobs();
+    if (multi_block_packed(layer, n_blocks, kn))
         return attend_packed(layer, n_blocks, anchors, q_diff, k_diff_blk, v_diff_blk, out, workspace,
-                             workspace_bytes, stream);
+                             workspace_bytes, stream, kn);
     return attend(&L, 0, q_diff, k_diff_blk, v_diff_blk, out, workspace, workspace_bytes, stream, n_blocks);
 }
 
@@ -521,7 +546,7 @@ orthrus_status_t orthrus_lm_head_consensus(const void *hidden, const void *lm_he
                                           static_cast<int32_t *>(workspace), st);
     if (e == cudaErrorNotSupported) return ORTHRUS_ERR_UNSUPPORTED;
     if (e == cudaSuccess)
-        e = launch_consensus_finalize_wide(parts, lm_head_vocab_tiles(batch * block, vocab), draft, batch, block, n_commit,
+        e = launch_consensus_finalize(parts, lm_head_vocab_tiles(batch * block, vocab), draft, batch, block, n_commit,
                                            committed, ar_argmax, next_anchor, st);
     return e == cudaSuccess ? ORTHRUS_OK : ORTHRUS_ERR_CUDA;
 }

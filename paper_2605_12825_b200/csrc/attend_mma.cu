@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(NWARPS * 32) attend_mma_kernel(AttnParams p)
     constexpr int NTHREADS = NWARPS * 32;
     extern __shared__ __align__(128) unsigned char smem_raw[];
 
+    pdl_begin();
     const int unit = blockIdx.x, split = blockIdx.y, rt = blockIdx.z;
     const int b = unit / p.Hkv, h = unit % p.Hkv;
     const int P = clamp_cache_len(p, b);
@@ -282,9 +283,7 @@ cudaError_t launch_one(const AttnParams &p, cudaStream_t st)
         configured = true;
     }
     dim3 grid(p.B * p.Hkv, p.n_splits, (p.M + MT - 1) / MT);
-    kern<<<grid, NWARPS * 32, smem, st>>>(p);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(p.early, kern, grid, NWARPS * 32, smem, st, p);
 }
 
 }  // namespace

@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(128) attend_simt_kernel(AttnParams p)
     float *sV = sK + TN * (D + 1);       // [TN][D]
     float *sQ = sV + TN * D;             // [MT][D]
 
+    pdl_begin();
     const int unit = blockIdx.x, split = blockIdx.y, rt = blockIdx.z;
     const int b = unit / p.Hkv, h = unit % p.Hkv;
     const int P = clamp_cache_len(p, b);
@@ -159,9 +160,7 @@ cudaError_t launch_one(const AttnParams &p, cudaStream_t st)
         if (e != cudaSuccess) return e;
     }
     dim3 grid(p.B * p.Hkv, p.n_splits, (p.M + MT - 1) / MT);
-    kern<<<grid, 128, smem, st>>>(p);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(p.early, kern, grid, 128, smem, st, p);
 }
 
 template <typename T>

@@ -11,6 +11,7 @@ namespace {
 template <typename T>
 __global__ void __launch_bounds__(256) combine_kernel(AttnParams p)
 {
+    pdl_begin();
     const int unit = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = blockIdx.y * 8 + warp;
@@ -49,10 +50,8 @@ __global__ void __launch_bounds__(256) combine_kernel(AttnParams p)
 cudaError_t launch_combine(const AttnParams &p, int dtype, cudaStream_t st)
 {
     dim3 grid(p.B * p.Hkv, (p.M + 7) / 8);
-    if (dtype == ORTHRUS_FP32) combine_kernel<float><<<grid, 256, 0, st>>>(p);
-    else combine_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(p);
-    count_launch();
-    return cudaGetLastError();
+    return dtype == ORTHRUS_FP32 ? launch_kernel(p.early, combine_kernel<float>, grid, 256, 0, st, p)
+                                 : launch_kernel(p.early, combine_kernel<__nv_bfloat16>, grid, 256, 0, st, p);
 }
 
 }  // namespace orthrus

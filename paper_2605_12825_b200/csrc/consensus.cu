@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const T *logits, in
                                                              ArgPart *parts)
 {
     constexpr int N = Vec<T>::N;
+    pdl_begin();
     const int row = blockIdx.y, seg = blockIdx.x;
     const int start = seg * seg_len;
     const int end = min(V, start + seg_len);
@@ -115,54 +116,18 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const T *logits, in
     }
 }
 
-// One CTA per sequence: thread i folds the segment partials of row i, then thread 0
-// walks the block left to right: drafts are kept while they equal the greedy token,
-// the first disagreeing position contributes the correction token, a fully agreeing
-// block commits K tokens.
-__global__ void consensus_finalize_kernel(const ArgPart *parts, int n_seg, const int32_t *draft,
-                                          int K, int32_t *n_commit, int32_t *committed,
-                                          int32_t *ar_argmax, int32_t *next_anchor)
-{
-    extern __shared__ int g[];
-    const int b = blockIdx.x;
-    for (int i = threadIdx.x; i < K; i += blockDim.x) {
-        const ArgPart *pp = parts + ((long long)b * K + i) * n_seg;
-        float bv = -INFINITY;
-        int bi = 0x7fffffff;
-        for (int s = 0; s < n_seg; ++s)
-            if (better(pp[s].v, pp[s].idx, bv, bi)) { bv = pp[s].v; bi = pp[s].idx; }
-        if (bi == 0x7fffffff) bi = 0;            // a row with no comparable value
-        g[i] = bi;
-        ar_argmax[(long long)b * K + i] = bi;
-    }
-    __syncthreads();
-    __shared__ int n_sh;
-    if (threadIdx.x == 0) {
-        int m = 0;
-        while (m < K && draft[(long long)b * K + m] == g[m]) ++m;
-        const int n = m + 1 < K ? m + 1 : K;
-        n_sh = n;
-        n_commit[b] = n;
-        next_anchor[b] = g[n - 1];
-    }
-    __syncthreads();
-    const int n = n_sh;
-    for (int i = threadIdx.x; i < K; i += blockDim.x)
-        committed[(long long)b * K + i] = i < n ? g[i] : -1;
-}
-
-// The same with many partials per row (one per vocabulary tile of the fused LM head): a warp
-// per row folds them, lanes striding over the tiles.
-__global__ void __launch_bounds__(256) consensus_finalize_wide_kernel(
+// One CTA per sequence: a warp per row folds the row's partials (one per segment of the streaming
+// argmax, or one per vocabulary tile of the fused LM head), lanes striding over them; then thread 0
+// walks the block left to right: drafts are kept while they equal the greedy token, the first
+// disagreeing position contributes the correction token, a fully agreeing block commits K tokens.
+__global__ void __launch_bounds__(1024) consensus_finalize_kernel(
         const ArgPart *parts, int n_seg, const int32_t *draft, int K, int32_t *n_commit,
         int32_t *committed, int32_t *ar_argmax, int32_t *next_anchor)
 {
     extern __shared__ int g[];
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // launched early (programmatic dependent launch): the pairs are complete once the kernel
-    // that writes them has finished
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = warp; i < K; i += 8) {
+    pdl_begin();
+    for (int i = warp; i < K; i += blockDim.x >> 5) {
         const ArgPart *pp = parts + ((long long)b * K + i) * n_seg;
         float bv = -INFINITY;
         int bi = 0x7fffffff;
@@ -197,26 +162,13 @@ __global__ void __launch_bounds__(256) consensus_finalize_wide_kernel(
 
 }  // namespace
 
-cudaError_t launch_consensus_finalize_wide(const ArgPart *parts, int n_seg, const int32_t *draft, int B,
-                                           int K, int32_t *n_commit, int32_t *committed,
-                                           int32_t *ar_argmax, int32_t *next_anchor, cudaStream_t st)
+cudaError_t launch_consensus_finalize(const ArgPart *parts, int n_seg, const int32_t *draft, int B,
+                                      int K, int32_t *n_commit, int32_t *committed,
+                                      int32_t *ar_argmax, int32_t *next_anchor, cudaStream_t st)
 {
-    // programmatic dependent launch: the CTAs are placed while the producer of `parts` is still
-    // running and wait for it on the device
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(B);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = K * sizeof(int);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, consensus_finalize_wide_kernel, parts, n_seg, draft, K, n_commit,
-                                       committed, ar_argmax, next_anchor);
-    count_launch();
-    return e;
+    const unsigned threads = K >= 32 ? 1024 : 32 * K;
+    return launch_kernel(true, consensus_finalize_kernel, dim3(B), threads, K * sizeof(int), st, parts, n_seg, draft, K,
+                         n_commit, committed, ar_argmax, next_anchor);
 }
 
 int consensus_segments(int B, int K, int V)
@@ -237,19 +189,13 @@ cudaError_t launch_consensus(const void *logits, int dtype, const int32_t *draft
     seg_len = (seg_len + 7) / 8 * 8;
     dim3 grid(n_seg, B * K);
     ArgPart *parts = static_cast<ArgPart *>(partials);
-    if (dtype == ORTHRUS_FP32)
-        argmax_partial_kernel<float><<<grid, 256, 0, st>>>(static_cast<const float *>(logits), V,
-                                                          seg_len, parts);
-    else
-        argmax_partial_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
-            static_cast<const __nv_bfloat16 *>(logits), V, seg_len, parts);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = dtype == ORTHRUS_FP32
+        ? launch_kernel(true, argmax_partial_kernel<float>, grid, 256, 0, st, static_cast<const float *>(logits), V,
+                        seg_len, parts)
+        : launch_kernel(true, argmax_partial_kernel<__nv_bfloat16>, grid, 256, 0, st,
+                        static_cast<const __nv_bfloat16 *>(logits), V, seg_len, parts);
     if (e != cudaSuccess) return e;
-    const int threads = K <= 32 ? 32 : ((K + 31) / 32 * 32 > 256 ? 256 : (K + 31) / 32 * 32);
-    consensus_finalize_kernel<<<B, threads, K * sizeof(int), st>>>(parts, n_seg, draft, K, n_commit,
-                                                                    committed, ar_argmax, next_anchor);
-    count_launch(2);
-    return cudaGetLastError();
+    return launch_consensus_finalize(parts, n_seg, draft, B, K, n_commit, committed, ar_argmax, next_anchor, st);
 }
 
 // ---------------------------------------------------------------- consensus without a workspace

@@ -11,6 +11,7 @@ __global__ void __launch_bounds__(256) kv_append_kernel(
     const int32_t *n_commit, int K, int Hkv, int row_vecs, long long capacity, int update_len,
     int32_t *status)
 {
+    pdl_begin();
     const int b = blockIdx.x;
     const int P = cache_len[b];
     const int n = n_commit[b];
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(128) kv_append_layers_kernel(
     const __grid_constant__ AppendBatch batch, const int32_t *n_commit, int K, int Hkv, int row_vecs,
     long long capacity, int32_t *status)
 {
+    pdl_begin();
     const int b = blockIdx.x, h = blockIdx.z;
     const AppendLayer &L = batch.layer[blockIdx.y];
     const int P = L.cache_len[b];
@@ -70,6 +72,7 @@ struct LenBatch { int32_t *len[128]; };
 __global__ void kv_append_bump_kernel(const __grid_constant__ LenBatch lens, int n_lens,
                                       const int32_t *n_commit, int B, int K, long long capacity)
 {
+    pdl_begin();
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * n_lens; e += gridDim.x * blockDim.x) {
         const int b = e % B;
         int32_t *len = lens.len[e / B];
@@ -91,10 +94,9 @@ cudaError_t launch_kv_append_layers(const orthrus_layer_t &shape, const AppendLa
         const int n = n_layers - l0 < kLayersPerLaunch ? n_layers - l0 : kLayersPerLaunch;
         for (int l = 0; l < n; ++l) batch.layer[l] = layers[l0 + l];
         for (int l = n; l < kLayersPerLaunch; ++l) batch.layer[l] = layers[l0];
-        kv_append_layers_kernel<<<dim3(shape.batch, n, shape.n_kv_heads), 128, 0, st>>>(
-            batch, n_commit, shape.block, shape.n_kv_heads, row_vecs, shape.capacity, status);
-        count_launch();
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_kernel(early_launch(shape), kv_append_layers_kernel, dim3(shape.batch, n, shape.n_kv_heads),
+                                      128, 0, st, batch, n_commit, shape.block, shape.n_kv_heads, row_vecs,
+                                      shape.capacity, status);
         if (e != cudaSuccess) return e;
     }
     if (n_len_arrays > 0) {
@@ -102,10 +104,8 @@ cudaError_t launch_kv_append_layers(const orthrus_layer_t &shape, const AppendLa
         for (int j = 0; j < 128; ++j) lb.len[j] = len_arrays[j < n_len_arrays ? j : 0];
         const int total = shape.batch * n_len_arrays;
         const int blocks = (total + 255) / 256 < 64 ? (total + 255) / 256 : 64;
-        kv_append_bump_kernel<<<blocks, 256, 0, st>>>(lb, n_len_arrays, n_commit, shape.batch, shape.block,
-                                                      shape.capacity);
-        count_launch();
-        return cudaGetLastError();
+        return launch_kernel(early_launch(shape), kv_append_bump_kernel, dim3(blocks), 256, 0, st, lb, n_len_arrays,
+                             n_commit, shape.batch, shape.block, shape.capacity);
     }
     return cudaSuccess;
 }
@@ -116,12 +116,10 @@ cudaError_t launch_kv_append(const orthrus_layer_t &L, const void *k_blk, const 
 {
     const int es = L.dtype == ORTHRUS_FP32 ? 4 : 2;
     const int row_vecs = L.head_dim * es / 16;
-    kv_append_kernel<<<L.batch, 256, 0, st>>>(
-        static_cast<uint4 *>(L.k_cache), static_cast<uint4 *>(L.v_cache), L.cache_len,
-        static_cast<const uint4 *>(k_blk), static_cast<const uint4 *>(v_blk), n_commit, L.block,
-        L.n_kv_heads, row_vecs, L.capacity, update_len, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(early_launch(L), kv_append_kernel, dim3(L.batch), 256, 0, st,
+                         static_cast<uint4 *>(L.k_cache), static_cast<uint4 *>(L.v_cache), L.cache_len,
+                         static_cast<const uint4 *>(k_blk), static_cast<const uint4 *>(v_blk), n_commit, L.block,
+                         L.n_kv_heads, row_vecs, L.capacity, update_len, status);
 }
 
 }  // namespace orthrus

@@ -137,7 +137,7 @@ lm_head_argmax_kernel(const __grid_constant__ HeadMaps tm, const int R, const in
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    griddep_launch();                         // the finalize kernel may be placed now; it waits for this grid
+    pdl_begin();                              // (the finalize kernel may be placed now; it waits for this grid)
 
     // accumulator and its use count for row half `a` of this CTA's item number `li`
     auto acc_of = [](int li, int a) { return MT == 1 ? (li & 1) : a; };
@@ -349,7 +349,7 @@ lm_head_argmax_pair_kernel(const __grid_constant__ HeadMaps tm, const int R, con
     cluster_sync_all();                       // the peer's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    griddep_launch();                         // the finalize kernel may be placed now; it waits for this grid
+    pdl_begin();                              // (the finalize kernel may be placed now; it waits for this grid)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer (both CTAs)
@@ -524,10 +524,8 @@ cudaError_t launch_shape(const HeadMaps &tm, int R, int V, int H, int bn, ArgPar
     const int n_m = (R + S::BM - 1) / S::BM, n_n = (V + bn - 1) / bn, n_k = (H + BK - 1) / BK;
     const long long n_items = (long long)n_m * n_n;
     const int grid = (int)(n_items < num_sms() ? n_items : num_sms());
-    lm_head_argmax_kernel<MT><<<grid, S::NTHREADS, S::SMEM_BYTES, st>>>(tm, R, V, n_k, n_m, n_n, bn, parts,
-                                                                       status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(true, lm_head_argmax_kernel<MT>, dim3(grid), S::NTHREADS, S::SMEM_BYTES, st, tm, R, V, n_k, n_m,
+                         n_n, bn, parts, status);
 }
 
 // Clusters of two CTAs of the pair kernel the current device can keep resident (0: not asked
@@ -570,10 +568,8 @@ cudaError_t launch_pair(const HeadMaps &tm, int R, int V, int H, int bn, int clu
     const int n_k = (H + pair::KPANELS * BK - 1) / (pair::KPANELS * BK);
     const long long n_items = (long long)n_m * n_n;
     const int n_cl = (int)(n_items < clusters ? n_items : clusters);
-    lm_head_argmax_pair_kernel<<<2 * n_cl, pair::NTHREADS, pair::SMEM_BYTES, st>>>(tm, R, V, n_k, n_m, n_n, bn,
-                                                                                  parts, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(true, lm_head_argmax_pair_kernel, dim3(2 * n_cl), pair::NTHREADS, pair::SMEM_BYTES, st, tm, R, V,
+                         n_k, n_m, n_n, bn, parts, status);
 }
 
 }  // namespace
