@@ -40,7 +40,7 @@ static int current_path()
 // search per variable: half a dozen searches were a tenth of a call's host time.
 struct Knobs {
     int splits = 0, min_chunk_tiles = 2, target_ctas = 0;     // 0: not forced / the default
-    bool no_early_launch = false, stream = false, pack = true;
+    bool no_early_launch = false, stream = false, pack = true, small_rows = true;
 };
 static Knobs read_knobs()
 {
@@ -61,6 +61,7 @@ static Knobs read_knobs()
         else if (is("TARGET_CTAS")) positive(k.target_ctas);
         else if (is("NO_EARLY_LAUNCH")) { positive(on); k.no_early_launch = on > 0; }
         else if (is("TC_SCHEDULE")) k.stream = !strcmp(val, "stream");
+        else if (is("TC_SMALL_ROWS")) k.small_rows = val[0] != '0';
         else if (is("MULTI_BLOCK_PACK")) k.pack = val[0] != '0';
     }
     return k;
@@ -198,6 +199,31 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
     return pl;
 }
 
+// Units of at most 64 query rows run with the keys on the MMA's rows (attend_keys.cu), head_dim 64
+// and 128.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the kernel for wide units (a measurement knob).
+static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
+{
+    const int M = L->n_q_heads / L->n_kv_heads * L->block;
+    if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || !keys_rows(M) || !kn.small_rows) return false;
+    const unsigned long long rows = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
+    return rows < 0x7fffffffull && (long long)L->batch * L->n_kv_heads <= 65535 && tc_driver_ok();
+}
+static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
+{
+    if (kn.splits > 0) return kn.splits < 16 ? kn.splits : 16;
+    // from prefix and block together: a decoder that bounds its lengths by capacity - block then cuts
+    // a block's verification and a width-1 step at the same keys, and both round alike
+    return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads * L->block, L->batch * L->n_kv_heads,
+                       max_len_of(L) + L->block);
+}
+static size_t keys_bytes(const orthrus_layer_t *L, int S, size_t *ml_off)
+{
+    const size_t ctas = S > 1 ? (size_t)L->batch * L->n_kv_heads * S : 0;
+    const size_t nr = keys_rows(L->n_q_heads / L->n_kv_heads * L->block);
+    if (ml_off) *ml_off = ctas * nr * L->head_dim * sizeof(float);
+    return ctas * nr * (L->head_dim + 2) * sizeof(float);
+}
+
 static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off, bool tc = false)
 {
     if (ml_off) *ml_off = 0;
@@ -235,7 +261,10 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     Plan pl = make_plan(L, tc, kn);
     if (stream_k) pl.n_splits = 1;
     size_t ml_off = 0;
+    const bool keys = !stream_k && (want == PATH_AUTO || (want == PATH_TCGEN05 && tc)) && keys_usable(L, kn);
+    if (keys) pl.n_splits = keys_plan(L, kn);
     const size_t need = kHeaderBytes + (stream_k ? tc_stream_workspace_bytes(L->batch, L->n_kv_heads, tc_stream_ctas())
+                                        : keys   ? keys_bytes(L, pl.n_splits, &ml_off)
                                                  : partial_bytes(L, pl, &ml_off, tc));
     if (ws_bytes < need) return ORTHRUS_ERR_WORKSPACE;
 
@@ -261,7 +290,11 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     bool merge_kernel = pl.n_splits > 1;
-    if (tc) {
+    if (keys) {
+        t_last_path = "tcgen05";
+        e = launch_attend_keys(p, flags, cs);
+        merge_kernel = false;
+    } else if (tc) {
         t_last_path = "tcgen05";
         if (stream_k) e = launch_attend_tc_stream(p, tc_stream_ctas(), base + kHeaderBytes, flags, cs);
         else e = launch_attend_tc(p, flags, cs);
@@ -293,6 +326,10 @@ size_t orthrus_attend_workspace_bytes(const orthrus_layer_t *layer)
     // enough for whichever kernel path a later call resolves to
     const Knobs kn = read_knobs();
     size_t need = partial_bytes(layer, make_plan(layer, false, kn), nullptr, false);
+    if (keys_usable(layer, kn)) {
+        const size_t n1 = keys_bytes(layer, keys_plan(layer, kn), nullptr);
+        if (n1 > need) need = n1;
+    }
     if (tc_usable(layer)) {
         const size_t n2 = partial_bytes(layer, make_plan(layer, true, kn), nullptr, true);
         if (n2 > need) need = n2;

@@ -17,8 +17,7 @@
 //              the MMAs consume them.
 //   warp 5     TMEM allocation and MMA issue: S = Q.K^T into one of two score buffers
 //              (so that QK(t+1) runs under softmax(t)), then O += P.V.
-// Units of at most 64 rows run a variant of this CTA (see the kernel's comment): probabilities
-// through shared memory, the two products issued by two warps.
+// (Units of at most 64 rows run on attend_keys.cu.)
 // The output accumulator O stays in TMEM for the whole CTA.  The running max is only
 // raised when a tile exceeds it by more than 2^8; then, and only then, the owner threads
 // rescale their O rows in TMEM.  Probabilities are bounded by 2^8, which fp32 sums and
@@ -89,10 +88,7 @@ template <int NT> struct Shape {
     static constexpr int BAR_PFULL = BAR_SFULL + 2 * NT;       // + ti * 2 + buffer
     static constexpr int BAR_PVDONE = BAR_PFULL + 2 * NT;      // + ti
     static constexpr int BAR_ALLDONE = BAR_PVDONE + NT;        // + ti
-    // small-row form of the narrow shape: "scores of buffer b read" and "P buffer b consumed"
-    static constexpr int BAR_SREAD = BAR_ALLDONE + NT;         // + buffer
-    static constexpr int BAR_PFREE = BAR_SREAD + 2;            // + buffer
-    static constexpr int BAR_DRAIN = BAR_PFREE + 2;            // + MMA warp: its MMAs retired, after a wait gave up
+    static constexpr int BAR_DRAIN = BAR_ALLDONE + NT;         // + MMA warp: its MMAs retired, after a wait gave up
     static constexpr int NUM_BARS = BAR_DRAIN + 2;
     static_assert(NUM_BARS <= MAX_BARS, "barrier area");
     // TMEM columns: the NT output accumulators, then two score buffers per query tile
@@ -162,7 +158,7 @@ __device__ inline void l2_merge_tasks(int S, int rank, int warp, int lane, int n
 // per lane) do not add to those of the streaming loop.  out_tile: the output row of the tile's
 // first block position and first head of the group; row R = i * G + g lies (i * Hq + g) rows on.
 template <int LOADS>
-__device__ __forceinline__ void merge_tile_body(int S, int rank, int warp, int lane, int n_warps, int rows_here,
+__device__ __noinline__ void merge_tile(int S, int rank, int warp, int lane, int n_warps, int rows_here,
                                                 const float4 *grp_o, const float2 *grp_ml, __nv_bfloat16 *out_tile,
                                                 int G, int Hq)
 {
@@ -180,13 +176,6 @@ __device__ __forceinline__ void merge_tile_body(int S, int rank, int warp, int l
     else if (S <= 8) run(std::integral_constant<int, 8>());
     else run(std::integral_constant<int, 16>());
 }
-template <int LOADS>
-__device__ __noinline__ void merge_tile(int S, int rank, int warp, int lane, int n_warps, int rows_here,
-                                        const float4 *grp_o, const float2 *grp_ml, __nv_bfloat16 *out_tile,
-                                        int G, int Hq)
-{
-    merge_tile_body<LOADS>(S, rank, warp, lane, n_warps, rows_here, grp_o, grp_ml, out_tile, G, Hq);
-}
 
 // Thread r of a softmax warpgroup owns query row r of its tile (TMEM lane r) and all 64 columns of
 // a key tile.  blockIdx.z counts groups of NT query tiles; warpgroup ti works on tile z * NT + ti.
@@ -197,23 +186,14 @@ __device__ __noinline__ void merge_tile(int S, int rank, int warp, int lane, int
 // j = i / kb_width, sees the prefix below its own anchor cache_len[b * nb + j] and the keys of its
 // own block only; the CTA streams up to the largest anchor among the blocks of its query tile,
 // then the 64-key tiles of the block axis that hold those blocks' keys.
-//
-// SM (at most 64 query rows, narrow shape, not packed): the chain score tile -> softmax -> P.V ->
-// next score tile is what a short chunk waits for, and an issuing thread is held about 110 cycles
-// per tcgen05.mma.  Here the probabilities go to shared memory (the unused upper halves of the
-// query tile's two sub-tiles) instead of back into the score buffer, so a score buffer is free
-// again as soon as its softmax threads have read it, and the two products are issued by two
-// warps.  256 threads: warps 0-3 softmax (200 registers after setmaxnreg), 4 producer, 5 Q.K^T,
-// 6 P.V, 7 idle (56 registers).
-template <int NT, bool PACK, bool SM>
-__global__ void __launch_bounds__(SM ? 256 : Shape<NT>::NTHREADS, NT == 1 ? 2 : 1)
+template <int NT, bool PACK>
+__global__ void __launch_bounds__(Shape<NT>::NTHREADS, NT == 1 ? 2 : 1)
 attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const int S, const int kb_rows,
                  const int quiescent)
 {
     using C = Shape<NT>;
     constexpr int W = TN;                     // score columns per softmax thread
-    static_assert(!SM || (NT == 1 && !PACK), "the small-row form is a variant of the plain narrow shape");
-    constexpr int NSLOT = C::NSLOT, NTHREADS = SM ? 256 : C::NTHREADS;
+    constexpr int NSLOT = C::NSLOT, NTHREADS = C::NTHREADS;
     constexpr int OFF_Q = C::OFF_Q, OFF_RING = C::OFF_RING, OFF_BAR = C::OFF_BAR, OFF_MISC = C::OFF_MISC;
     constexpr int BAR_FULL = C::BAR_FULL, BAR_EMPTY = C::BAR_EMPTY, BAR_QFULL = C::BAR_QFULL;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -253,11 +233,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             }
             mbar_init(bar(C::BAR_PVDONE + ti), 1);
             mbar_init(bar(C::BAR_ALLDONE + ti), 1);
-            if constexpr (SM)
-                for (int sb = 0; sb < 2; ++sb) {
-                    mbar_init(bar(C::BAR_SREAD + sb), n_act);
-                    mbar_init(bar(C::BAR_PFREE + sb), 1);
-                }
         }
         mbar_init(bar(C::BAR_DRAIN), 1);
         mbar_init(bar(C::BAR_DRAIN + 1), 1);
@@ -335,19 +310,13 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     // The ring holds K and V tiles in the order the MMAs consume them: K0, K1, V0, K2, V1, ...,
     // K(n-1), V(n-2), V(n-1) (the product P.V of a tile is issued after the scores of the next
     // one), so that slots are freed in the order they were filled and a V tile does not sit
-    // in the ring while its softmax is still to come.  Item j lives in slot j % NSLOT, except in the
-    // small-row form: there two warps consume the tiles, each waiting for its own kind only, so a
-    // slot holds tiles of one kind (K tile t in slot t % 3, V tile t in slot 3 + t % 2).  With
-    // mixed slots a warp skips the phases of the other's tiles, and a parity wait that is two
-    // phases ahead of its barrier succeeds at once: the QK^T warp could take a slot whose V tile
-    // had not even landed.
+    // in the ring while its softmax is still to come.  Item j lives in slot j % NSLOT.
     auto item_of_k = [&](int t) { return t == 0 ? 0 : 2 * t - 1; };
     auto item_of_v = [&](int t) { return min(2 * t + 2, 2 * n_tiles - 1); };
     auto v_item = [&](int j) { return j == 2 * n_tiles - 1 || (j > 0 && (j & 1) == 0); };
     auto tile_of = [&](int j) { return v_item(j) ? (j == 2 * n_tiles - 1 ? n_tiles - 1 : j / 2 - 1) : (j + 1) / 2; };
-    static_assert(!SM || NSLOT == 5, "three K slots, two V slots");
-    auto slot_of = [&](int j) { return !SM ? j % NSLOT : (v_item(j) ? 3 + tile_of(j) % 2 : tile_of(j) % 3); };
-    auto use_of = [&](int j) { return !SM ? j / NSLOT : (v_item(j) ? tile_of(j) / 2 : tile_of(j) / 3); };
+    auto slot_of = [&](int j) { return j % NSLOT; };
+    auto use_of = [&](int j) { return j / NSLOT; };
     const uint64_t stream_policy = policy_evict_first();
     auto issue_item = [&](int j) {
         const int slot = slot_of(j);
@@ -390,11 +359,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     }
     griddep_launch();
 
-    if constexpr (SM) {
-        // the softmax warps take the registers the other four warps do not need
-        if (warp < 4) asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    }
     if (warp < 4 * NT) {
         const int ti = warp >> 2, wq = warp & 3;              // query tile, quarter of its TMEM lanes
         const int r = tid - ti * MROWS;
@@ -429,11 +393,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
 #pragma unroll
                 for (int c = 0; c < W / 32; ++c) tmem_ld32(lane_base + TM_S + c * 32, s + c * 32);
                 tmem_ld_wait();
-                if constexpr (SM) {                            // the buffer may take the scores of tile t + 2
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(C::BAR_SREAD + sb));
-                }
                 // visible columns of this row in this tile: [lo, lim)
                 int lim, lo = 0;
                 if constexpr (PACK) {
@@ -477,14 +436,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                 }
                 const float m_new = fmaxf(m_run, mx * sc);
                 const bool need = m_new > m_run + RESCALE_THRESHOLD;   // also the first finite maximum
-                if constexpr (SM) {
-                    // the product of tile t - 2 has read P buffer sb (and with it BAR_PVDONE is at
-                    // most one phase behind tile t - 1, which is what a parity wait can tell)
-                    if (t >= 2) {
-                        ok = mbar_wait_warp(bar(C::BAR_PFREE + sb), ((t >> 1) - 1) & 1, abort_flag);
-                        if (!ok) break;
-                    }
-                }
                 if (__any_sync(0xffffffffu, need)) {
                     const float alpha = need ? ex2(m_run - m_new) : 1.f;
                     if (need) { m_run = m_new; l_run *= alpha; }
@@ -539,20 +490,10 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                     }
                 }
                 l_run += (acc0.x + acc0.y) + (acc1.x + acc1.y);
-                if constexpr (SM) {
-                    // P row r into shared memory buffer sb ([64 rows][64 keys] bf16, 128-byte swizzle)
-                    unsigned char *prow = smem + OFF_Q + (sb ? 3 : 1) * (QSUB_BYTES / 2) + r * 128;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        *reinterpret_cast<uint4 *>(prow + ((c ^ (r & 7)) << 4)) =
-                            make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
-                    fence_proxy_async();
-                } else {
-                    // P over the scores, 2 bf16 per 32-bit column
-                    tmem_st32(lane_base + TM_S, pk);
-                    tmem_st_wait();
-                    tc_fence_before();
-                }
+                // P over the scores, 2 bf16 per 32-bit column
+                tmem_st32(lane_base + TM_S, pk);
+                tmem_st_wait();
+                tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(C::BAR_PFULL + ti * 2 + sb));
             }
@@ -598,7 +539,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             if (have_o) {
                 // the narrow shape reads the whole row out at once (one wait instead of four), the
                 // wide one, with fewer registers per thread, in two halves; 16-byte stores follow
-                constexpr int PIECE = (NT == 1 && !SM) ? HD : HD / 2;
+                constexpr int PIECE = NT == 1 ? HD : HD / 2;
 #pragma unroll 1
                 for (int c0 = 0; c0 < HD; c0 += PIECE) {
                     uint32_t o[PIECE];
@@ -618,22 +559,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             if (valid) __stcg(my_ml + r, make_float2(have_o ? m_run : -INFINITY, have_o ? l_run : 0.f));
         }
         tc_fence_before();
-        if constexpr (SM) {
-            // These warps hold the registers the merge wants, so they finish the unit here: the
-            // CTA-wide barrier the other warps take below (after it the TMEM is freed), then the
-            // cluster barrier and this CTA's share of the merge.
-            asm volatile("bar.sync 0;" ::: "memory");
-            if (S == 1) return;
-            cluster_sync_all();
-            const int rows_here0 = tile_rows(0);
-            __nv_bfloat16 *out_tile = static_cast<__nv_bfloat16 *>(p.out) +
-                                      (((long long)b * p.K + tile_i0(0)) * p.Hq + h * p.G) * HD;
-            const long long grp_lin = ((long long)blockIdx.z * gridDim.y + order) * S;
-            merge_tile_body<16>(S, rank, warp, lane, 4, rows_here0,
-                                reinterpret_cast<const float4 *>(p.part_o + grp_lin * (MROWS * HD)),
-                                reinterpret_cast<const float2 *>(p.part_ml + grp_lin * (MROWS * 2)), out_tile, p.G, p.Hq);
-            return;
-        }
     } else if (warp == C::PRODUCER_WARP) {
         // ------------------------------------------------------------------ producer
         if (active && lane == 0) {
@@ -666,9 +591,9 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                 mbar_wait(bar(BAR_QFULL), 0, &dummy);
             }
         }
-    } else if (active && (SM ? warp <= C::MMA_WARP + 1 : tile_rows(warp - C::MMA_WARP) > 0)) {
+    } else if (active && tile_rows(warp - C::MMA_WARP) > 0) {
         // ------------------------------------------------------------------ MMA issue, query tile ti
-        const int ti = SM ? 0 : warp - C::MMA_WARP;
+        const int ti = warp - C::MMA_WARP;
         constexpr uint32_t IDESC_QK = make_idesc(TN, 0);      // A = Q, B = K tile, both K-major
         constexpr uint32_t IDESC_PV = make_idesc(HD, 1);      // A = P (TMEM), B = V tile (MN-major)
         const uint32_t q_addr = sbase + OFF_Q + ti * 2 * QSUB_BYTES;
@@ -719,47 +644,22 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
 #pragma unroll
                 for (int kk = 0; kk < TN / 16; ++kk) {        // 16 key positions per MMA
                     if (kk >= n_kk) break;
-                    if constexpr (SM)
-                        umma_ss(tmem + C::tm_o(ti),
-                                make_desc(sbase + OFF_Q + ((t & 1) ? 3 : 1) * (QSUB_BYTES / 2) + kk * 32, 16, 1024),
-                                make_desc(v_addr + kk * 2048, SUB_BYTES, 1024), IDESC_PV, (t > 0) || (kk > 0));
-                    else
-                        umma_ts(tmem + C::tm_o(ti), tmem + C::tm_s(ti, t & 1) + kk * 8,
-                                make_desc(v_addr + kk * 2048, SUB_BYTES, 1024), IDESC_PV, (t > 0) || (kk > 0));
+                    umma_ts(tmem + C::tm_o(ti), tmem + C::tm_s(ti, t & 1) + kk * 8,
+                            make_desc(v_addr + kk * 2048, SUB_BYTES, 1024), IDESC_PV, (t > 0) || (kk > 0));
                 }
                 umma_commit(bar(BAR_EMPTY + slot));
                 umma_commit(bar(C::BAR_PVDONE + ti));
-                if constexpr (SM) umma_commit(bar(C::BAR_PFREE + (t & 1)));
                 if (t == n_tiles - 1) umma_commit(bar(C::BAR_ALLDONE + ti));
             }
             __syncwarp();
             return true;
         };
         bool ok = true;
-        if constexpr (SM) {
-            if (warp == C::MMA_WARP) {
-                // scores of tile t go into buffer t & 1 once the softmax threads of tile t - 2 have
-                // read theirs out of it (one completion of that barrier per use of the buffer, so
-                // the waiter is never more than one phase behind)
-                ok = mbar_wait_warp(bar(BAR_QFULL), 0, abort_flag);
-                if (ok) tc_fence_after();
-                for (int t = 0; t < n_tiles && ok; ++t) {
-                    if (t >= 2) {
-                        ok = mbar_wait_warp(bar(C::BAR_SREAD + (t & 1)), ((t >> 1) - 1) & 1, abort_flag);
-                        if (ok) tc_fence_after();
-                    }
-                    if (ok) ok = issue_qk(t);
-                }
-            } else {
-                for (int t = 0; t < n_tiles && ok; ++t) ok = issue_pv(t);
-            }
-        } else {
-            ok = mbar_wait_warp(bar(BAR_QFULL), 0, abort_flag);
-            if (ok) { tc_fence_after(); ok = issue_qk(0); }
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                if (t + 1 < n_tiles) ok = issue_qk(t + 1);
-                if (ok) ok = issue_pv(t);
-            }
+        ok = mbar_wait_warp(bar(BAR_QFULL), 0, abort_flag);
+        if (ok) { tc_fence_after(); ok = issue_qk(0); }
+        for (int t = 0; t < n_tiles && ok; ++t) {
+            if (t + 1 < n_tiles) ok = issue_qk(t + 1);
+            if (ok) ok = issue_pv(t);
         }
         // every MMA of this warp must have retired before TMEM is freed
         if (ok) ok = mbar_wait_warp(bar(C::BAR_ALLDONE + ti), 0, abort_flag);
@@ -779,23 +679,21 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     tc_fence_after();
     if (warp == C::MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TM_COLS) : "memory");
-    if (tid == (SM ? 128 : 0) && *abort_flag && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
+    if (tid == 0 && *abort_flag && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
     if (S == 1) return;
     constexpr int NWARPS = NTHREADS / 32;
     // The cluster is what guarantees that the CTAs waiting for one another are resident
     // together.  Release / acquire at cluster scope: every CTA's partial rows are in place.
     cluster_sync_all();
-    if constexpr (!SM) {                  // (in the small-row form the softmax warps merge; they never come here)
-        for (int ti = 0; ti < NT; ++ti) {
-            const int rows_here = tile_rows(ti);
-            if (rows_here == 0) break;
-            __nv_bfloat16 *out_tile = static_cast<__nv_bfloat16 *>(p.out) +
-                                      (((long long)b * p.K + tile_i0(ti)) * p.Hq + h * p.G) * HD;
-            const long long grp_lin = (((long long)blockIdx.z * NT + ti) * gridDim.y + order) * S;
-            merge_tile<NT == 1 ? 16 : 8>(S, rank, warp, lane, NWARPS, rows_here,
-                       reinterpret_cast<const float4 *>(p.part_o + grp_lin * (MROWS * HD)),
-                       reinterpret_cast<const float2 *>(p.part_ml + grp_lin * (MROWS * 2)), out_tile, p.G, p.Hq);
-        }
+    for (int ti = 0; ti < NT; ++ti) {
+        const int rows_here = tile_rows(ti);
+        if (rows_here == 0) break;
+        __nv_bfloat16 *out_tile = static_cast<__nv_bfloat16 *>(p.out) +
+                                  (((long long)b * p.K + tile_i0(ti)) * p.Hq + h * p.G) * HD;
+        const long long grp_lin = (((long long)blockIdx.z * NT + ti) * gridDim.y + order) * S;
+        merge_tile<NT == 1 ? 16 : 8>(S, rank, warp, lane, NWARPS, rows_here,
+                   reinterpret_cast<const float4 *>(p.part_o + grp_lin * (MROWS * HD)),
+                   reinterpret_cast<const float2 *>(p.part_ml + grp_lin * (MROWS * 2)), out_tile, p.G, p.Hq);
     }
 }
 
@@ -821,39 +719,41 @@ EncodeTiledFn encode_fn()
 
 namespace {
 
-// Tensor maps over bf16 tensors whose innermost dimension is the 128-wide head: up to four
-// dimensions, boxes of 64 columns with the 128-byte swizzle.  Cached by (pointer, shape).
+// Tensor maps over bf16 tensors whose innermost dimension is the head (hd = 64 or 128 wide): up to
+// four dimensions, boxes of 64 columns with the 128-byte swizzle.  Cached by (pointer, shape).
 struct MapKey {
-    const void *ptr; unsigned long long d1, d2, d3; unsigned b1, b2;
+    const void *ptr; unsigned long long d1, d2, d3; unsigned b1, b2, hd;
     bool operator==(const MapKey &o) const {
-        return ptr == o.ptr && d1 == o.d1 && d2 == o.d2 && d3 == o.d3 && b1 == o.b1 && b2 == o.b2;
+        return ptr == o.ptr && hd == o.hd && d1 == o.d1 && d2 == o.d2 && d3 == o.d3 && b1 == o.b1 && b2 == o.b2;
     }
 };
 struct MapKeyHash {
     size_t operator()(const MapKey &k) const {
         size_t x = std::hash<const void *>()(k.ptr);
-        for (unsigned long long v : {k.d1, k.d2, k.d3, (unsigned long long)k.b1, (unsigned long long)k.b2})
+        for (unsigned long long v : {k.d1, k.d2, k.d3, (unsigned long long)k.b1 << 32 | k.b2, (unsigned long long)k.hd})
             x = (x ^ v) * 0x9E3779B97F4A7C15ull;
         return x;
     }
 };
 
-// dims: (128, d1, d2, d3) row-major with d3 outermost; box (64, b1, b2, 1).  rank = 2 when
+}  // namespace
+
+// dims: (hd, d1, d2, d3) row-major with d3 outermost; box (64, b1, b2, 1).  rank = 2 when
 // d2 == 0 (then the box is (64, b1)).
-bool get_map(const void *ptr, unsigned long long d1, unsigned long long d2, unsigned long long d3,
+bool tensor_map(const void *ptr, unsigned hd, unsigned long long d1, unsigned long long d2, unsigned long long d3,
              unsigned b1, unsigned b2, CUtensorMap *out)
 {
     static std::mutex mu;
     static std::unordered_map<MapKey, CUtensorMap, MapKeyHash> cache;
     std::lock_guard<std::mutex> lock(mu);
-    const MapKey key{ptr, d1, d2, d3, b1, b2};
+    const MapKey key{ptr, d1, d2, d3, b1, b2, hd};
     auto it = cache.find(key);
     if (it != cache.end()) { *out = it->second; return true; }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const int rank = d2 == 0 ? 2 : 4;
-    const cuuint64_t dims[4] = {(cuuint64_t)HD, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)d3};
-    const cuuint64_t strides[3] = {(cuuint64_t)HD * 2, (cuuint64_t)HD * 2 * d1, (cuuint64_t)HD * 2 * d1 * d2};
+    const cuuint64_t dims[4] = {(cuuint64_t)hd, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)d3};
+    const cuuint64_t strides[3] = {(cuuint64_t)hd * 2, (cuuint64_t)hd * 2 * d1, (cuuint64_t)hd * 2 * d1 * d2};
     const cuuint32_t box[4] = {64, b1, b2, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUtensorMap tm;
@@ -867,8 +767,6 @@ bool get_map(const void *ptr, unsigned long long d1, unsigned long long d2, unsi
     *out = tm;
     return true;
 }
-
-}  // namespace
 
 // block positions per query tile of 128 rows
 static int tc_kb_rows(int G, int K) { return K < MROWS / G ? K : MROWS / G; }
@@ -928,7 +826,7 @@ int tc_ctas_per_sm(int nt)
 
 namespace {
 
-template <int NT, bool PACK = false, bool SM = false>
+template <int NT, bool PACK = false>
 cudaError_t configure_kernel()
 {   // function attributes belong to a device: set them once on each device that launches
     constexpr int kMaxDevices = 64;
@@ -940,9 +838,9 @@ cudaError_t configure_kernel()
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!configured[dev]) {
-        e = cudaFuncSetAttribute(attend_tc_kernel<NT, PACK, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<NT>::SMEM_BYTES);
+        e = cudaFuncSetAttribute(attend_tc_kernel<NT, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<NT>::SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(attend_tc_kernel<NT, PACK, SM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(attend_tc_kernel<NT, PACK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
@@ -971,7 +869,7 @@ int max_cluster_of_shape()
             attr[0].val.clusterDim.x = s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr; cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, attend_tc_kernel<NT, false, false>, &cfg) == cudaSuccess && n > 0) { best = s; break; }
+            if (cudaOccupancyMaxActiveClusters(&n, attend_tc_kernel<NT, false>, &cfg) == cudaSuccess && n > 0) { best = s; break; }
             best = s >> 1;
         }
         if (best < 1) best = 1;
@@ -990,16 +888,16 @@ int max_cluster_of_shape()
 int tc_max_cluster(int nt) { return nt == 2 ? max_cluster_of_shape<2>() : max_cluster_of_shape<1>(); }
 int tc_tile_positions() { return TN; }
 
-template <int NT, bool PACK = false, bool SM = false>
+template <int NT, bool PACK = false>
 static cudaError_t launch_tc(const AttnParams &p, const TcMaps &tm, int kb, int flags, cudaStream_t st)
 {
     const int S = p.n_splits;
-    cudaError_t e = configure_kernel<NT, PACK, SM>();
+    cudaError_t e = configure_kernel<NT, PACK>();
     if (e != cudaSuccess) return e;
     const int row_tiles = (p.K + kb - 1) / kb;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, p.B * p.Hkv, (row_tiles + NT - 1) / NT);
-    cfg.blockDim = dim3(SM ? 256 : Shape<NT>::NTHREADS);
+    cfg.blockDim = dim3(Shape<NT>::NTHREADS);
     cfg.dynamicSmemBytes = Shape<NT>::SMEM_BYTES;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -1018,7 +916,7 @@ static cudaError_t launch_tc(const AttnParams &p, const TcMaps &tm, int kb, int 
     }
     cfg.attrs = attr;
     cfg.numAttrs = n_attr;
-    e = cudaLaunchKernelEx(&cfg, attend_tc_kernel<NT, PACK, SM>, p, tm, S, kb, (flags & ORTHRUS_LAYER_CACHE_QUIESCENT) ? 1 : 0);
+    e = cudaLaunchKernelEx(&cfg, attend_tc_kernel<NT, PACK>, p, tm, S, kb, (flags & ORTHRUS_LAYER_CACHE_QUIESCENT) ? 1 : 0);
     count_launch();
     return e;
 }
@@ -1038,12 +936,12 @@ cudaError_t launch_attend_tc_stream(const AttnParams &p, int n_ctas, void *ws_bo
 {
     TcMaps tm;
     const unsigned long long rows = (unsigned long long)(p.B / p.nb) * p.Hkv * p.capacity;
-    if (!get_map(p.k_cache, rows, 0, 0, TN, 0, &tm.k) || !get_map(p.v_cache, rows, 0, 0, TN, 0, &tm.v) ||
-        !get_map(p.q, p.Hq, p.K, p.B, p.G, p.K, &tm.q))
+    if (!tensor_map(p.k_cache, HD, rows, 0, 0, TN, 0, &tm.k) || !tensor_map(p.v_cache, HD, rows, 0, 0, TN, 0, &tm.v) ||
+        !tensor_map(p.q, HD, p.Hq, p.K, p.B, p.G, p.K, &tm.q))
         return cudaErrorInvalidValue;
     if (p.blk_in_cache) {
         tm.kb = tm.k; tm.vb = tm.v;
-    } else if (!get_map(p.k_blk, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !get_map(p.v_blk, p.Hkv, p.K, p.B, 1, TN, &tm.vb)) {
+    } else if (!tensor_map(p.k_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !tensor_map(p.v_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.vb)) {
         return cudaErrorInvalidValue;
     }
     {   // function attributes belong to a device: set them once on each device that launches
@@ -1090,19 +988,15 @@ cudaError_t launch_attend_tc(const AttnParams &p, int flags, cudaStream_t st)
     const int kb = tc_kb_rows(p.G, p.K);
     TcMaps tm;
     const unsigned long long rows = (unsigned long long)(p.B / p.nb) * p.Hkv * p.capacity;
-    if (!get_map(p.k_cache, rows, 0, 0, TN, 0, &tm.k) || !get_map(p.v_cache, rows, 0, 0, TN, 0, &tm.v) ||
-        !get_map(p.q, p.Hq, p.K, p.B, p.G, kb, &tm.q))
+    if (!tensor_map(p.k_cache, HD, rows, 0, 0, TN, 0, &tm.k) || !tensor_map(p.v_cache, HD, rows, 0, 0, TN, 0, &tm.v) ||
+        !tensor_map(p.q, HD, p.Hq, p.K, p.B, p.G, kb, &tm.q))
         return cudaErrorInvalidValue;
     if (p.blk_in_cache) {
         tm.kb = tm.k; tm.vb = tm.v;           // unused: the block tile comes through the cache maps
-    } else if (!get_map(p.k_blk, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !get_map(p.v_blk, p.Hkv, p.K, p.B, 1, TN, &tm.vb)) {
+    } else if (!tensor_map(p.k_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !tensor_map(p.v_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.vb)) {
         return cudaErrorInvalidValue;
     }
     if (tc_tiles_per_cta(p.G, p.K) == 2) return launch_tc<2>(p, tm, kb, flags, st);
-    // at most 64 query rows: the form with the probabilities in shared memory and two issuing warps
-    // (ORTHRUS_TC_SMALL_ROWS=0 keeps the common form: a measurement knob)
-    static const bool small_rows = [] { const char *e = getenv("ORTHRUS_TC_SMALL_ROWS"); return !(e && e[0] == '0'); }();
-    if (small_rows && p.G * p.K <= MROWS / 2) return launch_tc<1, false, true>(p, tm, kb, flags, st);
     return launch_tc<1>(p, tm, kb, flags, st);
 }
 
@@ -1113,9 +1007,9 @@ cudaError_t launch_attend_tc_packed(const AttnParams &p, int flags, cudaStream_t
     const int kb = tc_kb_rows(p.G, p.K);
     TcMaps tm;
     const unsigned long long rows = (unsigned long long)p.B * p.Hkv * p.capacity;
-    if (!get_map(p.k_cache, rows, 0, 0, TN, 0, &tm.k) || !get_map(p.v_cache, rows, 0, 0, TN, 0, &tm.v) ||
-        !get_map(p.q, p.Hq, p.K, p.B, p.G, kb, &tm.q) ||
-        !get_map(p.k_blk, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !get_map(p.v_blk, p.Hkv, p.K, p.B, 1, TN, &tm.vb))
+    if (!tensor_map(p.k_cache, HD, rows, 0, 0, TN, 0, &tm.k) || !tensor_map(p.v_cache, HD, rows, 0, 0, TN, 0, &tm.v) ||
+        !tensor_map(p.q, HD, p.Hq, p.K, p.B, p.G, kb, &tm.q) ||
+        !tensor_map(p.k_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.kb) || !tensor_map(p.v_blk, HD, p.Hkv, p.K, p.B, 1, TN, &tm.vb))
         return cudaErrorInvalidValue;
     return launch_tc<1, true>(p, tm, kb, flags, st);
 }

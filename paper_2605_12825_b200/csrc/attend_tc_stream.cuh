@@ -33,8 +33,8 @@
 // unit, at most 128 batch entries (their lengths are ranked in shared memory).
 
 constexpr int STREAM_MAX_B = 128;
-// two more barriers of the persistent kernel, in the place of two that only the small-row form has
-constexpr int SBAR_QFREE = Shape<1>::BAR_SREAD, SBAR_OFREE = SBAR_QFREE + 1, SBAR_NUM = Shape<1>::NUM_BARS;
+// extra barriers of the persistent kernel, behind those of Shape<1>
+constexpr int SBAR_QFREE = Shape<1>::NUM_BARS, SBAR_OFREE = SBAR_QFREE + 1, SBAR_NUM = SBAR_OFREE + 1;
 static_assert(SBAR_NUM <= 24, "the barrier area's last 128 bytes hold the ranking");
 // Two CTAs per SM leave 640 bytes beside Shape<1>'s map: the ranked sequences go into the unused
 // end of the barrier area, the flag into the spare words next to the TMEM address, the tile

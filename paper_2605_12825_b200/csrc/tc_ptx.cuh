@@ -186,5 +186,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_fn();
+bool tensor_map(const void *ptr, unsigned hd, unsigned long long d1, unsigned long long d2, unsigned long long d3,
+                unsigned b1, unsigned b2, CUtensorMap *out);
 
 }  // namespace orthrus
