@@ -3,34 +3,33 @@
 // With p = softmax(ar_logits / T) and q = softmax(diff_logits / T) per block position, the
 // drafts are visited left to right; draft y_k is kept iff u_accept * q_k(y_k) <= p_k(y_k);
 // the first position that fails gets a correction token drawn from max(0, p_k - q_k) by
-// inverting its running sum with u_resample.  Four kernels, all streaming:
-//   1. sample_stats      grid (segments, rows): one online pass over BOTH logit rows
-//                        giving, per segment, an integer reference at or above the maximum
-//                        and the sum of exponentials relative to it (16-byte loads, exp2 with the 1/T and
-//                        log2(e) factors folded into one multiply);
-//   2. sample_decide     one CTA per sequence: folds the segments (in order), evaluates
-//                        the K accept tests, finds the first failure;
-//   3. sample_residual   grid (segments, sequences): for the failing row only, the
-//                        per-segment sums of max(0, p - q) and of p;
-//   4. sample_pick       one CTA per sequence: walks the segment sums in order to the
-//                        segment that contains u * total, then scans that segment.
+// inverting its running sum with u_resample.  Two kernels (three for large problems):
+//   sample_stats   a warp per (row, stretch of the vocabulary): one online pass over BOTH logit rows
+//                  giving an integer reference at or above the maximum and the sum of exponentials
+//                  relative to it (16-byte loads, eight in flight per lane; 1/T and log2(e) folded into
+//                  one multiply).  Bound by the loads and, close behind, by the exponentials.
+//   sample_finish  a cluster of CTAs per sequence: folds the stretches, takes the accept tests, sums
+//                  the residual of the first rejected row (a share of the vocabulary per CTA, exchanged
+//                  through distributed shared memory), and the CTA whose share holds the drawn point
+//                  finds the token by block scans.
+// Verification halts at the first rejected draft, so rows behind it are not needed.  When the logits
+// are many times what the GPU holds in flight, the statistics pass takes the rows of all sequences in
+// the order of their block position; whoever completes a row takes its accept test and lowers the
+// sequence's first failure, and stretches behind a known failure are skipped.  Nobody waits: a row
+// that is read in vain costs time only, and the result is the smallest failing row either way.  (With
+// one statistics pass over a quarter of the block, a second one over the rest for the sequences still
+// open, and serial folds, the two configurations named in the benchmark took 124 and 41 us.)
 // Exponentials are fp32; every sum is carried in double and taken in a fixed order, and
 // references are integers so that rescaling is exact: the result is reproducible run to run
 // and departs from an exact evaluation only by the rounding of the individual exponentials.
-#include <cstdlib>
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace orthrus {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kPickSegMax = 4096;       // elements one CTA scans in sample_pick: 256 threads x 16
-
-__device__ inline float ex2f(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
+constexpr int kThreads = 256, kWarps = kThreads / 32;
+constexpr int kStretch = 4096;          // logits of a row a warp takes at a time (about), where there are plenty
 
 template <typename T> struct Elem;
 template <> struct Elem<__nv_bfloat16> {
@@ -69,303 +68,427 @@ __device__ inline RefSum combine(const RefSum &a, const RefSum &b) {
     const float M = fmaxf(a.m, b.m);
     return RefSum{M, a.s * (double)pow2i(a.m - M) + b.s * (double)pow2i(b.m - M)};
 }
-template <int N>
-__device__ inline void absorb_vec(RefSum &a, const float (&x)[N], float c) {
-    float y[N], mx = -INFINITY;
+// R x N raw logits; c > 0 scales them into the log2 domain.  The instruction count matters (the loop
+// is bound by the exponentials only while the rest stays below them): the maximum is taken over the
+// raw values, once for all R vectors (some lane of a warp raises its reference at nearly every check),
+// scaling and reference are one fused multiply-add, and the sum of a vector enters in double.
+template <int R, int N>
+__device__ inline void absorb(RefSum &a, const float (&x)[R][N], float c) {
+    float mx[R];
 #pragma unroll
-    for (int e = 0; e < N; ++e) { y[e] = x[e] * c; mx = fmaxf(mx, y[e]); }
-    if (mx == -INFINITY) return;
-    if (mx > a.m) {
-        const float m_new = ceilf(mx);
+    for (int q = 0; q < R; ++q) {
+        mx[q] = fmaxf(x[q][0], x[q][1]);
+#pragma unroll
+        for (int e = 2; e < N; e += 2) mx[q] = max3(mx[q], x[q][e], x[q][e + 1]);
+    }
+#pragma unroll
+    for (int q = 1; q < R; ++q) mx[0] = fmaxf(mx[0], mx[q]);
+    mx[0] *= c;
+    if (mx[0] > a.m) {
+        const float m_new = ceilf(mx[0]);
         if (a.m > -INFINITY) a.s *= (double)pow2i(a.m - m_new);
         a.m = m_new;
     }
-    float s = 0.f;
+    if (a.m == -INFINITY) return;
+    const float2 c2 = make_float2(c, c), m2 = make_float2(-a.m, -a.m);
+    float sum[R];
 #pragma unroll
-    for (int e = 0; e < N; ++e) s += ex2f(y[e] - a.m);
-    a.s += (double)s;
-}
-__device__ inline void absorb(RefSum &a, float x) {
-    const float v[1] = {x};
-    absorb_vec<1>(a, v, 1.f);
-}
-__device__ inline RefSum shfl_down(const RefSum &v, int off) {
-    return RefSum{__shfl_down_sync(0xffffffffu, v.m, off), __shfl_down_sync(0xffffffffu, v.s, off)};
-}
-// block-wide fold of one RefSum per thread, in a fixed order; the result is valid in thread 0
-__device__ inline RefSum block_fold(RefSum v, RefSum *sh) {
+    for (int q = 0; q < R; ++q) {
+        float2 s0 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int off = 16; off; off >>= 1) v = combine(v, shfl_down(v, off));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < kThreads / 32 ? sh[lane] : RefSum{-INFINITY, 0.0};
-#pragma unroll
-        for (int off = 4; off; off >>= 1) v = combine(v, shfl_down(v, off));
+        for (int e = 0; e < N; e += 2) {
+            const float2 y = __ffma2_rn(make_float2(x[q][e], x[q][e + 1]), c2, m2);
+            s0 = __fadd2_rn(s0, make_float2(ex2(y.x), ex2(y.y)));
+        }
+        sum[q] = s0.x + s0.y;
     }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < R; ++q) a.s += (double)sum[q];
+}
+// fold over a warp in a fixed order, known to every lane
+__device__ inline RefSum warp_fold(RefSum v) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1)
+        v = combine(v, RefSum{__shfl_xor_sync(0xffffffffu, v.m, off), __shfl_xor_sync(0xffffffffu, v.s, off)});
     return v;
 }
 
-// true when rows of V elements starting at `base` can be read with 16-byte loads
-template <typename T> __host__ __device__ inline bool vector_ok(const void *base, int V) {
-    return V % Elem<T>::N == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+struct alignas(8) StatPart { float ma, md; double sa, sd; };       // per (row, stretch)
+
+// The logits of one row as vectors of N elements on 16-byte boundaries: vector v holds elements
+// [v * N - a, v * N - a + N), of which those outside [0, V) do not exist.  Only the first and the last
+// can be incomplete.  `vec` false (the two tensors' rows are not aligned alike): no 16-byte loads.
+struct RowShape { int V, a, n_vec; bool vec; };
+template <typename T> __device__ inline RowShape row_shape(const T *ra, const T *rd, int V) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(ra) & 15, y = reinterpret_cast<uintptr_t>(rd) & 15;
+    RowShape s;
+    s.V = V;
+    s.vec = x == y;
+    s.a = s.vec ? (int)(x / sizeof(T)) : 0;
+    s.n_vec = (V + s.a + Elem<T>::N - 1) / Elem<T>::N;
+    return s;
+}
+template <typename T> __device__ inline bool whole(const RowShape &s, int v) {
+    return s.vec && v * Elem<T>::N >= s.a && v * Elem<T>::N - s.a + Elem<T>::N <= s.V;
+}
+// one vector of a row; elements that do not exist are -inf (their exponential is 0)
+template <typename T> __device__ inline void load_vec(const T *row, const RowShape &s, int v, float (&x)[Elem<T>::N]) {
+    const int i0 = v * Elem<T>::N - s.a;
+    if (whole<T>(s, v)) {
+        Elem<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(row + i0)), x);
+    } else {
+#pragma unroll
+        for (int e = 0; e < Elem<T>::N; ++e) x[e] = i0 + e >= 0 && i0 + e < s.V ? Elem<T>::load(row + i0 + e) : -INFINITY;
+    }
 }
 
-struct StatPart { float ma, md; double sa, sd; };       // per (row, segment)
-struct Sum2 { double x, y; };                           // (residual mass, AR mass) of a segment
-
-// 1. per (row, segment): (reference, sum) of both logit rows, in the log2 domain scaled by c = log2(e) / T.
-// The launch covers block positions [k0, k1) of every sequence; with `fail` given, sequences
-// whose first rejection is already known (fail[b] < K) are skipped: verification halts at the
-// first rejected draft, so their later rows are never looked at.
+// the accept test of one row, from its folded statistics
 template <typename T>
-__global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, const T *ld, int V, int seg_len,
-                                                                float c, StatPart *parts, int vec, int K, int k0,
-                                                                int k1, const int *fail)
+__device__ inline bool keeps(const T *ra, const T *rd, const RefSum &a, const RefSum &d, int draft, float u, int V, float c)
+{
+    const int y = min(max(draft, 0), V - 1);            // an out-of-range draft id is clamped, not dereferenced
+    // u * q(y) <= p(y), both sides times the two sums
+    return (double)u * (double)ex2(Elem<T>::load(rd + y) * c - d.m) * a.s <= (double)ex2(Elem<T>::load(ra + y) * c - a.m) * d.s;
+}
+// a warp folds the stretches of a row (four per lane requested together)
+__device__ inline void fold_row(const StatPart *parts, int n_seg, int lane, RefSum &a, RefSum &d) {
+    a = d = RefSum{-INFINITY, 0.0};
+    for (int s0 = lane; s0 < n_seg; s0 += 128) {
+        StatPart t[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            t[q] = StatPart{-INFINITY, -INFINITY, 0.0, 0.0};
+            if (s0 + q * 32 < n_seg) {                  // (written by other SMs: past L1)
+                const StatPart *x = parts + s0 + q * 32;
+                const float2 m = __ldcg(reinterpret_cast<const float2 *>(x));
+                t[q].ma = m.x; t[q].md = m.y;
+                t[q].sa = __ldcg(&x->sa); t[q].sd = __ldcg(&x->sd);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            a = combine(a, RefSum{t[q].ma, t[q].sa});
+            d = combine(d, RefSum{t[q].md, t[q].sd});
+        }
+    }
+    a = warp_fold(a);
+    d = warp_fold(d);
+}
+
+// per sequence: first row known to fail; per row: stretches done.  Only the skipping form reads them.
+__global__ void sample_init_kernel(int *fail, int *done, int B, int K)
+{
+    pdl_begin();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B * K; i += gridDim.x * blockDim.x) {
+        done[i] = 0;
+        if (i < B) fail[i] = K;
+    }
+}
+
+// A warp takes items (block position k, sequence b, stretch) in that order, k outermost.
+template <typename T, bool SKIP>
+__global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, const T *ld, int B, int K, int V, int n_seg,
+                                                                float c, const int32_t *draft, const float *u_accept,
+                                                                StatPart *parts, int *fail, int *done)
 {
     constexpr int N = Elem<T>::N;
-    __shared__ RefSum sh[kThreads / 32];
-    const int seq = blockIdx.y / (k1 - k0), seg = blockIdx.x;
-    if (fail != nullptr && fail[seq] < K) return;
-    const int row = seq * K + k0 + blockIdx.y % (k1 - k0);
-    const int start = seg * seg_len, end = min(V, start + seg_len);
-    const T *ra = la + (long long)row * V, *rd = ld + (long long)row * V;
-    RefSum a{-INFINITY, 0.0}, d{-INFINITY, 0.0};
-    if (vec) {                                  // seg_len and V are multiples of N, rows are 16-byte aligned
-        const uint4 *va = reinterpret_cast<const uint4 *>(ra + start), *vd = reinterpret_cast<const uint4 *>(rd + start);
-        const int n_vec = (end - start) / N;
-        for (int v = threadIdx.x; v < n_vec; v += 4 * kThreads) {     // up to 8 loads in flight per thread
-            uint4 av[4], dv[4];
+    pdl_begin();
+    const int lane = threadIdx.x & 31;
+    const long long n_items = (long long)K * B * n_seg, stride = (long long)gridDim.x * kWarps;
+    for (long long it = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); it < n_items; it += stride) {
+        const int seg = (int)(it % n_seg), kb = (int)(it / n_seg), b = kb % B, k = kb / B;
+        const long long row = (long long)b * K + k;
+        bool needed = true;
+        if (SKIP) needed = *reinterpret_cast<volatile int *>(fail + b) >= k;
+        if (SKIP) needed = __all_sync(0xffffffffu, needed);
+        if (needed) {
+            const T *ra = la + row * V, *rd = ld + row * V;
+            const RowShape sh = row_shape(ra, rd, V);
+            const int per = (sh.n_vec + n_seg - 1) / n_seg, v0 = seg * per, v1 = min(sh.n_vec, v0 + per);
+            RefSum a{-INFINITY, 0.0}, d{-INFINITY, 0.0};
+            // whole vectors, four of each row at a time; incomplete ones by one lane each
+            const int w0 = max(v0, sh.vec ? (sh.a + N - 1) / N : v1), w1 = min(v1, (V + sh.a) / N);
+            const uint4 *va = reinterpret_cast<const uint4 *>(ra - sh.a), *vd = reinterpret_cast<const uint4 *>(rd - sh.a);
+            int v = w0 + lane;
+            for (; v + 96 < w1; v += 128) {
+                uint4 x[4], y[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int w = min(v + k * kThreads, n_vec - 1);
-                av[k] = __ldg(va + w); dv[k] = __ldg(vd + w);
+                for (int q = 0; q < 4; ++q) { x[q] = __ldg(va + v + q * 32); y[q] = __ldg(vd + v + q * 32); }
+                float f[4][N];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) Elem<T>::unpack(x[q], f[q]);
+                absorb<4, N>(a, f, c);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) Elem<T>::unpack(y[q], f[q]);
+                absorb<4, N>(d, f, c);
+            }
+            for (; v < w1; v += 32) {
+                const uint4 x = __ldg(va + v), y = __ldg(vd + v);
+                float f[1][N];
+                Elem<T>::unpack(x, f[0]); absorb<1, N>(a, f, c);
+                Elem<T>::unpack(y, f[0]); absorb<1, N>(d, f, c);
+            }
+            for (int e = v0 + lane; e < v1; e += 32) {
+                if (e >= w0 && e < w1) continue;
+                float f[1][N];
+                load_vec<T>(ra, sh, e, f[0]); absorb<1, N>(a, f, c);
+                load_vec<T>(rd, sh, e, f[0]); absorb<1, N>(d, f, c);
+            }
+            a = warp_fold(a);
+            d = warp_fold(d);
+            if (lane == 0) parts[row * n_seg + seg] = StatPart{a.m, d.m, a.s, d.s};
+        }
+        // (a stretch that was skipped is not counted: its row is behind a failure, and nobody asks for it)
+        if (SKIP && needed) {
+            int before = 0;
+            if (lane == 0) {
+                __threadfence();                        // the statistics before the count
+                before = atomicAdd(done + row, 1);
+            }
+            before = __shfl_sync(0xffffffffu, before, 0);
+            // the row is complete
+            if (before == n_seg - 1 && *reinterpret_cast<volatile int *>(fail + b) >= k) {
+                __threadfence();
+                RefSum a, d;
+                fold_row(parts + row * n_seg, n_seg, lane, a, d);
+                if (lane == 0 && !keeps(la + row * V, ld + row * V, a, d, draft[row], u_accept[row], V, c)) atomicMin(fail + b, k);
+            }
+        }
+    }
+}
+
+struct RowStat { float ma, md; double inv_za, inv_zd; };  // of the first rejected row (1 / sums)
+
+__device__ inline void residual_of(float xa, float xd, float c, const RowStat &st, double &r, double &p) {
+    p = (double)ex2(xa * c - st.ma) * st.inv_za;
+    const double q = (double)ex2(xd * c - st.md) * st.inv_zd;
+    r = fmax(p - q, 0.0);
+}
+template <int N>
+__device__ inline void residual_vec(const float (&x)[N], const float (&y)[N], float c, const RowStat &st, double &sr, double &sp) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        double r, p;
+        residual_of(x[e], y[e], c, st, r, p);           // (an element that does not exist has p = r = 0)
+        sr += r; sp += p;
+    }
+}
+__device__ inline double warp_sum(double x) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+__device__ inline double peer_double(const double *mine, int rank) {
+    double x;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(map_to_rank(smem_u32(mine), rank)) : "memory");
+    return x;
+}
+
+// Grid (C, B) in clusters of C: one sequence.  The residual's running sum is taken over CTAs, then a
+// CTA's warps, then a warp's groups of rounds (a round is 32 vectors, a lane each), in index order, and
+// each level keeps its sums, so that the drawn point is found level by level.
+constexpr int kGroups = 64;
+template <typename T>
+__global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, const T *ld, int K, int V, int n_seg, float c,
+                                                                 const int32_t *draft, const float *u_accept,
+                                                                 const float *u_resample, const StatPart *parts,
+                                                                 const int *fail, int32_t *n_commit, int32_t *committed,
+                                                                 int32_t *next_anchor)
+{
+    constexpr int N = Elem<T>::N;
+    __shared__ double grp[2][kWarps][kGroups], wsum[2][kWarps], csum[2];
+    __shared__ double s_before, s_target;
+    __shared__ int s_first, s_owner, s_use_p, s_warp, s_group;
+    __shared__ RowStat s_stat;
+    extern __shared__ RefSum folded[];                  // [K][2], unless the failures are known already
+    const int b = blockIdx.y, rank = blockIdx.x, C = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_begin();
+    if (tid == 0) s_first = fail ? fail[b] : K;
+    __syncthreads();
+    if (!fail) {
+        for (int i = warp; i < K; i += kWarps) {
+            const long long row = (long long)b * K + i;
+            RefSum a, d;
+            fold_row(parts + row * n_seg, n_seg, lane, a, d);
+            if (lane == 0) {
+                folded[2 * i] = a; folded[2 * i + 1] = d;
+                if (!keeps(la + row * V, ld + row * V, a, d, draft[row], u_accept[row], V, c)) atomicMin(&s_first, i);
+            }
+        }
+        __syncthreads();
+    }
+    const int j = s_first;                              // K: every draft is kept
+    if (rank == 0) {
+        for (int i = tid; i < K; i += kThreads)
+            if (i != j) committed[(long long)b * K + i] = i < j ? draft[(long long)b * K + i] : -1;
+        if (tid == 0) {
+            n_commit[b] = j < K ? j + 1 : K;
+            if (j >= K) next_anchor[b] = draft[(long long)b * K + K - 1];
+        }
+    }
+    if (j >= K) return;                                 // (the whole cluster)
+    const long long row = (long long)b * K + j;
+    const T *ra = la + row * V, *rd = ld + row * V;
+    if (warp == 0) {
+        RefSum a, d;
+        if (fail) fold_row(parts + row * n_seg, n_seg, lane, a, d);
+        else { a = folded[2 * j]; d = folded[2 * j + 1]; }
+        if (lane == 0) s_stat = RowStat{a.m, d.m, 1.0 / a.s, 1.0 / d.s};
+    }
+    __syncthreads();
+    const RowStat st = s_stat;
+    const RowShape sh = row_shape(ra, rd, V);
+    const int per = (sh.n_vec + C - 1) / C, v0 = rank * per, v1 = min(sh.n_vec, v0 + per);
+    const int per_w = (per + kWarps - 1) / kWarps, w0 = min(v1, v0 + warp * per_w), w1 = min(v1, w0 + per_w);
+    // (a group costs two warp sums, a round in the end two loads: two rounds and up to a group)
+    const int rounds = (per_w + 31) / 32, gsz = max(2, (rounds + kGroups - 1) / kGroups), n_grp = (rounds + gsz - 1) / gsz;
+    {
+        double tr = 0.0, tp = 0.0, sr = 0.0, sp = 0.0;
+        for (int r0 = 0; r0 < rounds; r0 += 4) {        // the loads of four rounds together
+            float x[4][N], y[4][N];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int v = w0 + (r0 + i) * 32 + lane;
+                if (r0 + i < rounds && v < w1) {
+                    load_vec<T>(ra, sh, v, x[i]);
+                    load_vec<T>(rd, sh, v, y[i]);
+                }
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (v + k * kThreads < n_vec) {
-                    float x[N];
-                    Elem<T>::unpack(av[k], x); absorb_vec<N>(a, x, c);
-                    Elem<T>::unpack(dv[k], x); absorb_vec<N>(d, x, c);
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + i;
+                if (r >= rounds) break;
+                if (w0 + r * 32 + lane < w1) residual_vec<N>(x[i], y[i], c, st, sr, sp);
+                if ((r + 1) % gsz == 0 || r == rounds - 1) {
+                    sr = warp_sum(sr); sp = warp_sum(sp);
+                    if (lane == 0) { grp[0][warp][r / gsz] = sr; grp[1][warp][r / gsz] = sp; }
+                    tr += sr; tp += sp;
+                    sr = sp = 0.0;
                 }
             }
         }
-    } else {
-        for (int i = start + threadIdx.x; i < end; i += kThreads) {
-            absorb(a, Elem<T>::load(ra + i) * c);
-            absorb(d, Elem<T>::load(rd + i) * c);
-        }
-    }
-    a = block_fold(a, sh);
-    d = block_fold(d, sh);
-    if (threadIdx.x == 0) parts[(long long)row * gridDim.x + seg] = StatPart{a.m, d.m, a.s, d.s};
-}
-
-struct RowStat { float ma, md; double inv_za, inv_zd; int row; int pad; };   // of the first rejected row (1 / sums); row = -1: none
-
-// 2. per sequence: fold the segments, take the accept tests, find the first failure
-template <typename T>
-// for block positions [k0, k1); fail[b] carries the outcome between the stages (K: no rejection
-// so far).  A sequence's results are written by the stage that settles it: the one that finds
-// its first rejection, or the last one.
-__global__ void sample_decide_kernel(const T *la, const T *ld, const StatPart *parts, int n_seg, int K, int V,
-                                     float c, const int32_t *draft, const float *u_accept,
-                                     int32_t *n_commit, int32_t *committed, int32_t *next_anchor,
-                                     RowStat *stat, int k0, int k1, int *fail)
-{
-    extern __shared__ StatPart folded[];        // [K]
-    __shared__ int first_fail;
-    const int b = blockIdx.x;
-    if (k0 > 0 && fail[b] < K) return;          // settled by an earlier stage
-    if (threadIdx.x == 0) first_fail = K;
-    __syncthreads();
-    for (int i = k0 + threadIdx.x; i < k1; i += blockDim.x) {
-        const long long row = (long long)b * K + i;
-        RefSum a{-INFINITY, 0.0}, d{-INFINITY, 0.0};
-        for (int s = 0; s < n_seg; ++s) {
-            const StatPart t = parts[row * n_seg + s];
-            a = combine(a, RefSum{t.ma, t.sa});
-            d = combine(d, RefSum{t.md, t.sd});
-        }
-        folded[i] = StatPart{a.m, d.m, a.s, d.s};
-        int y = draft[row];
-        y = min(max(y, 0), V - 1);              // an out-of-range draft id is clamped, not dereferenced
-        const double py = (double)ex2f(Elem<T>::load(la + row * V + y) * c - a.m) / a.s;
-        const double qy = (double)ex2f(Elem<T>::load(ld + row * V + y) * c - d.m) / d.s;
-        if (!((double)u_accept[row] * qy <= py)) atomicMin(&first_fail, i);
+        if (lane == 0) { wsum[0][warp] = tr; wsum[1][warp] = tp; }
     }
     __syncthreads();
-    const int j = first_fail;                   // K: every draft so far kept
-    if (threadIdx.x == 0) fail[b] = j;
-    if (j >= K && k1 < K) return;               // still open: the next stage goes on
-    const int n = j < K ? j + 1 : K;
-    for (int i = threadIdx.x; i < K; i += blockDim.x)
-        committed[(long long)b * K + i] = i < min(j, K) ? draft[(long long)b * K + i] : -1;
-    if (threadIdx.x == 0) {
-        n_commit[b] = n;
-        RowStat st;
-        st.row = j < K ? j : -1;
-        const StatPart f = j < K ? folded[j] : StatPart{0.f, 0.f, 1.0, 1.0};
-        st.ma = f.ma; st.inv_za = 1.0 / f.sa; st.md = f.md; st.inv_zd = 1.0 / f.sd;
-        st.pad = 0;
-        stat[b] = st;
-        if (j >= K) next_anchor[b] = draft[(long long)b * K + K - 1];
+    if (tid < 2) {
+        double s = 0.0;
+        for (int w = 0; w < kWarps; ++w) s += wsum[tid][w];
+        csum[tid] = s;
     }
-}
-
-__device__ inline void residual_of(float xa, float xd, float c, const RowStat &st, double &r, double &p) {
-    p = (double)ex2f(xa * c - st.ma) * st.inv_za;
-    const double q = (double)ex2f(xd * c - st.md) * st.inv_zd;
-    r = fmax(p - q, 0.0);
-}
-
-// 3. per (sequence, segment) of the rejected row: sum of max(0, p - q) and of p
-template <typename T>
-__global__ void __launch_bounds__(kThreads) sample_residual_kernel(const T *la, const T *ld, int K, int V,
-                                                                   int seg_len, float c, const RowStat *stat,
-                                                                   Sum2 *seg_sums)
-{
-    __shared__ Sum2 sh[kThreads];
-    const int b = blockIdx.y, seg = blockIdx.x;
-    const RowStat st = stat[b];
-    if (st.row < 0) return;
-    const long long row = (long long)b * K + st.row;
-    const int start = seg * seg_len, end = min(V, start + seg_len);
-    // every thread owns a contiguous run of the segment; the runs are added up in order
-    const int per = (seg_len + kThreads - 1) / kThreads;
-    const int i0 = start + threadIdx.x * per, i1 = min(end, i0 + per);
-    double sr = 0.0, sp = 0.0;
-    for (int i = i0; i < i1; ++i) {
-        double r, p;
-        residual_of(Elem<T>::load(la + row * V + i), Elem<T>::load(ld + row * V + i), c, st, r, p);
-        sr += r; sp += p;
-    }
-    sh[threadIdx.x] = Sum2{sr, sp};
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, p = 0.0;
-        for (int t = 0; t < kThreads; ++t) { a += sh[t].x; p += sh[t].y; }
-        seg_sums[(long long)b * gridDim.x + seg] = Sum2{a, p};
-    }
-}
-
-// 4. per sequence: invert the running sum of the residual (of p itself if the residual is empty)
-template <typename T>
-__global__ void __launch_bounds__(kThreads) sample_pick_kernel(const T *la, const T *ld, int K, int V, int seg_len,
-                                                               int n_seg, float c, const RowStat *stat,
-                                                               const Sum2 *seg_sums, const float *u_resample,
-                                                               int32_t *committed, int32_t *next_anchor)
-{
-    __shared__ double run_sh[kThreads];
-    __shared__ int seg_sh, use_p_sh;
-    __shared__ double before_sh, target_sh;
-    const int b = blockIdx.x;
-    const RowStat st = stat[b];
-    if (st.row < 0) return;
-    const long long row = (long long)b * K + st.row;
-    if (threadIdx.x == 0) {
+    cluster_sync_all();
+    // every CTA finds the share that holds the drawn point: the first whose running sum exceeds the target,
+    // the last that is not empty if rounding leaves the target at or past the total
+    if (warp == 0) {
+        const double xr = lane < C ? peer_double(&csum[0], lane) : 0.0, xp = lane < C ? peer_double(&csum[1], lane) : 0.0;
         double tot_r = 0.0, tot_p = 0.0;
-        for (int s = 0; s < n_seg; ++s) { tot_r += seg_sums[(long long)b * n_seg + s].x; tot_p += seg_sums[(long long)b * n_seg + s].y; }
+        for (int s = 0; s < C; ++s) { tot_r += __shfl_sync(0xffffffffu, xr, s); tot_p += __shfl_sync(0xffffffffu, xp, s); }
         const int use_p = !(tot_r > 0.0);
-        const double total = use_p ? tot_p : tot_r;
-        const double target = (double)u_resample[row] * total;
-        // the first segment whose running sum exceeds the target (the last non-empty one otherwise)
+        const double x = use_p ? xp : xr, target = (double)u_resample[row] * (use_p ? tot_p : tot_r);
         double run = 0.0, before = 0.0;
         int pick = -1, last = 0;
-        for (int s = 0; s < n_seg; ++s) {
-            const Sum2 t = seg_sums[(long long)b * n_seg + s];
-            const double v = use_p ? t.y : t.x;
+        for (int s = 0; s < C; ++s) {
+            const double v = __shfl_sync(0xffffffffu, x, s);
             if (v > 0.0) {
                 last = s;
                 if (pick < 0 && run + v > target) { pick = s; before = run; }
                 run += v;
             }
         }
-        if (pick < 0) { pick = last; before = run; }      // rounding: the target is at or past the total
-        seg_sh = pick; use_p_sh = use_p; before_sh = before; target_sh = target;
+        if (pick < 0) { pick = last; before = run; }
+        if (lane == 0) { s_owner = pick; s_use_p = use_p; s_before = before; s_target = target; }
     }
     __syncthreads();
-    const int seg = seg_sh, use_p = use_p_sh;
-    const double before = before_sh, target = target_sh;
-    const int start = seg * seg_len, end = min(V, start + seg_len);
-    const int per = (seg_len + kThreads - 1) / kThreads;
-    const int i0 = start + threadIdx.x * per, i1 = min(end, i0 + per);
-    double mine = 0.0;
-    for (int i = i0; i < i1; ++i) {
-        double r, p;
-        residual_of(Elem<T>::load(la + row * V + i), Elem<T>::load(ld + row * V + i), c, st, r, p);
-        mine += use_p ? p : r;
-    }
-    run_sh[threadIdx.x] = mine;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // walk the threads' runs in order, then the elements of the run that contains the target
-        double run = before;
-        int t_pick = -1, t_last = -1;
-        for (int t = 0; t < kThreads; ++t) {
-            if (run_sh[t] > 0.0) {
-                t_last = t;
-                if (run + run_sh[t] > target) { t_pick = t; break; }
-                run += run_sh[t];
+    if (rank == s_owner && warp == 0) {
+        // the warp and the group of rounds, by the same rule (a lane's warp total, then a lane's two groups)
+        const int use_p = s_use_p;
+        const double target = s_target;
+        double run = s_before;
+        int pw = -1, last = 0;
+        double at = run;
+        for (int w = 0; w < kWarps; ++w) {
+            const double v = wsum[use_p][w];
+            if (v > 0.0) {
+                last = w;
+                if (pw < 0 && run + v > target) { pw = w; at = run; }
+                run += v;
             }
         }
-        const bool past_end = t_pick < 0;                // rounding again: take the last positive element
-        if (past_end) t_pick = t_last;
-        int z = -1, z_last = -1;
-        if (t_pick >= 0) {
-            const int j0 = start + t_pick * per, j1 = min(end, j0 + per);
-            double acc = run;
-            for (int i = j0; i < j1; ++i) {
-                double r, p;
-                residual_of(Elem<T>::load(la + row * V + i), Elem<T>::load(ld + row * V + i), c, st, r, p);
-                const double v = use_p ? p : r;
-                if (v > 0.0) {
-                    z_last = i;
-                    if (!past_end) { acc += v; if (acc > target) { z = i; break; } }
-                }
+        const bool past = pw < 0;                       // rounding: take the last element that is positive
+        if (past) { pw = last; at = run; }
+        int pg = -1, last_g = 0;
+        run = at;
+        for (int g = 0; g < n_grp; ++g) {
+            const double v = grp[use_p][pw][g];
+            if (v > 0.0) {
+                last_g = g;
+                if (pg < 0 && !past && run + v > target) { pg = g; at = run; }
+                run += v;
             }
+        }
+        if (pg < 0) { pg = last_g; at = run; }
+        // the vector and the element
+        const int q0 = min(v1, v0 + pw * per_w), q1 = min(v1, q0 + per_w);
+        int z = -1, z_last = -1;
+        run = at;
+        for (int r = pg * gsz; r < min(rounds, (pg + 1) * gsz) && z < 0; ++r) {
+            const int v = q0 + r * 32 + lane;
+            float x[N], y[N];
+            double mine[N], sum = 0.0;
+            if (v < q1) { load_vec<T>(ra, sh, v, x); load_vec<T>(rd, sh, v, y); }
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                double rr = 0.0, pp = 0.0;
+                if (v < q1) residual_of(x[e], y[e], c, st, rr, pp);
+                mine[e] = use_p ? pp : rr;
+                sum += mine[e];
+            }
+            double incl = sum;                          // running sum over the lanes
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const double o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, !past && sum > 0.0 && run + incl > target);
+            int my_last = -1, my_z = -1;
+            double acc = run + (incl - sum);
+#pragma unroll
+            for (int e = 0; e < N; ++e)
+                if (mine[e] > 0.0) {
+                    my_last = v * N - sh.a + e;
+                    acc += mine[e];
+                    if (my_z < 0 && acc > target) my_z = my_last;
+                }
+            if (hit) {
+                const int l = __ffs(hit) - 1;
+                z = __shfl_sync(0xffffffffu, my_z >= 0 ? my_z : my_last, l);
+            }
+            const unsigned some = __ballot_sync(0xffffffffu, my_last >= 0);
+            if (some) z_last = __shfl_sync(0xffffffffu, my_last, 31 - __clz(some));
+            run += __shfl_sync(0xffffffffu, incl, 31);
         }
         if (z < 0) z = z_last >= 0 ? z_last : 0;
-        committed[(long long)b * K + st.row] = z;
-        next_anchor[b] = z;
+        if (lane == 0) {
+            committed[(long long)b * K + j] = z;
+            next_anchor[b] = z;
+        }
     }
+    cluster_sync_all();                                 // the peers have read this CTA's sums
 }
 
 }  // namespace
 
-int sample_stat_segments(int B, int K, int V)
+// Stretches per row: about kStretch logits each, shorter ones (down to 512) where the rows are too few
+// to give every SM 16 warps.
+static int sample_stat_segments(int B, int K, int V)
 {
-    const long long rows = (long long)B * K;
-    long long want = (8LL * num_sms() + rows - 1) / rows;           // more CTAs than fit at once, for balance
-    const long long max_by_len = (V + 4095) / 4096;
-    if (want > max_by_len) want = max_by_len;
-    return (int)(want < 1 ? 1 : want);
+    const long long want = (16LL * num_sms() + (long long)B * K - 1) / ((long long)B * K);
+    const int lo = (V + kStretch - 1) / kStretch, hi = (V + 511) / 512;
+    return want < lo ? lo : want > hi ? hi : (int)want;
 }
-
-int sample_pick_segments(int V) { return (V + kPickSegMax - 1) / kPickSegMax; }
 
 size_t sample_workspace_bytes(int B, int K, int V)
 {
-    return (size_t)B * K * sample_stat_segments(B, K, V) * sizeof(StatPart) + (size_t)B * sizeof(RowStat) +
-           (size_t)B * sample_pick_segments(V) * sizeof(Sum2) + (size_t)B * sizeof(int);
-}
-
-// Block positions verified by the first statistics pass.  Verification halts at the first
-// rejected draft, so rows behind it need not be looked at: when the two logit tensors are
-// large enough for the pass to be bound by throughput, the first pass covers a quarter of the
-// block (at least 4 positions) and a second pass the rest, for the sequences still open only.
-// More stages were measured slower (each costs two dependent launches), and small problems
-// are bound by launch latency and take one pass.  ORTHRUS_SAMPLE_FIRST_STAGE overrides.
-int sample_first_stage(int B, int K, int V)
-{
-    const long long bytes = 2LL * B * K * V * 2;
-    static const int forced = [] { const char *e = getenv("ORTHRUS_SAMPLE_FIRST_STAGE"); return e ? atoi(e) : 0; }();
-    if (forced > 0) return forced < K ? forced : K;
-    if (K <= 4 || bytes < (64LL << 20)) return K;
-    const int k1 = (K + 3) / 4;
-    return k1 < 4 ? 4 : k1;
+    return (size_t)B * K * sample_stat_segments(B, K, V) * sizeof(StatPart) + (size_t)B * K * sizeof(int) + (size_t)B * sizeof(int);
 }
 
 template <typename T>
@@ -374,41 +497,54 @@ static cudaError_t launch_sample_t(const void *ar_logits, const void *diff_logit
                                    int V, int32_t *n_commit, int32_t *committed, int32_t *next_anchor,
                                    unsigned char *ws, cudaStream_t st)
 {
-    constexpr int N = Elem<T>::N;
     const T *la = static_cast<const T *>(ar_logits), *ld = static_cast<const T *>(diff_logits);
     const float c = 1.4426950408889634f / temperature;
     const int n_seg = sample_stat_segments(B, K, V);
-    int seg_len = (V + n_seg - 1) / n_seg;
-    seg_len = (seg_len + N - 1) / N * N;
-    const int vec = vector_ok<T>(la, V) && vector_ok<T>(ld, V);
     StatPart *parts = reinterpret_cast<StatPart *>(ws);
-    RowStat *stat = reinterpret_cast<RowStat *>(ws + (size_t)B * K * n_seg * sizeof(StatPart));
-    const int n_seg2 = sample_pick_segments(V);
-    Sum2 *seg_sums = reinterpret_cast<Sum2 *>(reinterpret_cast<unsigned char *>(stat) + (size_t)B * sizeof(RowStat));
-    int *fail = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(seg_sums) + (size_t)B * n_seg2 * sizeof(Sum2));
-    const int threads = K <= 32 ? 32 : ((K + 31) / 32 * 32 > 256 ? 256 : (K + 31) / 32 * 32);
-    const int k_first = sample_first_stage(B, K, V);
-    cudaError_t e = cudaSuccess;
-    int launches = 2;
-    for (int k0 = 0, k1 = k_first; k0 < K; k0 = k1, k1 = K) {
-        sample_stats_kernel<T><<<dim3(n_seg, B * (k1 - k0)), kThreads, 0, st>>>(la, ld, V, seg_len, c, parts, vec, K,
-                                                                               k0, k1, k0 > 0 ? fail : nullptr);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        sample_decide_kernel<T><<<B, threads, K * sizeof(StatPart), st>>>(la, ld, parts, n_seg, K, V, c, draft,
-                                                                      u_accept, n_commit, committed, next_anchor,
-                                                                      stat, k0, k1, fail);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        launches += 2;
+    int *done = reinterpret_cast<int *>(ws + (size_t)B * K * n_seg * sizeof(StatPart)), *fail = done + (size_t)B * K;
+    // The skipping form pays for its counters and its extra launch once the logits are several waves
+    // of the grid below: then whole rows behind the first rejection are left out.
+    const long long n_items = (long long)B * K * n_seg;
+    // (every resident warp more is a stretch more that may be read in vain)
+    const bool skip = K > 1 && n_items > 64LL * num_sms();
+    const int ctas_per_sm = skip ? 3 : 4;
+    const int grid = (int)((n_items + kWarps - 1) / kWarps < (long long)ctas_per_sm * num_sms()
+                               ? (n_items + kWarps - 1) / kWarps : (long long)ctas_per_sm * num_sms());
+    cudaError_t e;
+    if (skip) {
+        const int n = (B * K + 255) / 256;
+        e = launch_kernel(true, sample_init_kernel, dim3(n < 64 ? n : 64), 256, 0, st, fail, done, B, K);
+        if (e == cudaSuccess)
+            e = launch_kernel(true, sample_stats_kernel<T, true>, dim3(grid), kThreads, 0, st, la, ld, B, K, V, n_seg, c, draft,
+                              u_accept, parts, fail, done);
+    } else {
+        e = launch_kernel(true, sample_stats_kernel<T, false>, dim3(grid), kThreads, 0, st, la, ld, B, K, V, n_seg, c, draft,
+                          u_accept, parts, fail, done);
     }
-    sample_residual_kernel<T><<<dim3(n_seg2, B), kThreads, 0, st>>>(la, ld, K, V, kPickSegMax, c, stat, seg_sums);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    sample_pick_kernel<T><<<B, kThreads, 0, st>>>(la, ld, K, V, kPickSegMax, n_seg2, c, stat, seg_sums, u_resample,
-                                                  committed, next_anchor);
-    count_launch(launches);
-    return cudaGetLastError();
+    // CTAs per sequence: 16 for the first few, 8 (the portable cluster size) while that does not crowd the GPU
+    int C = B <= 4 ? 16 : 8;
+    while (C > 1 && (long long)B * C > 4LL * num_sms()) C /= 2;
+    if (C > 8) {
+        e = cudaFuncSetAttribute(sample_finish_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C, B);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = skip ? 0 : (size_t)K * 2 * sizeof(RefSum);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, sample_finish_kernel<T>, la, ld, K, V, n_seg, c, draft, u_accept, u_resample,
+                              static_cast<const StatPart *>(parts), static_cast<const int *>(skip ? fail : nullptr), n_commit,
+                              committed, next_anchor);
 }
 
 cudaError_t launch_consensus_sample(const void *ar_logits, const void *diff_logits, int dtype, const int32_t *draft,
