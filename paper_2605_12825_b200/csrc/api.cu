@@ -199,27 +199,37 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
     return pl;
 }
 
-// Units of at most 64 query rows run with the keys on the MMA's rows (attend_keys.cu), head_dim 64
-// and 128.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the kernel for wide units (a measurement knob).
+// Units of at most 64 query rows, and wider ones at head_dim 64, run with the keys on the MMA's rows
+// (attend_keys.cu).  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels (a measurement knob).
+// Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
+// and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
+// from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).
 static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
 {
-    const int M = L->n_q_heads / L->n_kv_heads * L->block;
-    if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || !keys_rows(M) || !kn.small_rows) return false;
-    const unsigned long long rows = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
-    return rows < 0x7fffffffull && (long long)L->batch * L->n_kv_heads <= 65535 && tc_driver_ok();
+    if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || !kn.small_rows) return false;
+    const int G = L->n_q_heads / L->n_kv_heads;
+    const int rows = keys_rows(L->head_dim, G, L->block);
+    if (!rows || (rows > 64 && max_len_of(L) <= 320)) return false;
+    const unsigned long long cache = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
+    return cache < 0x7fffffffull && (long long)L->batch * L->n_kv_heads <= 65535 && tc_driver_ok();
+}
+static int keys_tiles(const orthrus_layer_t *L)
+{
+    const int kb = tc_kb_rows(L->n_q_heads / L->n_kv_heads, L->block);
+    return (L->block + kb - 1) / kb;
 }
 static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (kn.splits > 0) return kn.splits < 16 ? kn.splits : 16;
     // from prefix and block together: a decoder that bounds its lengths by capacity - block then cuts
     // a block's verification and a width-1 step at the same keys, and both round alike
-    return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads * L->block, L->batch * L->n_kv_heads,
+    return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
                        max_len_of(L) + L->block);
 }
 static size_t keys_bytes(const orthrus_layer_t *L, int S, size_t *ml_off)
 {
-    const size_t ctas = S > 1 ? (size_t)L->batch * L->n_kv_heads * S : 0;
-    const size_t nr = keys_rows(L->n_q_heads / L->n_kv_heads * L->block);
+    const size_t ctas = S > 1 ? (size_t)L->batch * L->n_kv_heads * keys_tiles(L) * S : 0;
+    const size_t nr = keys_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
     if (ml_off) *ml_off = ctas * nr * L->head_dim * sizeof(float);
     return ctas * nr * (L->head_dim + 2) * sizeof(float);
 }

@@ -1,7 +1,7 @@
-// Block attention for units of at most 64 query rows (M = G*K), bf16, head_dim 64 and 128, both
-// views, on tcgen05 with the KEYS on the rows of the MMA:
+// Block attention for units of at most 64 query rows (M = G*K), bf16, head_dim 64 and 128, and of more
+// at head_dim 64 (in tiles of up to 128 rows), both views, on tcgen05 with the KEYS on the MMA's rows:
 //     S^T [128 keys x NR rows] = K_tile . Q^T        O^T [d x NR rows] = V_tile^T . P^T
-// NR = M rounded up to 16, 32 or 64 is the MMA's N.  With the query rows there instead, an M of 4 to 64
+// NR = M rounded up to 16, 32, 64 or 128 is the MMA's N.  With the query rows there instead, an M of 4 to 64
 // is padded to 128, and only the threads that own real rows take part in the softmax and the
 // read-out; here all 128 lanes of the tensor memory hold keys (or head columns), every thread of
 // a softmax warpgroup works whatever M is, and a width-1 call costs a quarter of the exponentials.
@@ -15,9 +15,12 @@
 // of 64 rows and 4000 keys 10.9 -> 9.9 us; 16 units of 4 rows and 2700 keys 16.4 -> 8.5 us; 32 units of
 // 64 rows and 1800 keys 13.6 -> 12.5 us; head_dim 64, which ran on mma.sync with a second launch for
 // the merge, 10 units of 49 rows and 800 keys 10.9 -> 7.0 us, 2 units of 32 rows and 512 keys 10.4 ->
-// 6.2 us.  A batch of 256 such units at 4000 keys streams at 6.4 TB/s.
+// 6.2 us.  A batch of 256 such units at 4000 keys streams at 6.4 TB/s.  At 128 rows the exponentials
+// bound it, and the wide-unit kernel, whose softmax is spread over more warps, is the better one at
+// head_dim 128 (256 units, about 3000 keys: 30 against 50 us); head_dim 64 had mma.sync alone: one unit
+// of 4000 keys 15.1 -> 9.4 us, 64 of 1500 31 -> 26 us, 256 of 2000 103 -> 68 us.
 //
-// One CTA (320 threads, at most 113 KB of shared memory and 256 TMEM columns: two fit an SM, so that
+// One CTA (320 threads, up to 64 rows at most 113 KB of shared memory and 256 TMEM columns: two fit an SM, so that
 // with programmatic dependent launch the next call's CTAs are resident and, if the caller promised
 // a quiescent cache, load their first tiles while this call computes):
 //   warps 0-3, 4-7  softmax of tiles 0, 2, 4, ... and 1, 3, 5, ...; thread = key; also the query
@@ -65,19 +68,23 @@ constexpr float RAISE = 8.f;               // log2 units
 struct KeysMaps { CUtensorMap k, v, kb, vb; };
 struct KeysArgs {
     int S, quiescent, ranked;
-    uint32_t inv_g;            // ceil(2^16 / G): r / G = r * inv_g >> 16 for r < 64
+    uint32_t inv_g;            // ceil(2^16 / G): r / G = r * inv_g >> 16 for r < 128
     int slice;                 // elements of the merge per CTA, a multiple of 8
+    int kb_rows;               // block positions per query tile (blockIdx.z counts the tiles of a unit)
 };
 
 template <int HD, int NR> struct KeysShape {
     static constexpr int PANELS = HD / 64;
     static constexpr int KV_BYTES = PANELS * PANEL;
-    static constexpr int NSLOT = HD == 128 ? 2 : 4;
+    // up to 64 rows two CTAs share an SM; 128 rows take all of its tensor memory
+    static constexpr int CTAS = NR <= 64 ? 2 : 1;
+    static constexpr int NSLOT = HD == 128 && NR <= 64 ? 2 : 4;
     static constexpr int Q_BYTES = NR * HD * 2;
+    static constexpr int P_PANELS = (NR + 63) / 64, P_BYTES = P_PANELS * PANEL;   // probabilities of a tile
     static constexpr int OFF_RING = 0;
-    static constexpr int OFF_P = NSLOT * KV_BYTES;             // per warpgroup [128 keys][128 bytes]
-    static constexpr int OFF_Q = OFF_P + 2 * PANEL;
-    static constexpr int END_Q = OFF_Q + (Q_BYTES > 4608 ? Q_BYTES : 4608);   // (later the tables of the read-out)
+    static constexpr int OFF_P = NSLOT * KV_BYTES;             // per warpgroup [panel][128 keys][128 bytes]
+    static constexpr int OFF_Q = OFF_P + 2 * P_BYTES;
+    static constexpr int END_Q = OFF_Q + (Q_BYTES > 6144 ? Q_BYTES : 6144);   // (later the tables of the read-out)
     static constexpr int OFF_REF = END_Q;                      // float [2][NR]: references of the current tiles
     static constexpr int OFF_BAR = OFF_REF + 2 * NR * 4;
     static constexpr int BAR_FULL = 0, BAR_Q = NSLOT, BAR_S = BAR_Q + 1, BAR_P = BAR_S + 2, BAR_PV = BAR_P + 2,
@@ -88,7 +95,7 @@ template <int HD, int NR> struct KeysShape {
     static constexpr uint32_t TM_COLS = 4 * NR;                // two score buffers, two accumulators
     static constexpr uint32_t tm_s(int w) { return (uint32_t)(w * NR); }
     static constexpr uint32_t tm_o(int w) { return (uint32_t)(2 * NR + w * NR); }
-    static_assert(2 * (SMEM_BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
+    static_assert(CTAS * (SMEM_BYTES + 1024) <= 228 * 1024, "shared memory of an SM");
 };
 
 __device__ inline float warp_max(float x) {
@@ -144,8 +151,81 @@ __device__ inline bool elect_one() {
     return p != 0;
 }
 
+// A CTA's share [e, e_end) of the merge of S <= 4 U partial results, an element being a head column of
+// a group of four rows; called by each softmax warp, no barrier.  A warp takes eight columns at a time,
+// its lane groups every fourth partial, a lane U of them; all loads of 8 / U such steps are requested
+// together (a step waits for L2 once, about 0.9 us; two CTAs had sixteen steps of two for 128 rows).
+template <int HD, int NR, int U, class RowOff>
+__device__ inline void merge(const float4 *po, const float2 *pml, float *wt, int e, const int e_end, int M, int S,
+                             __nv_bfloat16 *out, const RowOff &row_off)
+{
+    constexpr int MX = 8 / U, MSTEP = 8 * SW, JS = U == 4 ? 16 : 8, R4 = NR / 4 * HD;
+    const int lane = threadIdx.x & 31, el = lane & 7, jg = lane >> 3, r = lane >> 3, j0 = lane & 7;
+    e += (threadIdx.x >> 5) * 8;
+    po += el + (long long)jg * R4;
+    for (; e < e_end; e += MX * MSTEP) {
+        float2 ml[MX][U == 4 ? 2 : 1];
+        float4 v[MX][U];
+        int at[MX];                           // where this lane's result goes (-1: no such row)
+#pragma unroll
+        for (int x = 0; x < MX; ++x) {
+            // rows 4g..4g+3 of the element's group g: lane = (row, partial), with U = 4 twice
+            const int ex = e + x * MSTEP, row = ex / HD * 4 + r;
+            const bool live = ex < e_end;
+#pragma unroll
+            for (int w = 0; w < (U == 4 ? 2 : 1); ++w)
+                ml[x][w] = live && row < M && j0 + 8 * w < S ? __ldcg(pml + (j0 + 8 * w) * NR + row) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                v[x][u] = live && jg + 4 * u < S ? __ldcg(po + ex + u * (4 * R4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int x = 0; x < MX; ++x) {
+            const int ex = e + x * MSTEP, row = ex / HD * 4 + jg;
+            at[x] = ex < e_end && row < M ? row_off(row) + ex % HD + el : -1;
+        }
+#pragma unroll
+        for (int x = 0; x < MX; ++x) {
+            if (e + x * MSTEP >= e_end) break;
+            float m = ml[x][0].x;
+            if constexpr (U == 4) m = fmaxf(m, ml[x][1].x);
+#pragma unroll
+            for (int off = 4; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+            const float w0 = ml[x][0].y > 0.f ? ex2(ml[x][0].x - m) : 0.f;
+            float w1 = 0.f, L = w0 * ml[x][0].y;
+            if constexpr (U == 4) {
+                w1 = ml[x][1].y > 0.f ? ex2(ml[x][1].x - m) : 0.f;
+                L = fmaf(w1, ml[x][1].y, L);
+            }
+#pragma unroll
+            for (int off = 4; off; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+            const float inv = L > 0.f ? 1.f / L : 0.f;
+            float *wx = wt + x * (JS * 4);    // weights [partial][row]
+            wx[j0 * 4 + r] = w0 * inv;
+            if constexpr (U == 4) wx[(j0 + 8) * 4 + r] = w1 * inv;
+            __syncwarp();
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float4 w = *reinterpret_cast<const float4 *>(wx + (jg + 4 * u) * 4);
+                acc.x = fmaf(w.x, v[x][u].x, acc.x); acc.y = fmaf(w.y, v[x][u].y, acc.y);
+                acc.z = fmaf(w.z, v[x][u].z, acc.z); acc.w = fmaf(w.w, v[x][u].w, acc.w);
+            }
+            // the four lane groups add up and end with a row each
+            const float2 send = jg & 1 ? make_float2(acc.x, acc.z) : make_float2(acc.y, acc.w);
+            float2 keep = jg & 1 ? make_float2(acc.y, acc.w) : make_float2(acc.x, acc.z);
+            keep.x += __shfl_xor_sync(0xffffffffu, send.x, 8);
+            keep.y += __shfl_xor_sync(0xffffffffu, send.y, 8);
+            const float give = jg & 2 ? keep.x : keep.y;
+            const float y = (jg & 2 ? keep.y : keep.x) + __shfl_xor_sync(0xffffffffu, give, 16);
+            if (at[x] >= 0) out[at[x]] = __float2bfloat16_rn(y);
+        }
+        __syncwarp();
+    }
+}
+
 template <int HD, int NR>
-__global__ void __launch_bounds__(NTHREADS, 2)
+__global__ void __launch_bounds__(NTHREADS, KeysShape<HD, NR>::CTAS)
 attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, const KeysArgs args)
 {
     using C = KeysShape<HD, NR>;
@@ -158,6 +238,8 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
     auto bar = [&](int i) { return sbase + C::OFF_BAR + i * 8; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = blockIdx.x, S = args.S, quiescent = args.quiescent;
+    // query tile: block positions [i0, i0 + kb_rows) of the unit, M rows
+    const int zt = blockIdx.z, i0 = zt * args.kb_rows, M = min(p.K - i0, args.kb_rows) * p.G;
     // element offset of query row r within the tensor rows of this unit's sequence and head group
     auto row_off = [&](int r) {
         const int i = (int)((uint32_t)r * args.inv_g >> 16);
@@ -191,24 +273,12 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
     // where this thread's query chunks (16 bytes each) come from; rows past M are zero
     constexpr int QCH = HD / 8, QN = (NR * QCH + ST - 1) / ST;
     int q_src[QN];
-    // this thread's elements of the merge: (group of four query rows, head column); a warp takes eight
-    // columns, its lane groups every fourth partial result
-    constexpr int MX = 2, MSTEP = 8 * SW;                     // elements of a lane per step, their distance
-    const int n4 = (p.M + 3) >> 2, el = lane & 7, jg = lane >> 3;
-    const int e_end = min(n4 * HD, (rank + 1) * args.slice);
-    int e_first = rank * args.slice + (warp < SW ? warp : 0) * 8, o_at[MX];
-    auto out_at = [&](int e) {                // where the result of this lane for element e goes (-1: no such row)
-        const int row = e / HD * 4 + jg;
-        return row < p.M ? row_off(row) + e % HD + el : -1;
-    };
     if (warp < SW) {
 #pragma unroll
         for (int u = 0; u < QN; ++u) {
             const int e = tid + u * ST, r = e / QCH;
-            q_src[u] = r < p.M ? row_off(r) / 8 + e % QCH : -1;
+            q_src[u] = r < M ? row_off(r) / 8 + e % QCH : -1;
         }
-#pragma unroll
-        for (int x = 0; x < MX; ++x) o_at[x] = out_at(e_first + x * MSTEP);
     }
     tc_fence_before();
     __syncthreads();
@@ -239,9 +309,9 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         P = P < 0 ? 0 : len_hi;
     }
     // the unit's halves: n_pre of 64 prefix keys, then the block's keys, shared out evenly
-    const int n_pre = (P + HALF - 1) / HALF;
-    const int a0 = (int)((long long)rank * (n_pre + 1) / S), a1 = (int)((long long)(rank + 1) * (n_pre + 1) / S);
-    const int nh = a1 - a0, n_mine = min(nh, n_pre - a0);     // halves of this CTA, prefix halves among them
+    const int n_pre = (P + HALF - 1) / HALF, n_all = n_pre + 1;
+    const int a0 = (int)((long long)rank * n_all / S), a1 = (int)((long long)(rank + 1) * n_all / S);
+    const int nh = a1 - a0, n_mine = max(0, min(nh, n_pre - a0));     // halves of this CTA, prefix halves among them
     const int n_tiles = (nh + 1) >> 1;
     const int row_base = (int)(((long long)(b / p.nb) * p.Hkv + h) * p.capacity);
     // keys of half a (CTA-local): 0 past the end
@@ -262,14 +332,14 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll
             for (int s = 0; s < PANELS; ++s) {
                 const uint32_t d = dst + s * PANEL + (a & 1) * (HALF * 128);
-                if (a < n_mine || p.blk_in_cache)             // (rows behind the keys hold anything: masked, cleared in V)
+                if (a < n_mine || p.blk_in_cache)  // (rows behind the keys hold anything: masked, cleared in V)
                     tma_load_2d(d, v ? &tm.v : &tm.k, s * 64, row_base + (a < n_mine ? (a0 + a) * HALF : P), fb, policy);
                 else                                          // rows >= K are out of bounds and arrive as zeros
                     tma_load_4d(d, v ? &tm.vb : &tm.kb, s * 64, h, 0, b, fb);
             }
         }
     };
-    const long long unit_row = ((long long)b * p.K * p.Hq + h * p.G) * HD;
+    const long long unit_row = (((long long)b * p.K + i0) * p.Hq + h * p.G) * HD;
     const uint4 *q = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.q) + unit_row);
     __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(p.out) + unit_row;
     int produced = 0;
@@ -301,18 +371,19 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         const int wg = warp >> 2, wq = warp & 3, kt = tid & 127;
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
         const uint32_t TS = lane_base + C::tm_s(wg), TO = lane_base + C::tm_o(wg);
-        unsigned char *p_buf = smem + C::OFF_P + wg * PANEL, *p_row = p_buf + kt * 128;
+        unsigned char *p_buf = smem + C::OFF_P + wg * C::P_BYTES, *p_row = p_buf + kt * 128;
         float *red = reinterpret_cast<float *>(p_buf);        // [4 warps][NR] until the probabilities take its place
         float *ref = reinterpret_cast<float *>(smem + C::OFF_REF) + wg * NR;
         const float sc = p.scale_log2;
         float m_run = -INFINITY;                              // of row kt (threads kt < NR)
-        constexpr int RP = NR / 2, LG = 32 / RP;              // row pairs, lane groups that share a warp's keys
-        float2 l_run = make_float2(0.f, 0.f);                 // of row pair lane % RP over this warp's keys
+        constexpr int PP = C::P_PANELS, RP = NR / 2 / PP, LG = 32 / RP;   // row pairs of a panel, lane groups that share a warp's keys
+        float2 l_run[PP];                                     // of row pair lane % RP of each panel over this warp's keys
+#pragma unroll
+        for (int x = 0; x < PP; ++x) l_run[x] = make_float2(0.f, 0.f);
         for (int t = wg, u = 0; t < n_tiles; t += 2, ++u) {
             const int a = 2 * t + (kt >> 6), j = kt & 63;     // this thread's half and key in it
-            const bool blk = a >= n_mine;
             // rows below lo do not see the key (all, if the key does not exist)
-            const int lo = j >= half_keys(a) ? NR : (blk && p.causal ? j * p.G : 0);
+            const int lo = j >= half_keys(a) ? NR : (a >= n_mine && p.causal ? (j - i0) * p.G : 0);
             const bool masks = __any_sync(0xffffffffu, lo > 0);
             mbar_wait_warp(bar(C::BAR_S + wg), u & 1, abort_flag);
             if (u > 0) mbar_wait_warp(bar(C::BAR_PV + wg), (u - 1) & 1, abort_flag);   // P buffer and O^T at rest
@@ -352,8 +423,11 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             }
             if (bar_group_or(wg, raised && u > 0)) {
                 // rescale what the earlier tiles have added up
-                const float2 al = *reinterpret_cast<const float2 *>(red + 2 * (lane % RP));
-                l_run.x *= al.x; l_run.y *= al.y;
+#pragma unroll
+                for (int x = 0; x < PP; ++x) {
+                    const float2 al = *reinterpret_cast<const float2 *>(red + x * 64 + 2 * (lane % RP));
+                    l_run[x].x *= al.x; l_run[x].y *= al.y;
+                }
 #pragma unroll 1
                 for (int c = 0; c < NR; c += 16) {
                     uint32_t o[16];
@@ -386,43 +460,49 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             }
 #pragma unroll
             for (int c = 0; c < NR / 8; ++c)
-                *reinterpret_cast<uint4 *>(p_row + ((c ^ (kt & 7)) << 4)) =
+                *reinterpret_cast<uint4 *>(p_row + (c >> 3) * PANEL + (((c & 7) ^ (kt & 7)) << 4)) =
                     make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
             fence_proxy_async();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(C::BAR_P + wg));
             // while the product runs: the sums of this warp's 32 keys, lane = row pair
-            {
+#pragma unroll
+            for (int pn = 0; pn < PP; ++pn) {
                 const int rp = lane % RP;
                 float2 l0 = make_float2(0.f, 0.f), l1 = l0;
 #pragma unroll 8
                 for (int k = lane / RP; k < 32; k += 2 * LG) {
-                    const uint32_t x = *reinterpret_cast<const uint32_t *>(p_buf + (wq * 32 + k) * 128 +
+                    const uint32_t x = *reinterpret_cast<const uint32_t *>(p_buf + pn * PANEL + (wq * 32 + k) * 128 +
                                                                            (((rp >> 2) ^ (k & 7)) << 4) + (rp & 3) * 4);
                     const int k2 = k + LG;
-                    const uint32_t y = *reinterpret_cast<const uint32_t *>(p_buf + (wq * 32 + k2) * 128 +
+                    const uint32_t y = *reinterpret_cast<const uint32_t *>(p_buf + pn * PANEL + (wq * 32 + k2) * 128 +
                                                                            (((rp >> 2) ^ (k2 & 7)) << 4) + (rp & 3) * 4);
                     l0.x += __uint_as_float(x << 16); l0.y += __uint_as_float(x & 0xffff0000u);
                     l1.x += __uint_as_float(y << 16); l1.y += __uint_as_float(y & 0xffff0000u);
                 }
-                l_run.x += l0.x + l1.x; l_run.y += l0.y + l1.y;
+                l_run[pn].x += l0.x + l1.x; l_run[pn].y += l0.y + l1.y;
             }
         }
         // ------------------------------------------------------------------ weights of the two warpgroups
 #pragma unroll
-        for (int off = RP; off < 32; off <<= 1) {
-            l_run.x += __shfl_xor_sync(0xffffffffu, l_run.x, off);
-            l_run.y += __shfl_xor_sync(0xffffffffu, l_run.y, off);
-        }
+        for (int off = RP; off < 32; off <<= 1)
+#pragma unroll
+            for (int x = 0; x < PP; ++x) {
+                l_run[x].x += __shfl_xor_sync(0xffffffffu, l_run[x].x, off);
+                l_run[x].y += __shfl_xor_sync(0xffffffffu, l_run[x].y, off);
+            }
         // the query rows have served: their place takes the tables
         float *t_l = reinterpret_cast<float *>(smem + C::OFF_Q);              // [8 warps][NR] sums
         float *t_m = t_l + 8 * NR, *t_w = t_m + 2 * NR;                       // [2][NR] references, weights
         static_assert((8 + 4) * NR * 4 <= C::END_Q - C::OFF_Q, "tables");
-        const long long cta = (long long)blockIdx.y * S + rank;
+        const int n4 = (M + 3) >> 2;                          // groups of four rows
+        const long long cta0 = ((long long)zt * gridDim.y + blockIdx.y) * S, cta = cta0 + rank;
         if (n_tiles > 0) mbar_wait_warp(bar(C::BAR_QKALL), 0, abort_flag);
         else bar_pair();                                      // (no product reads them: every warp has written its own)
-        if (lane < RP) *reinterpret_cast<float2 *>(t_l + warp * NR + 2 * lane) = l_run;
+        if (lane < RP)
+#pragma unroll
+            for (int x = 0; x < PP; ++x) *reinterpret_cast<float2 *>(t_l + warp * NR + x * 64 + 2 * lane) = l_run[x];
         if (kt < NR) t_m[wg * NR + kt] = m_run;
         bar_pair();
         if (tid < NR) {
@@ -476,76 +556,21 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll
                 for (int i = 0; i < CW; ++i) {
                     const float4 y = x[i / 4];
-                    if (c + i < p.M)
+                    if (c + i < M)
                         out[row_off(c + i) + d] = __float2bfloat16_rn(i % 4 == 0 ? y.x : i % 4 == 1 ? y.y : i % 4 == 2 ? y.z : y.w);
                 }
             }
         }
         tc_fence_before();
         if (S > 1) {
-            // -------------------------------------------------------------- merge: no barrier but the cluster's
-            float *wt = reinterpret_cast<float *>(smem) + warp * 128;        // this warp's weights [2][16 CTAs][4 rows]
-            const long long cta0 = (long long)blockIdx.y * S;
-            const float4 *po = reinterpret_cast<const float4 *>(p.part_o) + cta0 * (NR / 4 * HD) + (e_first + el) +
-                               (long long)jg * (NR / 4 * HD);
+            float *wt = reinterpret_cast<float *>(smem) + warp * 256;
+            const float4 *po = reinterpret_cast<const float4 *>(p.part_o) + cta0 * (NR / 4 * HD);
             const float2 *pml = reinterpret_cast<const float2 *>(p.part_ml) + cta0 * NR;
             cluster_sync_all();
-            // all loads of a step are requested together
-            for (; e_first < e_end; e_first += MX * MSTEP, po += MX * MSTEP) {
-                const int r = lane >> 3, j0 = lane & 7;
-                float2 ml[MX][2];
-                float4 v[MX][4];
-#pragma unroll
-                for (int x = 0; x < MX; ++x) {
-                    // rows 4g..4g+3 of the element's group g: lane = (row, partial) twice
-                    const int row = (e_first + x * MSTEP) / HD * 4 + r;
-                    const bool live = e_first + x * MSTEP < e_end;
-                    ml[x][0] = ml[x][1] = make_float2(-INFINITY, 0.f);
-                    if (live && row < p.M) {
-                        if (j0 < S) ml[x][0] = __ldcg(pml + j0 * NR + row);
-                        if (j0 + 8 < S) ml[x][1] = __ldcg(pml + (j0 + 8) * NR + row);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        v[x][u] = live && jg + 4 * u < S ? __ldcg(po + x * MSTEP + u * (4 * (NR / 4 * HD))) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-#pragma unroll
-                for (int x = 0; x < MX; ++x) {
-                    if (e_first + x * MSTEP >= e_end) break;
-                    float M = fmaxf(ml[x][0].x, ml[x][1].x);
-#pragma unroll
-                    for (int off = 4; off; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-                    const float w0 = ml[x][0].y > 0.f ? ex2(ml[x][0].x - M) : 0.f, w1 = ml[x][1].y > 0.f ? ex2(ml[x][1].x - M) : 0.f;
-                    float L = fmaf(w0, ml[x][0].y, w1 * ml[x][1].y);
-#pragma unroll
-                    for (int off = 4; off; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
-                    const float inv = L > 0.f ? 1.f / L : 0.f;
-                    float *wx = wt + x * 64;
-                    wx[j0 * 4 + r] = w0 * inv;
-                    wx[(j0 + 8) * 4 + r] = w1 * inv;
-                    __syncwarp();
-                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float4 w = *reinterpret_cast<const float4 *>(wx + (jg + 4 * u) * 4);
-                        acc.x = fmaf(w.x, v[x][u].x, acc.x); acc.y = fmaf(w.y, v[x][u].y, acc.y);
-                        acc.z = fmaf(w.z, v[x][u].z, acc.z); acc.w = fmaf(w.w, v[x][u].w, acc.w);
-                    }
-                    // the four lane groups add up and end with a row each
-                    const float2 send = jg & 1 ? make_float2(acc.x, acc.z) : make_float2(acc.y, acc.w);
-                    float2 keep = jg & 1 ? make_float2(acc.y, acc.w) : make_float2(acc.x, acc.z);
-                    keep.x += __shfl_xor_sync(0xffffffffu, send.x, 8);
-                    keep.y += __shfl_xor_sync(0xffffffffu, send.y, 8);
-                    const float give = jg & 2 ? keep.x : keep.y;
-                    const float y = (jg & 2 ? keep.y : keep.x) + __shfl_xor_sync(0xffffffffu, give, 16);
-                    if (o_at[x] >= 0) out[o_at[x]] = __float2bfloat16_rn(y);
-                }
-                if (e_first + MX * MSTEP < e_end) {
-#pragma unroll
-                    for (int x = 0; x < MX; ++x) o_at[x] = out_at(e_first + (MX + x) * MSTEP);
-                    __syncwarp();
-                }
-            }
+            const int e0 = rank * args.slice, e1 = min(n4 * HD, e0 + args.slice);
+            if (S <= 4) merge<HD, NR, 1>(po, pml, wt, e0, e1, M, S, out, row_off);
+            else if (S <= 8) merge<HD, NR, 2>(po, pml, wt, e0, e1, M, S, out, row_off);
+            else merge<HD, NR, 4>(po, pml, wt, e0, e1, M, S, out, row_off);
             return;
         }
     } else if (warp == PRODUCER_WARP) {
@@ -611,7 +636,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             if (!mbar_wait_warp(bar(C::BAR_P + w), (t >> 1) & 1, abort_flag)) return false;
             tc_fence_after();
             if (elect_one()) {
-                const uint32_t v_addr = sbase + C::OFF_RING + slot * C::KV_BYTES, p_addr = sbase + C::OFF_P + w * PANEL;
+                const uint32_t v_addr = sbase + C::OFF_RING + slot * C::KV_BYTES, p_addr = sbase + C::OFF_P + w * C::P_BYTES;
                 const int g0 = (k0 + 15) >> 4, g1 = (k1 + 15) >> 4;
 #pragma unroll
                 for (int g = 0; g < 8; ++g)
@@ -687,11 +712,12 @@ template <int HD, int NR> int resident_clusters(int S)
     constexpr int kMaxDevices = 64;
     static std::atomic<int> cached[kMaxDevices][MAX_CLUSTER + 1];
     int dev = 0;
-    if (configure<HD, NR>(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 2 * kDefaultSMs / S; }
+    constexpr int CTAS = KeysShape<HD, NR>::CTAS;
+    if (configure<HD, NR>(&dev) != cudaSuccess) { (void)cudaGetLastError(); return CTAS * kDefaultSMs / S; }
     int n = cached[dev][S].load(std::memory_order_relaxed);
     if (n != 0) return n > 0 ? n : 0;
     cudaLaunchConfig_t cfg = {};
-    const int sms = (S + 1) / 2;
+    const int sms = (S + CTAS - 1) / CTAS;
     cfg.gridDim = dim3(sms, 1);
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = KeysShape<HD, NR>::SMEM_BYTES;
@@ -704,29 +730,31 @@ template <int HD, int NR> int resident_clusters(int S)
         (void)cudaGetLastError();
         n = sms <= 8 ? num_sms() / sms : 0;       // a size the device cannot schedule is not chosen
     }
-    if (S == 1) n *= 2;
+    if (S == 1) n *= CTAS;
     cached[dev][S].store(n < 1 ? -1 : n, std::memory_order_relaxed);
     return n;
 }
 
-// CTAs per unit.  A CTA's time is that of its tiles one after the other, except that the two
-// warpgroups take two side by side; a second wave of clusters costs more than any split gains.  So:
-// the fewest tiles, but no fewer than two, among the sizes at which all units are resident together.
-// Of sizes with the same number of tiles the largest up to 8 (lengths are often below the bound the
-// plan is made for, and then the larger size has fewer), else the smallest (sizes above 8 were up to
-// 1 us slower at the same number of tiles).  Measured per call, bf16, d = 128: 16 units of 61 halves
-// 8.5 us at 11 CTAs (3 tiles), 10.0 at 8 (4), 13.7 at 14 (second wave); 8 units of 63 halves 9.9 us at
-// 16 (2 tiles), 12.3 at 15 (3); 256 units 82 us at 1, 106 at 2; d = 64, 10 units of 25 halves 7.0 us
-// at 8, 7.8 at 10.
+// CTAs per unit.  A CTA's time is that of its tiles one after the other; a merge costs as much as one
+// tile and, for what it moves, up to two more; a second wave of clusters costs more than any split
+// gains.  So: the cheapest by that count among the sizes at which all units are resident together.
+// Of sizes that cost the same the largest up to 8 (lengths are often below the bound the plan is
+// made for, and then the larger size has fewer tiles), else the smallest; above 10 a single tile per
+// CTA gains nothing over two.  Measured per call, chained in a graph, lengths 0.7 to 1 times the bound:
+// d = 128, 64 rows: 8 units, bound 150, 7.3 us at 1 CTA, 11.5 at 2; bound 2000, 9.1 us at 10, 10.1 at 8;
+// bound 4000, 10.7 us at 16, 12.0 at 8; 128 units, bound 400, 13.2 us at 1, 16.5 at 2; 256 units,
+// bound 2000, 46.5 us at 1, 61 at 2; 4 rows: 8 units, bound 400, 5.2 us at 5, 7.4 at 1; bound 4000,
+// 7.6 at 16, 9.5 at 8; d = 64, 32 rows: 2 units, bound 1000, 5.2 us at 10, 5.8 at 8, 11.8 at 1.
 template <int HD, int NR> int choose_splits(int units, int halves)
 {
-    int best = 1, best_tiles = 1 << 30;
+    int best = 1, best_cost = 1 << 30;
     for (int S = 1; S <= MAX_CLUSTER && S <= halves; ++S) {
-        const int tiles = max(2, ((halves + S - 1) / S + 1) / 2);
-        if (S <= 8 ? tiles > best_tiles : tiles >= best_tiles) continue;
+        const int tiles = max(S <= 10 ? 1 : 2, ((halves + S - 1) / S + 1) / 2);
+        const int cost = 2 * tiles + (S > 1 ? 2 + NR * HD / 2048 : 0);
+        if (S <= 8 ? cost > best_cost : cost >= best_cost) continue;
         if (S > 1 && units > resident_clusters<HD, NR>(S)) continue;
         best = S;
-        best_tiles = tiles;
+        best_cost = cost;
     }
     return best;
 }
@@ -739,9 +767,9 @@ cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cud
     int dev = 0;
     cudaError_t e = configure<HD, NR>(&dev);
     if (e != cudaSuccess) return e;
-    const int S = p.n_splits, units = p.B * p.Hkv;
+    const int S = p.n_splits, units = p.B * p.Hkv, kb = tc_kb_rows(p.G, p.K), tiles = (p.K + kb - 1) / kb;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S, units);
+    cfg.gridDim = dim3(S, units, tiles);
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = C::SMEM_BYTES;
     cfg.stream = st;
@@ -762,9 +790,10 @@ cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cud
     KeysArgs args;
     args.S = S;
     args.quiescent = (flags & ORTHRUS_LAYER_CACHE_QUIESCENT) ? 1 : 0;
-    args.ranked = units * S > 2 * num_sms() && p.B > 1 && p.B <= 128;
+    args.ranked = units * tiles * S > C::CTAS * num_sms() && p.B > 1 && p.B <= 128;
     args.inv_g = (65536u + p.G - 1) / p.G;
-    args.slice = (((p.M + 3) / 4 * HD + S - 1) / S + 7) & ~7;
+    args.slice = (((kb * p.G + 3) / 4 * HD + S - 1) / S + 7) & ~7;
+    args.kb_rows = kb;
     e = cudaLaunchKernelEx(&cfg, kern, p, tm, args);
     count_launch();
     return e;
@@ -773,30 +802,38 @@ cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cud
 template <int HD>
 cudaError_t launch_rows(const AttnParams &p, const KeysMaps &tm, int flags, cudaStream_t st)
 {
-    switch (keys_rows(p.M)) {
+    switch (keys_rows(HD, p.G, p.K)) {
     case 16: return launch_shape<HD, 16>(p, tm, flags, st);
     case 32: return launch_shape<HD, 32>(p, tm, flags, st);
-    default: return launch_shape<HD, 64>(p, tm, flags, st);
+    case 64: return launch_shape<HD, 64>(p, tm, flags, st);
     }
+    if constexpr (HD == 64) return launch_shape<HD, 128>(p, tm, flags, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-// columns of the MMA that M query rows take (0: too many)
-int keys_rows(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 0; }
+// columns of the MMA that a unit's query rows take (0: not a shape of this kernel)
+int keys_rows(int d, int G, int K)
+{
+    const int M = G * K;
+    if (d == 64 && M > 64) return G <= 128 ? 128 : 0;
+    return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 0;
+}
 
-int keys_splits(int d, int M, int units, int max_keys)
+int keys_splits(int d, int G, int K, int units, int max_keys)
 {
     // the layers of a pass ask the same question: the last answer of this thread is kept
     struct Key { int dev, d, nr, units, halves, S; };
     static thread_local Key last = {-1, 0, 0, 0, 0, 0};
-    Key k = {-1, d, keys_rows(M), units, (max_keys + HALF - 1) / HALF, 0};
+    Key k = {-1, d, keys_rows(d, G, K), units, (max_keys + HALF - 1) / HALF + 1, 0};   // (prefix and block in halves of their own)
     if (cudaGetDevice(&k.dev) != cudaSuccess) { (void)cudaGetLastError(); k.dev = -2; }
     if (k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.units == last.units && k.halves == last.halves) return last.S;
     switch (k.nr) {
     case 16: k.S = d == 64 ? choose_splits<64, 16>(units, k.halves) : choose_splits<128, 16>(units, k.halves); break;
     case 32: k.S = d == 64 ? choose_splits<64, 32>(units, k.halves) : choose_splits<128, 32>(units, k.halves); break;
-    default: k.S = d == 64 ? choose_splits<64, 64>(units, k.halves) : choose_splits<128, 64>(units, k.halves);
+    case 64: k.S = d == 64 ? choose_splits<64, 64>(units, k.halves) : choose_splits<128, 64>(units, k.halves); break;
+    default: k.S = choose_splits<64, 128>(units, k.halves);
     }
     last = k;
     return k.S;

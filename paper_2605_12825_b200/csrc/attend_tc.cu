@@ -769,7 +769,7 @@ bool tensor_map(const void *ptr, unsigned hd, unsigned long long d1, unsigned lo
 }
 
 // block positions per query tile of 128 rows
-static int tc_kb_rows(int G, int K) { return K < MROWS / G ? K : MROWS / G; }
+int tc_kb_rows(int G, int K) { return K < MROWS / G ? K : MROWS / G; }
 
 int tc_row_tiles(int G, int K)
 {

@@ -1,5 +1,5 @@
-"""The kernel for units of few query rows (bf16, "auto" path): up to 64 rows at head_dim 64 and 128.
-Edges of its row counts (16, 32, 64), of its key tiles, of the cluster split (CTAs without a
+"""The kernel with the keys on the MMA's rows (bf16, "auto" path), head_dim 64 and 128.
+Edges of its row counts (16, 32, 64, 128, several tiles of 128), of its key tiles, of the cluster split (CTAs without a
 tile included), both masks, the block as a tensor and in the cache, NaN behind the keys."""
 import pytest
 import torch
@@ -10,9 +10,10 @@ from _gpu_util import Guarded, assert_close, binding, oracle_attend, run_attend,
 
 pytestmark = pytest.mark.gpu
 VIEWS = [oracle.VIEW_DIFFUSION, oracle.VIEW_AR]
-# (Hq, Hkv, head_dim, K): 1, 4, 16, 17, 32, 33, 49 and 64 query rows
+# (Hq, Hkv, head_dim, K): 1, 4, 16, 17, 32, 33, 49, 64, then 72, 128, 129 and 320 query rows
 SHAPES = [(2, 2, 64, 1), (8, 2, 64, 1), (8, 2, 64, 4), (3, 3, 64, 17), (8, 2, 64, 8), (3, 1, 64, 11), (14, 2, 64, 7), (4, 2, 64, 32),
-          (1, 1, 128, 1), (8, 2, 128, 1), (8, 2, 128, 4), (2, 2, 128, 17), (16, 4, 128, 8), (7, 1, 128, 4)]
+          (1, 1, 128, 1), (8, 2, 128, 1), (8, 2, 128, 4), (2, 2, 128, 17), (16, 4, 128, 8), (7, 1, 128, 4),
+          (8, 1, 128, 9), (8, 2, 64, 32), (16, 2, 128, 16), (3, 1, 128, 43), (10, 2, 64, 64)]
 NAN = float("nan")
 
 
@@ -38,7 +39,8 @@ def test_shapes_and_splits(view, shape, splits):
         assert_close(got, oracle_attend(view, t), torch.bfloat16, f"{shape} lens={lens} splits={splits}")
 
 
-@pytest.mark.parametrize("shape", [(14, 2, 64, 7), (8, 2, 64, 1), (8, 2, 128, 1), (16, 4, 128, 8)])
+@pytest.mark.parametrize("shape", [(14, 2, 64, 7), (8, 2, 64, 1), (8, 2, 128, 1), (16, 4, 128, 8), (8, 2, 128, 20),
+                                   (3, 1, 128, 43)])
 @pytest.mark.parametrize("view", VIEWS)
 def test_block_in_the_cache(view, shape):
     b = binding()
@@ -61,7 +63,7 @@ def test_block_in_the_cache(view, shape):
         assert_close(out.t.cpu(), ref, torch.bfloat16, f"{shape} {lens}")
 
 
-@pytest.mark.parametrize("shape", [(16, 4, 64, 8), (32, 8, 128, 1)])
+@pytest.mark.parametrize("shape", [(16, 4, 64, 8), (32, 8, 128, 1), (32, 8, 128, 32)])
 def test_many_units_of_unequal_length(shape):
     """More clusters than fit at once: handed out longest prefix first; peaked scores move the running maximum."""
     lens = [int(x) for x in torch.randint(0, 3000, (40,), generator=torch.Generator().manual_seed(3))]
