@@ -145,11 +145,6 @@ template <int N> __device__ inline void tmem_ld(uint32_t addr, uint32_t *r) {
 __host__ __device__ constexpr uint32_t keys_idesc(uint32_t n, uint32_t a_mn, uint32_t b_mn) {
     return make_idesc(n, b_mn) | (a_mn << 15);
 }
-__device__ inline bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
-    return p != 0;
-}
 
 // A CTA's share [e, e_end) of the merge of S <= 4 U partial results, an element being a head column of
 // a group of four rows; called by each softmax warp, no barrier.  A warp takes eight columns at a time,

@@ -596,20 +596,18 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
         const int ti = warp - C::MMA_WARP;
         constexpr uint32_t IDESC_QK = make_idesc(TN, 0);      // A = Q, B = K tile, both K-major
         constexpr uint32_t IDESC_PV = make_idesc(HD, 1);      // A = P (TMEM), B = V tile (MN-major)
-        const uint32_t q_addr = sbase + OFF_Q + ti * 2 * QSUB_BYTES;
+        const uint64_t q_desc = make_desc(sbase + OFF_Q + ti * 2 * QSUB_BYTES, 16, 1024);
         auto issue_qk = [&](int t) -> bool {
             const int j = item_of_k(t), slot = slot_of(j);
             if (!mbar_wait_warp(bar(BAR_FULL + slot), use_of(j) & 1, abort_flag)) return false;
             tc_fence_after();
-            if (lane == 0) {
-                const uint32_t k_addr = sbase + OFF_RING + slot * SLOT_BYTES;
+            if (elect_one()) {
+                const uint64_t kd = make_desc(sbase + OFF_RING + slot * SLOT_BYTES, 16, 1024);
+                const uint32_t d = tmem + C::tm_s(ti, t & 1);
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {        // 16 head-dim columns per MMA
-                    umma_ss(tmem + C::tm_s(ti, t & 1),
-                            make_desc(q_addr + (kk >> 2) * QSUB_BYTES + (kk & 3) * 32, 16, 1024),
-                            make_desc(k_addr + (kk >> 2) * SUB_BYTES + (kk & 3) * 32, 16, 1024),
-                            IDESC_QK, kk > 0);
-                }
+                for (int kk = 0; kk < HD / 16; ++kk)          // 16 head-dim columns per MMA
+                    umma_ss(d, q_desc + (((kk >> 2) * QSUB_BYTES + (kk & 3) * 32) >> 4),
+                            kd + (((kk >> 2) * SUB_BYTES + (kk & 3) * 32) >> 4), IDESC_QK, kk > 0);
                 umma_commit(bar(BAR_EMPTY + slot));
                 umma_commit(bar(C::BAR_SFULL + ti * 2 + (t & 1)));
             }
@@ -639,14 +637,13 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
             }
             if (!mbar_wait_warp(bar(C::BAR_PFULL + ti * 2 + (t & 1)), (t >> 1) & 1, abort_flag)) return false;
             tc_fence_after();
-            if (lane == 0) {
-                const uint32_t v_addr = sbase + OFF_RING + slot * SLOT_BYTES;
+            if (elect_one()) {
+                const uint64_t vd = make_desc(sbase + OFF_RING + slot * SLOT_BYTES, SUB_BYTES, 1024);
+                const uint32_t a = tmem + C::tm_s(ti, t & 1);
 #pragma unroll
-                for (int kk = 0; kk < TN / 16; ++kk) {        // 16 key positions per MMA
-                    if (kk >= n_kk) break;
-                    umma_ts(tmem + C::tm_o(ti), tmem + C::tm_s(ti, t & 1) + kk * 8,
-                            make_desc(v_addr + kk * 2048, SUB_BYTES, 1024), IDESC_PV, (t > 0) || (kk > 0));
-                }
+                for (int kk = 0; kk < TN / 16; ++kk)          // 16 key positions per MMA
+                    if (kk < n_kk)
+                        umma_ts(tmem + C::tm_o(ti), a + kk * 8, vd + (kk * 2048 >> 4), IDESC_PV, (t > 0) || (kk > 0));
                 umma_commit(bar(BAR_EMPTY + slot));
                 umma_commit(bar(C::BAR_PVDONE + ti));
                 if (t == n_tiles - 1) umma_commit(bar(C::BAR_ALLDONE + ti));

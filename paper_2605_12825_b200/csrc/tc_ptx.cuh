@@ -119,6 +119,13 @@ __device__ inline void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uin
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc) : "memory");
 }
+// true in one lane of a converged warp, the same one each time.  (Behind a test of the lane index
+// the compiler moves the operands of every tcgen05.mma to uniform registers lane by lane.)
+__device__ inline bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
 __device__ inline void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  ::"r"(bar) : "memory");
