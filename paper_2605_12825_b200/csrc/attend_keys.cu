@@ -124,23 +124,6 @@ __device__ inline bool bar_group_or(int wg, bool pred) {
                      " selp.u32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((uint32_t)pred) : "memory");
     return r != 0;
 }
-// N consecutive columns of this thread's lane, no wait
-template <int N> __device__ inline void tmem_ld(uint32_t addr, uint32_t *r) {
-    static_assert(N == 8 || N == 16 || N % 32 == 0, "");
-    if constexpr (N >= 32)
-#pragma unroll
-        for (int c = 0; c < N; c += 32) tmem_ld32(addr + c, r + c);
-    else if constexpr (N == 16)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                     "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                       "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                     : "r"(addr));
-    else
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(addr));
-}
 // D fp32, A and B bf16, M = 128, N = n; bit 15 / 16: A / B is MN-major
 __host__ __device__ constexpr uint32_t keys_idesc(uint32_t n, uint32_t a_mn, uint32_t b_mn) {
     return make_idesc(n, b_mn) | (a_mn << 15);

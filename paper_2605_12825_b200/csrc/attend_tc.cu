@@ -98,6 +98,8 @@ template <int NT> struct Shape {
 };
 static_assert(2 * (Shape<1>::SMEM_BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
 static_assert(Shape<2>::SMEM_BYTES <= 227 * 1024, "one CTA per SM");
+constexpr int EXCHANGE_BYTES = 72 * 1024;                 // of the ring per query tile, in the merge
+static_assert(Shape<1>::NSLOT * SLOT_BYTES >= EXCHANGE_BYTES && Shape<2>::NSLOT * SLOT_BYTES >= 2 * EXCHANGE_BYTES, "merge");
 constexpr float RESCALE_THRESHOLD = 8.f;                  // log2 units
 struct TcMaps { CUtensorMap k, v, q, kb, vb; };
 
@@ -177,6 +179,76 @@ __device__ __noinline__ void merge_tile(int S, int rank, int warp, int lane, int
     else run(std::integral_constant<int, 16>());
 }
 
+// The merge of clusters of SP = 2, 4 or 8, through distributed shared memory: CTA q ends with columns
+// [q W, q W + W) of all rows, W = 128 / SP.  Each softmax thread (one query row) sends the other CTAs
+// their columns of its row, as 16-byte chunks [source][chunk][row] so that a warp's store is 512
+// contiguous bytes, into the ring, which every CTA has done with; then it sums up what it got.
+// Called by the softmax warps between the cluster's two barriers, the second of which is in here.
+template <int SP>
+__device__ inline void exchange_merge(uint32_t tm_row, const unsigned char *buf, int rank, int r, bool valid, bool have_o,
+                                      float m, float l, __nv_bfloat16 *out_row)
+{
+    constexpr int W = HD / SP, SRC = W / 4 * MROWS * 16;      // bytes a source sends
+    static_assert(SP * SRC + SP * MROWS * 8 <= EXCHANGE_BYTES, "exchange buffer");
+    if (!have_o) { m = -INFINITY; l = 0.f; }
+#pragma unroll 1
+    for (int k = 1; k < SP; ++k) {
+        const int q = (rank + k) & (SP - 1);
+        uint32_t o[W];
+        tmem_ld<W>(tm_row + q * W, o);
+        tmem_ld_wait();
+        const uint32_t dst = map_to_rank(smem_u32(buf), q);
+        if (valid) {
+            st_cluster(dst + SP * SRC + (rank * MROWS + r) * 8, m, l);
+            if (have_o) {
+#pragma unroll
+                for (int c = 0; c < W / 4; ++c) st_cluster(dst + rank * SRC + (c * MROWS + r) * 16, o + 4 * c);
+            }
+        }
+    }
+    uint32_t o[W];
+    tmem_ld<W>(tm_row + rank * W, o);
+    tmem_ld_wait();
+    tc_fence_before();
+    cluster_sync_all();
+    if (!valid) return;
+    float2 ml[SP];
+    float mmax = m, L = 0.f;
+#pragma unroll
+    for (int j = 0; j < SP; ++j) {
+        ml[j] = j == rank ? make_float2(m, l) : *reinterpret_cast<const float2 *>(buf + SP * SRC + (j * MROWS + r) * 8);
+        mmax = fmaxf(mmax, ml[j].x);
+    }
+    const float w_own = l > 0.f ? ex2(m - mmax) : 0.f;
+#pragma unroll
+    for (int i = 0; i < W; ++i) o[i] = l > 0.f ? __float_as_uint(w_own * __uint_as_float(o[i])) : 0u;
+#pragma unroll
+    for (int j = 0; j < SP; ++j) {
+        if (!(ml[j].y > 0.f)) continue;                       // a CTA without keys sent no row
+        const float w = ex2(ml[j].x - mmax);
+        L = fmaf(w, ml[j].y, L);
+        if (j == rank) continue;
+#pragma unroll
+        for (int c = 0; c < W / 4; ++c) {
+            const float4 x = *reinterpret_cast<const float4 *>(buf + j * SRC + (c * MROWS + r) * 16);
+            o[4 * c] = __float_as_uint(fmaf(w, x.x, __uint_as_float(o[4 * c])));
+            o[4 * c + 1] = __float_as_uint(fmaf(w, x.y, __uint_as_float(o[4 * c + 1])));
+            o[4 * c + 2] = __float_as_uint(fmaf(w, x.z, __uint_as_float(o[4 * c + 2])));
+            o[4 * c + 3] = __float_as_uint(fmaf(w, x.w, __uint_as_float(o[4 * c + 3])));
+        }
+    }
+    const float inv = 1.f / L;
+#pragma unroll
+    for (int i = 0; i < W; i += 8) {
+        uint4 w;
+        w.x = pack_bf16(__uint_as_float(o[i]) * inv, __uint_as_float(o[i + 1]) * inv);
+        w.y = pack_bf16(__uint_as_float(o[i + 2]) * inv, __uint_as_float(o[i + 3]) * inv);
+        w.z = pack_bf16(__uint_as_float(o[i + 4]) * inv, __uint_as_float(o[i + 5]) * inv);
+        w.w = pack_bf16(__uint_as_float(o[i + 6]) * inv, __uint_as_float(o[i + 7]) * inv);
+        reinterpret_cast<uint4 *>(out_row + rank * W)[i / 8] = w;
+    }
+}
+
 // Thread r of a softmax warpgroup owns query row r of its tile (TMEM lane r) and all 64 columns of
 // a key tile.  blockIdx.z counts groups of NT query tiles; warpgroup ti works on tile z * NT + ti.
 //
@@ -213,6 +285,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     const int zt = PACK ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
     auto tile_i0 = [&](int ti) { return (zt * NT + ti) * kb_rows; };
     auto tile_rows = [&](int ti) { return max(0, min(p.K - tile_i0(ti), kb_rows)) * p.G; };
+    const bool exchange = S == 2 || S == 4 || S == 8;         // how the cluster merges
     const bool aligned = (sbase & 1023u) == 0;                // swizzled tiles need 1 KB alignment
 
     // ------------------------------------------------------------------ prologue
@@ -529,6 +602,15 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                     }
                 }
             }
+        } else if (exchange) {
+            cluster_sync_all();                               // every CTA is through with its ring
+            tc_fence_after();
+            const unsigned char *buf = smem + OFF_RING + ti * EXCHANGE_BYTES;
+            __nv_bfloat16 *row = static_cast<__nv_bfloat16 *>(p.out) + (((long long)b * p.K + i_row) * p.Hq + h * p.G + r % p.G) * HD;
+            const uint32_t tm_row = lane_base + TM_O;
+            if (S == 2) exchange_merge<2>(tm_row, buf, rank, r, valid, have_o, m_run, l_run, row);
+            else if (S == 4) exchange_merge<4>(tm_row, buf, rank, r, valid, have_o, m_run, l_run, row);
+            else exchange_merge<8>(tm_row, buf, rank, r, valid, have_o, m_run, l_run, row);
         } else {
             // ---------------------------------------------------------- partial rows to the workspace
             // straight from the registers of the TMEM read-out: element (chunk c, row r) of this
@@ -672,6 +754,18 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     }
 
     // ---------------------------------------------------------------------- merge
+    if (exchange) {
+        if (warp >= 4 * NT) {
+            __syncwarp();
+            cluster_sync_all();
+            cluster_sync_all();                               // the softmax warps have read their TMEM
+            tc_fence_after();
+            if (warp == C::MMA_WARP)
+                asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TM_COLS) : "memory");
+            if (warp == C::MMA_WARP && lane == 0 && *abort_flag && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
+        }
+        return;
+    }
     __syncthreads();
     tc_fence_after();
     if (warp == C::MMA_WARP)
