@@ -174,7 +174,10 @@ cudaError_t launch_consensus_finalize(const ArgPart *parts, int n_seg, const int
 int consensus_segments(int B, int K, int V)
 {
     const long long rows = (long long)B * K;
-    long long want = (4LL * num_sms() + rows - 1) / rows;          // enough CTAs to fill the GPU
+    // Enough CTAs to fill the GPU.  Many rows: three each, more than fit at once.  CTAs placed early, while the
+    // preceding kernel still holds part of the SMs, are spread unevenly, and only a second wave evens that
+    // out (1024 rows of 128256: 82 us at one each, 64 at three).
+    long long want = rows > 4LL * num_sms() ? 3 : (4LL * num_sms() + rows - 1) / rows;
     const long long max_by_len = (V + 2047) / 2048;              // at least 2048 logits each
     if (want > max_by_len) want = max_by_len;
     if (want < 1) want = 1;
