@@ -165,7 +165,12 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
         if (forced > 0) {
             S = forced;
         } else if (units * 2 <= slots) {
-            while (S < 16 && units * S * 2 <= slots && tiles / (S * 2) >= kn.min_chunk_tiles) S *= 2;
+            // Up to four CTAs for a tile each where they leave most SMs idle (8 units of 300 keys 7.6 us
+            // a call at 4, 8.1 at 2).  Sixteen only with an SM for each CTA: clusters of that size do not
+            // fill the second places (16 units of 4000 keys 16.2 us at 8, 23.2 at 16; of 16000 keys
+            // 40 and 45), and their merge goes through L2.
+            while (S < 16 && units * S * 2 <= (S == 8 ? num_sms() : slots) &&
+                   tiles / (S * 2) >= (S < 4 && units * 8 <= num_sms() ? 1 : kn.min_chunk_tiles)) S *= 2;
         } else {
             // (a lone CTA streams slower than an SM's share of HBM, so the longest unit is
             //  still split; many small CTAs would spend their time starting and merging)
