@@ -471,7 +471,7 @@ attend_tc_stream_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, c
                 const int j = jg0 + item_of_k(t), slot = j % NSLOT, tg = tg0 + t;
                 if (!mbar_wait_warp(bar(BAR_FULL + slot), (j / NSLOT) & 1, abort_flag)) return false;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t k_addr = sbase + OFF_RING + slot * SLOT_BYTES;
 #pragma unroll
                     for (int kk = 0; kk < HD / 16; ++kk) {    // 16 head-dim columns per MMA
@@ -507,7 +507,7 @@ attend_tc_stream_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, c
                 if (t == 0 && pcidx > 0 && !mbar_wait_warp(bar(SBAR_OFREE), (pcidx - 1) & 1, abort_flag)) return false;
                 if (!mbar_wait_warp(bar(BAR_PFULL + (tg & 1)), (tg >> 1) & 1, abort_flag)) return false;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t v_addr = sbase + OFF_RING + slot * SLOT_BYTES;
 #pragma unroll
                     for (int kk = 0; kk < TN / 16; ++kk) {    // 16 key positions per MMA
@@ -534,7 +534,7 @@ attend_tc_stream_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, c
         // every MMA must have retired before TMEM is freed
         if (ok && pcidx > 0) ok = mbar_wait_warp(bar(BAR_ALLDONE), (pcidx - 1) & 1, abort_flag);
         if (!ok) {                            // a wait gave up: the MMAs in flight end before TMEM is freed
-            if (lane == 0) umma_commit(bar(C::BAR_DRAIN));
+            if (elect_one()) umma_commit(bar(C::BAR_DRAIN));
             __syncwarp();
             int dummy = 0;
             mbar_wait_warp(bar(C::BAR_DRAIN), 0, &dummy);

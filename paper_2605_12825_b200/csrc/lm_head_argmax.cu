@@ -183,7 +183,8 @@ lm_head_argmax_kernel(const __grid_constant__ HeadMaps tm, const int R, const in
                 const int stage = g % NSTAGE, suse = g / NSTAGE;
                 ok = mbar_wait_warp(bar(BAR_FULL + stage), suse & 1, abort_flag);
                 if (!ok) break;
-                const uint32_t x_addr = sbase + stage * STAGE_BYTES, w_addr = x_addr + X_BYTES;
+                const uint32_t x_addr = sbase + stage * STAGE_BYTES;
+                const uint64_t wd = make_desc(x_addr + X_BYTES, 16, 1024);
 #pragma unroll
                 for (int a = 0; a < MT; ++a) {
                     const int acc = acc_of(li, a);
@@ -193,11 +194,11 @@ lm_head_argmax_kernel(const __grid_constant__ HeadMaps tm, const int R, const in
                         if (!ok) break;
                     }
                     tc_fence_after();
-                    if (lane == 0) {
+                    if (elect_one()) {
+                        const uint64_t xd = make_desc(x_addr + a * XSUB_BYTES, 16, 1024);
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk)
-                            umma_ss(tmem + acc * BN, make_desc(x_addr + a * XSUB_BYTES + kk * 32, 16, 1024),
-                                    make_desc(w_addr + kk * 32, 16, 1024), IDESC, (ks > 0) || (kk > 0));
+                            umma_ss(tmem + acc * BN, xd + (kk * 32 >> 4), wd + (kk * 32 >> 4), IDESC, (ks > 0) || (kk > 0));
                         if (a == MT - 1) umma_commit(bar(BAR_EMPTY + stage));
                         if (ks == n_k - 1) umma_commit(bar(BAR_TFULL + acc));
                     }
@@ -206,7 +207,7 @@ lm_head_argmax_kernel(const __grid_constant__ HeadMaps tm, const int R, const in
             }
         }
         // every MMA issued so far must have retired before TMEM is freed
-        if (lane == 0) umma_commit(bar(BAR_DONE));
+        if (elect_one()) umma_commit(bar(BAR_DONE));
         __syncwarp();
         { int dummy = 0; mbar_wait_warp(bar(BAR_DONE), 0, &dummy); }
         tc_fence_before();
@@ -401,14 +402,13 @@ lm_head_argmax_pair_kernel(const __grid_constant__ HeadMaps tm, const int R, con
                     ok = mbar_wait_warp(bar(BAR_FULL + stage), use & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t x_addr = sbase + stage * STAGE_BYTES, w_addr = x_addr + X_BYTES;
+                    if (elect_one()) {
+                        const uint32_t x_addr = sbase + stage * STAGE_BYTES;
+                        const uint64_t xd = make_desc(x_addr, 16, 1024), wd = make_desc(x_addr + X_BYTES, 16, 1024);
 #pragma unroll
                         for (int kk = 0; kk < KPANELS * BK / 16; ++kk)
-                            umma_ss_pair(tmem + buf * BN,
-                                         make_desc(x_addr + (kk >> 2) * XSUB_BYTES + (kk & 3) * 32, 16, 1024),
-                                         make_desc(w_addr + (kk >> 2) * WPANEL_BYTES + (kk & 3) * 32, 16, 1024),
-                                         IDESC, (ks > 0) || (kk > 0));
+                            umma_ss_pair(tmem + buf * BN, xd + (((kk >> 2) * XSUB_BYTES + (kk & 3) * 32) >> 4),
+                                         wd + (((kk >> 2) * WPANEL_BYTES + (kk & 3) * 32) >> 4), IDESC, (ks > 0) || (kk > 0));
                         umma_commit_both(bar(BAR_EMPTY + stage));
                         if (ks == n_k - 1) umma_commit_both(bar(BAR_TFULL + buf));
                     }
@@ -416,7 +416,7 @@ lm_head_argmax_pair_kernel(const __grid_constant__ HeadMaps tm, const int R, con
                 }
             }
             // every MMA issued so far must have retired before TMEM is freed
-            if (lane == 0) umma_commit_pair(bar(BAR_DONE));
+            if (elect_one()) umma_commit_pair(bar(BAR_DONE));
             __syncwarp();
             { int dummy = 0; mbar_wait_warp(bar(BAR_DONE), 0, &dummy); }
         }
