@@ -16,7 +16,10 @@
 //              cache, the block K/V tile) into a ring of five 16 KB slots, in the order
 //              the MMAs consume them.
 //   warp 5     TMEM allocation and MMA issue: S = Q.K^T into one of two score buffers
-//              (so that QK(t+1) runs under softmax(t)), then O += P.V.
+//              (so that QK(t+1) runs under softmax(t)), then O += P.V.  This chain sets the pace
+//              of a lone CTA, 1450 cycles per tile: 480 to issue the eight MMAs of QK, 250 for the
+//              four of P.V, the rest waits and fences.  (Behind a test of the lane index instead
+//              of elect.sync, the descriptors built in the loop: 660, 640 and 2020 per tile.)
 // (Units of at most 64 rows run on attend_keys.cu.)
 // The output accumulator O stays in TMEM for the whole CTA.  The running max is only
 // raised when a tile exceeds it by more than 2^8; then, and only then, the owner threads
@@ -24,16 +27,19 @@
 // bf16 operands carry without loss, and the result is the exact softmax because the
 // same shift is used for the numerator and the denominator.
 //
-// Merge of the S partial results of a unit, inside the kernel (there is no second launch),
-// through the workspace, which stays in L2: every softmax thread stores its partial row (max, sum, unnormalised O) straight from the
+// Merge of the S partial results of a unit, inside the kernel (there is no second launch).  Clusters of 2,
+// 4 and 8 exchange through distributed shared memory: each row's thread sends the other CTAs their
+// 128 / S columns of it (exchange_merge).  Other sizes go through the workspace, which stays in L2:
+// every softmax thread stores its partial row (max, sum, unnormalised O) straight from the
 // registers its TMEM read-out filled, in a chunk-major layout ([16-byte column chunk][row])
 // so that a warp's 32 rows land in 512 contiguous bytes; one cluster barrier publishes the
 // rows; then the work is shared out as (32-row group, column chunk) tasks, one warp each,
 // round-robin over the cluster's CTAs and their warps: lane = row, all S partials of the
 // task are requested at once (again 512 contiguous bytes per request), weighted, summed,
-// normalised and written.  A CTA leaves as soon as its tasks are done.  (Reading the peers'
-// shared memory instead was measured slower at every cluster size: remote loads are round
-// trips with few requests in flight.)
+// normalised and written.  A CTA leaves as soon as its tasks are done.  A CTA's end took about 10 us
+// through L2 with clusters of 2 (a ragged batch of 32, 128 rows: 292 us a pass, 271 with the exchange; a packed
+// multi-block call 66.8 and 57.9); with clusters of 16 the exchange is the slower one (8 units of
+// 4000 keys 14.3 against 12.6 us a call: as many messages of 8 columns).
 //
 // Programmatic dependent launch.  The kernel waits for the preceding kernel of the
 // stream (griddepcontrol.wait) before it reads anything that kernel may have written,
@@ -72,8 +78,8 @@ constexpr int MAX_BARS = 40;
 template <int NT> struct Shape {
     static constexpr int NSLOT = NT == 1 ? 5 : 10;             // ring slots, one K or V tile each
     // warps: 4 softmax warps per query tile, the producer, one MMA-issuing warp per query tile
-    // (a thread is held for about a hundred cycles per tcgen05.mma it issues, whatever the
-    //  shape: the two tiles' MMAs of a key tile are issued side by side, not one after the other)
+    // (a thread is held for about fifty cycles per tcgen05.mma it issues, whatever the shape: the
+    //  two tiles' MMAs of a key tile are issued side by side, not one after the other)
     static constexpr int NTHREADS = 32 * (4 * NT + 1 + NT);
     static constexpr int PRODUCER_WARP = 4 * NT, MMA_WARP = 4 * NT + 1;    // MMA warps: MMA_WARP + ti
     // shared memory map (offsets from a 1024-byte aligned base)
