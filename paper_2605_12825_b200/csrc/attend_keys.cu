@@ -39,12 +39,12 @@
 // bf16 rows [key][row], which is the MN-major B operand of the second product; their sums are taken
 // over the same rounded values, while that product runs.
 //
-// Merge of the S CTAs of a cluster (one unit), through the workspace, which stays in L2: every thread
-// stores its head column of four query rows per 16 bytes, so that a warp's store is 512 contiguous
-// bytes; a cluster barrier publishes them; each CTA then sums its share of the (row group, column)
-// elements over the S partials, a lane every fourth partial.  Through distributed shared memory
-// (remote loads, remote stores or bulk copies between the CTAs) the merge was measured slower for
-// 64 rows (11.8 against 9.9 us a call) and no faster for fewer.
+// Merge of the S CTAs of a cluster (one unit).  A thread of the read-out holds its head column of four
+// query rows per 16 bytes.  Where the CTAs have much to tell one another (`exchanges`), it sends them into
+// the ring of the CTA that sums up that column; a cluster barrier before that (every ring is idle; the
+// CTAs arrive ahead of the read-out, which hides it), one behind it.  Else through the workspace, which
+// stays in L2: a warp's store is 512 contiguous bytes; a cluster barrier publishes them; each CTA then
+// sums its share of the (row group, column) elements over the S partials, a lane every fourth partial.
 //
 // Every mbarrier wait is bounded: on expiry the CTA raises ORTHRUS_DEV_WAIT_TIMEOUT, its warps go
 // on through their barriers with void results, the MMAs and copies in flight are waited for, and it ends.
@@ -70,6 +70,7 @@ struct KeysArgs {
     int S, quiescent, ranked;
     uint32_t inv_g;            // ceil(2^16 / G): r / G = r * inv_g >> 16 for r < 128
     int slice;                 // elements of the merge per CTA, a multiple of 8
+    int width;                 // XCH: columns that each CTA sums up
     int kb_rows;               // block positions per query tile (blockIdx.z counts the tiles of a unit)
 };
 
@@ -85,6 +86,10 @@ template <int HD, int NR> struct KeysShape {
     static constexpr int OFF_P = NSLOT * KV_BYTES;             // per warpgroup [panel][128 keys][128 bytes]
     static constexpr int OFF_Q = OFF_P + 2 * P_BYTES;
     static constexpr int END_Q = OFF_Q + (Q_BYTES > 6144 ? Q_BYTES : 6144);   // (later the tables of the read-out)
+    // merge through distributed shared memory, in the ring: partial sums [CTA][row group][column], maxima and
+    // sums [CTA][row], weights [CTA][row]
+    static constexpr int OFF_XML = 40 * 1024, OFF_XW = OFF_XML + 16 * NR * 8;
+    static_assert(HD / 4 * NR * 19 <= OFF_XML && OFF_XW + 16 * NR * 4 <= NSLOT * KV_BYTES, "exchange buffer");
     static constexpr int OFF_REF = END_Q;                      // float [2][NR]: references of the current tiles
     static constexpr int OFF_BAR = OFF_REF + 2 * NR * 4;
     static constexpr int BAR_FULL = 0, BAR_Q = NSLOT, BAR_S = BAR_Q + 1, BAR_P = BAR_S + 2, BAR_PV = BAR_P + 2,
@@ -202,7 +207,8 @@ __device__ inline void merge(const float4 *po, const float2 *pml, float *wt, int
     }
 }
 
-template <int HD, int NR>
+// XCH: the merge goes through distributed shared memory
+template <int HD, int NR, bool XCH>
 __global__ void __launch_bounds__(NTHREADS, KeysShape<HD, NR>::CTAS)
 attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, const KeysArgs args)
 {
@@ -483,17 +489,20 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             for (int x = 0; x < PP; ++x) *reinterpret_cast<float2 *>(t_l + warp * NR + x * 64 + 2 * lane) = l_run[x];
         if (kt < NR) t_m[wg * NR + kt] = m_run;
         bar_pair();
+        float2 ml_row = make_float2(-INFINITY, 0.f);          // of row tid
         if (tid < NR) {
             const float la = (t_l[tid] + t_l[NR + tid]) + (t_l[2 * NR + tid] + t_l[3 * NR + tid]);
             const float lb = (t_l[4 * NR + tid] + t_l[5 * NR + tid]) + (t_l[6 * NR + tid] + t_l[7 * NR + tid]);
             const float ma = t_m[tid], mb = t_m[NR + tid], M = fmaxf(ma, mb);
             float wa = la > 0.f ? ex2(ma - M) : 0.f, wb = lb > 0.f ? ex2(mb - M) : 0.f;
             const float L = wa * la + wb * lb;
+            ml_row = make_float2(M, L);
             if (S == 1) { wa /= L; wb /= L; }
-            else __stcg(reinterpret_cast<float2 *>(p.part_ml) + cta * NR + tid, make_float2(M, L));
+            else if (!XCH) __stcg(reinterpret_cast<float2 *>(p.part_ml) + cta * NR + tid, make_float2(M, L));
             t_w[tid] = wa; t_w[NR + tid] = wb;
         }
         if (n_tiles > 0) mbar_wait_warp(bar(C::BAR_ALL), 0, abort_flag);
+        if constexpr (XCH) cluster_arrive();                     // the ring is idle
         bar_pair();
         tc_fence_after();
         // ------------------------------------------------------------------ read-out: lane = head column
@@ -526,7 +535,14 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                     y.z = fmaf(w.z, __uint_as_float(ob[i + 2]), y.z); y.w = fmaf(w.w, __uint_as_float(ob[i + 3]), y.w);
                 }
             }
-            if (S > 1) {
+            if constexpr (XCH) {
+                const int q = d / args.width;                 // the CTA that sums up column d
+                const uint32_t dst = map_to_rank(sbase, q) + ((rank * (NR / 4) + c / 4) * args.width + d - q * args.width) * 16;
+                cluster_wait();
+#pragma unroll
+                for (int i = 0; i < CW / 4; ++i)
+                    if (c / 4 + i < n4) st_cluster(dst + i * args.width * 16, x[i]);
+            } else if (S > 1) {
 #pragma unroll
                 for (int i = 0; i < CW / 4; ++i)
                     if (c / 4 + i < n4) __stcg(part + (c / 4 + i) * HD, x[i]);
@@ -538,9 +554,47 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                         out[row_off(c + i) + d] = __float2bfloat16_rn(i % 4 == 0 ? y.x : i % 4 == 1 ? y.y : i % 4 == 2 ? y.z : y.w);
                 }
             }
+        } else if constexpr (XCH) {
+            cluster_wait();
         }
         tc_fence_before();
-        if (S > 1) {
+        if constexpr (XCH) {
+            if (tid < M)
+                for (int q = 0; q < S; ++q) st_cluster(map_to_rank(sbase + C::OFF_XML + (rank * NR + tid) * 8, q), ml_row.x, ml_row.y);
+            cluster_sync_all();
+            float *wt = reinterpret_cast<float *>(smem + C::OFF_XW);
+            if (tid < M) {
+                const float2 *ml = reinterpret_cast<const float2 *>(smem + C::OFF_XML) + tid;
+                float m = -INFINITY, L = 0.f;
+                for (int j = 0; j < S; ++j) m = fmaxf(m, ml[j * NR].x);
+                for (int j = 0; j < S; ++j) {
+                    const float2 y = ml[j * NR];
+                    const float w = y.y > 0.f ? ex2(y.x - m) : 0.f;
+                    L = fmaf(w, y.y, L);
+                    wt[j * NR + tid] = w;
+                }
+                const float inv = L > 0.f ? 1.f / L : 0.f;
+                for (int j = 0; j < S; ++j) wt[j * NR + tid] *= inv;
+            }
+            bar_pair();
+            const int w0 = rank * args.width, wn = min(args.width, HD - w0);
+            for (int e = tid; e < n4 * wn; e += ST) {
+                const int g = e / wn, col = e - g * wn;
+                const float4 *v = reinterpret_cast<const float4 *>(smem) + g * args.width + col;
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                for (int j = 0; j < S; ++j) {
+                    const float4 a = v[j * (NR / 4) * args.width], w = *reinterpret_cast<const float4 *>(wt + j * NR + 4 * g);
+                    acc.x = fmaf(w.x, a.x, acc.x); acc.y = fmaf(w.y, a.y, acc.y);
+                    acc.z = fmaf(w.z, a.z, acc.z); acc.w = fmaf(w.w, a.w, acc.w);
+                }
+                const float y[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (4 * g + k < M) out[row_off(4 * g + k) + w0 + col] = __float2bfloat16_rn(y[k]);
+            }
+            return;
+        } else if (S > 1) {
             float *wt = reinterpret_cast<float *>(smem) + warp * 256;
             const float4 *po = reinterpret_cast<const float4 *>(p.part_o) + cta0 * (NR / 4 * HD);
             const float2 *pml = reinterpret_cast<const float2 *>(p.part_ml) + cta0 * NR;
@@ -571,6 +625,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 }
         }
         __syncwarp();
+        if (XCH) cluster_sync_all();
         if (S > 1) cluster_sync_all();
     } else {
         // ------------------------------------------------------------------ MMA issue
@@ -642,6 +697,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         }
         tc_fence_before();
         if (S > 1) {
+            if (XCH) cluster_sync_all();
             cluster_sync_all();                               // every warp of this CTA has read its TMEM
             tc_fence_after();
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TM_COLS) : "memory");
@@ -659,7 +715,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 }
 
 // function attributes belong to a device: set them once on each device that launches
-template <int HD, int NR> cudaError_t configure(int *dev)
+template <int HD, int NR, bool XCH> cudaError_t configure(int *dev)
 {
     constexpr int kMaxDevices = 64;
     static std::mutex mu;
@@ -669,7 +725,7 @@ template <int HD, int NR> cudaError_t configure(int *dev)
     if (*dev < 0 || *dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!configured[*dev]) {
-        auto kern = attend_keys_kernel<HD, NR>;
+        auto kern = attend_keys_kernel<HD, NR, XCH>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, KeysShape<HD, NR>::SMEM_BYTES);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess)
@@ -691,7 +747,7 @@ template <int HD, int NR> int resident_clusters(int S)
     static std::atomic<int> cached[kMaxDevices][MAX_CLUSTER + 1];
     int dev = 0;
     constexpr int CTAS = KeysShape<HD, NR>::CTAS;
-    if (configure<HD, NR>(&dev) != cudaSuccess) { (void)cudaGetLastError(); return CTAS * kDefaultSMs / S; }
+    if (configure<HD, NR, false>(&dev) != cudaSuccess) { (void)cudaGetLastError(); return CTAS * kDefaultSMs / S; }
     int n = cached[dev][S].load(std::memory_order_relaxed);
     if (n != 0) return n > 0 ? n : 0;
     cudaLaunchConfig_t cfg = {};
@@ -704,7 +760,7 @@ template <int HD, int NR> int resident_clusters(int S)
     attr[0].val.clusterDim.x = sms; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, attend_keys_kernel<HD, NR>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, attend_keys_kernel<HD, NR, false>, &cfg) != cudaSuccess || n < 1) {
         (void)cudaGetLastError();
         n = sms <= 8 ? num_sms() / sms : 0;       // a size the device cannot schedule is not chosen
     }
@@ -712,6 +768,12 @@ template <int HD, int NR> int resident_clusters(int S)
     cached[dev][S].store(n < 1 ? -1 : n, std::memory_order_relaxed);
     return n;
 }
+
+// Clusters of up to four CTAs that exchange 4 KB or more with each other merge through distributed shared
+// memory.  Measured per call, L2 against exchange, d = 128: 128 units of 64 rows, 1000 keys (2 CTAs) 23.1 and
+// 19.0 us; 64 units, 2000 keys (4 CTAs) 18.5 and 17.1; 128 units of 32 rows, 400 keys (2) 11.5 and 9.9; but 32
+// units of 64 rows, 1000 keys (8) 11.6 and 11.9, 8 units of 4000 keys (16) 11.5 and 12.7, 4 rows (2) 8.5 and 8.8.
+constexpr bool exchanges(int d, int nr, int S) { return S > 1 && S <= 4 && nr >= 32 && nr * d >= 1024 * S; }
 
 // CTAs per unit.  A CTA's time is that of its tiles one after the other; a merge costs as much as one
 // tile and, for what it moves, up to two more; a second wave of clusters costs more than any split
@@ -737,13 +799,15 @@ template <int HD, int NR> int choose_splits(int units, int halves)
     return best;
 }
 
-template <int HD, int NR>
+template <int HD, int NR, bool XCH = false>
 cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cudaStream_t st)
 {
     using C = KeysShape<HD, NR>;
-    auto kern = attend_keys_kernel<HD, NR>;
+    if constexpr (!XCH && exchanges(HD, NR, 2))
+        if (exchanges(HD, NR, p.n_splits)) return launch_shape<HD, NR, true>(p, tm, flags, st);
+    auto kern = attend_keys_kernel<HD, NR, XCH>;
     int dev = 0;
-    cudaError_t e = configure<HD, NR>(&dev);
+    cudaError_t e = configure<HD, NR, XCH>(&dev);
     if (e != cudaSuccess) return e;
     const int S = p.n_splits, units = p.B * p.Hkv, kb = tc_kb_rows(p.G, p.K), tiles = (p.K + kb - 1) / kb;
     cudaLaunchConfig_t cfg = {};
@@ -772,6 +836,7 @@ cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cud
     args.inv_g = (65536u + p.G - 1) / p.G;
     args.slice = (((kb * p.G + 3) / 4 * HD + S - 1) / S + 7) & ~7;
     args.kb_rows = kb;
+    args.width = (HD + S - 1) / S;
     e = cudaLaunchKernelEx(&cfg, kern, p, tm, args);
     count_launch();
     return e;

@@ -30,7 +30,7 @@ def inputs(shape, lens, hint=1024):
 
 @pytest.mark.parametrize("view", VIEWS)
 @pytest.mark.parametrize("shape", SHAPES)
-@pytest.mark.parametrize("splits", [None, 1, 3, 16])
+@pytest.mark.parametrize("splits", [None, 1, 2, 3, 8, 16])
 def test_shapes_and_splits(view, shape, splits):
     for lens in ([0, 1], [15, 64], [65, 130], [700, 257], [1024, 1000]):
         wl, t = inputs(shape, lens)
