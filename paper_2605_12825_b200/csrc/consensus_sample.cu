@@ -62,12 +62,6 @@ __device__ inline float pow2i(float k) {                 // 2^k for integer-valu
     const int e = (int)k + 127;
     return e > 0 ? __int_as_float(e << 23) : 0.f;
 }
-__device__ inline RefSum combine(const RefSum &a, const RefSum &b) {
-    if (b.m == -INFINITY) return a;
-    if (a.m == -INFINITY) return b;
-    const float M = fmaxf(a.m, b.m);
-    return RefSum{M, a.s * (double)pow2i(a.m - M) + b.s * (double)pow2i(b.m - M)};
-}
 // R x N raw logits; c > 0 scales them into the log2 domain.  The instruction count matters (the loop
 // is bound by the exponentials only while the rest stays below them): the maximum is taken over the
 // raw values, once for all R vectors (some lane of a warp raises its reference at nearly every check),
@@ -105,12 +99,21 @@ __device__ inline void absorb(RefSum &a, const float (&x)[R][N], float c) {
 #pragma unroll
     for (int q = 0; q < R; ++q) a.s += (double)sum[q];
 }
-// fold over a warp in a fixed order, known to every lane
-__device__ inline RefSum warp_fold(RefSum v) {
+__device__ inline double warp_sum(double x) {
 #pragma unroll
-    for (int off = 16; off; off >>= 1)
-        v = combine(v, RefSum{__shfl_xor_sync(0xffffffffu, v.m, off), __shfl_xor_sync(0xffffffffu, v.s, off)});
-    return v;
+    for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+__device__ inline float warp_max(float x) {
+    float y;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
+}
+// fold over a warp in a fixed order, known to every lane: the reference first, then each lane's sum is
+// scaled to it once (scaling at each of the five steps is a chain of three dependent double operations)
+__device__ inline RefSum warp_fold(const RefSum &v) {
+    const float M = warp_max(v.m);
+    return RefSum{M, warp_sum(v.m > -INFINITY ? v.s * (double)pow2i(v.m - M) : 0.0)};
 }
 
 struct alignas(8) StatPart { float ma, md; double sa, sd; };       // per (row, stretch)
@@ -165,11 +168,14 @@ __device__ inline void fold_row(const StatPart *parts, int n_seg, int lane, RefS
                 t[q].sa = __ldcg(&x->sa); t[q].sd = __ldcg(&x->sd);
             }
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            a = combine(a, RefSum{t[q].ma, t[q].sa});
-            d = combine(d, RefSum{t[q].md, t[q].sd});
-        }
+        auto add = [](RefSum &v, float m0, double s0, float m1, double s1, float m2, double s2, float m3, double s3) {
+            const float M = fmaxf(fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)), v.m);
+            if (M == -INFINITY) return;
+            auto at = [M](float m, double x) { return m > -INFINITY ? x * (double)pow2i(m - M) : 0.0; };
+            v = RefSum{M, at(v.m, v.s) + ((at(m0, s0) + at(m1, s1)) + (at(m2, s2) + at(m3, s3)))};
+        };
+        add(a, t[0].ma, t[0].sa, t[1].ma, t[1].sa, t[2].ma, t[2].sa, t[3].ma, t[3].sa);
+        add(d, t[0].md, t[0].sd, t[1].md, t[1].sd, t[2].md, t[2].sd, t[3].md, t[3].sd);
     }
     a = warp_fold(a);
     d = warp_fold(d);
@@ -259,24 +265,11 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, con
 
 struct RowStat { float ma, md; double inv_za, inv_zd; };  // of the first rejected row (1 / sums)
 
-__device__ inline void residual_of(float xa, float xd, float c, const RowStat &st, double &r, double &p) {
-    p = (double)ex2(xa * c - st.ma) * st.inv_za;
-    const double q = (double)ex2(xd * c - st.md) * st.inv_zd;
-    r = fmax(p - q, 0.0);
-}
-template <int N>
-__device__ inline void residual_vec(const float (&x)[N], const float (&y)[N], float c, const RowStat &st, double &sr, double &sp) {
-#pragma unroll
-    for (int e = 0; e < N; ++e) {
-        double r, p;
-        residual_of(x[e], y[e], c, st, r, p);           // (an element that does not exist has p = r = 0)
-        sr += r; sp += p;
-    }
-}
-__device__ inline double warp_sum(double x) {
-#pragma unroll
-    for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    return x;
+// an element's share of the residual max(0, p - q), or (use_p) of p; 0 for one that does not exist
+__device__ inline double mass_of(float xa, float xd, float c, const RowStat &st, bool use_p) {
+    const double p = (double)ex2(xa * c - st.ma) * st.inv_za;
+    const double r = use_p ? p : fma(-(double)ex2(xd * c - st.md), st.inv_zd, p);
+    return r > 0.0 ? r : 0.0;
 }
 __device__ inline double peer_double(const double *mine, int rank) {
     double x;
@@ -286,19 +279,22 @@ __device__ inline double peer_double(const double *mine, int rank) {
 
 // Grid (C, B) in clusters of C: one sequence.  The residual's running sum is taken over CTAs, then a
 // CTA's warps, then a warp's groups of rounds (a round is 32 vectors, a lane each), in index order, and
-// each level keeps its sums, so that the drawn point is found level by level.
-constexpr int kGroups = 64;
+// each level keeps its sums, so that the drawn point is found level by level.  Bound by latencies (dependent
+// double operations, loads from L2), hence 16 warps a CTA, the mass of p only where the residual turns out to be
+// empty, and sums in several chains.  With 8 warps and both masses in one chain each the residual of a row of
+// 128256 took 13 us in clusters of 8; whole passes 102 -> 93 us (batch 32) and 23.8 -> 18.8 us (batch 1).
+constexpr int kFinishThreads = 512, kFinishWarps = kFinishThreads / 32, kGroups = 64;
 template <typename T>
-__global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, const T *ld, int K, int V, int n_seg, float c,
+__global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const T *la, const T *ld, int K, int V, int n_seg, float c,
                                                                  const int32_t *draft, const float *u_accept,
                                                                  const float *u_resample, const StatPart *parts,
                                                                  const int *fail, int32_t *n_commit, int32_t *committed,
                                                                  int32_t *next_anchor)
 {
     constexpr int N = Elem<T>::N;
-    __shared__ double grp[2][kWarps][kGroups], wsum[2][kWarps], csum[2];
+    __shared__ double grp[kFinishWarps][kGroups], wsum[kFinishWarps], csum[2];
     __shared__ double s_before, s_target;
-    __shared__ int s_first, s_owner, s_use_p, s_warp, s_group;
+    __shared__ int s_first, s_owner, s_use_p, s_empty;
     __shared__ RowStat s_stat;
     extern __shared__ RefSum folded[];                  // [K][2], unless the failures are known already
     const int b = blockIdx.y, rank = blockIdx.x, C = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -306,7 +302,7 @@ __global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, co
     if (tid == 0) s_first = fail ? fail[b] : K;
     __syncthreads();
     if (!fail) {
-        for (int i = warp; i < K; i += kWarps) {
+        for (int i = warp; i < K; i += kFinishWarps) {
             const long long row = (long long)b * K + i;
             RefSum a, d;
             fold_row(parts + row * n_seg, n_seg, lane, a, d);
@@ -319,7 +315,7 @@ __global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, co
     }
     const int j = s_first;                              // K: every draft is kept
     if (rank == 0) {
-        for (int i = tid; i < K; i += kThreads)
+        for (int i = tid; i < K; i += kFinishThreads)
             if (i != j) committed[(long long)b * K + i] = i < j ? draft[(long long)b * K + i] : -1;
         if (tid == 0) {
             n_commit[b] = j < K ? j + 1 : K;
@@ -339,15 +335,16 @@ __global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, co
     const RowStat st = s_stat;
     const RowShape sh = row_shape(ra, rd, V);
     const int per = (sh.n_vec + C - 1) / C, v0 = rank * per, v1 = min(sh.n_vec, v0 + per);
-    const int per_w = (per + kWarps - 1) / kWarps, w0 = min(v1, v0 + warp * per_w), w1 = min(v1, w0 + per_w);
+    const int per_w = (per + kFinishWarps - 1) / kFinishWarps, w0 = min(v1, v0 + warp * per_w), w1 = min(v1, w0 + per_w);
     // (a group costs two warp sums, a round in the end two loads: two rounds and up to a group)
     const int rounds = (per_w + 31) / 32, gsz = max(2, (rounds + kGroups - 1) / kGroups), n_grp = (rounds + gsz - 1) / gsz;
-    {
-        double tr = 0.0, tp = 0.0, sr = 0.0, sp = 0.0;
-        for (int r0 = 0; r0 < rounds; r0 += 4) {        // the loads of four rounds together
-            float x[4][N], y[4][N];
+    // the residual; if it is empty (p and q agree to the last bit), the mass of p
+    for (int use_p = 0; use_p < 2; ++use_p) {
+        double total = 0.0, sum = 0.0;
+        for (int r0 = 0; r0 < rounds; r0 += 2) {        // the loads of two rounds together
+            float x[2][N], y[2][N];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 2; ++i) {
                 const int v = w0 + (r0 + i) * 32 + lane;
                 if (r0 + i < rounds && v < w1) {
                     load_vec<T>(ra, sh, v, x[i]);
@@ -355,77 +352,75 @@ __global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, co
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 2; ++i) {
                 const int r = r0 + i;
                 if (r >= rounds) break;
-                if (w0 + r * 32 + lane < w1) residual_vec<N>(x[i], y[i], c, st, sr, sp);
+                if (w0 + r * 32 + lane < w1) {
+                    double m[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                    for (int e = 0; e < N; ++e) m[e & 3] += mass_of(x[i][e], y[i][e], c, st, use_p);
+                    sum += (m[0] + m[1]) + (m[2] + m[3]);
+                }
                 if ((r + 1) % gsz == 0 || r == rounds - 1) {
-                    sr = warp_sum(sr); sp = warp_sum(sp);
-                    if (lane == 0) { grp[0][warp][r / gsz] = sr; grp[1][warp][r / gsz] = sp; }
-                    tr += sr; tp += sp;
-                    sr = sp = 0.0;
+                    sum = warp_sum(sum);
+                    if (lane == 0) grp[warp][r / gsz] = sum;
+                    total += sum;
+                    sum = 0.0;
                 }
             }
         }
-        if (lane == 0) { wsum[0][warp] = tr; wsum[1][warp] = tp; }
-    }
-    __syncthreads();
-    if (tid < 2) {
-        double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += wsum[tid][w];
-        csum[tid] = s;
-    }
-    cluster_sync_all();
-    // every CTA finds the share that holds the drawn point: the first whose running sum exceeds the target,
-    // the last that is not empty if rounding leaves the target at or past the total
-    if (warp == 0) {
-        const double xr = lane < C ? peer_double(&csum[0], lane) : 0.0, xp = lane < C ? peer_double(&csum[1], lane) : 0.0;
-        double tot_r = 0.0, tot_p = 0.0;
-        for (int s = 0; s < C; ++s) { tot_r += __shfl_sync(0xffffffffu, xr, s); tot_p += __shfl_sync(0xffffffffu, xp, s); }
-        const int use_p = !(tot_r > 0.0);
-        const double x = use_p ? xp : xr, target = (double)u_resample[row] * (use_p ? tot_p : tot_r);
-        double run = 0.0, before = 0.0;
-        int pick = -1, last = 0;
-        for (int s = 0; s < C; ++s) {
-            const double v = __shfl_sync(0xffffffffu, x, s);
-            if (v > 0.0) {
-                last = s;
-                if (pick < 0 && run + v > target) { pick = s; before = run; }
-                run += v;
-            }
+        if (lane == 0) wsum[warp] = total;
+        __syncthreads();
+        if (warp == 0) {
+            const double s = warp_sum(lane < kFinishWarps ? wsum[lane] : 0.0);
+            if (lane == 0) csum[use_p] = s;
         }
-        if (pick < 0) { pick = last; before = run; }
-        if (lane == 0) { s_owner = pick; s_use_p = use_p; s_before = before; s_target = target; }
+        cluster_sync_all();
+        // every CTA finds the share that holds the drawn point: the first whose running sum exceeds the target,
+        // the last that is not empty if rounding leaves the target at or past the total
+        if (warp == 0) {
+            const double x = lane < C ? peer_double(&csum[use_p], lane) : 0.0;
+            double incl = x;                            // running sum over the CTAs
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const double o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            const double tot = __shfl_sync(0xffffffffu, incl, 31), target = (double)u_resample[row] * tot;
+            const unsigned hit = __ballot_sync(0xffffffffu, x > 0.0 && incl > target), some = __ballot_sync(0xffffffffu, x > 0.0);
+            const int pick = hit ? __ffs(hit) - 1 : some ? 31 - __clz(some) : 0;
+            const double upto = __shfl_sync(0xffffffffu, incl - x, pick);
+            if (lane == 0) { s_owner = pick; s_use_p = use_p; s_before = hit ? upto : tot; s_target = target; s_empty = !(tot > 0.0); }
+        }
+        __syncthreads();
+        if (!s_empty) break;
     }
-    __syncthreads();
     if (rank == s_owner && warp == 0) {
         // the warp and the group of rounds, by the same rule (a lane's warp total, then a lane's two groups)
         const int use_p = s_use_p;
         const double target = s_target;
-        double run = s_before;
-        int pw = -1, last = 0;
-        double at = run;
-        for (int w = 0; w < kWarps; ++w) {
-            const double v = wsum[use_p][w];
-            if (v > 0.0) {
-                last = w;
-                if (pw < 0 && run + v > target) { pw = w; at = run; }
-                run += v;
+        double run = s_before, at = run;
+        int last = 0;
+        auto pick = [&](const double *sums, int n, bool none) {   // -1: past the end
+            int z = -1;
+            for (int i = 0; i < n; ++i) {
+                const double v = sums[i];
+                if (v > 0.0) {
+                    last = i;
+                    if (z < 0 && !none && run + v > target) { z = i; at = run; }
+                    run += v;
+                }
             }
-        }
+            if (z < 0) at = run;
+            return z;
+        };
+        int pw = pick(wsum, kFinishWarps, false);
         const bool past = pw < 0;                       // rounding: take the last element that is positive
-        if (past) { pw = last; at = run; }
-        int pg = -1, last_g = 0;
+        if (past) pw = last;
         run = at;
-        for (int g = 0; g < n_grp; ++g) {
-            const double v = grp[use_p][pw][g];
-            if (v > 0.0) {
-                last_g = g;
-                if (pg < 0 && !past && run + v > target) { pg = g; at = run; }
-                run += v;
-            }
-        }
-        if (pg < 0) { pg = last_g; at = run; }
+        last = 0;
+        int pg = pick(grp[pw], n_grp, past);
+        if (pg < 0) pg = last;
         // the vector and the element
         const int q0 = min(v1, v0 + pw * per_w), q1 = min(v1, q0 + per_w);
         int z = -1, z_last = -1;
@@ -437,9 +432,7 @@ __global__ void __launch_bounds__(kThreads) sample_finish_kernel(const T *la, co
             if (v < q1) { load_vec<T>(ra, sh, v, x); load_vec<T>(rd, sh, v, y); }
 #pragma unroll
             for (int e = 0; e < N; ++e) {
-                double rr = 0.0, pp = 0.0;
-                if (v < q1) residual_of(x[e], y[e], c, st, rr, pp);
-                mine[e] = use_p ? pp : rr;
+                mine[e] = v < q1 ? mass_of(x[e], y[e], c, st, use_p) : 0.0;
                 sum += mine[e];
             }
             double incl = sum;                          // running sum over the lanes
@@ -531,7 +524,7 @@ static cudaError_t launch_sample_t(const void *ar_logits, const void *diff_logit
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, B);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kFinishThreads);
     cfg.dynamicSmemBytes = skip ? 0 : (size_t)K * 2 * sizeof(RefSum);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
