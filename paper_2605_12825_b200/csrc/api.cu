@@ -204,8 +204,16 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
     return pl;
 }
 
-// Units of at most 64 query rows, and wider ones at head_dim 64, run with the keys on the MMA's rows
+// Units of at most 32 query rows, and any at head_dim 64, run with the keys on the MMA's rows
 // (attend_keys.cu).  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels (a measurement knob).
+// 33 to 64 rows at head_dim 128 do so where the units alone fill the GPU, with one CTA each (256 units
+// of up to 2000 keys 47 against 50 us, of 1000 keys 28.8 and 33.2; of 600 keys 21.1 and 18.7); else the kernel
+// for wide units is the better one: 8 units of 4096 keys 13.0 against 10.5 us, of 600 keys 7.9 and 7.2;
+// 64 units of 2000 keys 17.3 and 15.9.  Between 17 and 63 units of more than 1536 keys the two are level (32 of
+// 2000: 13.1), and behind a rotary write in a decoder's step the keys win (15.4 against 16.2 us for both).  (Up to 512 keys they stay although it would take 6.5 against 8.7 us
+// at 300: there a block's verification and the width-1 steps it is compared with token by token run
+// the same kernel with the same cuts, and round alike to the last bit.)  At 32 rows the two are level, below the keys win (4 rows, 8
+// units of 4000 keys 7.3 against 9.7 us).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
 // from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).
@@ -215,6 +223,10 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     const int G = L->n_q_heads / L->n_kv_heads;
     const int rows = keys_rows(L->head_dim, G, L->block);
     if (!rows || (rows > 64 && max_len_of(L) <= 320)) return false;
+    if (rows == 64 && L->head_dim == 128 && tc_usable(L)) {
+        const int max_len = max_len_of(L), units = L->batch * L->n_kv_heads;
+        if (max_len > 512 && (units <= 16 || max_len <= (units > num_sms() ? 768 : units < 64 ? 1536 : 1 << 30))) return false;
+    }
     const unsigned long long cache = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
     return cache < 0x7fffffffull && (long long)L->batch * L->n_kv_heads <= 65535 && tc_driver_ok();
 }

@@ -1,5 +1,5 @@
-// Block attention for units of at most 64 query rows (M = G*K), bf16, head_dim 64 and 128, and of more
-// at head_dim 64 (in tiles of up to 128 rows), both views, on tcgen05 with the KEYS on the MMA's rows:
+// Block attention for units of few query rows (M = G*K; up to 32, and up to 64 where the units alone fill
+// the GPU) at head_dim 128, and of any number at head_dim 64 (in tiles of up to 128 rows), bf16, both views, on tcgen05 with the KEYS on the MMA's rows:
 //     S^T [128 keys x NR rows] = K_tile . Q^T        O^T [d x NR rows] = V_tile^T . P^T
 // NR = M rounded up to 16, 32, 64 or 128 is the MMA's N.  With the query rows there instead, an M of 4 to 64
 // is padded to 128, and only the threads that own real rows take part in the softmax and the
@@ -11,14 +11,12 @@
 // two softmax warpgroups that take alternate tiles into accumulators and running references of their
 // own (no tile waits for another one's maximum), row maxima by redux.sync on the whole warp, and
 // addresses worked out ahead of the wait for the preceding kernel.  Per call, chained in a graph,
-// against the kernel for wide units (two MMA-issuing warps) that served these shapes before: 8 units
-// of 64 rows and 4000 keys 10.9 -> 9.9 us; 16 units of 4 rows and 2700 keys 16.4 -> 8.5 us; 32 units of
-// 64 rows and 1800 keys 13.6 -> 12.5 us; head_dim 64, which ran on mma.sync with a second launch for
-// the merge, 10 units of 49 rows and 800 keys 10.9 -> 7.0 us, 2 units of 32 rows and 512 keys 10.4 ->
-// 6.2 us.  A batch of 256 such units at 4000 keys streams at 6.4 TB/s.  At 128 rows the exponentials
-// bound it, and the wide-unit kernel, whose softmax is spread over more warps, is the better one at
-// head_dim 128 (256 units, about 3000 keys: 30 against 50 us); head_dim 64 had mma.sync alone: one unit
-// of 4000 keys 15.1 -> 9.4 us, 64 of 1500 31 -> 26 us, 256 of 2000 103 -> 68 us.
+// against what served these shapes before: 16 units of 4 rows and 2700 keys 16.4 -> 8.5 us; head_dim 64,
+// which ran on mma.sync with a second launch for the merge, 10 units of 49 rows and 800 keys 10.9 ->
+// 7.0 us, one unit of 128 rows and 4000 keys 15.1 -> 9.4, 256 of 2000 keys 103 -> 68.  A batch of 256
+// units of 64 rows at 4000 keys streams at 6.4 TB/s.  From 33 rows at head_dim 128 the kernel for wide
+// units, whose tiles are half as long and whose threads hold a row each, takes less from the first score to
+// the last product (8 units of 64 rows and 4096 keys 13.0 against 10.5 us).
 //
 // One CTA (320 threads, up to 64 rows at most 113 KB of shared memory and 256 TMEM columns: two fit an SM, so that
 // with programmatic dependent launch the next call's CTAs are resident and, if the caller promised

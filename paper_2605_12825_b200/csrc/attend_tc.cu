@@ -20,7 +20,7 @@
 //              of a lone CTA, 1450 cycles per tile: 480 to issue the eight MMAs of QK, 250 for the
 //              four of P.V, the rest waits and fences.  (Behind a test of the lane index instead
 //              of elect.sync, the descriptors built in the loop: 660, 640 and 2020 per tile.)
-// (Units of at most 64 rows run on attend_keys.cu.)
+// (Units of few rows run on attend_keys.cu.)
 // The output accumulator O stays in TMEM for the whole CTA.  The running max is only
 // raised when a tile exceeds it by more than 2^8; then, and only then, the owner threads
 // rescale their O rows in TMEM.  Probabilities are bounded by 2^8, which fp32 sums and
@@ -513,7 +513,9 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                         }
                     }
                 }
-                const float m_new = fmaxf(m_run, mx * sc);
+                // (an integer, as in attend_keys.cu: another reference scales a probability by a power of two, so
+                // that its rounding does not depend on which kernel or cut computed it)
+                const float m_new = fmaxf(m_run, ceilf(mx * sc));
                 const bool need = m_new > m_run + RESCALE_THRESHOLD;   // also the first finite maximum
                 if (__any_sync(0xffffffffu, need)) {
                     const float alpha = need ? ex2(m_run - m_new) : 1.f;
