@@ -240,9 +240,10 @@ orthrus_status_t orthrus_consensus_sample(const void *ar_logits, const void *dif
  * Here that scratch is an array compiled into the library
  * (ORTHRUS_STATIC_CONSENSUS_SCRATCH_BYTES of device memory on every GPU that loads the
  * library, held until the process exits).  The call allocates nothing and frees nothing.
- *   - Limit: batch * block * segments * 8 bytes must fit in the array, where segments is
- *     the split of the vocabulary the library chooses (at most about 600 / (batch*block),
- *     at least 1): in practice batch * block <= 8192 rows.  A larger problem returns
+ *   - Limit: 8 bytes per row and vocabulary segment must fit in the array.  The library
+ *     splits a row's vocabulary into as many segments as orthrus_consensus_accept would, or
+ *     fewer where the array has no room for them, so that every problem of batch * block <=
+ *     8192 rows is served, whatever its vocabulary.  A larger problem returns
  *     ORTHRUS_ERR_WORKSPACE and launches nothing; use orthrus_consensus_accept then.
  *   - The first call on each device looks up the array's device address (with that device
  *     current).  Make that first call outside of any stream capture.

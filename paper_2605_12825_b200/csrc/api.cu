@@ -571,8 +571,7 @@ orthrus_status_t orthrus_consensus_accept_static(const void *ar_logits, int32_t 
           reinterpret_cast<uintptr_t>(next_anchor)) & 3))
         return ORTHRUS_ERR_INVALID_ARG;
     // the built-in scratch has a fixed size: larger problems need the workspace variant
-    if (static_consensus_scratch_needed(batch, block, vocab) > (size_t)ORTHRUS_STATIC_CONSENSUS_SCRATCH_BYTES)
-        return ORTHRUS_ERR_WORKSPACE;
+    if (static_consensus_segments(batch, block, vocab) < 1) return ORTHRUS_ERR_WORKSPACE;
     cudaError_t e = launch_consensus_static(ar_logits, dtype, draft, batch, block, vocab, n_commit,
                                             committed, ar_argmax, next_anchor,
                                             static_cast<cudaStream_t>(stream));

@@ -103,7 +103,7 @@ int lm_head_max_vocab_tiles(int V);        // the most any row count needs
 bool lm_head_supported();
 cudaError_t launch_lm_head_argmax(const void *hidden, const void *lm_head, int R, int V, int H,
                                   ArgPart *parts, int32_t *status, cudaStream_t st);
-size_t static_consensus_scratch_needed(int B, int K, int V);
+int static_consensus_segments(int B, int K, int V);   // 0: the built-in scratch is too small
 cudaError_t launch_consensus_static(const void *logits, int dtype, const int32_t *draft, int B, int K,
                                     int V, int32_t *n_commit, int32_t *committed, int32_t *ar_argmax,
                                     int32_t *next_anchor, cudaStream_t st);

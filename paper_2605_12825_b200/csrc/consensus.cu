@@ -232,9 +232,13 @@ static cudaError_t static_scratch_address(void **out)
     return cudaSuccess;
 }
 
-size_t static_consensus_scratch_needed(int B, int K, int V)
+// The segments of the workspace variant, or as many as the array has room for (many rows fill the GPU
+// with one each; the others only even out the start).  0: not even one a row.
+int static_consensus_segments(int B, int K, int V)
 {
-    return (size_t)B * K * consensus_segments(B, K, V) * sizeof(ArgPart);
+    const long long room = (long long)(kStaticScratchBytes / sizeof(ArgPart)) / ((long long)B * K);
+    const int want = consensus_segments(B, K, V);
+    return room < want ? (int)room : want;
 }
 
 cudaError_t launch_consensus_static(const void *logits, int dtype, const int32_t *draft, int B, int K,
@@ -247,7 +251,7 @@ cudaError_t launch_consensus_static(const void *logits, int dtype, const int32_t
     // every (row, segment) pair the second kernel reads is written by the first one in the
     // same call, so nothing in the array has to start at zero
     return launch_consensus(logits, dtype, draft, B, K, V, n_commit, committed, ar_argmax, next_anchor,
-                            scratch, consensus_segments(B, K, V), st);
+                            scratch, static_consensus_segments(B, K, V), st);
 }
 
 }  // namespace orthrus

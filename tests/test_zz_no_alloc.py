@@ -58,3 +58,22 @@ def test_static_consensus_refuses_what_does_not_fit():
     rc = f(0x1000, 0, 0x2000, 9000, 1, 64, 0x3000, 0x4000, 0x5000, 0x6000, None)
     assert rc == 4 and b.orthrus_launch_count() == n0
     assert b.STATIC_CONSENSUS_SCRATCH_BYTES < 9000 * 8
+
+
+# the array holds 8192 (value, index) pairs: rows for which the workspace variant cuts the vocabulary into
+# more segments than fit (three a row above four rows per SM; two where a row is short), and the last row
+# count that fits at all
+@pytest.mark.parametrize("B,K,V", [(128, 32, 6200), (171, 16, 4097), (512, 16, 2050), (129, 32, 6145), (8192, 1, 100)])
+def test_static_consensus_serves_every_row_count_that_fits(B, K, V):
+    from paper_2605_12825_b200 import binding as b
+    g = torch.Generator().manual_seed(B + V)
+    logits = torch.randn(B, K, V, generator=g).to(torch.bfloat16)
+    greedy = logits.float().argmax(-1).to(torch.int32)
+    coin = torch.rand(B, K, generator=g) < 0.8
+    draft = torch.where(coin, greedy, torch.randint(0, V, (B, K), generator=g, dtype=torch.int32))
+    ref, got = _both(b, logits, draft.contiguous())
+    for r, o, name in zip(ref, got, ("n_commit", "committed", "ar_argmax", "next_anchor")):
+        assert torch.equal(r, o), name
+    # the value at the token is the row's largest (bf16 logits tie)
+    top = logits.float().max(-1).values
+    assert torch.equal(torch.gather(logits.float(), 2, got[2].long().unsqueeze(2)).squeeze(2), top)
