@@ -99,7 +99,9 @@ typedef struct {
  * flag they request the first prefix K/V tiles before that wait.  Without it nothing
  * is read early and any caller is safe.
  *
- * ORTHRUS_LAYER_NO_EARLY_LAUNCH: launch with ordinary stream order only.
+ * ORTHRUS_LAYER_NO_EARLY_LAUNCH: launch with ordinary stream order only.  (Calls without a
+ * layer are always launched early; ORTHRUS_NO_EARLY_LAUNCH=1 in the environment, read at
+ * every call, puts all calls of the library into ordinary stream order.)
  *
  * ORTHRUS_LAYER_BLOCK_IN_CACHE (attention calls only): the K/V rows of the block are not
  * passed as tensors but already sit in the cache, at rows [P_b, P_b + K) of every KV

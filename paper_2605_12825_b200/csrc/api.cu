@@ -66,6 +66,7 @@ static Knobs read_knobs()
     }
     return k;
 }
+bool early_launch_allowed() { return !read_knobs().no_early_launch; }
 
 }  // namespace orthrus
 

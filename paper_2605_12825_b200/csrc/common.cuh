@@ -142,6 +142,7 @@ __device__ inline void pdl_begin()
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+bool early_launch_allowed();             // false: ORTHRUS_NO_EARLY_LAUNCH is set in the environment
 // `early` false: ordinary stream order
 template <class... Params, class... Args>
 cudaError_t launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem,
@@ -156,7 +157,7 @@ cudaError_t launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, unsi
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = early && early_launch_allowed() ? 1 : 0;
     count_launch();
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }

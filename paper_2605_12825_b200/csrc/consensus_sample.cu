@@ -533,7 +533,7 @@ static cudaError_t launch_sample_t(const void *ar_logits, const void *diff_logit
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = early_launch_allowed() ? 2 : 1;
     count_launch();
     return cudaLaunchKernelEx(&cfg, sample_finish_kernel<T>, la, ld, K, V, n_seg, c, draft, u_accept, u_resample,
                               static_cast<const StatPart *>(parts), static_cast<const int *>(skip ? fail : nullptr), n_commit,

@@ -109,3 +109,47 @@ def assert_close(got, ref, dtype, what=""):
 def small_workload(B, K, Hq, Hkv, d, pmin, pmax, dtype="bf16", V=64, std=1.0, name=None):
     return W.Workload(name or f"t_{B}_{K}_{Hq}_{Hkv}_{d}_{pmin}_{pmax}_{dtype}", B, Hq, Hkv, d, K,
                       V, pmin, pmax, value_std=std, dtype=dtype)
+
+
+def captured_launches(call):
+    """The kernels that `call` enqueues on the current stream, taken from a stream capture behind a kernel of the
+    library user's own: [(kernel name, launched as a programmatic dependent)] in launch order.  Nothing runs."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    x = torch.zeros(8, device="cuda")
+    x.add_(1)                                   # (loaded before the capture)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        x.add_(1)
+        call()
+    graph = ctypes.c_void_p(g.raw_cuda_graph())
+
+    def ok(rc):
+        assert rc == 0, f"driver error {rc}"
+
+    n = ctypes.c_size_t(0)
+    ok(cu.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)))
+    src, dst = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)()
+    data = (ctypes.c_ubyte * (8 * n.value))()   # CUgraphEdgeData: from_port, to_port, type, 5 reserved
+    ok(cu.cuGraphGetEdges_v2(graph, src, dst, data, ctypes.byref(n)))
+    edges = {src[i]: (dst[i], data[8 * i + 2] == 1) for i in range(n.value)}
+    assert len(edges) == n.value and len({d for d, _ in edges.values()}) == n.value, "not a chain"
+
+    class KernelParams(ctypes.Structure):       # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", ctypes.c_void_p), ("dims", ctypes.c_uint * 7), ("params", ctypes.c_void_p),
+                    ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    def name(node):
+        p, s = KernelParams(), ctypes.c_char_p()
+        ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        ok(cu.cuFuncGetName(ctypes.byref(s), ctypes.c_void_p(p.func)) if p.func else
+           cu.cuKernelGetName(ctypes.byref(s), ctypes.c_void_p(p.kern)))
+        return s.value.decode()
+
+    node = (set(edges) - {d for d, _ in edges.values()}).pop()
+    out = []
+    while node in edges:
+        node, early = edges[node]
+        out.append((name(node), early))
+    return out
