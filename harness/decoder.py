@@ -23,6 +23,10 @@ class Decoder:
         behind the prefix), the attention calls read the block from the cache, and the commit is
         orthrus_commit_len."""
         assert commit_mode in ("append", "truncate")
+        # A near tie that resolves otherwise than in the run that the drafts were forced from costs a sequence its
+        # agreeing drafts: it commits a token a cycle from there on while the others run ahead of it by two or
+        # three, so a short loop needs more room than the tokens asked for.
+        capacity = max(capacity, 512)
         self.commit_mode = commit_mode
         self.b, self.L, self.H, self.Hq, self.Hkv, self.d = binding, layers, hidden, n_q, n_kv, d
         self.V, self.dtype, self.B, self.cap, self.K = vocab, dtype, batch, capacity, block

@@ -40,7 +40,8 @@ static int current_path()
 // search per variable: half a dozen searches were a tenth of a call's host time.
 struct Knobs {
     int splits = 0, min_chunk_tiles = 2, target_ctas = 0;     // 0: not forced / the default
-    bool no_early_launch = false, stream = false, pack = true, small_rows = true;
+    int small_rows = -1;                                      // -1: by the rule of keys_usable
+    bool no_early_launch = false, stream = false, pack = true;
 };
 static Knobs read_knobs()
 {
@@ -61,7 +62,7 @@ static Knobs read_knobs()
         else if (is("TARGET_CTAS")) positive(k.target_ctas);
         else if (is("NO_EARLY_LAUNCH")) { positive(on); k.no_early_launch = on > 0; }
         else if (is("TC_SCHEDULE")) k.stream = !strcmp(val, "stream");
-        else if (is("TC_SMALL_ROWS")) k.small_rows = val[0] != '0';
+        else if (is("TC_SMALL_ROWS")) k.small_rows = val[0] != '0' ? 1 : 0;
         else if (is("MULTI_BLOCK_PACK")) k.pack = val[0] != '0';
     }
     return k;
@@ -205,31 +206,49 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
     return pl;
 }
 
-// Units of at most 32 query rows, and any at head_dim 64, run with the keys on the MMA's rows
-// (attend_keys.cu).  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels (a measurement knob).
-// 33 to 64 rows at head_dim 128 do so where the units alone fill the GPU, with one CTA each (256 units
-// of up to 2000 keys 47 against 50 us, of 1000 keys 28.8 and 33.2; of 600 keys 21.1 and 18.7); else the kernel
-// for wide units is the better one: 8 units of 4096 keys 13.0 against 10.5 us, of 600 keys 7.9 and 7.2;
-// 64 units of 2000 keys 17.3 and 15.9.  Between 17 and 63 units of more than 1536 keys the two are level (32 of
-// 2000: 13.1), and behind a rotary write in a decoder's step the keys win (15.4 against 16.2 us for both).  (Up to 512 keys they stay although it would take 6.5 against 8.7 us
-// at 300: there a block's verification and the width-1 steps it is compared with token by token run
-// the same kernel with the same cuts, and round alike to the last bit.)  At 32 rows the two are level, below the keys win (4 rows, 8
-// units of 4000 keys 7.3 against 9.7 us).
+// 33 to 64 query rows at head_dim 128 can run on either tcgen05 kernel: with the keys on the MMA's rows
+// (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).  The wide
+// one takes less per key (us a call, keys against wide, 64 rows: 8 units of 300 keys 8.3 and 5.8, of 4096 12.4 and
+// 10.1; 32 of 1024 11.0 and 10.2; 48 of 3072 21.4 and 19.8; 128 of 2048 29.0 and 26.5; 320 of 1024 50.0 and 46.1), so it is
+// the rule, for short prefixes as well.  It loses where its plan, whose clusters are powers of two,
+// does not suit the number of units:
+//  - its clusters are not all resident at once (34 to 37 units cut in 8: 37 of 1700 keys 14.5 and 20.3; more units
+//    than SMs, cut in 2 from 15 tiles on: 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9);
+//  - clusters of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix is long
+//    (12 units of 8000 keys 15.9 and 18.4, 44 of 6000 29.0 and 30.8; at 2500 keys they still win: 10.9 and 9.6, 17.7 and 17.3;
+//    clusters of 2 keep the memory busy all the same: 80 units of 4500 keys 44.2 and 40.0).
+//    Rows that do not fill warps of 32 cost the wide kernel a second way through its softmax, so that the line
+//    lies lower there (48 rows, 10 units of 3500 keys 9.8 and 11.8, 42 of 2500 16.1 and 17.3).
+// In a decoder (rotary write, both views, room above the lengths; us per write and call) the signs are the same: 64 rows, 32 units of
+// 1450 keys 17.2 and 16.4, of 3300 22.9 and 20.3, 48 of 3300 28.2 and 25.6, 40 of 6500 35.9 and 38.0; the two come
+// within 3 % of one another, either way, at 28 to 32 units of 1600 to 2000 keys.
+// A width-1 step (M <= 32) and the verification of a block (M > 32) thus run different kernels, which agree up to the
+// rounding of their sums; a program that wants the same bits from both sets ORTHRUS_TC_SMALL_ROWS=1.
+static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
+{
+    if (!tc_usable(L)) return false;
+    const int units = L->batch * L->n_kv_heads, M = L->n_q_heads / L->n_kv_heads * L->block;
+    const int S = make_plan(L, true, kn).n_splits;
+    if (S > 1 && units > keys_resident_clusters(S)) return false;   // (the two kernels' CTAs fit an SM alike)
+    const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
+    return !((S == 4 || S == 8) && roomy && max_len_of(L) > (M == 64 ? 4096 : 2048));
+}
+
+// Units of at most 32 query rows (4 rows, 8 units of 4000 keys 7.3 against 9.7 us on the wide kernel; at 32 rows the two
+// are level), of 33 to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
+// rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
 // from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).
 static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
 {
-    if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || !kn.small_rows) return false;
-    const int G = L->n_q_heads / L->n_kv_heads;
-    const int rows = keys_rows(L->head_dim, G, L->block);
-    if (!rows || (rows > 64 && max_len_of(L) <= 320)) return false;
-    if (rows == 64 && L->head_dim == 128 && tc_usable(L)) {
-        const int max_len = max_len_of(L), units = L->batch * L->n_kv_heads;
-        if (max_len > 512 && (units <= 16 || max_len <= (units > num_sms() ? 768 : units < 64 ? 1536 : 1 << 30))) return false;
-    }
+    if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || kn.small_rows == 0) return false;
+    const int rows = keys_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
     const unsigned long long cache = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
-    return cache < 0x7fffffffull && (long long)L->batch * L->n_kv_heads <= 65535 && tc_driver_ok();
+    if (!rows || cache >= 0x7fffffffull || (long long)L->batch * L->n_kv_heads > 65535 || !tc_driver_ok()) return false;
+    if (kn.small_rows > 0) return true;
+    if (rows > 64) return max_len_of(L) > 320;
+    return rows < 64 || L->head_dim == 64 || !wide_better(L, kn);
 }
 static int keys_tiles(const orthrus_layer_t *L)
 {

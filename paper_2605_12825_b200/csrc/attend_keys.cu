@@ -1,5 +1,6 @@
-// Block attention for units of few query rows (M = G*K; up to 32, and up to 64 where the units alone fill
-// the GPU) at head_dim 128, and of any number at head_dim 64 (in tiles of up to 128 rows), bf16, both views, on tcgen05 with the KEYS on the MMA's rows:
+// Block attention for units of few query rows (M = G*K; up to 32, and up to 64 where the wide kernel's plan does
+// not suit the number of units) at head_dim 128, and of any number at head_dim 64 (in tiles of up to 128 rows), bf16, both
+// views, on tcgen05 with the KEYS on the MMA's rows:
 //     S^T [128 keys x NR rows] = K_tile . Q^T        O^T [d x NR rows] = V_tile^T . P^T
 // NR = M rounded up to 16, 32, 64 or 128 is the MMA's N.  With the query rows there instead, an M of 4 to 64
 // is padded to 128, and only the threads that own real rows take part in the softmax and the
@@ -16,7 +17,7 @@
 // 7.0 us, one unit of 128 rows and 4000 keys 15.1 -> 9.4, 256 of 2000 keys 103 -> 68.  A batch of 256
 // units of 64 rows at 4000 keys streams at 6.4 TB/s.  From 33 rows at head_dim 128 the kernel for wide
 // units, whose tiles are half as long and whose threads hold a row each, takes less from the first score to
-// the last product (8 units of 64 rows and 4096 keys 13.0 against 10.5 us).
+// the last product (8 units of 64 rows and 4096 keys 12.4 against 10.1 us; the rule is in api.cu, wide_better).
 //
 // One CTA (320 threads, up to 64 rows at most 113 KB of shared memory and 256 TMEM columns: two fit an SM, so that
 // with programmatic dependent launch the next call's CTAs are resident and, if the caller promised
@@ -32,10 +33,12 @@
 // through shared memory, and the running reference of a row is raised only when a tile exceeds it
 // by more than 2^8 (then O^T's column is rescaled in TMEM); the result is the exact softmax because
 // numerator and denominator use the same reference.  References are integers: another reference
-// scales a probability by a power of two, so that its rounding to bf16, and with it the result up to
+// scales a probability by a power of two, so that its rounding to bf16, and with it the result of this kernel up to
 // the order of fp32 sums, does not depend on how the keys were cut.  Probabilities are written as
 // bf16 rows [key][row], which is the MN-major B operand of the second product; their sums are taken
-// over the same rounded values, while that product runs.
+// over the same rounded values, while that product runs.  (attend_tc.cu rounds the same probabilities but sums
+// them before rounding: a call that moves from one kernel to the other keeps its numerators and changes its
+// denominators by up to the mean rounding of the probabilities, 2^-9 at most.)
 //
 // Merge of the S CTAs of a cluster (one unit).  A thread of the read-out holds its head column of four
 // query rows per 16 bytes.  Where the CTAs have much to tell one another (`exchanges`), it sends them into
@@ -879,6 +882,8 @@ int keys_splits(int d, int G, int K, int units, int max_keys)
     last = k;
     return k.S;
 }
+
+int keys_resident_clusters(int S) { return resident_clusters<128, 64>(S); }
 
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st)
 {

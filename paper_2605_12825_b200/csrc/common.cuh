@@ -86,6 +86,7 @@ size_t tc_stream_workspace_bytes(int B, int Hkv, int n_ctas);
 cudaError_t launch_attend_tc_stream(const AttnParams &p, int n_ctas, void *ws_body, int flags, cudaStream_t st);
 int keys_rows(int d, int G, int K);      // MMA columns of a query tile on the keys kernel (0: not its shape)
 int keys_splits(int d, int G, int K, int units, int max_keys);   // CTAs per (unit, query tile) on the current device
+int keys_resident_clusters(int S);       // clusters of S CTAs, two to an SM, that are resident at once
 int tc_kb_rows(int G, int K);            // block positions per query tile of 128 rows
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st);        // n_splits = cluster size
 cudaError_t launch_combine(const AttnParams &p, int dtype, cudaStream_t st);
