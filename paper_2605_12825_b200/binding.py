@@ -3,16 +3,21 @@ module, everything else through ctypes.
 
 Every function has the name of the C entry point it calls; tensors are torch CUDA
 tensors whose device pointers are handed over unchanged.  torch is used for device
-memory and streams, nothing else.  There is no fallback: if the library has not
-been built, importing this module raises.
+memory and streams, nothing else.  There is no fallback for the library: if it has not
+been built, importing this module raises.  The native module only marshals arguments and is tied to one
+interpreter and one torch; without one for this pair the same calls go through ctypes, with a warning.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import warnings
 from typing import Optional
 
 import torch
+
+from .build import native_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liborthrus.so")
@@ -119,15 +124,31 @@ _lib = None
 _lib = _load()
 
 
-# after torch and liborthrus.so, whose symbols it uses
-from . import _native  # noqa: E402
-
-
 def _raise(code: int, where: str) -> None:
     raise OrthrusError(code, where)
 
 
-_native.set_raiser(_raise)
+def _load_native():
+    """The native marshalling, after torch and liborthrus.so, whose symbols it uses; else the ctypes one."""
+    path, why = native_path(), "it has not been built"
+    if os.path.exists(path):
+        try:
+            spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+            mod = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(mod)
+            mod.set_raiser(_raise)
+            return mod
+        except ImportError as e:
+            why = str(e)
+    warnings.warn(f"no native argument marshalling for this Python and torch ({os.path.basename(path)}: {why}); calls go "
+                  "through ctypes and cost the host several microseconds more.  `python -m paper_2605_12825_b200.build` "
+                  "compiles it.", RuntimeWarning, stacklevel=3)
+    from . import _marshal
+    _marshal.bind(_lib, _raise)
+    return _marshal
+
+
+_native = _load_native()
 
 
 def lib() -> ctypes.CDLL:

@@ -1,21 +1,30 @@
 """Builds liborthrus.so (sm_100a) with nvcc and the native argument marshalling with g++, in-tree.
-Usable without a GPU."""
+Usable without a GPU.  The library needs nvcc alone; without a C++ compiler or torch's headers there is no
+native marshalling, and binding.py uses ctypes."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liborthrus.so")
 NATIVE_SRC = os.path.join(CSRC, "native_binding.cpp")
-NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
+
+
+def native_path() -> str:
+    """The native marshalling for this interpreter and this torch, whose binary interfaces it is compiled against:
+    one file for each pair, so that none is loaded into another."""
+    import torch
+    return os.path.join(HERE, f"_native.{sys.implementation.cache_tag}-torch{torch.__version__}.so")
 
 
 def sources():
@@ -23,20 +32,19 @@ def sources():
 
 
 def stale_native() -> bool:
-    if not os.path.exists(NATIVE):
+    if not os.path.exists(native_path()):
         return True
-    t = os.path.getmtime(NATIVE)
+    t = os.path.getmtime(native_path())
     return any(os.path.getmtime(f) > t for f in [NATIVE_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h")))
 
 
 def start_native():
     """Starts the compilation of the native argument marshalling (it needs torch's and Python's
     headers and links against torch and liborthrus.so); finish_native() links it."""
-    import sysconfig
     import torch
     inc = os.path.join(os.path.dirname(torch.__file__), "include")
     obj = os.path.join(HERE, "_build", "native_binding.o")
-    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-w",
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-Wall", "-Wextra",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I", os.path.join(ROOT, "include"), "-isystem", inc,
            "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
@@ -50,14 +58,14 @@ def finish_native(started) -> None:
     import torch
     obj, pr = started
     out = pr.communicate()[0].decode()
+    sys.stderr.write(out)
     if pr.returncode != 0:
-        sys.stderr.write(out)
         raise RuntimeError("compiling native_binding.cpp failed")
-    tmp = NATIVE + f".tmp{os.getpid()}"
+    tmp = native_path() + f".tmp{os.getpid()}"
     subprocess.run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, "-L", HERE, "-l:liborthrus.so",
                     "-Wl,-rpath,$ORIGIN", "-L", os.path.join(os.path.dirname(torch.__file__), "lib"),
                     "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
-    os.replace(tmp, NATIVE)
+    os.replace(tmp, native_path())
 
 
 def stale() -> bool:
@@ -72,11 +80,20 @@ def stale() -> bool:
 def build(force: bool = False, verbose: bool = False) -> str:
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
-    native = start_native() if force or stale_native() else None
+    native = why = None
+    try:
+        native = start_native() if force or stale_native() else None
+    except OSError as e:                        # no compiler
+        why = e
     if force or stale():
         build_lib(objdir, verbose)
-    if native:
-        finish_native(native)
+    try:
+        if native:
+            finish_native(native)
+    except (RuntimeError, OSError, subprocess.CalledProcessError) as e:
+        why = e
+    if why:
+        warnings.warn(f"no native argument marshalling, calls will go through ctypes: {why}", RuntimeWarning)
     return LIB
 
 
