@@ -1,6 +1,8 @@
-"""The kernel with the keys on the MMA's rows (bf16, "auto" path), head_dim 64 and 128.
+"""The kernel with the keys on the MMA's rows (bf16, "auto" path), head_dim 64 and, up to 32 rows, 128.
 Edges of its row counts (16, 32, 64, 128, several tiles of 128), of its key tiles, of the cluster split (CTAs without a
-tile included), both masks, the block as a tensor and in the cache, NaN behind the keys."""
+tile included), both masks, the block as a tensor and in the cache, NaN behind the keys.  33 to 64 rows at head_dim 128, which
+the library may put there, are in test_gpu_rows_33_to_64.py; the shapes of more rows at 128 belong to the wide
+kernel and stand for the other side of the line."""
 import pytest
 import torch
 

@@ -13,18 +13,21 @@ import pytest
 import torch
 
 import oracle
-from _gpu_util import Guarded, binding
+from _gpu_util import Guarded, binding, captured_launches
 
 pytestmark = pytest.mark.gpu
 MARGIN_ACCEPT, MARGIN_PICK = 1e-4, 1e-2
 
 
-def run_gpu(la, ld, draft, ua, ur, T):
+def run_gpu(la, ld, draft, ua, ur, T, shift=0):
+    """shift: elements by which the second logit tensor lies off its 16-byte alignment."""
     b = binding()
     B, K, V = la.shape
+    pad = torch.empty(ld.numel() + 16, dtype=ld.dtype, device="cuda")
+    ld = pad[shift:shift + ld.numel()].view(ld.shape).copy_(ld)
     ws = b.new_workspace(b.orthrus_consensus_sample_workspace_bytes(B, K, V))
     outs = [Guarded((B,), torch.int32), Guarded((B, K), torch.int32), Guarded((B,), torch.int32)]
-    b.orthrus_consensus_sample(la.cuda(), ld.cuda(), draft.cuda(), ua.float().cuda(), ur.float().cuda(), T,
+    b.orthrus_consensus_sample(la.cuda(), ld, draft.cuda(), ua.float().cuda(), ur.float().cuda(), T,
                                outs[0].t, outs[1].t, outs[2].t, ws)
     torch.cuda.synchronize()
     assert all(o.intact() for o in outs)
@@ -42,8 +45,8 @@ def make_case(B, K, V, dtype, seed, keep=0.7, spread=1.0):
     return la, ld, draft.contiguous(), ua, ur
 
 
-def check(la, ld, draft, ua, ur, T, min_decided=0.9):
-    n, com, nxt = run_gpu(la, ld, draft, ua, ur, T)
+def check(la, ld, draft, ua, ur, T, min_decided=0.9, shift=0):
+    n, com, nxt = run_gpu(la, ld, draft, ua, ur, T, shift)
     rn, rcom, rnxt, margin = oracle.consensus_sample(la, ld, draft, ua.double(), ur.double(), T)
     B, K, V = la.shape
     decided = (margin[:, 0] > MARGIN_ACCEPT) & (margin[:, 1] > MARGIN_PICK)
@@ -135,17 +138,24 @@ def test_rejects_bad_arguments_on_the_host():
     assert b.orthrus_launch_count() == n0
 
 
-def test_staged_verification_in_a_child_process():
-    """Large problems verify the block in two stages (the second only for sequences without a
-    rejection so far).  The stage boundary is chosen when the library is first used, so the
-    small cases above are repeated in a child process with the boundary forced to 2 positions:
-    rejections before, at and after the boundary, and blocks kept whole."""
-    import os
-    import subprocess
-    import sys
-    env = dict(os.environ, ORTHRUS_SAMPLE_FIRST_STAGE="2")
-    r = subprocess.run([sys.executable, "-m", "pytest", os.path.abspath(__file__), "-x", "-q",
-                        "-k", "matches_oracle or temperatures or every_draft_kept or distribution"],
-                       env=env, capture_output=True, text=True, timeout=900)
-    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
-    assert " passed" in r.stdout
+# The skipping form of the statistics pass (more than 64 stretches per SM: rows behind a known rejection are left out),
+# with rows that start at every alignment (odd vocabulary), logit tensors aligned differently from one another
+# (no vector loads), fp32, and blocks kept whole, rejected at once and rejected somewhere in the same call.
+@pytest.mark.parametrize("B,K,V,dtype,shift", [(64, 32, 20001, torch.bfloat16, 0), (64, 32, 20001, torch.bfloat16, 1),
+                                               (300, 17, 8195, torch.bfloat16, 3), (40, 32, 32003, torch.float32, 0),
+                                               (40, 32, 32003, torch.float32, 1), (12, 24, 151937, torch.bfloat16, 0)])
+def test_rows_behind_a_rejection_are_skipped(B, K, V, dtype, shift):
+    la, ld, draft, ua, ur = make_case(B, K, V, dtype, seed=B + K + shift)
+    ld[0::4] = la[0::4]                                  # p == q: kept whole
+    ua[1::4, 0] = 1.0 - 2.0 ** -20                       # rejected at once: a draft the AR view does not expect
+    for s in range(1, B, 4):
+        la[s, 0, draft[s, 0]] = -30.0
+    rn = check(la, ld, draft, ua, ur, 1.0, shift=shift)
+    assert (rn[0::4] == K).all() and (rn[1::4] == 1).all() and int(rn[2::4].max()) > 1
+
+    b = binding()
+    z = torch.zeros(B, K, dtype=torch.int32, device="cuda")
+    lg, u, n = torch.empty(B, K, V, dtype=dtype, device="cuda"), torch.zeros(B, K, device="cuda"), z[:, 0].contiguous()
+    ws = b.new_workspace(b.orthrus_consensus_sample_workspace_bytes(B, K, V))
+    names = [x for x, _ in captured_launches(lambda: b.orthrus_consensus_sample(lg, lg, z, u, u, 1.0, n, z, n, ws))]
+    assert len(names) == 3 and "sample_init_kernel" in names[0], names      # (it clears the failures)
