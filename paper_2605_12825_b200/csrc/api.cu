@@ -259,7 +259,7 @@ static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (kn.splits > 0) return kn.splits < 16 ? kn.splits : 16;
     // from prefix and block together: a decoder that bounds its lengths by capacity - block then cuts
-    // a block's verification and a width-1 step at the same keys, and both round alike
+    // a block's verification and a width-1 step at the same keys, and where both run on this kernel they round alike
     return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
                        max_len_of(L) + L->block);
 }

@@ -771,9 +771,10 @@ template <int HD, int NR> int resident_clusters(int S)
 }
 
 // Clusters of up to four CTAs that exchange 4 KB or more with each other merge through distributed shared
-// memory.  Measured per call, L2 against exchange, d = 128: 128 units of 64 rows, 1000 keys (2 CTAs) 23.1 and
-// 19.0 us; 64 units, 2000 keys (4 CTAs) 18.5 and 17.1; 128 units of 32 rows, 400 keys (2) 11.5 and 9.9; but 32
-// units of 64 rows, 1000 keys (8) 11.6 and 11.9, 8 units of 4000 keys (16) 11.5 and 12.7, 4 rows (2) 8.5 and 8.8.
+// memory.  Measured per call, through L2 against exchanged: d = 128, 32 rows: 128 units of 1000 keys (2 CTAs) 17.5 and
+// 16.2 us, of 400 10.9 and 9.4, 64 of 2000 (4) 15.8 and 15.1; 64 rows: 128 of 1000 (2) 22.1 and 18.4, 64 of 2000 (4)
+// 19.2 and 17.8; d = 64, 128 rows: 64 of 2000 (2) 26.3 and 23.6; but d = 128, 32 rows: 32 units of 1000 keys (8) 8.3 and 8.8,
+// 8 of 4000 (16) 8.3 and 9.7; d = 64, 64 rows: 32 of 1000 (8) 8.8 and 9.5.
 constexpr bool exchanges(int d, int nr, int S) { return S > 1 && S <= 4 && nr >= 32 && nr * d >= 1024 * S; }
 
 // CTAs per unit.  A CTA's time is that of its tiles one after the other; a merge costs as much as one
@@ -782,10 +783,11 @@ constexpr bool exchanges(int d, int nr, int S) { return S > 1 && S <= 4 && nr >=
 // Of sizes that cost the same the largest up to 8 (lengths are often below the bound the plan is
 // made for, and then the larger size has fewer tiles), else the smallest; above 10 a single tile per
 // CTA gains nothing over two.  Measured per call, chained in a graph, lengths 0.7 to 1 times the bound:
-// d = 128, 64 rows: 8 units, bound 150, 7.3 us at 1 CTA, 11.5 at 2; bound 2000, 9.1 us at 10, 10.1 at 8;
-// bound 4000, 10.7 us at 16, 12.0 at 8; 128 units, bound 400, 13.2 us at 1, 16.5 at 2; 256 units,
-// bound 2000, 46.5 us at 1, 61 at 2; 4 rows: 8 units, bound 400, 5.2 us at 5, 7.4 at 1; bound 4000,
-// 7.6 at 16, 9.5 at 8; d = 64, 32 rows: 2 units, bound 1000, 5.2 us at 10, 5.8 at 8, 11.8 at 1.
+// d = 128, 32 rows: 8 units, bound 150, 5.1 us at 1 CTA, 5.8 at 2; bound 2000, 6.6 us at 10, 8.1 at 8; bound 4000,
+// 8.2 us at 16, 10.4 at 8; 32 units, bound 2000, 10.1 at 8, 16.8 at 9 (not all resident); 128 units, bound 400, 9.5 us at 2, 10.7 at 1;
+// 256 units, bound 2000, 43 us at 1, 49 at 2; 4 rows: 8 units, bound 400, 4.6 us at 5, 7.2 at 1; bound 4000, 7.2 at 16,
+// 9.4 at 8; 64 rows: 12 units, bound 8000, 15.2 us at 16, 19.5 at 8; 42 units, bound 6000, 27.1 at 6, 31.6 at 4, 38.0 at 7 (not
+// all resident); 256 units, bound 2000, 45 us at 1, 54 at 2; d = 64, 32 rows: 2 units, bound 1000, 4.5 us at 10, 5.0 at 8, 10.8 at 1.
 template <int HD, int NR> int choose_splits(int units, int halves)
 {
     int best = 1, best_cost = 1 << 30;
