@@ -220,10 +220,14 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 //    Rows that do not fill warps of 32 cost the wide kernel a second way through its softmax, so that the line
 //    lies lower there (48 rows, 10 units of 3500 keys 9.8 and 11.8, 42 of 2500 16.1 and 17.3).
 // In a decoder (rotary write, both views, room above the lengths; us per write and call) the signs are the same: 64 rows, 32 units of
-// 1450 keys 17.2 and 16.4, of 3300 22.9 and 20.3, 48 of 3300 28.2 and 25.6, 40 of 6500 35.9 and 38.0; the two come
-// within 3 % of one another, either way, at 28 to 32 units of 1600 to 2000 keys.
-// A width-1 step (M <= 32) and the verification of a block (M > 32) thus run different kernels, which agree up to the
-// rounding of their sums; a program that wants the same bits from both sets ORTHRUS_TC_SMALL_ROWS=1.
+// 1450 keys 17.2 and 16.4, of 3300 22.9 and 20.3, 48 of 3300 28.2 and 25.6, 40 of 6500 35.9 and 38.0.
+//  - Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys are a draw: 32 units of 64 rows +3 to -5 %
+//    in a decoder, 24 and 28 units 0 to -7, 52 rows +7 to 0.  There the equal rounding with width-1 steps decides for the keys
+//    kernel: a width-1 step (M <= 32) runs on it too, and cut into as many CTAs the two agree to the last bit, where the two
+//    kernels agree up to the rounding of their sums.  In the bf16 decoder of 12 layers, 32 units and 2048 to 2560 keys no token of
+//    2340 then differs from plain decoding, against 72 near ties that resolve differently with the block on the wide kernel
+//    (45 if that one summed the rounded probabilities too).  Elsewhere the faster kernel is taken; a program that wants
+//    the same bits from both widths throughout sets ORTHRUS_TC_SMALL_ROWS=1.
 static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (!tc_usable(L)) return false;
@@ -231,7 +235,9 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
     const int S = make_plan(L, true, kn).n_splits;
     if (S > 1 && units > keys_resident_clusters(S)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
-    return !((S == 4 || S == 8) && roomy && max_len_of(L) > (M == 64 ? 4096 : 2048));
+    const int max_len = max_len_of(L);
+    if (S == 8 && !roomy) return max_len <= 1536 || max_len > 3072;
+    return !((S == 4 || S == 8) && roomy && max_len > (M == 64 ? 4096 : 2048));
 }
 
 // Units of at most 32 query rows (4 rows, 8 units of 4000 keys 7.3 against 9.7 us on the wide kernel; at 32 rows the two

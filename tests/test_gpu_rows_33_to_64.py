@@ -96,14 +96,16 @@ def test_cuts_that_many_units_pick_by_themselves(B, K, monkeypatch):
 
 # (units, rows, bound, kernel)
 PICKS = [(8, 64, 100, "wide"), (8, 64, 300, "wide"), (8, 64, 512, "wide"), (8, 64, 4096, "wide"), (8, 64, 20000, "wide"),
-         (32, 64, 2000, "wide"), (48, 64, 3000, "wide"), (128, 64, 2000, "wide"), (256, 64, 300, "wide"),
+         (32, 64, 500, "wide"), (48, 64, 3000, "wide"), (128, 64, 2000, "wide"), (256, 64, 300, "wide"), (8, 36, 4096, "wide"),
          # clusters of the wide kernel that are not all resident
-         (33, 64, 1700, "wide"), (34, 64, 1700, "keys"), (37, 64, 1700, "keys"), (38, 64, 1700, "wide"),
+         (33, 64, 1300, "wide"), (34, 64, 1300, "keys"), (37, 64, 1700, "keys"), (38, 64, 1700, "wide"),
          (160, 64, 960, "wide"), (160, 64, 961, "keys"), (296, 64, 1024, "wide"), (320, 64, 1024, "wide"),
          # half-empty grids
          (12, 64, 4096, "wide"), (12, 64, 4097, "keys"), (44, 64, 4097, "keys"), (46, 64, 4097, "wide"), (80, 64, 4500, "wide"),
          (12, 36, 2048, "wide"), (12, 36, 2049, "keys"), (42, 60, 2049, "keys"), (46, 36, 3000, "wide"),
-         (32, 36, 2049, "wide"), (8, 36, 4096, "wide")]
+         # clusters of eight that fill the grid
+         (22, 64, 2000, "wide"), (23, 64, 2000, "keys"), (32, 64, 1536, "wide"), (32, 64, 1537, "keys"), (32, 64, 3072, "keys"),
+         (32, 64, 3073, "wide"), (32, 36, 1536, "wide"), (32, 36, 3072, "keys")]
 
 
 @pytest.mark.parametrize("units,rows,bound,kernel", PICKS)
