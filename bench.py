@@ -63,10 +63,11 @@ def measured_tensor_peak():
 # DRAM bytes (read + write) per launch from the ncu captures summarised under profiles/, each
 # with the first 16 hex digits of the SHA-256 of the kernel sources the capture was taken
 # from: once those files change the figure is stale and None is reported.
-NCU_TRAFFIC = {"cfg2_8b_b1": (17068288, "40cd1b2b5bbcc023")}
+NCU_TRAFFIC = {"cfg2_8b_b1": (17064576, "b761ffb8afe492c6"), "cfg3_ragged": (512661248, "b761ffb8afe492c6"),
+               "cfg4_long": (542857088, "b761ffb8afe492c6")}
 NCU_TRAFFIC_SOURCES = ("attend_tc.cu", "tc_ptx.cuh")
-NCU_TRAFFIC_LM_HEAD = {("cfg2_8b_b1", 4096): (1249568280, "5112ef6ba5d70c0f"),
-                       ("cfg3_ragged", 4096): (1067102904, "5112ef6ba5d70c0f")}
+NCU_TRAFFIC_LM_HEAD = {("cfg2_8b_b1", 4096): (1247972200, "a99646786b164572"),
+                       ("cfg3_ragged", 4096): (1066815368, "a99646786b164572")}
 NCU_TRAFFIC_LM_HEAD_SOURCES = ("lm_head_argmax.cu", "tc_ptx.cuh")
 
 
