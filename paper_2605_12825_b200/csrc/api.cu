@@ -240,8 +240,13 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
     return !((S == 4 || S == 8) && roomy && max_len > (M == 64 ? 4096 : 2048));
 }
 
-// Units of at most 32 query rows (4 rows, 8 units of 4000 keys 7.3 against 9.7 us on the wide kernel; at 32 rows the two
-// are level), of 33 to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
+static int keys_tiles(const orthrus_layer_t *L)
+{
+    const int kb = tc_kb_rows(L->n_q_heads / L->n_kv_heads, L->block);
+    return (L->block + kb - 1) / kb;
+}
+
+// Units of at most 32 query rows (4 rows, 8 units of 4000 keys 5.7 against 9.7 us on the wide kernel, 32 rows 6.9), of 33 to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
 // rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
@@ -251,15 +256,10 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     if (L->dtype != ORTHRUS_BF16 || (L->head_dim != 64 && L->head_dim != 128) || kn.small_rows == 0) return false;
     const int rows = keys_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
     const unsigned long long cache = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
-    if (!rows || cache >= 0x7fffffffull || (long long)L->batch * L->n_kv_heads > 65535 || !tc_driver_ok()) return false;
+    if (!rows || cache >= 0x7fffffffull || L->batch > 65535 || (long long)L->n_kv_heads * keys_tiles(L) > 65535 || !tc_driver_ok()) return false;
     if (kn.small_rows > 0) return true;
     if (rows > 64) return max_len_of(L) > 320;
     return rows < 64 || L->head_dim == 64 || !wide_better(L, kn);
-}
-static int keys_tiles(const orthrus_layer_t *L)
-{
-    const int kb = tc_kb_rows(L->n_q_heads / L->n_kv_heads, L->block);
-    return (L->block + kb - 1) / kb;
 }
 static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
 {
@@ -269,14 +269,6 @@ static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
     return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
                        max_len_of(L) + L->block);
 }
-static size_t keys_bytes(const orthrus_layer_t *L, int S, size_t *ml_off)
-{
-    const size_t ctas = S > 1 ? (size_t)L->batch * L->n_kv_heads * keys_tiles(L) * S : 0;
-    const size_t nr = keys_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
-    if (ml_off) *ml_off = ctas * nr * L->head_dim * sizeof(float);
-    return ctas * nr * (L->head_dim + 2) * sizeof(float);
-}
-
 static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off, bool tc = false)
 {
     if (ml_off) *ml_off = 0;
@@ -317,7 +309,7 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     const bool keys = !stream_k && (want == PATH_AUTO || (want == PATH_TCGEN05 && tc)) && keys_usable(L, kn);
     if (keys) pl.n_splits = keys_plan(L, kn);
     const size_t need = kHeaderBytes + (stream_k ? tc_stream_workspace_bytes(L->batch, L->n_kv_heads, tc_stream_ctas())
-                                        : keys   ? keys_bytes(L, pl.n_splits, &ml_off)
+                                        : keys   ? 0
                                                  : partial_bytes(L, pl, &ml_off, tc));
     if (ws_bytes < need) return ORTHRUS_ERR_WORKSPACE;
 
@@ -379,10 +371,6 @@ size_t orthrus_attend_workspace_bytes(const orthrus_layer_t *layer)
     // enough for whichever kernel path a later call resolves to
     const Knobs kn = read_knobs();
     size_t need = partial_bytes(layer, make_plan(layer, false, kn), nullptr, false);
-    if (keys_usable(layer, kn)) {
-        const size_t n1 = keys_bytes(layer, keys_plan(layer, kn), nullptr);
-        if (n1 > need) need = n1;
-    }
     if (tc_usable(layer)) {
         const size_t n2 = partial_bytes(layer, make_plan(layer, true, kn), nullptr, true);
         if (n2 > need) need = n2;

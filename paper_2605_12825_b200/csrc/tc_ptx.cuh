@@ -35,8 +35,8 @@ __device__ inline bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false (and raises the CTA's abort flag) if the phase does not
 // complete within about a second, or if another thread already gave up.
-__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
-    if (mbar_test(bar, parity)) return true;
+// (The loop is one function for all waits of a kernel: its copies filled the instruction cache.)
+static __device__ __noinline__ bool mbar_wait_loop(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
     const long long t0 = clock64();
     for (uint32_t it = 1; it < (1u << 24); ++it) {
         if (mbar_try(bar, parity)) return true;
@@ -48,10 +48,25 @@ __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *ab
     *abort_flag = 1;
     return false;
 }
+__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    return mbar_try(bar, parity) || mbar_wait_loop(bar, parity, abort_flag);
+}
 // the same for a whole warp: every lane learns the common outcome, so that warp-wide
 // (.aligned) instructions behind it are executed by all lanes or by none
 __device__ inline bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
+// a wait for CTAs of the same cluster, whose own waits end within seconds whatever happens to them
+__device__ inline bool mbar_wait_long(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t ok;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                     " selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if (clock64() - t0 > (1ll << 35)) return false;
+    }
 }
 
 // L2 policy for data that is read exactly once (the streamed cache tiles)
@@ -72,6 +87,10 @@ __device__ inline void tma_load_4d(uint32_t dst, const CUtensorMap *tm, int c0, 
                  " [%0], [%1, {%2, %3, %4, %5}], [%6];"
                  ::"r"(dst), "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar) : "memory");
 }
+__device__ inline void prefetch_l2_bulk(const void *p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+__device__ inline void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ inline void prefetch_map(const CUtensorMap *tm) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
@@ -84,6 +103,8 @@ __device__ inline void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// (without the release, which waits for the thread's stores: 330 cycles against 18)
+__device__ inline void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ inline uint32_t cluster_rank() {
     uint32_t r;
@@ -104,6 +125,11 @@ __device__ inline void st_cluster(uint32_t addr, const float4 &v) {
 }
 __device__ inline void st_cluster(uint32_t addr, const uint32_t *v) {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+// the same, counted (16 bytes) by an mbarrier of that CTA
+__device__ inline void st_async(uint32_t addr, const float4 &v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
 }
 // shared-memory matrix descriptor, 128-byte swizzle
 __device__ inline uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
