@@ -135,10 +135,21 @@ template <typename T> __device__ inline bool whole(const RowShape &s, int v) {
     return s.vec && v * Elem<T>::N >= s.a && v * Elem<T>::N - s.a + Elem<T>::N <= s.V;
 }
 // one vector of a row; elements that do not exist are -inf (their exponential is 0)
-template <typename T> __device__ inline void load_vec(const T *row, const RowShape &s, int v, float (&x)[Elem<T>::N]) {
+template <typename T> struct VecOf { float x[Elem<T>::N]; };
+template <typename T> __device__ __noinline__ VecOf<T> load_part(const T *row, int i0, int V) {
+    VecOf<T> r;
+#pragma unroll
+    for (int e = 0; e < Elem<T>::N; ++e) r.x[e] = i0 + e >= 0 && i0 + e < V ? Elem<T>::load(row + i0 + e) : -INFINITY;
+    return r;
+}
+template <typename T, bool CALL> __device__ inline void load_vec(const T *row, const RowShape &s, int v, float (&x)[Elem<T>::N]) {
     const int i0 = v * Elem<T>::N - s.a;
     if (whole<T>(s, v)) {
         Elem<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(row + i0)), x);
+    } else if (CALL) {
+        const VecOf<T> r = load_part<T>(row, i0, s.V);
+#pragma unroll
+        for (int e = 0; e < Elem<T>::N; ++e) x[e] = r.x[e];
     } else {
 #pragma unroll
         for (int e = 0; e < Elem<T>::N; ++e) x[e] = i0 + e >= 0 && i0 + e < s.V ? Elem<T>::load(row + i0 + e) : -INFINITY;
@@ -181,6 +192,14 @@ __device__ inline void fold_row(const StatPart *parts, int n_seg, int lane, RefS
     d = warp_fold(d);
 }
 
+// the same out of line, for the finish kernel, where it stands twice and its code counts
+struct RowFold { RefSum a, d; };
+__device__ __noinline__ RowFold fold_row_call(const StatPart *parts, int n_seg, int lane) {
+    RowFold f;
+    fold_row(parts, n_seg, lane, f.a, f.d);
+    return f;
+}
+
 // per sequence: first row known to fail; per row: stretches done.  Only the skipping form reads them.
 __global__ void sample_init_kernel(int *fail, int *done, int B, int K)
 {
@@ -212,7 +231,7 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, con
             const RowShape sh = row_shape(ra, rd, V);
             const int per = (sh.n_vec + n_seg - 1) / n_seg, v0 = seg * per, v1 = min(sh.n_vec, v0 + per);
             RefSum a{-INFINITY, 0.0}, d{-INFINITY, 0.0};
-            // whole vectors, four of each row at a time; incomplete ones by one lane each
+            // whole vectors, four of each row at a time; the ends of the row by a lane an element
             const int w0 = max(v0, sh.vec ? (sh.a + N - 1) / N : v1), w1 = min(v1, (V + sh.a) / N);
             const uint4 *va = reinterpret_cast<const uint4 *>(ra - sh.a), *vd = reinterpret_cast<const uint4 *>(rd - sh.a);
             int v = w0 + lane;
@@ -234,11 +253,23 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, con
                 Elem<T>::unpack(x, f[0]); absorb<1, N>(a, f, c);
                 Elem<T>::unpack(y, f[0]); absorb<1, N>(d, f, c);
             }
-            for (int e = v0 + lane; e < v1; e += 32) {
-                if (e >= w0 && e < w1) continue;
+            if (sh.vec) {
+                // the elements in front of the first whole vector, then those behind the last one
+                const int lo = max(v0 * N - sh.a, 0), hi = min(v1 * N - sh.a, V);
+                const int h = min(w0 * N - sh.a, hi), t = max(w1 * N - sh.a, h);
+                if (lo < h || t < hi) {
+                    const int e = lane < 8 ? lo + lane : t + lane - 8;
+                    const bool mine = lane < 8 ? e < h : lane < 16 && e < hi;
+                    float f[1][2];
+                    f[0][1] = -INFINITY;
+                    f[0][0] = mine ? Elem<T>::load(ra + e) : -INFINITY; absorb<1, 2>(a, f, c);
+                    f[0][0] = mine ? Elem<T>::load(rd + e) : -INFINITY; absorb<1, 2>(d, f, c);
+                }
+            }
+            else for (int e = v0 + lane; e < v1; e += 32) {
                 float f[1][N];
-                load_vec<T>(ra, sh, e, f[0]); absorb<1, N>(a, f, c);
-                load_vec<T>(rd, sh, e, f[0]); absorb<1, N>(d, f, c);
+                load_vec<T, true>(ra, sh, e, f[0]); absorb<1, N>(a, f, c);
+                load_vec<T, true>(rd, sh, e, f[0]); absorb<1, N>(d, f, c);
             }
             a = warp_fold(a);
             d = warp_fold(d);
@@ -283,6 +314,10 @@ __device__ inline double peer_double(const double *mine, int rank) {
 // double operations, loads from L2), hence 16 warps a CTA, the mass of p only where the residual turns out to be
 // empty, and sums in several chains.  With 8 warps and both masses in one chain each the residual of a row of
 // 128256 took 13 us in clusters of 8; whole passes 102 -> 93 us (batch 32) and 23.8 -> 18.8 us (batch 1).
+// An SM's instruction cache holds 32 KB, and every warp runs through this code once: one round per turn of the loop, the next
+// one's vectors asked for ahead, incomplete vectors and the fold of a row out of line (66 -> 49 KB), in the statistics
+// the ends of a row by a lane an element: 93.6 -> 85.9 us (batch 32), 19.2 -> 18.0 us (batch 1).  The fold out of line in the
+// statistics as well, where it writes to the stack: 118 us.
 constexpr int kFinishThreads = 512, kFinishWarps = kFinishThreads / 32, kGroups = 64;
 template <typename T>
 __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const T *la, const T *ld, int K, int V, int n_seg, float c,
@@ -304,11 +339,10 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
     if (!fail) {
         for (int i = warp; i < K; i += kFinishWarps) {
             const long long row = (long long)b * K + i;
-            RefSum a, d;
-            fold_row(parts + row * n_seg, n_seg, lane, a, d);
+            const RowFold f = fold_row_call(parts + row * n_seg, n_seg, lane);
             if (lane == 0) {
-                folded[2 * i] = a; folded[2 * i + 1] = d;
-                if (!keeps(la + row * V, ld + row * V, a, d, draft[row], u_accept[row], V, c)) atomicMin(&s_first, i);
+                folded[2 * i] = f.a; folded[2 * i + 1] = f.d;
+                if (!keeps(la + row * V, ld + row * V, f.a, f.d, draft[row], u_accept[row], V, c)) atomicMin(&s_first, i);
             }
         }
         __syncthreads();
@@ -326,10 +360,10 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
     const long long row = (long long)b * K + j;
     const T *ra = la + row * V, *rd = ld + row * V;
     if (warp == 0) {
-        RefSum a, d;
-        if (fail) fold_row(parts + row * n_seg, n_seg, lane, a, d);
-        else { a = folded[2 * j]; d = folded[2 * j + 1]; }
-        if (lane == 0) s_stat = RowStat{a.m, d.m, 1.0 / a.s, 1.0 / d.s};
+        RowFold f;
+        if (fail) f = fold_row_call(parts + row * n_seg, n_seg, lane);
+        else f = RowFold{folded[2 * j], folded[2 * j + 1]};
+        if (lane == 0) s_stat = RowStat{f.a.m, f.d.m, 1.0 / f.a.s, 1.0 / f.d.s};
     }
     __syncthreads();
     const RowStat st = s_stat;
@@ -339,34 +373,41 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
     // (a group costs two warp sums, a round in the end two loads: two rounds and up to a group)
     const int rounds = (per_w + 31) / 32, gsz = max(2, (rounds + kGroups - 1) / kGroups), n_grp = (rounds + gsz - 1) / gsz;
     // the residual; if it is empty (p and q agree to the last bit), the mass of p
+#pragma unroll 1
     for (int use_p = 0; use_p < 2; ++use_p) {
         double total = 0.0, sum = 0.0;
-        for (int r0 = 0; r0 < rounds; r0 += 2) {        // the loads of two rounds together
-            float x[2][N], y[2][N];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int v = w0 + (r0 + i) * 32 + lane;
-                if (r0 + i < rounds && v < w1) {
-                    load_vec<T>(ra, sh, v, x[i]);
-                    load_vec<T>(rd, sh, v, y[i]);
-                }
+        // (whole vectors are asked for one round ahead, as they come)
+        uint4 nx = make_uint4(0, 0, 0, 0), ny = nx;
+        auto ask = [&](int r) {
+            const int v = w0 + r * 32 + lane;
+            if (r < rounds && v < w1 && whole<T>(sh, v)) {
+                nx = __ldg(reinterpret_cast<const uint4 *>(ra + v * N - sh.a));
+                ny = __ldg(reinterpret_cast<const uint4 *>(rd + v * N - sh.a));
             }
+        };
+        ask(0);
+        int left = gsz, g = 0;                          // rounds left in this group
+#pragma unroll 1
+        for (int r = 0; r < rounds; ++r) {
+            const uint4 cx = nx, cy = ny;
+            ask(r + 1);
+            const int v = w0 + r * 32 + lane;
+            if (v < w1) {
+                float x[N], y[N];
+                if (whole<T>(sh, v)) { Elem<T>::unpack(cx, x); Elem<T>::unpack(cy, y); }
+                else { load_vec<T, true>(ra, sh, v, x); load_vec<T, true>(rd, sh, v, y); }
+                double m[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r = r0 + i;
-                if (r >= rounds) break;
-                if (w0 + r * 32 + lane < w1) {
-                    double m[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-                    for (int e = 0; e < N; ++e) m[e & 3] += mass_of(x[i][e], y[i][e], c, st, use_p);
-                    sum += (m[0] + m[1]) + (m[2] + m[3]);
-                }
-                if ((r + 1) % gsz == 0 || r == rounds - 1) {
-                    sum = warp_sum(sum);
-                    if (lane == 0) grp[warp][r / gsz] = sum;
-                    total += sum;
-                    sum = 0.0;
-                }
+                for (int e = 0; e < N; ++e) m[e & 3] += mass_of(x[e], y[e], c, st, use_p);
+                sum += (m[0] + m[1]) + (m[2] + m[3]);
+            }
+            if (--left == 0 || r == rounds - 1) {
+                sum = warp_sum(sum);
+                if (lane == 0) grp[warp][g] = sum;
+                total += sum;
+                sum = 0.0;
+                left = gsz;
+                ++g;
             }
         }
         if (lane == 0) wsum[warp] = total;
@@ -403,6 +444,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
         int last = 0;
         auto pick = [&](const double *sums, int n, bool none) {   // -1: past the end
             int z = -1;
+#pragma unroll 4
             for (int i = 0; i < n; ++i) {
                 const double v = sums[i];
                 if (v > 0.0) {
@@ -425,11 +467,12 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
         const int q0 = min(v1, v0 + pw * per_w), q1 = min(v1, q0 + per_w);
         int z = -1, z_last = -1;
         run = at;
+#pragma unroll 1
         for (int r = pg * gsz; r < min(rounds, (pg + 1) * gsz) && z < 0; ++r) {
             const int v = q0 + r * 32 + lane;
             float x[N], y[N];
             double mine[N], sum = 0.0;
-            if (v < q1) { load_vec<T>(ra, sh, v, x); load_vec<T>(rd, sh, v, y); }
+            if (v < q1) { load_vec<T, true>(ra, sh, v, x); load_vec<T, true>(rd, sh, v, y); }
 #pragma unroll
             for (int e = 0; e < N; ++e) {
                 mine[e] = v < q1 ? mass_of(x[e], y[e], c, st, use_p) : 0.0;
