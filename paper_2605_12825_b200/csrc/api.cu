@@ -170,7 +170,7 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
             // Up to four CTAs for a tile each where they leave most SMs idle (8 units of 300 keys 7.6 us
             // a call at 4, 8.1 at 2).  Sixteen only with an SM for each CTA: clusters of that size do not
             // fill the second places (16 units of 4000 keys 16.2 us at 8, 23.2 at 16; of 16000 keys
-            // 40 and 45), and their merge goes through L2.
+            // 40 and 45).
             while (S < 16 && units * S * 2 <= (S == 8 ? num_sms() : slots) &&
                    tiles / (S * 2) >= (S < 4 && units * 8 <= num_sms() ? 1 : kn.min_chunk_tiles)) S *= 2;
         } else {
@@ -178,9 +178,19 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
             //  still split; many small CTAs would spend their time starting and merging)
             while (S < 16 && units * S < slots && tiles / (S * 2) >= 8) S *= 2;
         }
+        // Sixteen only while a call and the next one, which starts early, find SMs of their own, too: on shared ones the CTAs of
+        // a cluster share the way to the others, which the merge of more than 64 rows fills.  As many CTAs as do find some,
+        // then (8 units of 128 rows, 2000, 4000, 8000 and 16000 keys 12.4, 13.6, 17.6 and 26.0 us at 16, 9.1, 11.4, 15.8 and 25.3 at
+        // 10), until streaming the keys is nearly all there is (32000 keys 42.7 and 43.7).
+        const int rows = G * L->block;
+        if (forced <= 0 && S == 16 && 2 * units * S > num_sms() && tiles < (rows > 96 ? 160 : rows > 64 ? 64 : 48)) {
+            S = num_sms() / (2 * units);
+            if (S < 8) S = 8;
+        }
         const int max_cluster = tc_max_cluster(nt);
         if (S > max_cluster) S = max_cluster;
         if (S > tiles) S = tiles;
+        if (S > 12 && S < 16) S = 12;             // (the merge shares 128 columns out by eights; its buffer)
         if (S < 1) S = 1;
         pl.n_splits = S;
         pl.chunk = ((tiles + S - 1) / S) * tn;
@@ -207,31 +217,31 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 }
 
 // 33 to 64 query rows at head_dim 128 can run on either tcgen05 kernel: with the keys on the MMA's rows
-// (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).  The wide
-// one takes less per key (us a call, keys against wide, 64 rows: 8 units of 300 keys 8.3 and 5.8, of 4096 12.4 and
-// 10.1; 32 of 1024 11.0 and 10.2; 48 of 3072 21.4 and 19.8; 128 of 2048 29.0 and 26.5; 320 of 1024 50.0 and 46.1), so it is
-// the rule, for short prefixes as well.  It loses where its plan, whose clusters are powers of two,
-// does not suit the number of units:
-//  - its clusters are not all resident at once (34 to 37 units cut in 8: 37 of 1700 keys 14.5 and 20.3; more units
-//    than SMs, cut in 2 from 15 tiles on: 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9);
-//  - clusters of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix is long
-//    (12 units of 8000 keys 15.9 and 18.4, 44 of 6000 29.0 and 30.8; at 2500 keys they still win: 10.9 and 9.6, 17.7 and 17.3;
-//    clusters of 2 keep the memory busy all the same: 80 units of 4500 keys 44.2 and 40.0).
+// (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).
+//  - Where the caller promises a quiescent cache, the keys kernel has its first three tiles in shared memory by the time the
+//    query rows come, and is the rule up to 64 units (us a call, keys against wide, 64 rows: 8 units of 1000 keys 5.3 and
+//    6.8, of 4000 8.6 and 10.0; 16 of 2000 8.7 and 9.9; 32 of 1000 9.0 and 10.0, of 3500 14.3 and 14.9; 40 of 4000 18.8 and 22.2; 48
+//    of 3000 17.4 and 18.6; 64 of 500 9.3 and 9.7, of 2000 16.8 and 16.7; level at 8 of 300, 5.7 and 5.6).
+//  - With more units the SMs are full in any case, and the wide kernel's takes less per key (128 units of 500, 1000 and 2000 keys
+//    13.5 and 11.8, 18.3 and 16.8, 28.0 and 26.3; 320 of 1000 51.5 and 46.5), unless its clusters are not all resident at
+//    once (256 of 2000, cut in two, 46.3 and 53.6; 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9).
+//  - Without the promise every load waits for the preceding kernel, and the two are within ten per cent of one another
+//    either way (8 units of 300 keys 6.6 and 6.4, of 1000 6.7 and 7.8, of 4096 11.5 and 11.3; 32 of 2000 13.0 and 12.7; 64 of 2000 18.3 and
+//    17.7).  There the wide kernel is the rule, short prefixes included, where its plan, whose clusters are powers of two, suits
+//    the number of units: not where its clusters are not all resident (34 to 37 units cut in 8: 37 of 1700 keys 14.5 and
+//    20.3), nor where clusters of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix
+//    is long (12 units of 8000 keys 15.9 and 18.4, 44 of 6000 29.0 and 30.8; at 2500 keys the wide one still won).
 //    Rows that do not fill warps of 32 cost the wide kernel a second way through its softmax, so that the line
 //    lies lower there (48 rows, 10 units of 3500 keys 9.8 and 11.8, 42 of 2500 16.1 and 17.3).
-// In a decoder (rotary write, both views, room above the lengths; us per write and call) the signs are the same: 64 rows, 32 units of
-// 1450 keys 17.2 and 16.4, of 3300 22.9 and 20.3, 48 of 3300 28.2 and 25.6, 40 of 6500 35.9 and 38.0.
-//  - Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys are a draw: 32 units of 64 rows +3 to -5 %
-//    in a decoder, 24 and 28 units 0 to -7, 52 rows +7 to 0.  There the equal rounding with width-1 steps decides for the keys
-//    kernel: a width-1 step (M <= 32) runs on it too, and cut into as many CTAs the two agree to the last bit, where the two
-//    kernels agree up to the rounding of their sums.  In the bf16 decoder of 12 layers, 32 units and 2048 to 2560 keys no token of
-//    2340 then differs from plain decoding, against 72 near ties that resolve differently with the block on the wide kernel
-//    (45 if that one summed the rounded probabilities too).  Elsewhere the faster kernel is taken; a program that wants
-//    the same bits from both widths throughout sets ORTHRUS_TC_SMALL_ROWS=1.
+//    Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys are a draw, and the equal rounding with
+//    width-1 steps decides for the keys kernel: a width-1 step (M <= 32) runs on it too, and cut into as many CTAs the two
+//    agree to the last bit, where the two kernels agree up to the rounding of their sums.  A program that wants the same
+//    bits from both widths throughout promises a quiescent cache or sets ORTHRUS_TC_SMALL_ROWS=1.
 static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (!tc_usable(L)) return false;
     const int units = L->batch * L->n_kv_heads, M = L->n_q_heads / L->n_kv_heads * L->block;
+    if ((L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units <= 64 && (units < 24 || max_len_of(L) >= 1024)) return false;
     const int S = make_plan(L, true, kn).n_splits;
     if (S > 1 && units > keys_resident_clusters(S)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
@@ -242,7 +252,7 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
 
 static int keys_tiles(const orthrus_layer_t *L)
 {
-    const int kb = tc_kb_rows(L->n_q_heads / L->n_kv_heads, L->block);
+    const int kb = keys_kb_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
     return (L->block + kb - 1) / kb;
 }
 
@@ -257,6 +267,10 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     const int rows = keys_rows(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block);
     const unsigned long long cache = (unsigned long long)L->batch * L->n_kv_heads * (unsigned long long)L->capacity;
     if (!rows || cache >= 0x7fffffffull || L->batch > 65535 || (long long)L->n_kv_heads * keys_tiles(L) > 65535 || !tc_driver_ok()) return false;
+    const int M = L->n_q_heads / L->n_kv_heads * L->block, units = L->batch * L->n_kv_heads;
+    if (L->head_dim == 128 && M > 64)
+        return kn.small_rows < 0 && (L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units * keys_tiles(L) <= 16 &&
+               max_len_of(L) <= 8192;
     if (kn.small_rows > 0) return true;
     if (rows > 64) return max_len_of(L) > 320;
     return rows < 64 || L->head_dim == 64 || !wide_better(L, kn);
@@ -269,14 +283,12 @@ static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
     return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
                        max_len_of(L) + L->block);
 }
-static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off, bool tc = false)
+// Split partials of the mma and SIMT paths (the tcgen05 kernels merge through shared memory)
+static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off)
 {
     if (ml_off) *ml_off = 0;
     if (pl.n_splits == 1) return 0;
-    // the tcgen05 path keeps one 128-row partial tile per CTA
-    const size_t units = (size_t)L->batch * L->n_kv_heads *
-                         (tc ? tc_row_tiles(L->n_q_heads / L->n_kv_heads, L->block) : 1);
-    const size_t M = tc ? 128 : (size_t)(L->n_q_heads / L->n_kv_heads) * L->block;
+    const size_t units = (size_t)L->batch * L->n_kv_heads, M = (size_t)(L->n_q_heads / L->n_kv_heads) * L->block;
     const size_t o_bytes = units * pl.n_splits * M * L->head_dim * sizeof(float);
     const size_t ml_bytes = units * pl.n_splits * M * 2 * sizeof(float);
     if (ml_off) *ml_off = o_bytes;
@@ -309,8 +321,7 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     const bool keys = !stream_k && (want == PATH_AUTO || (want == PATH_TCGEN05 && tc)) && keys_usable(L, kn);
     if (keys) pl.n_splits = keys_plan(L, kn);
     const size_t need = kHeaderBytes + (stream_k ? tc_stream_workspace_bytes(L->batch, L->n_kv_heads, tc_stream_ctas())
-                                        : keys   ? 0
-                                                 : partial_bytes(L, pl, &ml_off, tc));
+                                        : keys || tc ? 0 : partial_bytes(L, pl, &ml_off));
     if (ws_bytes < need) return ORTHRUS_ERR_WORKSPACE;
 
     AttnParams p;
@@ -370,14 +381,10 @@ size_t orthrus_attend_workspace_bytes(const orthrus_layer_t *layer)
     if (check_layer(layer) != ORTHRUS_OK) return 0;
     // enough for whichever kernel path a later call resolves to
     const Knobs kn = read_knobs();
-    size_t need = partial_bytes(layer, make_plan(layer, false, kn), nullptr, false);
-    if (tc_usable(layer)) {
-        const size_t n2 = partial_bytes(layer, make_plan(layer, true, kn), nullptr, true);
-        if (n2 > need) need = n2;
-        if (tc_use_stream(layer, kn)) {
-            const size_t n3 = tc_stream_workspace_bytes(layer->batch, layer->n_kv_heads, tc_stream_ctas());
-            if (n3 > need) need = n3;
-        }
+    size_t need = partial_bytes(layer, make_plan(layer, false, kn), nullptr);
+    if (tc_usable(layer) && tc_use_stream(layer, kn)) {
+        const size_t n3 = tc_stream_workspace_bytes(layer->batch, layer->n_kv_heads, tc_stream_ctas());
+        if (n3 > need) need = n3;
     }
     return kHeaderBytes + need;
 }
@@ -450,16 +457,14 @@ static orthrus_status_t attend_packed(const orthrus_layer_t *layer, int32_t n_bl
         return ORTHRUS_ERR_INVALID_ARG;
     const orthrus_layer_t L = packed_layer(layer, n_blocks);
     const Plan pl = make_plan(&L, true, kn);
-    size_t ml_off = 0;
-    if (ws_bytes < kHeaderBytes + partial_bytes(&L, pl, &ml_off, true)) return ORTHRUS_ERR_WORKSPACE;
+    if (ws_bytes < (size_t)kHeaderBytes) return ORTHRUS_ERR_WORKSPACE;
 
     AttnParams p;
     p.q = q; p.k_blk = k_blk; p.v_blk = v_blk; p.k_cache = layer->k_cache; p.v_cache = layer->v_cache;
     p.cache_len = anchors; p.out = out;
     unsigned char *base = static_cast<unsigned char *>(ws);
     p.status = reinterpret_cast<int32_t *>(base);
-    p.part_o = reinterpret_cast<float *>(base + kHeaderBytes);
-    p.part_ml = reinterpret_cast<float *>(base + kHeaderBytes + ml_off);
+    p.part_o = p.part_ml = nullptr;
     p.B = layer->batch; p.K = L.block; p.Hq = layer->n_q_heads; p.Hkv = layer->n_kv_heads;
     p.G = p.Hq / p.Hkv; p.M = p.G * p.K; p.d = layer->head_dim; p.capacity = layer->capacity;
     p.chunk = pl.chunk; p.n_splits = pl.n_splits; p.causal = 0; p.blk_in_cache = 0;
@@ -478,15 +483,8 @@ size_t orthrus_multi_block_workspace_bytes(const orthrus_layer_t *layer, int32_t
 {
     orthrus_layer_t L;
     if (!multi_block_layer(layer, n_blocks, nullptr, &L)) return 0;
-    // enough for either form
-    size_t need = orthrus_attend_workspace_bytes(&L);
-    if (need && check_layer(layer) == ORTHRUS_OK && tc_usable(layer) && n_blocks >= 2 &&
-        (long long)n_blocks * layer->block <= (1 << 20)) {
-        const orthrus_layer_t Lp = packed_layer(layer, n_blocks);
-        const size_t n2 = kHeaderBytes + partial_bytes(&Lp, make_plan(&Lp, true, read_knobs()), nullptr, true);
-        if (n2 > need) need = n2;
-    }
-    return need;
+    // enough for either form (the packed one needs the header alone)
+    return orthrus_attend_workspace_bytes(&L);
 }
 
 orthrus_status_t orthrus_multi_block_attend(const orthrus_layer_t *layer, int32_t n_blocks,

@@ -181,6 +181,9 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
     const int my_tasks = (int)((uint32_t)(n_tasks - rank + S - 1) * args.inv_s >> 16);
 
     // ------------------------------------------------------------------ prologue
+    int b = blockIdx.z, P = 0;
+    const bool len_first = quiescent && !args.ranked;         // the length is on its way while the barriers are set up
+    if (len_first) P = p.cache_len[b];
     // The producer is to ask for its first tiles as early as can be: it sets up the barriers of the ring and waits for nobody.
     if (warp == PRODUCER_WARP) {
         if (lane == 0) {
@@ -191,47 +194,31 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         }
         __syncwarp();
         bar_start_arrive();
+    } else if (warp == MMA_WARP) {
+        if (lane == 0) {
+            *abort_flag = (sbase & 1023u) == 0 ? 0 : 1;   // swizzled tiles need 1 KB alignment
+#pragma unroll
+            for (int i = C::BAR_Q; i < C::NUM_BARS; ++i) mbar_init(bar(i), i == C::BAR_Q ? SW : 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_proxy_async();
+            if (XCH) mbar_expect_tx(bar(C::BAR_X), (uint32_t)(my_tasks * S * MSG));
+            prefetch_map(&tm.kb); prefetch_map(&tm.vb);
+        }
+        __syncwarp();
+        bar_issue_arrive();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(C::TM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else if (tid < 2 * NR) {
+        reinterpret_cast<float *>(smem + C::OFF_REF)[tid] = 0.f;
     }
     // which unit: when the clusters do not all fit at once they go out longest prefix first (every warp finds out by itself)
     if (!quiescent) griddep_wait();
-    int b = blockIdx.z;
     const int h = blockIdx.y - zt * p.Hkv;
     const int len_hi = (int)p.len_cap;
-    if (args.ranked) {
-        int mine = -1;
-#pragma unroll 1
-        for (int i = lane; i < p.B; i += 32) {
-            const int Pi = min(max(__ldg(p.cache_len + i), 0), len_hi);
-            int before = 0;
-#pragma unroll 1
-            for (int j = 0; j < p.B; ++j) {
-                const int Pj = min(max(__ldg(p.cache_len + j), 0), len_hi);
-                before += (Pj > Pi) || (Pj == Pi && j < i);
-            }
-            if (before == b) mine = i;
-        }
-        b = __shfl_sync(0xffffffffu, mine, __ffs(__ballot_sync(0xffffffffu, mine >= 0)) - 1);
-    }
-    int P = p.cache_len[b];
+    if (args.ranked) b = rank_by_length(p, b, len_hi, lane);
+    if (!len_first) P = p.cache_len[b];
     if (warp != PRODUCER_WARP) {
-        if (warp == MMA_WARP) {
-            if (lane == 0) {
-                *abort_flag = (sbase & 1023u) == 0 ? 0 : 1;   // swizzled tiles need 1 KB alignment
-#pragma unroll
-                for (int i = C::BAR_Q; i < C::NUM_BARS; ++i) mbar_init(bar(i), i == C::BAR_Q ? SW : 1);
-                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-                fence_proxy_async();
-                if (XCH) mbar_expect_tx(bar(C::BAR_X), (uint32_t)(my_tasks * S * MSG));
-                prefetch_map(&tm.kb); prefetch_map(&tm.vb);
-            }
-            __syncwarp();
-            bar_issue_arrive();
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                         ::"r"(smem_u32(tmem_slot)), "r"(C::TM_COLS) : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        } else if (tid < 2 * NR) {
-            reinterpret_cast<float *>(smem + C::OFF_REF)[tid] = 0.f;
-        }
         tc_fence_before();
         bar_start_wait();
         tc_fence_after();
@@ -324,8 +311,8 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             // rows below lo do not see the key (all, if the key does not exist)
             const int lo = j >= half_keys(a) ? NR : (a >= n_mine && p.causal ? (j - i0) * p.G : 0);
             const bool masks = __any_sync(0xffffffffu, lo > 0);
-            if (u > 0) mbar_wait_warp(bar(C::BAR_PV + wg), (u - 1) & 1, abort_flag);   // P buffer and O^T at rest
-            mbar_wait_warp(bar(C::BAR_S + wg), u & 1, abort_flag);
+            if (u > 0) mbar_wait_warp_call(bar(C::BAR_PV + wg), (u - 1) & 1, abort_flag);   // P buffer and O^T at rest
+            mbar_wait_warp_call(bar(C::BAR_S + wg), u & 1, abort_flag);
             tc_fence_after();
             bool exact = false;                               // the references are at or above the maxima of this tile
 #pragma unroll 1
@@ -447,7 +434,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         float *t_l = reinterpret_cast<float *>(smem + C::OFF_Q);              // [8 warps][NR] sums
         float *t_w = t_l + 8 * NR, *t_ml = t_w + 2 * NR;                      // [2][NR] weights, [2][NR] reference and sum of the CTA
         static_assert((8 + 4) * NR * 4 <= C::END_Q - C::OFF_Q, "tables");
-        if (n_tiles > 0) mbar_wait_warp(bar(C::BAR_QKALL), 0, abort_flag);
+        if (n_tiles > 0) mbar_wait_warp_call(bar(C::BAR_QKALL), 0, abort_flag);
         else bar_pair();                                      // (no product reads them: every warp has written its own)
         if (lane < RP)
 #pragma unroll
@@ -482,7 +469,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             }
         };
         if constexpr (XCH) addresses(wg * CW);
-        if (n_tiles > 0) mbar_wait_warp(bar(C::BAR_ALL), 0, abort_flag);
+        if (n_tiles > 0) mbar_wait_warp_call(bar(C::BAR_ALL), 0, abort_flag);
         if constexpr (XCH) cluster_arrive_relaxed();                  // the ring is idle
         bar_pair();
         tc_fence_after();
@@ -625,7 +612,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                         // (Item 3 is K2, so that with four slots the barrier of K0 can be two phases on before it is looked
                         // at here.  K1's cannot, and its scores come behind those of K0.)
                         const int it = iv ? i / 2 - 1 : C::NSLOT == 4 && i == 0 ? 1 : (i + 1) / 2;
-                        ok = mbar_wait(bar((iv ? C::BAR_PV : C::BAR_S) + (it & 1)), (it >> 1) & 1, abort_flag);
+                        ok = mbar_wait_call(bar((iv ? C::BAR_PV : C::BAR_S) + (it & 1)), (it >> 1) & 1, abort_flag);
                         if (!ok) continue;
                     }
                     if (n < 32) loaded |= 1u << n;
@@ -642,7 +629,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 for (int i = fold ? 0 : max(0, end - C::NSLOT); i < max(end, n_slots); ++i) {
                     int dummy = 0;
                     if (fold && i == 1 && (loaded >> 3 & 1)) continue;
-                    if (i < 32 ? loaded >> i & 1 : i < end) mbar_wait(bar(C::BAR_FULL + slot_of(i)), use_of(i) & 1, &dummy);
+                    if (i < 32 ? loaded >> i & 1 : i < end) mbar_wait_call(bar(C::BAR_FULL + slot_of(i)), use_of(i) & 1, &dummy);
                 }
             }
         }
@@ -675,8 +662,8 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         for (int t = 0; t <= n_tiles && n_tiles > 0 && ok; ++t) {
             if (t < n_tiles && t >= scored) {
                 const int i = item_of_k(t), slot = slot_of(i);
-                ok = mbar_wait_warp(bar(C::BAR_FULL + slot), use_of(i) & 1, abort_flag);
-                if (ok && t == 0) ok = mbar_wait_warp(bar(C::BAR_Q), 0, abort_flag);
+                ok = mbar_wait_warp_call(bar(C::BAR_FULL + slot), use_of(i) & 1, abort_flag);
+                if (ok && t == 0) ok = mbar_wait_warp_call(bar(C::BAR_Q), 0, abort_flag);
                 if (!ok) break;
                 // (the second tile's scores with the first one's, if its keys are there)
                 scored = t + 1;
@@ -700,7 +687,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             }
             if (t > 0) {
                 const int pt = t - 1, i = item_of_v(pt), slot = slot_of(i), w = pt & 1;
-                ok = mbar_wait_warp(bar(C::BAR_FULL + slot), use_of(i) & 1, abort_flag);
+                ok = mbar_wait_warp_call(bar(C::BAR_FULL + slot), use_of(i) & 1, abort_flag);
                 if (!ok) break;
                 // only the 16-key groups that hold keys are multiplied; V rows behind the keys in the last
                 // group may hold anything where they come from the cache, and 0 * NaN would poison the product
@@ -719,7 +706,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                     fence_proxy_async();
                     __syncwarp();
                 }
-                ok = mbar_wait_warp(bar(C::BAR_P + w), (pt >> 1) & 1, abort_flag);
+                ok = mbar_wait_warp_call(bar(C::BAR_P + w), (pt >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
@@ -738,12 +725,12 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 __syncwarp();
             }
         }
-        if (ok && n_tiles > 0) ok = mbar_wait_warp(bar(C::BAR_ALL), 0, abort_flag);
+        if (ok && n_tiles > 0) ok = mbar_wait_warp_call(bar(C::BAR_ALL), 0, abort_flag);
         if (!ok) {                                            // the MMAs in flight end before TMEM is freed
             if (elect_one()) umma_commit(bar(C::BAR_DRAIN));
             __syncwarp();
             int dummy = 0;
-            mbar_wait_warp(bar(C::BAR_DRAIN), 0, &dummy);
+            mbar_wait_warp_call(bar(C::BAR_DRAIN), 0, &dummy);
         }
         if constexpr (XCH) cluster_arrive_relaxed();
         bar_tmem_wait();                                      // the softmax warps have read their TMEM
@@ -859,7 +846,7 @@ cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cud
     int dev = 0;
     cudaError_t e = configure<HD, NR, XCH>(&dev);
     if (e != cudaSuccess) return e;
-    const int S = p.n_splits, units = p.B * p.Hkv, kb = tc_kb_rows(p.G, p.K), tiles = (p.K + kb - 1) / kb;
+    const int S = p.n_splits, units = p.B * p.Hkv, kb = keys_kb_rows(HD, p.G, p.K), tiles = (p.K + kb - 1) / kb;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, p.Hkv * tiles, p.B);
     cfg.blockDim = dim3(NTHREADS);
@@ -912,7 +899,16 @@ int keys_rows(int d, int G, int K)
 {
     const int M = G * K;
     if (d == 64 && M > 64) return G <= 128 ? 128 : 0;
-    return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 0;
+    return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 || (M <= 128 && G <= 64) ? 64 : 0;
+}
+
+// Block positions of a query tile.  At head_dim 128 up to 128 rows are cut into tiles of at most 64, as equal as can be,
+// which read the same keys (from L2, but for the first).
+int keys_kb_rows(int d, int G, int K)
+{
+    if (d == 64 || G * K <= 64) return tc_kb_rows(G, K);
+    const int most = 64 / G, tiles = (K + most - 1) / most;
+    return (K + tiles - 1) / tiles;
 }
 
 int keys_splits(int d, int G, int K, int units, int max_keys)

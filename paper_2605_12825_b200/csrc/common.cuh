@@ -67,6 +67,33 @@ __device__ inline int clamp_cache_len(const AttnParams &p, int b) {
     return P;
 }
 
+// The batch entry with the want-th longest prefix (ties by index), of at most 128; every lane of a warp calls it.  A lane counts
+// what comes before its entry; of more than 32, for up to four entries at a time, so that the lengths are read once.
+template <int N> __device__ inline int rank_by_length_of(const AttnParams &p, int want, int len_hi, int lane)
+{
+    int len[N], before[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int i = lane + 32 * k;
+        len[k] = i < p.B ? min(max(__ldg(p.cache_len + i), 0), len_hi) : 0;
+        before[k] = 0;
+    }
+#pragma unroll 4
+    for (int j = 0; j < p.B; ++j) {
+        const int x = min(max(__ldg(p.cache_len + j), 0), len_hi);
+#pragma unroll
+        for (int k = 0; k < N; ++k) before[k] += x > len[k] || (x == len[k] && j < lane + 32 * k);
+    }
+    int mine = -1;
+#pragma unroll
+    for (int k = 0; k < N; ++k) if (lane + 32 * k < p.B && before[k] == want) mine = lane + 32 * k;
+    return __shfl_sync(0xffffffffu, mine, __ffs(__ballot_sync(0xffffffffu, mine >= 0)) - 1);
+}
+static __device__ __noinline__ int rank_by_length(const AttnParams &p, int want, int len_hi, int lane)
+{
+    return p.B <= 32 ? rank_by_length_of<1>(p, want, len_hi, lane) : rank_by_length_of<4>(p, want, len_hi, lane);
+}
+
 // launchers (each returns the cudaError of its launches)
 cudaError_t launch_attend_simt(const AttnParams &p, int dtype, cudaStream_t st);
 bool mma_path_supports(const AttnParams &p, int dtype);
@@ -85,6 +112,7 @@ bool tc_stream_shape(int B, int G, int K);                  // the persistent ke
 size_t tc_stream_workspace_bytes(int B, int Hkv, int n_ctas);
 cudaError_t launch_attend_tc_stream(const AttnParams &p, int n_ctas, void *ws_body, int flags, cudaStream_t st);
 int keys_rows(int d, int G, int K);      // MMA columns of a query tile on the keys kernel (0: not its shape)
+int keys_kb_rows(int d, int G, int K);   // block positions of such a query tile
 int keys_splits(int d, int G, int K, int units, int max_keys);   // CTAs per (unit, query tile) on the current device
 int keys_resident_clusters(int S);       // clusters of S CTAs, two to an SM, that are resident at once
 int tc_kb_rows(int G, int K);            // block positions per query tile of 128 rows

@@ -35,8 +35,8 @@ __device__ inline bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false (and raises the CTA's abort flag) if the phase does not
 // complete within about a second, or if another thread already gave up.
-// (The loop is one function for all waits of a kernel: its copies filled the instruction cache.)
-static __device__ __noinline__ bool mbar_wait_loop(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
     for (uint32_t it = 1; it < (1u << 24); ++it) {
         if (mbar_try(bar, parity)) return true;
@@ -48,13 +48,31 @@ static __device__ __noinline__ bool mbar_wait_loop(uint32_t bar, uint32_t parity
     *abort_flag = 1;
     return false;
 }
-__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
-    return mbar_try(bar, parity) || mbar_wait_loop(bar, parity, abort_flag);
-}
 // the same for a whole warp: every lane learns the common outcome, so that warp-wide
 // (.aligned) instructions behind it are executed by all lanes or by none
 __device__ inline bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+// The same again for kernels whose code has to be short: the first try here, the loop in one function for all waits of a
+// kernel.  (An arrival is seen 54 cycles later by mbarrier.try_wait, 107 by a test and then the loop.)
+static __device__ __noinline__ bool mbar_wait_loop(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    return mbar_wait(bar, parity, abort_flag);
+}
+__device__ inline bool mbar_wait_call(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    return mbar_try(bar, parity) || mbar_wait_loop(bar, parity, abort_flag);
+}
+__device__ inline bool mbar_wait_warp_call(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait_call(bar, parity, abort_flag));
+}
+// and without a call, for a place where many registers are live or that is run through often
+__device__ inline bool mbar_wait_warp_inline(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    bool ok = true;
+    if (!mbar_try(bar, parity)) {
+        const long long t0 = clock64();
+        while (ok && !mbar_try(bar, parity))
+            if (*abort_flag || clock64() - t0 > (1ll << 31)) { *abort_flag = 1; ok = false; }
+    }
+    return __all_sync(0xffffffffu, ok);
 }
 
 // a wait for CTAs of the same cluster, whose own waits end within seconds whatever happens to them
@@ -130,6 +148,10 @@ __device__ inline void st_cluster(uint32_t addr, const uint32_t *v) {
 __device__ inline void st_async(uint32_t addr, const float4 &v, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+__device__ inline void st_async(uint32_t addr, float x, float y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+                 ::"r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
 }
 // shared-memory matrix descriptor, 128-byte swizzle
 __device__ inline uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
