@@ -179,13 +179,14 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
             while (S < 16 && units * S < slots && tiles / (S * 2) >= 8) S *= 2;
         }
         // Sixteen only while a call and the next one, which starts early, find SMs of their own, too: on shared ones the CTAs of
-        // a cluster share the way to the others, which the merge of more than 64 rows fills.  As many CTAs as do find some,
-        // then (8 units of 128 rows, 2000, 4000, 8000 and 16000 keys 12.4, 13.6, 17.6 and 26.0 us at 16, 9.1, 11.4, 15.8 and 25.3 at
-        // 10), until streaming the keys is nearly all there is (32000 keys 42.7 and 43.7).
+        // a cluster share the way to the others, which the merge fills.  As many CTAs as do find some, then (8 units of 128
+        // rows, 2000, 4000, 8000 and 16000 keys 12.4, 13.6, 17.6 and 26.0 us at 16, 9.1, 11.4, 15.8 and 25.3 at 10; behind a rotary
+        // write, whose CTAs are in between, 4000 and 8000 keys 15.6 and 19.7 at 16, 16.9 and 22.9 at 10, 15.0 and 19.3 at 9), until
+        // streaming the keys is nearly all there is (32000 keys 42.7 and 43.7; 68 rows, 8000 keys 17.6 and 18.3).
         const int rows = G * L->block;
-        if (forced <= 0 && S == 16 && 2 * units * S > num_sms() && tiles < (rows > 96 ? 160 : rows > 64 ? 64 : 48)) {
-            S = num_sms() / (2 * units);
-            if (S < 8) S = 8;
+        if (forced <= 0 && S == 16 && tiles < (rows > 96 ? 160 : rows > 64 ? 64 : 48)) {
+            const int fit = L->flags & ORTHRUS_LAYER_BLOCK_IN_CACHE ? num_sms() / (2 * units) : 5 * num_sms() / (9 * units);
+            if (fit < S) S = fit > 8 ? fit : 8;
         }
         const int max_cluster = tc_max_cluster(nt);
         if (S > max_cluster) S = max_cluster;
@@ -221,7 +222,9 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 //  - Where the caller promises a quiescent cache, the keys kernel has its first three tiles in shared memory by the time the
 //    query rows come, and is the rule up to 64 units (us a call, keys against wide, 64 rows: 8 units of 1000 keys 5.3 and
 //    6.8, of 4000 8.6 and 10.0; 16 of 2000 8.7 and 9.9; 32 of 1000 9.0 and 10.0, of 3500 14.3 and 14.9; 40 of 4000 18.8 and 22.2; 48
-//    of 3000 17.4 and 18.6; 64 of 500 9.3 and 9.7, of 2000 16.8 and 16.7; level at 8 of 300, 5.7 and 5.6).
+//    of 3000 17.4 and 18.6; 64 of 2000 16.8 and 16.7; level at 8 of 300, 5.7 and 5.6).  From 24 units on only with bounds of
+//    1024 keys and more: below, the wide kernel is level where the lengths reach the bound (32 of 300 6.5 and 6.3) and the
+//    faster one where they do not (40 of 71 to 435 under a bound of 690, two layers of a decoder 65 and 60).
 //  - With more units the SMs are full in any case, and the wide kernel's takes less per key (128 units of 500, 1000 and 2000 keys
 //    13.5 and 11.8, 18.3 and 16.8, 28.0 and 26.3; 320 of 1000 51.5 and 46.5), unless its clusters are not all resident at
 //    once (256 of 2000, cut in two, 46.3 and 53.6; 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9).
@@ -256,8 +259,12 @@ static int keys_tiles(const orthrus_layer_t *L)
     return (L->block + kb - 1) / kb;
 }
 
-// Units of at most 32 query rows (4 rows, 8 units of 4000 keys 5.7 against 9.7 us on the wide kernel, 32 rows 6.9), of 33 to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
+// Units of at most 32 query rows (4 rows, 8 units of 4000 keys 5.7 against 9.7 us on the wide kernel, 32 rows 6.9), of 33
+// to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
 // rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
+// 65 to 128 rows at head_dim 128 are two tiles there, which read the same keys: the faster way where latency counts, that is, with
+// the promise of a quiescent cache, up to 16 tiles and 8192 keys (keys against wide: 2 units of 77 rows, 3000 keys 5.9 and
+// 8.6 us, 4 of 128, 2000 keys 6.1 and 9.0, 8 of 128, 500, 2000 and 8000 keys 5.9 and 8.0, 8.7 and 9.1, 16.4 and 16.4).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
 // from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).

@@ -1,5 +1,5 @@
-// Block attention for units of few query rows (M = G*K; up to 32, and up to 64 where the wide kernel's plan does
-// not suit the number of units) at head_dim 128, and of any number at head_dim 64 (in tiles of up to 128 rows), bf16, both
+// Block attention for units of few query rows (M = G*K; up to 64, up to 128 in two tiles where latency counts; the lines are in
+// api.cu) at head_dim 128, and of any number at head_dim 64 (in tiles of up to 128 rows), bf16, both
 // views, on tcgen05 with the KEYS on the MMA's rows:
 //     S^T [128 keys x NR rows] = K_tile . Q^T        O^T [d x NR rows] = V_tile^T . P^T
 // NR = M rounded up to 16, 32, 64 or 128 is the MMA's N.  With the query rows there instead, an M of 4 to 64

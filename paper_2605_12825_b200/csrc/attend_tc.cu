@@ -20,7 +20,7 @@
 //              of a lone CTA, 1450 cycles per tile: 480 to issue the eight MMAs of QK, 250 for the
 //              four of P.V, the rest waits and fences.  (Behind a test of the lane index instead
 //              of elect.sync, the descriptors built in the loop: 660, 640 and 2020 per tile.)
-// (Units of few rows run on attend_keys.cu.)
+// (Units of few rows run on attend_keys.cu; api.cu, keys_usable and wide_better.)
 // The output accumulator O stays in TMEM for the whole CTA.  A row's reference starts at 0 and is left alone as long as no
 // probability exceeds 2^40 and, in the first tile that shows the row a key, the largest is not below 2^-60: floating-point
 // numbers keep their relative precision whatever the reference, so that no tile pays for its row maxima.  Otherwise the
@@ -34,10 +34,11 @@
 //
 // The kernel's code matters at its two ends, which every CTA runs through once: an SM's instruction cache holds 32 KB, and the
 // kernel was 113 KB of it (softmax and read-outs in three forms each, a merge per cluster size, one of them through L2, all barrier waits
-// inlined), now 44.  With that, the references, the producer's loads ahead of everything else and the merge above: a
-// ragged batch of 32 units x 8 heads of 128 rows 294 -> 278 us a pass (consensus and commit included), 64 units of 128 rows and
-// 4000 keys 28.4 -> 27.4 us a call, 8 of 2000 keys 10.3 -> 9.1.  One instance of the merge for each of 1, 2 and 4 column groups at
-// a time is faster for clusters of 2 to 8 by itself, and slower for those of 16 by the code it adds (10.8 -> 11.3 us).
+// inlined), now 54.  With that, the references, the producer's loads ahead of everything else and the merge above, us a call:
+// 64 units of 128 rows and 4000 keys 28.4 -> 27.5, 32 of 256 rows and 32768 keys 89 -> 86, 320 of 96 rows and 300 keys 23.0 -> 21.5, 8 of
+// 128 rows and 2000 keys 10.3 -> 9.1.  One instance of the merge for each of 1, 2 and 4 column groups at a time gained 0.2 us at clusters
+// of 4 and lost 0.5 at those of 16 by the code it adds.  Clusters of 16 are slower than with the merge through L2 (8 units of 64
+// rows, 4096 keys, without the promise below 10.6 -> 11.3 us); api.cu has fewer of them.
 //
 // Programmatic dependent launch.  The kernel waits for the preceding kernel of the
 // stream (griddepcontrol.wait) before it reads anything that kernel may have written,
@@ -217,7 +218,7 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
 template <int NT, bool PACK>
 __global__ void __launch_bounds__(Shape<NT>::NTHREADS, NT == 1 ? 2 : 1)
 attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const int S, const int kb_rows,
-                 const int quiescent)
+                 const int quiescent, const int ranked)
 {
     using C = Shape<NT>;
     constexpr int W = TN;                     // score columns per softmax thread
@@ -290,12 +291,13 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     if (!quiescent) griddep_wait();
 
     // ------------------------------------------------------------------ which unit
-    // clusters are ordered longest prefix first (ties by sequence index); every warp finds out by itself
+    // when the clusters do not all fit at once they go out longest prefix first (ties by sequence index); every warp finds
+    // out by itself
     const int len_hi = (int)p.len_cap;
     static_assert(!PACK || NT == 1, "the packed form runs one query tile per CTA");
     int b = order / p.Hkv;
     const int h = order % p.Hkv;
-    if (!PACK && p.B > 1 && p.B <= 128) b = rank_by_length(p, b, len_hi, lane);
+    if (!PACK && ranked) b = rank_by_length(p, b, len_hi, lane);
     int P;
     int bt_lo = 0, n_blk = 1;               // first tile of block keys on the block axis, how many
     if constexpr (PACK) {
@@ -918,7 +920,9 @@ static cudaError_t launch_tc(const AttnParams &p, const TcMaps &tm, int kb, int 
     }
     cfg.attrs = attr;
     cfg.numAttrs = n_attr;
-    e = cudaLaunchKernelEx(&cfg, attend_tc_kernel<NT, PACK>, p, tm, S, kb, (flags & ORTHRUS_LAYER_CACHE_QUIESCENT) ? 1 : 0);
+    const long long ctas = (long long)S * p.B * p.Hkv * cfg.gridDim.z;
+    const int ranked = !PACK && p.B > 1 && p.B <= 128 && ctas > (long long)tc_ctas_per_sm(NT) * num_sms();
+    e = cudaLaunchKernelEx(&cfg, attend_tc_kernel<NT, PACK>, p, tm, S, kb, (flags & ORTHRUS_LAYER_CACHE_QUIESCENT) ? 1 : 0, ranked);
     count_launch();
     return e;
 }
