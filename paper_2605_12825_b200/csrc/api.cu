@@ -228,9 +228,10 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 //  - With more units the SMs are full in any case, and the wide kernel's takes less per key (128 units of 500, 1000 and 2000 keys
 //    13.5 and 11.8, 18.3 and 16.8, 28.0 and 26.3; 320 of 1000 51.5 and 46.5), unless its clusters are not all resident at
 //    once (256 of 2000, cut in two, 46.3 and 53.6; 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9).
-//  - Without the promise every load waits for the preceding kernel, and the two are within ten per cent of one another
-//    either way (8 units of 300 keys 6.6 and 6.4, of 1000 6.7 and 7.8, of 4096 11.5 and 11.3; 32 of 2000 13.0 and 12.7; 64 of 2000 18.3 and
-//    17.7).  There the wide kernel is the rule, short prefixes included, where its plan, whose clusters are powers of two, suits
+//  - Without the promise every load waits for the preceding kernel.  Up to 9 units, whose clusters of 16 the wide kernel merges
+//    slowly, the keys kernel is still the faster one while sixteen CTAs have two tiles each or fewer (8 units of 600 keys 6.6 and 8.0, of
+//    2000 7.8 and 9.7, of 3500 10.0 and 10.9; 2 of 1000 6.2 and 7.6; but of 300 6.6 and 6.4, of 4096 11.5 and 11.3).  For more units the
+//    two are within ten per cent of one another either way (32 of 2000 13.0 and 12.7; 64 of 2000 18.3 and 17.7).  There the wide kernel is the rule, short prefixes included, where its plan, whose clusters are powers of two, suits
 //    the number of units: not where its clusters are not all resident (34 to 37 units cut in 8: 37 of 1700 keys 14.5 and
 //    20.3), nor where clusters of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix
 //    is long (12 units of 8000 keys 15.9 and 18.4, 44 of 6000 29.0 and 30.8; at 2500 keys the wide one still won).
@@ -245,6 +246,7 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
     if (!tc_usable(L)) return false;
     const int units = L->batch * L->n_kv_heads, M = L->n_q_heads / L->n_kv_heads * L->block;
     if ((L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units <= 64 && (units < 24 || max_len_of(L) >= 1024)) return false;
+    if (units <= 9 && max_len_of(L) > 512 && max_len_of(L) + L->block <= 4032) return false;
     const int S = make_plan(L, true, kn).n_splits;
     if (S > 1 && units > keys_resident_clusters(S)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();

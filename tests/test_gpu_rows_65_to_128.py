@@ -78,6 +78,22 @@ def test_which_side_many_units_and_long_prefixes_are_on():
         assert ("attend_keys_kernel" if kernel == "keys" else "attend_tc_kernel") in name
 
 
+def test_few_units_of_33_to_64_rows_without_the_promise():
+    """Two tiles for each of sixteen CTAs are the line: bound and block together in 62 halves of 64 keys and one of the block's."""
+    b = binding()
+    z = lambda *s: torch.zeros(s, dtype=torch.bfloat16, device="cuda")
+    for B, Hkv, K, hint, flags, kernel in ((2, 4, 16, 512, 0, "wide"), (2, 4, 16, 513, 0, "keys"), (2, 4, 16, 4016, 0, "keys"),
+                                           (2, 4, 16, 4017, 0, "wide"), (9, 1, 9, 4000, 0, "keys"), (10, 1, 9, 2000, 0, "wide"),
+                                           (2, 4, 16, 4096, b.LAYER_CACHE_QUIESCENT, "keys"), (3, 8, 16, 1023, b.LAYER_CACHE_QUIESCENT, "wide"),
+                                           (3, 8, 16, 1024, b.LAYER_CACHE_QUIESCENT, "keys"), (65, 1, 16, 2000, b.LAYER_CACHE_QUIESCENT, "wide")):
+        kc, ln = z(B, Hkv, hint + K, 128), torch.zeros(B, dtype=torch.int32, device="cuda")
+        layer = b.make_layer(kc, kc, ln, 4 * Hkv, K, hint, 0.0, flags)
+        ws = b.new_workspace(b.orthrus_attend_workspace_bytes(layer))
+        q, kb = z(B, K, 4 * Hkv, 128), z(B, K, Hkv, 128)
+        (name, _), = captured_launches(lambda: b.orthrus_ar_verify_attend(layer, q, kb, kb, torch.empty_like(q), ws))
+        assert ("attend_keys_kernel" if kernel == "keys" else "attend_tc_kernel") in name, (B, Hkv, K, hint, flags)
+
+
 @pytest.mark.parametrize("splits", [3, 6, 7, 9, 10, 11, 12, 14, 16])
 @pytest.mark.parametrize("peak", [1.0, 40.0])
 def test_uneven_clusters_of_the_wide_kernel(splits, peak, monkeypatch):
