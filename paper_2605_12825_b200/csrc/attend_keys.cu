@@ -213,10 +213,10 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         reinterpret_cast<float *>(smem + C::OFF_REF)[tid] = 0.f;
     }
     // which unit: when the clusters do not all fit at once they go out longest prefix first (every warp finds out by itself)
-    if (!quiescent) griddep_wait();
+    if (__builtin_expect(!quiescent, 0)) griddep_wait();
     const int h = blockIdx.y - zt * p.Hkv;
     const int len_hi = (int)p.len_cap;
-    if (args.ranked) b = rank_by_length(p, b, len_hi, lane);
+    if (__builtin_expect(args.ranked, 0)) b = rank_by_length(p, b, len_hi, lane);
     if (!len_first) P = p.cache_len[b];
     if (warp != PRODUCER_WARP) {
         tc_fence_before();
@@ -325,7 +325,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                     const float4 *rf = reinterpret_cast<const float4 *>(ref + c0);
                     float4 ra = rf[0], rb = rf[1];
                     tmem_ld_wait();
-                    if (masks) {
+                    if (__builtin_expect(masks, 0)) {
 #pragma unroll
                         for (int i = 0; i < CH; ++i) if (i < lo - c0) s[i] = 0xff800000u;
                     }
@@ -355,7 +355,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 // A reference of 0, with which a row starts, will do as long as no probability is out of all proportion and
                 // (first tile; its first key is one that every row sees) no row has nothing but tiny ones.
                 const bool off = max(top & 0xffffu, top >> 16) > P_HIGH || (u == 0 && kt == 0 && min(low & 0xffffu, low >> 16) < P_LOW);
-                if (!bar_group_or(wg, off && !exact)) break;
+                if (__builtin_expect(!bar_group_or(wg, off && !exact), 1)) break;
                 // ------------------------------------------------ all references are set to the maxima of the tile, or, behind
                 // the first, raised to them, and what the earlier tiles have added up is rescaled
                 tc_fence_after();
@@ -621,7 +621,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll 1
                 for (int a = 2 * t; a < last; ++a) load_half(v, a, slot);
             }
-            if (*abort_flag) {
+            if (__builtin_expect(*abort_flag, 0)) {
                 // Copies in flight land before the CTA ends: the last of each slot.  (`ok` false: item n - 1 was
                 // not asked for, later ones only if they were early.)
                 const int end = ok ? n : max(n - 1, 0);
@@ -692,7 +692,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 // only the 16-key groups that hold keys are multiplied; V rows behind the keys in the last
                 // group may hold anything where they come from the cache, and 0 * NaN would poison the product
                 const int k0 = half_keys(2 * pt), k1 = half_keys(2 * pt + 1);
-                if ((k0 | k1) & 15) {
+                if (__builtin_expect((k0 | k1) & 15, 0)) {
 #pragma unroll 1
                     for (int a = 0; a < 2; ++a) {
                         const int n = a ? k1 : k0, pad = -n & 15;
@@ -726,7 +726,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             }
         }
         if (ok && n_tiles > 0) ok = mbar_wait_warp_call(bar(C::BAR_ALL), 0, abort_flag);
-        if (!ok) {                                            // the MMAs in flight end before TMEM is freed
+        if (__builtin_expect(!ok, 0)) {                       // the MMAs in flight end before TMEM is freed
             if (elect_one()) umma_commit(bar(C::BAR_DRAIN));
             __syncwarp();
             int dummy = 0;

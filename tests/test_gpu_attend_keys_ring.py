@@ -20,7 +20,7 @@ def test_early_tiles_in_a_chain_of_calls(shape, splits, peak, monkeypatch):
     Hq, Hkv, d, K = shape
     monkeypatch.setenv("ORTHRUS_TC_SMALL_ROWS", "1")
     monkeypatch.setenv("ORTHRUS_SPLITS", str(splits))
-    for lens in ([127, 640], [193, 1024], [64, 577]):
+    for lens in ([127, 640], [193, 1024], [64, 577], [256, 576], [897, 310]):        # (256, 576, 897: five halves of 64 keys for each of 1, 2, 3 CTAs)
         wl = small_workload(2, K, Hq, Hkv, d, 1024, 1024, std=0.5, name=f"ring_{Hq}_{Hkv}_{d}_{K}")
         t = W.attention_inputs(wl)
         t["cache_len"][:] = torch.tensor(lens, dtype=torch.int32)
