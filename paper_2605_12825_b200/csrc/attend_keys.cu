@@ -478,6 +478,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll 1
             for (int c = wg * CW; c < (wg + 1) * CW; c += CR) {
                 uint32_t oa[CR], ob[CR];
+                __syncwarp();                                 // (the messages below are not every lane's, these loads are)
                 if (n_tiles > 0) tmem_ld<CR>(lane_base + C::tm_o(0) + c, oa);
                 if (n_tiles > 1) tmem_ld<CR>(lane_base + C::tm_o(1) + c, ob);
                 tmem_ld_wait();
@@ -516,6 +517,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 }
             }
         }
+        __syncwarp();
         tc_fence_before();
         bar_tmem_arrive();
         if (XCH && warp < my_tasks) {

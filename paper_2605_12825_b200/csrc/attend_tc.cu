@@ -125,6 +125,7 @@ __device__ inline void bar_tmem_wait(int n) { asm volatile("bar.sync 3, %0;" ::"
 // eight-column groups [first_group(q), first_group(q + 1)) of all rows.  A thread sends the other CTAs their groups of
 // its row with its reference and sum, as 16-byte chunks [source][group][half][row] so that a warp's store is 512
 // contiguous bytes, by stores that the destination's barrier counts; then it waits for its own count and sums up, two groups at a time.
+// (Lanes without a row store nothing, but the loads from tensor memory are the whole warp's: each is reached behind a __syncwarp().)
 __device__ inline int first_group(int q, int S) { return (int)((uint32_t)(16 * q) * ((65536u + S - 1) / (uint32_t)S) >> 16); }
 __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf, uint32_t x_bar, int S, int rank, int r, bool valid,
                              bool have_o, float m, float l, __nv_bfloat16 *row, int32_t *status)
@@ -143,6 +144,7 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
             uint32_t o[16];                                   // (the second group need not be one of q's)
 #pragma unroll
             for (int i = 0; i < 16; ++i) o[i] = 0u;           // (a CTA without keys sends zeros)
+            __syncwarp();
             if (have_o) { tmem_ld<16>(tm_row + g * 8, o); tmem_ld_wait(); }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -180,29 +182,31 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
         uint32_t o[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) o[i] = 0u;
+        __syncwarp();
         if (have_o) { tmem_ld<16>(tm_row + (g0 + g) * 8, o); tmem_ld_wait(); }
-        if (!valid) continue;
-        float acc[16];
+        if (valid) {
+            float acc[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = own * __uint_as_float(o[i]);
+            for (int i = 0; i < 16; ++i) acc[i] = own * __uint_as_float(o[i]);
 #pragma unroll 4
-        for (int k = 0; k < S - 1; ++k) {
-            const int j = k + (k >= rank);
-            const float w = ml[j * MROWS].x;
+            for (int k = 0; k < S - 1; ++k) {
+                const int j = k + (k >= rank);
+                const float w = ml[j * MROWS].x;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (i < 2 || two) {
-                    const float4 x = *reinterpret_cast<const float4 *>(src + (j * n + g) * 4096 + i * 2048);
-                    acc[4 * i] = fmaf(w, x.x, acc[4 * i]); acc[4 * i + 1] = fmaf(w, x.y, acc[4 * i + 1]);
-                    acc[4 * i + 2] = fmaf(w, x.z, acc[4 * i + 2]); acc[4 * i + 3] = fmaf(w, x.w, acc[4 * i + 3]);
-                }
+                for (int i = 0; i < 4; ++i)
+                    if (i < 2 || two) {
+                        const float4 x = *reinterpret_cast<const float4 *>(src + (j * n + g) * 4096 + i * 2048);
+                        acc[4 * i] = fmaf(w, x.x, acc[4 * i]); acc[4 * i + 1] = fmaf(w, x.y, acc[4 * i + 1]);
+                        acc[4 * i + 2] = fmaf(w, x.z, acc[4 * i + 2]); acc[4 * i + 3] = fmaf(w, x.w, acc[4 * i + 3]);
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < 16; i += 8)
+                if (i == 0 || two)
+                    *reinterpret_cast<uint4 *>(row + (g0 + g) * 8 + i) =
+                        make_uint4(pack_bf16(acc[i] * inv, acc[i + 1] * inv), pack_bf16(acc[i + 2] * inv, acc[i + 3] * inv),
+                                   pack_bf16(acc[i + 4] * inv, acc[i + 5] * inv), pack_bf16(acc[i + 6] * inv, acc[i + 7] * inv));
         }
-#pragma unroll
-        for (int i = 0; i < 16; i += 8)
-            if (i == 0 || two)
-                *reinterpret_cast<uint4 *>(row + (g0 + g) * 8 + i) =
-                    make_uint4(pack_bf16(acc[i] * inv, acc[i + 1] * inv), pack_bf16(acc[i + 2] * inv, acc[i + 3] * inv),
-                               pack_bf16(acc[i + 4] * inv, acc[i + 5] * inv), pack_bf16(acc[i + 6] * inv, acc[i + 7] * inv));
     }
 }
 
@@ -510,6 +514,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
 #pragma unroll 1
                 for (int c = 0; c < HD; c += 32) {
                     uint32_t o[32];
+                    __syncwarp();                             // (the stores below are not every lane's, this load is)
                     tmem_ld32(tm_row + c, o);
                     tmem_ld_wait();
                     if (valid) {

@@ -83,6 +83,7 @@ __device__ inline void scan_accumulator(uint32_t taddr, int n_valid, int v0, flo
 #pragma unroll 1
     for (int c = 0; c < n_valid; c += 64) {
         uint32_t r[64];
+        __syncwarp();                         // (the comparisons below may part the lanes)
         tmem_ld32(taddr + c, r);
         tmem_ld32(taddr + c + 32, r + 32);
         tmem_ld_wait();
