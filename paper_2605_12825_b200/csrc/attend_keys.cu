@@ -478,7 +478,6 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll 1
             for (int c = wg * CW; c < (wg + 1) * CW; c += CR) {
                 uint32_t oa[CR], ob[CR];
-                __syncwarp();                                 // (the messages below are not every lane's, these loads are)
                 if (n_tiles > 0) tmem_ld<CR>(lane_base + C::tm_o(0) + c, oa);
                 if (n_tiles > 1) tmem_ld<CR>(lane_base + C::tm_o(1) + c, ob);
                 tmem_ld_wait();
@@ -505,9 +504,9 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                     if (c == wg * CW) cluster_wait();
 #pragma unroll
                     for (int i = 0; i < CR / 4; ++i)
-                        if (to[i]) {
-                            st_async(to[i], make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]), to_bar[i]);
-                            if (lane < 2) st_async(to[i] + 512, *reinterpret_cast<const float4 *>(t_ml + lane * NR + c + 4 * i), to_bar[i]);
+                        if (to[i]) {                          // (the same for the whole warp)
+                            st_async_if(true, to[i], make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]), to_bar[i]);
+                            st_async_if(lane < 2, to[i] + 512, *reinterpret_cast<const float4 *>(t_ml + (lane & 1) * NR + c + 4 * i), to_bar[i]);
                         }
                     if (CR < CW) addresses(c + CR);
                 } else {
@@ -517,7 +516,6 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 }
             }
         }
-        __syncwarp();
         tc_fence_before();
         bar_tmem_arrive();
         if (XCH && warp < my_tasks) {

@@ -125,7 +125,8 @@ __device__ inline void bar_tmem_wait(int n) { asm volatile("bar.sync 3, %0;" ::"
 // eight-column groups [first_group(q), first_group(q + 1)) of all rows.  A thread sends the other CTAs their groups of
 // its row with its reference and sum, as 16-byte chunks [source][group][half][row] so that a warp's store is 512
 // contiguous bytes, by stores that the destination's barrier counts; then it waits for its own count and sums up, two groups at a time.
-// (Lanes without a row store nothing, but the loads from tensor memory are the whole warp's: each is reached behind a __syncwarp().)
+// Lanes without a row go the same way with predicated stores: the loads from tensor memory are the whole warp's.  (A branch around
+// their stores and a __syncwarp() ahead of each load cost 0.1 us a call.)
 __device__ inline int first_group(int q, int S) { return (int)((uint32_t)(16 * q) * ((65536u + S - 1) / (uint32_t)S) >> 16); }
 __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf, uint32_t x_bar, int S, int rank, int r, bool valid,
                              bool have_o, float m, float l, __nv_bfloat16 *row, int32_t *status)
@@ -138,19 +139,18 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
         const int g0 = first_group(q, S), n = first_group(q + 1, S) - g0;
         const uint32_t base = map_to_rank(sbase, q), xb = base + (x_bar - sbase);
         uint32_t dst = base + buf + rank * n * 4096 + r * 16;
-        if (valid) st_async(base + buf + S * n * 4096 + (rank * MROWS + r) * 8, m, l, xb);
+        st_async_if(valid, base + buf + S * n * 4096 + (rank * MROWS + r) * 8, m, l, xb);
 #pragma unroll 1
         for (int g = g0; g < g0 + n; g += 2, dst += 2 * 4096) {
             uint32_t o[16];                                   // (the second group need not be one of q's)
 #pragma unroll
             for (int i = 0; i < 16; ++i) o[i] = 0u;           // (a CTA without keys sends zeros)
-            __syncwarp();
             if (have_o) { tmem_ld<16>(tm_row + g * 8, o); tmem_ld_wait(); }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (valid && (i < 2 || g + 1 < g0 + n))
-                    st_async(dst + i * 2048, make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
-                                                         __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3])), xb);
+                st_async_if(valid && (i < 2 || g + 1 < g0 + n), dst + i * 2048,
+                            make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
+                                        __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3])), xb);
         }
     }
     // (the wait outlasts every other one: a CTA of the cluster that gave one up sends all the same)
@@ -161,19 +161,17 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
     float2 *ml = reinterpret_cast<float2 *>(smem + buf + S * n * 4096) + r;
     // weights, in the place of the references
     float mmax = -INFINITY, L = 0.f, own = 0.f;
-    if (valid) {
-        ml[rank * MROWS] = make_float2(m, l);
+    ml[rank * MROWS] = make_float2(m, l);
 #pragma unroll 8
-        for (int j = 0; j < S; ++j) { const float2 x = ml[j * MROWS]; mmax = fmaxf(mmax, x.y > 0.f ? x.x : -INFINITY); }
+    for (int j = 0; j < S; ++j) { const float2 x = ml[j * MROWS]; mmax = fmaxf(mmax, x.y > 0.f ? x.x : -INFINITY); }
 #pragma unroll 8
-        for (int j = 0; j < S; ++j) {
-            const float2 x = ml[j * MROWS];
-            // (a sum that is not a number has no order: its row is void with it)
-            const float w = x.y > 0.f ? ex2(x.x - mmax) : x.y;
-            L = fmaf(w, x.y, L);
-            if (j == rank) own = w;
-            ml[j * MROWS].x = w;
-        }
+    for (int j = 0; j < S; ++j) {
+        const float2 x = ml[j * MROWS];
+        // (a sum that is not a number has no order: its row is void with it)
+        const float w = x.y > 0.f ? ex2(x.x - mmax) : x.y;
+        L = fmaf(w, x.y, L);
+        if (j == rank) own = w;
+        ml[j * MROWS].x = w;
     }
     const float inv = 1.f / L;
 #pragma unroll 1
@@ -182,31 +180,27 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
         uint32_t o[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) o[i] = 0u;
-        __syncwarp();
         if (have_o) { tmem_ld<16>(tm_row + (g0 + g) * 8, o); tmem_ld_wait(); }
-        if (valid) {
-            float acc[16];
+        float acc[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) acc[i] = own * __uint_as_float(o[i]);
+        for (int i = 0; i < 16; ++i) acc[i] = own * __uint_as_float(o[i]);
 #pragma unroll 4
-            for (int k = 0; k < S - 1; ++k) {
-                const int j = k + (k >= rank);
-                const float w = ml[j * MROWS].x;
+        for (int k = 0; k < S - 1; ++k) {
+            const int j = k + (k >= rank);
+            const float w = ml[j * MROWS].x;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (i < 2 || two) {
-                        const float4 x = *reinterpret_cast<const float4 *>(src + (j * n + g) * 4096 + i * 2048);
-                        acc[4 * i] = fmaf(w, x.x, acc[4 * i]); acc[4 * i + 1] = fmaf(w, x.y, acc[4 * i + 1]);
-                        acc[4 * i + 2] = fmaf(w, x.z, acc[4 * i + 2]); acc[4 * i + 3] = fmaf(w, x.w, acc[4 * i + 3]);
-                    }
-            }
-#pragma unroll
-            for (int i = 0; i < 16; i += 8)
-                if (i == 0 || two)
-                    *reinterpret_cast<uint4 *>(row + (g0 + g) * 8 + i) =
-                        make_uint4(pack_bf16(acc[i] * inv, acc[i + 1] * inv), pack_bf16(acc[i + 2] * inv, acc[i + 3] * inv),
-                                   pack_bf16(acc[i + 4] * inv, acc[i + 5] * inv), pack_bf16(acc[i + 6] * inv, acc[i + 7] * inv));
+            for (int i = 0; i < 4; ++i)
+                if (i < 2 || two) {
+                    const float4 x = *reinterpret_cast<const float4 *>(src + (j * n + g) * 4096 + i * 2048);
+                    acc[4 * i] = fmaf(w, x.x, acc[4 * i]); acc[4 * i + 1] = fmaf(w, x.y, acc[4 * i + 1]);
+                    acc[4 * i + 2] = fmaf(w, x.z, acc[4 * i + 2]); acc[4 * i + 3] = fmaf(w, x.w, acc[4 * i + 3]);
+                }
         }
+#pragma unroll
+        for (int i = 0; i < 16; i += 8)
+            st_global_if(valid && (i == 0 || two), row + (g0 + g) * 8 + i,
+                         make_uint4(pack_bf16(acc[i] * inv, acc[i + 1] * inv), pack_bf16(acc[i + 2] * inv, acc[i + 3] * inv),
+                                    pack_bf16(acc[i + 4] * inv, acc[i + 5] * inv), pack_bf16(acc[i + 6] * inv, acc[i + 7] * inv)));
     }
 }
 
@@ -514,18 +508,15 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
 #pragma unroll 1
                 for (int c = 0; c < HD; c += 32) {
                     uint32_t o[32];
-                    __syncwarp();                             // (the stores below are not every lane's, this load is)
                     tmem_ld32(tm_row + c, o);
                     tmem_ld_wait();
-                    if (valid) {
 #pragma unroll
-                        for (int i = 0; i < 32; i += 8)
-                            *reinterpret_cast<uint4 *>(row + c + i) = make_uint4(
-                                pack_bf16(__uint_as_float(o[i]) * inv, __uint_as_float(o[i + 1]) * inv),
-                                pack_bf16(__uint_as_float(o[i + 2]) * inv, __uint_as_float(o[i + 3]) * inv),
-                                pack_bf16(__uint_as_float(o[i + 4]) * inv, __uint_as_float(o[i + 5]) * inv),
-                                pack_bf16(__uint_as_float(o[i + 6]) * inv, __uint_as_float(o[i + 7]) * inv));
-                    }
+                    for (int i = 0; i < 32; i += 8)
+                        st_global_if(valid, row + c + i, make_uint4(
+                            pack_bf16(__uint_as_float(o[i]) * inv, __uint_as_float(o[i + 1]) * inv),
+                            pack_bf16(__uint_as_float(o[i + 2]) * inv, __uint_as_float(o[i + 3]) * inv),
+                            pack_bf16(__uint_as_float(o[i + 4]) * inv, __uint_as_float(o[i + 5]) * inv),
+                            pack_bf16(__uint_as_float(o[i + 6]) * inv, __uint_as_float(o[i + 7]) * inv)));
                 }
             }
         } else {

@@ -134,24 +134,22 @@ __device__ inline uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
-// stores to the shared memory of a CTA of the cluster (address from map_to_rank)
-__device__ inline void st_cluster(uint32_t addr, float x, float y) {
-    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
+// Stores to the shared memory of a CTA of the cluster (address from map_to_rank), counted (16 or 8 bytes) by an mbarrier of that
+// CTA, by the lanes that bring `p`: a predicate and no branch, so that the warp stays together for the collective loads around them.
+__device__ inline void st_async_if(bool p, uint32_t addr, const float4 &v, uint32_t bar) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %6, 0;\n"
+                 "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n}"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar), "r"((uint32_t)p) : "memory");
 }
-__device__ inline void st_cluster(uint32_t addr, const float4 &v) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+__device__ inline void st_async_if(bool p, uint32_t addr, float x, float y, uint32_t bar) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+                 "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n}"
+                 ::"r"(addr), "f"(x), "f"(y), "r"(bar), "r"((uint32_t)p) : "memory");
 }
-__device__ inline void st_cluster(uint32_t addr, const uint32_t *v) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
-}
-// the same, counted (16 bytes) by an mbarrier of that CTA
-__device__ inline void st_async(uint32_t addr, const float4 &v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
-}
-__device__ inline void st_async(uint32_t addr, float x, float y, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-                 ::"r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
+// 16 bytes to global memory by the lanes that bring `p`, likewise
+__device__ inline void st_global_if(bool p, void *ptr, const uint4 &v) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n@p st.global.v4.b32 [%0], {%1, %2, %3, %4};\n}"
+                 ::"l"(ptr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)p) : "memory");
 }
 // shared-memory matrix descriptor, 128-byte swizzle
 __device__ inline uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
