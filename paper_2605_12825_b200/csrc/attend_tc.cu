@@ -677,7 +677,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                 // a wait gave up: this warp's MMAs in flight still read shared memory and write TMEM, and the query rows may
                 // still be on their way
                 const int drain = C::BAR_DRAIN + ti;
-                if (lane == 0) umma_commit(bar(drain));
+                if (elect_one()) umma_commit(bar(drain));     // (a commit tells of its own thread's MMAs)
                 __syncwarp();
                 int dummy = 0;
                 mbar_wait_warp_call(bar(drain), 0, &dummy);
