@@ -90,6 +90,47 @@ int orthrus::num_sms()
     return n;
 }
 
+// What the query below asks for: the occupancy of an attention kernel's cluster without its tensor memory, for which the runtime
+// counts one CTA per SM whatever it allocates.  (Clusters of 5, 6, 8, 10, 11, 12, 13 and 14 with two CTAs per SM: 56, 45, 33,
+// 26, 21, 21, 17 and 14 by this query, and measured to run in one wave up to there; half-sized clusters with an SM each,
+// asked before, say 52, 45, 33, 26, 22, 22, 15 and 15.)
+__global__ void __launch_bounds__(320) cluster_probe_kernel() {}
+
+int orthrus::clusters_resident(int S, int per_sm)
+{
+    constexpr int kMaxDevices = 64, kMaxCluster = 16, kBytes[2] = {200 * 1024, 113 * 1024};
+    static std::atomic<int> cached[2][kMaxDevices][kMaxCluster + 1];      // 0: not asked; else the number plus one
+    int dev = 0;
+    if (S < 1 || S > kMaxCluster || per_sm < 1 || per_sm > 2) return 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+        (void)cudaGetLastError();
+        return per_sm * kDefaultSMs / S;
+    }
+    std::atomic<int> &known = cached[per_sm - 1][dev][S];
+    int n = known.load(std::memory_order_relaxed);
+    if (n > 0) return n - 1;
+    n = per_sm * num_sms();
+    if (S > 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(S);
+        cfg.blockDim = dim3(320);
+        cfg.dynamicSmemBytes = kBytes[per_sm - 1];
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = S; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(cluster_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes[0]) != cudaSuccess ||
+            cudaFuncSetAttribute(cluster_probe_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, cluster_probe_kernel, &cfg) != cudaSuccess || n < 1) {
+            (void)cudaGetLastError();
+            n = S <= 8 ? num_sms() / S : 0;           // a size the device cannot schedule is not chosen
+        }
+    }
+    known.store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
 namespace orthrus {
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -248,7 +289,7 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
     if ((L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units <= 64 && (units < 24 || max_len_of(L) >= 1024)) return false;
     if (units <= 9 && max_len_of(L) > 512 && max_len_of(L) + L->block <= 4032) return false;
     const int S = make_plan(L, true, kn).n_splits;
-    if (S > 1 && units > keys_resident_clusters(S)) return false;   // (the two kernels' CTAs fit an SM alike)
+    if (S > 1 && units > clusters_resident(S, 2)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
     const int max_len = max_len_of(L);
     if (S == 8 && !roomy) return max_len <= 1536 || max_len > 3072;
@@ -287,10 +328,8 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
 static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (kn.splits > 0) return kn.splits < 16 ? kn.splits : 16;
-    // from prefix and block together: a decoder that bounds its lengths by capacity - block then cuts
-    // a block's verification and a width-1 step at the same keys, and where both run on this kernel they round alike
     return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
-                       max_len_of(L) + L->block);
+                       max_len_of(L));
 }
 // Split partials of the mma and SIMT paths (the tcgen05 kernels merge through shared memory)
 static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off)

@@ -763,73 +763,45 @@ template <int HD, int NR, bool XCH> cudaError_t configure(int *dev)
     return cudaSuccess;
 }
 
-// Clusters of S CTAs the current device keeps resident at once.  Two CTAs fit an SM, and a cluster
-// stays within a GPC, so that this is less than 2 x 148 / S.  The query counts one CTA per SM for
-// kernels that allocate tensor memory: asked for clusters of S / 2 (rounded up) it tells how many
-// groups of that many SMs there are (33 of 4, 15 of 8 on a B200; 32 clusters of 8 CTAs were measured
-// to run in one wave, 16 of 16 not); of an odd size two share S SMs (48 clusters of 5 run in one wave).
-// Asked once per device and size.
-template <int HD, int NR> int resident_clusters(int S)
-{
-    constexpr int kMaxDevices = 64;
-    static std::atomic<int> cached[kMaxDevices][MAX_CLUSTER + 1];
-    int dev = 0;
-    constexpr int CTAS = KeysShape<HD, NR>::CTAS;
-    if (configure<HD, NR, true>(&dev) != cudaSuccess) { (void)cudaGetLastError(); return CTAS * kDefaultSMs / S; }
-    int known = cached[dev][S].load(std::memory_order_relaxed);
-    if (known != 0) return known > 0 ? known : 0;
-    auto groups = [](int sms) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(sms, 1);
-        cfg.blockDim = dim3(NTHREADS);
-        cfg.dynamicSmemBytes = KeysShape<HD, NR>::SMEM_BYTES;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = sms; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, attend_keys_kernel<HD, NR, true>, &cfg) != cudaSuccess || n < 1) {
-            (void)cudaGetLastError();
-            n = sms <= 8 ? num_sms() / sms : 0;   // a size the device cannot schedule is not chosen
-        }
-        return n;
-    };
-    int n = groups((S + CTAS - 1) / CTAS);
-    if (S == 1) n *= CTAS;
-    else if (CTAS == 2 && S % 2) n = max(n, 2 * groups(S));
-    cached[dev][S].store(n < 1 ? -1 : n, std::memory_order_relaxed);
-    return n;
-}
-
 // CTAs per unit: the cheapest by this count (in 0.1 us) among the sizes at which all units are resident together.
 //  - Tiles follow one another.  Two cost little more than one (a warpgroup each; at head_dim 128 both tiles' keys and the
 //    first one's values wait in shared memory), from the third on each waits for its slot of the ring: 8 units
 //    of 4 rows, 500 keys, 1, 2, 3 and 5 tiles a CTA 3.5, 4.4, 5.9 and 8.6 us; d = 64, 32 rows, 2 units of 500 keys 3.5, 4.2, 5.1, 7.0.
 //  - The merge: a warp takes some 0.4 us for a task, and the CTAs share the tasks (64 rows, 8 units of 300 keys, one tile
-//    each: 7.2 us at 2 CTAs, 6.2 at 3, 5.7 at 4 to 6).
-//  - Once a call and the next one, which starts early, no longer find SMs of their own, CTAs of a cluster share an SM and with
-//    it the way to the others, which counts where they have much to tell (64 rows, 8 units of 1500 keys 6.0 us at 10
-//    CTAs, 7.6 at 11; 16 units of 700 keys 6.2 at 6, 7.4 at 7; with 4 rows no difference); once they do not fit
-//    together at all, the next call starts late (32 units of 1000 keys, 4 rows 5.8 us at 5 CTAs, 6.3 at 8; 64 rows, 300 keys 6.7
-//    at 4, 8.0 at 5).
+//    each: 7.2 us at 2 CTAs, 6.2 at 3, 5.7 at 4 to 6).  At 64 rows that is worth CTAs without a key of their own (one unit of 100
+//    keys 6.0 us at 3, 5.0 at 8).
+//  - From 32 rows on there is much to tell, and CTAs that share an SM share the way to the others: once the clusters of a call do not all
+//    find SMs of their own, it takes 1 to 1.5 us more at 64 rows, 0.5 at 32.  A cluster stays within a GPC, so that this depends on the size of the
+//    cluster (a B200 has SMs for 45, 33, 26, 22, 15, 15, 15, 11 and 7 clusters of 3 to 11 CTAs and for 7 of 12 to 16; us a call, 300 keys:
+//    clusters of 3, 36 units 6.7 and 48 8.4; of 4, 28 6.3 and 36 8.0; of 5, 24 6.5 and 28 7.6; of 6, 20 6.6 and 24 8.1; of 7, 14
+//    6.1 and 16 7.4).  A line at five ninths of the SMs, which stood here before, kept 28 units of 200 keys at 2 CTAs: 7.3 us, 6.3 at 4.
+//  - Once they do not fit beside one another at all, the next call starts late (32 units of 1000 keys, 4 rows 5.8 us at 5 CTAs, 6.3
+//    at 8), the more so where clusters fill the GPU to the last place (56 units of 32 rows, 3000 keys 17.1 us at 4, 19.9 at 5).
 // Of sizes that cost the same the largest up to 8 (lengths are often below the bound the plan is
-// made for, and then the larger size has fewer tiles), else the smallest.  A second wave of clusters costs more than any
-// split gains (32 units of 64 rows, 1000 keys 9.1 us at 8, 12.8 at 9).
+// made for, and then the larger size has fewer tiles), else the smallest, and so where a CTA has one tile in any case
+// and half the SMs are taken (16 units of 64 rows, 300 keys 5.8 us at 4, 6.3 at 6; but 8 of 4 rows 3.6 at 3, 3.4 at 6).  A second wave of clusters costs more than any
+// split gains (32 units of 64 rows, 1000 keys 9.1 us at 8, 12.8 at 9; 22 of 4000 keys 13.7 at 10, 20.7 at 11; 72 units of 32 rows,
+// 1000 keys 10.4 at 3, 17.4 at 4).
+// Against sweeps of 1 to 92 units, 64 to 8000 keys and all sizes, the choice is 0.5 to 0.6 % above the best size in the mean at
+// 4, 32 and 64 rows and both head sizes, where the count of residents by half-sized clusters and the line at five ninths took 3.8 to 4.9 %.
+// Where it misses most: 16 or 17 units of 24 to 26 halves, which get 13 CTAs and are 5 to 12 % faster with 8.
 template <int HD, int NR> int choose_splits(int units, int halves)
 {
+    constexpr bool FULL = HD == 128 && NR == 64;
     constexpr int TILE2 = HD == 128 ? 9 : 6, TILE3 = HD == 128 ? 16 : NR == 128 ? 15 : 10;
-    constexpr int TASKS = NR / 4 * (HD / 32);
+    constexpr int TASKS = NR / 4 * (HD / 32), ALONE = NR >= 64 ? 10 : 6, MERGE = FULL ? 10 : 7;
+    constexpr int SHARED = NR == 64 ? (HD == 128 ? 15 : 8) : NR == 32 ? 5 : 0;    // CTAs of a call share SMs
+    constexpr int PER_SM = KeysShape<HD, NR>::CTAS;
     const int sms = num_sms();
     int best = 1, best_cost = 1 << 30;
-    for (int S = 1; S <= MAX_CLUSTER && S <= halves; ++S) {
+    for (int S = 1; S <= MAX_CLUSTER && S <= (FULL ? max(halves, 8) : halves); ++S) {
         const int tiles = ((halves + S - 1) / S + 1) / 2, ctas = units * S;
         int cost = (tiles > 1 ? TILE2 : 0) + (tiles > 2 ? min(tiles - 2, 1 << 20) * TILE3 : 0);
-        cost += S == 1 ? (NR >= 64 ? 10 : 5) : 7 + 4 * ((TASKS + 8 * S - 1) / (8 * S));
-        if (NR == 64 && S > 1 && 9 * ctas > 5 * sms) cost += HD == 128 ? 15 : 8;
-        if (S > 1 && ctas > sms) cost += NR == 64 && HD == 128 ? 15 : 5 + min(5 * (ctas - sms) / sms, 10);
-        if (S <= 8 ? cost > best_cost : cost >= best_cost) continue;
-        if (S > 1 && units > resident_clusters<HD, NR>(S)) continue;
+        cost += S == 1 ? ALONE : MERGE + 4 * ((TASKS + 8 * S - 1) / (8 * S));
+        if (SHARED && S > (NR == 32 ? 2 : 1) && units > clusters_resident(S, 1)) cost += SHARED;
+        if (S > 1 && ctas > sms) cost += FULL ? 3 + 4 * (ctas - sms) / sms : 5 + min(5 * (ctas - sms) / sms, 10);
+        if (S <= 8 && (tiles > 1 || 2 * ctas <= sms) ? cost > best_cost : cost >= best_cost) continue;
+        if (S > 1 && (units > clusters_resident(S, PER_SM) || (S > 2 && 16 * ctas > 15 * PER_SM * sms))) continue;
         best = S;
         best_cost = cost;
     }
@@ -911,12 +883,12 @@ int keys_kb_rows(int d, int G, int K)
     return (K + tiles - 1) / tiles;
 }
 
-int keys_splits(int d, int G, int K, int units, int max_keys)
+int keys_splits(int d, int G, int K, int units, int max_len)
 {
     // the layers of a pass ask the same question: the last answer of this thread is kept
     struct Key { int dev, d, nr, units, halves, S; };
     static thread_local Key last = {-1, 0, 0, 0, 0, 0};
-    Key k = {-1, d, keys_rows(d, G, K), units, (max_keys + HALF - 1) / HALF + 1, 0};   // (prefix and block in halves of their own)
+    Key k = {-1, d, keys_rows(d, G, K), units, (max_len + HALF - 1) / HALF + 1, 0};   // (prefix and block in halves of their own)
     if (cudaGetDevice(&k.dev) != cudaSuccess) { (void)cudaGetLastError(); k.dev = -2; }
     if (k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.units == last.units && k.halves == last.halves) return last.S;
     switch (k.nr) {
@@ -928,8 +900,6 @@ int keys_splits(int d, int G, int K, int units, int max_keys)
     last = k;
     return k.S;
 }
-
-int keys_resident_clusters(int S) { return resident_clusters<128, 64>(S); }
 
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st)
 {

@@ -16,6 +16,11 @@ constexpr int kDefaultSMs = 148;      // a full B200; used only when no device c
 // there is no device, so that size queries still work on a host without a GPU).
 int num_sms();
 
+// Clusters of S <= 16 CTAs that are resident at once where per_sm (1 or 2) of the attention kernels' CTAs fit an SM.  A cluster
+// stays within a GPC, and GPCs have unequal numbers of SMs, so that this is less than per_sm * num_sms() / S.  Asked once per
+// device; per_sm * kDefaultSMs / S when there is no device.
+int clusters_resident(int S, int per_sm);
+
 // Parameters common to every attention kernel.  Rows of one (sequence, KV head)
 // unit are ordered r = i * G + g  (block position i, head g within the group), so
 // that the G query heads sharing a KV head and all K block positions form one tile
@@ -126,8 +131,7 @@ size_t tc_stream_workspace_bytes(int B, int Hkv, int n_ctas);
 cudaError_t launch_attend_tc_stream(const AttnParams &p, int n_ctas, void *ws_body, int flags, cudaStream_t st);
 int keys_rows(int d, int G, int K);      // MMA columns of a query tile on the keys kernel (0: not its shape)
 int keys_kb_rows(int d, int G, int K);   // block positions of such a query tile
-int keys_splits(int d, int G, int K, int units, int max_keys);   // CTAs per (unit, query tile) on the current device
-int keys_resident_clusters(int S);       // clusters of S CTAs, two to an SM, that are resident at once
+int keys_splits(int d, int G, int K, int units, int max_len);   // CTAs per (unit, query tile) on the current device
 int tc_kb_rows(int G, int K);            // block positions per query tile of 128 rows
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st);        // n_splits = cluster size
 cudaError_t launch_combine(const AttnParams &p, int dtype, cudaStream_t st);

@@ -111,9 +111,10 @@ def small_workload(B, K, Hq, Hkv, d, pmin, pmax, dtype="bf16", V=64, std=1.0, na
                       V, pmin, pmax, value_std=std, dtype=dtype)
 
 
-def captured_launches(call):
+def captured_launches(call, grids=None):
     """The kernels that `call` enqueues on the current stream, taken from a stream capture behind a kernel of the
-    library user's own: [(kernel name, launched as a programmatic dependent)] in launch order.  Nothing runs."""
+    library user's own: [(kernel name, launched as a programmatic dependent)] in launch order.  Nothing runs.
+    A list passed as `grids` takes their grids (x, y, z) in the same order."""
     import ctypes
     cu = ctypes.CDLL("libcuda.so.1")
     x = torch.zeros(8, device="cuda")
@@ -143,6 +144,8 @@ def captured_launches(call):
     def name(node):
         p, s = KernelParams(), ctypes.c_char_p()
         ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        if grids is not None:
+            grids.append(tuple(p.dims[:3]))
         ok(cu.cuFuncGetName(ctypes.byref(s), ctypes.c_void_p(p.func)) if p.func else
            cu.cuKernelGetName(ctypes.byref(s), ctypes.c_void_p(p.kern)))
         return s.value.decode()
