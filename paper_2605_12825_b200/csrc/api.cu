@@ -219,16 +219,18 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
             //  still split; many small CTAs would spend their time starting and merging)
             while (S < 16 && units * S < slots && tiles / (S * 2) >= 8) S *= 2;
         }
-        // Sixteen only while a call and the next one, which starts early, find SMs of their own, too: on shared ones the CTAs of
-        // a cluster share the way to the others, which the merge fills.  As many CTAs as do find some, then (8 units of 128
-        // rows, 2000, 4000, 8000 and 16000 keys 12.4, 13.6, 17.6 and 26.0 us at 16, 9.1, 11.4, 15.8 and 25.3 at 10; behind a rotary
-        // write, whose CTAs are in between, 4000 and 8000 keys 15.6 and 19.7 at 16, 16.9 and 22.9 at 10, 15.0 and 19.3 at 9), until
-        // streaming the keys is nearly all there is (32000 keys 42.7 and 43.7; 68 rows, 8000 keys 17.6 and 18.3).
+        // Sixteen only where every cluster finds SMs of its own (up to 7 units on a B200; a cluster stays within a GPC): on shared ones
+        // the CTAs of a cluster share the way to the others, which the merge fills.  Else the largest size that does and has a
+        // merge of its own (128 rows, 8 units of 500, 2000, 4000 and 16000 keys 7.9, 11.7, 13.1 and 25.7 us at 16, 6.7, 8.9, 11.1 and 25.3
+        // at 10; 6 units of 8000 13.1 at 16, 15.8 at 10), until streaming the keys is nearly all there is (24000 keys 34.6 and 34.9; 64
+        // rows, 2000 and 4000 keys 8.4 and 9.9 at 16, 7.8 and 10.0 at 10).  Behind a rotary write, whose CTAs are in between, 128 rows
+        // and clusters of 10 do not go together (4000, 8000 and 16000 keys 14.1, 20.0 and 32.0 at 8, 16.5, 22.8 and 35.3 at 10, 15.6, 19.1
+        // and 27.5 at 16).
         const int rows = G * L->block;
-        if (forced <= 0 && S == 16 && tiles < (rows > 96 ? 160 : rows > 64 ? 64 : 48)) {
-            const int fit = L->flags & ORTHRUS_LAYER_BLOCK_IN_CACHE ? num_sms() / (2 * units) : 5 * num_sms() / (9 * units);
-            if (fit < S) S = fit > 8 ? fit : 8;
-        }
+        const bool behind_write = (L->flags & ORTHRUS_LAYER_BLOCK_IN_CACHE) && rows > 96;
+        if (forced <= 0 && S == 16 && units > clusters_resident(16, 1) &&
+            tiles < (behind_write ? 112 : rows > 96 ? 320 : rows > 64 ? 64 : 48))
+            S = units <= clusters_resident(10, 1) && !behind_write ? 10 : 8;
         const int max_cluster = tc_max_cluster(nt);
         if (S > max_cluster) S = max_cluster;
         if (S > tiles) S = tiles;

@@ -11,10 +11,10 @@ pytestmark = pytest.mark.gpu
 TWO = (296, 148, 93, 71, 56, 45, 37, 33, 30, 26, 21, 21, 17, 14, 14, 14)
 
 
-def planned(units, rows, bound, monkeypatch, flags=0, d=128):
+def planned(units, rows, bound, monkeypatch, flags=0, d=128, kernel="attend_keys_kernel"):
     """(CTAs per unit, query tiles) of a call of `units` units of `rows` = 4 x block query rows."""
     b = binding()
-    monkeypatch.setenv("ORTHRUS_TC_SMALL_ROWS", "1")
+    monkeypatch.setenv("ORTHRUS_TC_SMALL_ROWS", "1" if kernel == "attend_keys_kernel" else "0")
     K = rows // 4
     cache = torch.empty(units, 1, bound + K, d, dtype=torch.bfloat16, device="cuda")
     ln = torch.zeros(units, dtype=torch.int32, device="cuda")
@@ -23,8 +23,8 @@ def planned(units, rows, bound, monkeypatch, flags=0, d=128):
     ws = b.new_workspace(b.orthrus_attend_workspace_bytes(layer))
     grids = []
     (name, _), = captured_launches(lambda: b.orthrus_ar_verify_attend(layer, q, kb, kb, q, ws), grids)
-    assert "attend_keys_kernel" in name
-    return grids[0][0], grids[0][1]
+    assert kernel in name
+    return grids[0][0], grids[0][1] // (units if kernel == "attend_tc_kernel" else 1)
 
 
 @pytest.fixture(autouse=True)
@@ -47,3 +47,13 @@ def test_clusters_are_all_resident(rows, monkeypatch):
     (22, 4000, 8), (24, 500, 5), (32, 1000, 8)])
 def test_clusters_at_the_lines(units, bound, splits, monkeypatch):
     assert planned(units, 64, bound, monkeypatch) == (splits, 1)
+
+
+# wide kernel: units, rows, bound, block in the cache, CTAs per unit
+@pytest.mark.parametrize("units,rows,bound,in_cache,splits", [
+    (6, 128, 8000, 0, 16), (7, 128, 8000, 0, 16), (8, 128, 2000, 0, 10), (8, 128, 16000, 0, 10), (8, 128, 20481, 0, 16), (9, 128, 4000, 0, 10),
+    (8, 128, 4000, 1, 8), (8, 128, 8000, 1, 16), (8, 80, 4000, 0, 10), (8, 80, 5000, 0, 16), (8, 64, 3000, 0, 10), (8, 64, 3073, 0, 16),
+    (4, 64, 3000, 0, 16)])
+def test_clusters_of_sixteen_of_the_wide_kernel(units, rows, bound, in_cache, splits, monkeypatch):
+    flags = binding().LAYER_BLOCK_IN_CACHE if in_cache else 0
+    assert planned(units, rows, bound, monkeypatch, flags, kernel="attend_tc_kernel") == (splits, 1)
