@@ -327,11 +327,12 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     if (rows > 64) return max_len_of(L) > 320;
     return rows < 64 || L->head_dim == 64 || !wide_better(L, kn);
 }
-static int keys_plan(const orthrus_layer_t *L, const Knobs &kn)
+static int keys_plan(const orthrus_layer_t *L, const Knobs &kn, bool *apart)
 {
+    *apart = false;
     if (kn.splits > 0) return kn.splits < 16 ? kn.splits : 16;
     return keys_splits(L->head_dim, L->n_q_heads / L->n_kv_heads, L->block, L->batch * L->n_kv_heads * keys_tiles(L),
-                       max_len_of(L));
+                       max_len_of(L), apart);
 }
 // Split partials of the mma and SIMT paths (the tcgen05 kernels merge through shared memory)
 static size_t partial_bytes(const orthrus_layer_t *L, const Plan &pl, size_t *ml_off)
@@ -369,7 +370,8 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
     if (stream_k) pl.n_splits = 1;
     size_t ml_off = 0;
     const bool keys = !stream_k && (want == PATH_AUTO || (want == PATH_TCGEN05 && tc)) && keys_usable(L, kn);
-    if (keys) pl.n_splits = keys_plan(L, kn);
+    bool apart = false;
+    if (keys) pl.n_splits = keys_plan(L, kn, &apart);
     const size_t need = kHeaderBytes + (stream_k ? tc_stream_workspace_bytes(L->batch, L->n_kv_heads, tc_stream_ctas())
                                         : keys || tc ? 0 : partial_bytes(L, pl, &ml_off));
     if (ws_bytes < need) return ORTHRUS_ERR_WORKSPACE;
@@ -391,6 +393,7 @@ static orthrus_status_t attend(const orthrus_layer_t *L, int causal, const void 
 
     int flags = (int)(L->flags & (ORTHRUS_LAYER_CACHE_QUIESCENT | ORTHRUS_LAYER_NO_EARLY_LAUNCH));
     if (kn.no_early_launch) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
+    p.apart = apart;
     p.early = !(flags & ORTHRUS_LAYER_NO_EARLY_LAUNCH);
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
@@ -524,6 +527,7 @@ static orthrus_status_t attend_packed(const orthrus_layer_t *layer, int32_t n_bl
     t_last_path = "tcgen05";
     int flags = (int)(layer->flags & (ORTHRUS_LAYER_CACHE_QUIESCENT | ORTHRUS_LAYER_NO_EARLY_LAUNCH));
     if (kn.no_early_launch) flags |= ORTHRUS_LAYER_NO_EARLY_LAUNCH;
+    p.apart = 0;
     p.early = !(flags & ORTHRUS_LAYER_NO_EARLY_LAUNCH);
     return launch_attend_tc_packed(p, flags, static_cast<cudaStream_t>(stream)) == cudaSuccess
                ? ORTHRUS_OK : ORTHRUS_ERR_CUDA;

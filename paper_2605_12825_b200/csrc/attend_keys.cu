@@ -109,7 +109,8 @@ template <int HD, int NR> struct KeysShape {
     // the merge, in the ring: [task of this CTA][CTA] messages, then weights [warp][CTA][row]
     static constexpr int TASKS = NR / 4 * (HD / 32);
     static constexpr int OFF_XW = (TASKS + MAX_CLUSTER) * MSG;
-    static_assert(OFF_XW + SW * MAX_CLUSTER * 16 <= OFF_Q, "exchange buffer");
+    static constexpr int OFF_XB = OFF_XW + SW * (MAX_CLUSTER + 1) * 16;       // a task's part from the block's own keys [warp][row][column]
+    static_assert(OFF_XB + SW * 512 <= OFF_Q, "exchange buffer");
     static constexpr uint32_t TM_COLS = 4 * NR;                // two score buffers, two accumulators
     static constexpr uint32_t tm_s(int w) { return (uint32_t)(w * NR); }
     static constexpr uint32_t tm_o(int w) { return (uint32_t)(2 * NR + w * NR); }
@@ -153,12 +154,83 @@ __host__ __device__ constexpr uint32_t keys_idesc(uint32_t n, uint32_t a_mn, uin
     return make_idesc(n, b_mn) | (a_mn << 15);
 }
 
+// A block's own keys apart from the tiles (APART): what a unit's query rows 4 g to 4 g + 3 get from them in 32 head columns, by the
+// warp that merges these.  Sixteen keys at a time by mma.sync, query rows (four of the sixteen) on its rows, the 128 head columns of the
+// first product in an order of their own, the same for both sides; probabilities, references and sums as a tile's.
+struct BlockPart { float m, l, o[4][2]; };                   // of row lane / 4 (lanes below 16); columns 8 t + 2 (lane % 4), + 1
+__device__ inline void mma_16x8x16(float *d, uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {      // (rows 8 to 15 of A are zero)
+    float x = 0.f, y = 0.f;
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(x), "+f"(y) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+}
+__device__ inline uint32_t transposed_8x8(uint32_t x) {
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+// q: query row lane / 4 (any where there is none); k, v: row 0 of the block's keys and of the 32 columns of its values, `stride`
+// elements apart; sees: keys that the row sees
+__device__ inline BlockPart block_part(const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v, long long stride, int K,
+                                       int sees, float sc, int lane)
+{
+    constexpr int HD = 128;
+    BlockPart r = {-INFINITY, 0.f, {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}};
+    const int part = (lane & 3) * 8, key = lane >> 2, j0 = (lane & 3) * 2;
+    uint4 qv[HD / 32];
+#pragma unroll
+    for (int x = 0; x < HD / 32; ++x) qv[x] = *reinterpret_cast<const uint4 *>(q + x * 32 + part);
+#pragma unroll 1
+    for (int k0 = 0; k0 < K; k0 += 16) {
+        // (rows behind the block's last are that one again: their probabilities are zero)
+        const long long row0 = min(k0 + key, K - 1) * stride, row1 = min(k0 + key + 8, K - 1) * stride;
+        uint4 ka[HD / 32], kb[HD / 32];
+        uint32_t va[4], vb[4];
+#pragma unroll
+        for (int x = 0; x < HD / 32; ++x) {
+            ka[x] = *reinterpret_cast<const uint4 *>(k + row0 + x * 32 + part);
+            kb[x] = *reinterpret_cast<const uint4 *>(k + row1 + x * 32 + part);
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            va[t] = *reinterpret_cast<const uint32_t *>(v + row0 + t * 8 + j0);
+            vb[t] = *reinterpret_cast<const uint32_t *>(v + row1 + t * 8 + j0);
+        }
+        float d[2][2] = {{0.f, 0.f}, {0.f, 0.f}};             // keys k0 + j0, + 1 and those 8 on
+#pragma unroll
+        for (int x = 0; x < HD / 32; ++x) {
+            mma_16x8x16(d[0], qv[x].x, qv[x].y, ka[x].x, ka[x].y);
+            mma_16x8x16(d[1], qv[x].x, qv[x].y, kb[x].x, kb[x].y);
+            mma_16x8x16(d[0], qv[x].z, qv[x].w, ka[x].z, ka[x].w);
+            mma_16x8x16(d[1], qv[x].z, qv[x].w, kb[x].z, kb[x].w);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) if (k0 + j0 + (i & 1) + (i & 2) * 4 >= sees) d[i >> 1][i & 1] = -INFINITY;
+        float top = fmaxf(fmaxf(d[0][0], d[0][1]), fmaxf(d[1][0], d[1][1]));
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+        const float m = fmaxf(r.m, ceilf(top * sc)), ref = m == -INFINITY ? 0.f : m, al = ex2(r.m - ref);     // (of nothing so far: 0)
+        r.m = m;
+        const uint32_t wa = pack_bf16(ex2(fmaf(d[0][0], sc, -ref)), ex2(fmaf(d[0][1], sc, -ref)));
+        const uint32_t wb = pack_bf16(ex2(fmaf(d[1][0], sc, -ref)), ex2(fmaf(d[1][1], sc, -ref)));
+        r.l = fmaf(r.l, al, (__uint_as_float(wa << 16) + __uint_as_float(wa & 0xffff0000u)) + (__uint_as_float(wb << 16) + __uint_as_float(wb & 0xffff0000u)));
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            r.o[t][0] *= al; r.o[t][1] *= al;
+            mma_16x8x16(r.o[t], wa, wb, transposed_8x8(va[t]), transposed_8x8(vb[t]));
+        }
+    }
+    r.l += __shfl_xor_sync(0xffffffffu, r.l, 1);
+    r.l += __shfl_xor_sync(0xffffffffu, r.l, 2);
+    return r;
+}
+
 // XCH: several CTAs share a unit and exchange their partial results.
+// APART: the tiles hold prefix keys only; the block's own, which would be one CTA's third tile, are left to the warps that merge, while
+// they wait for messages (8 units of 64 rows, 4096 keys and blocks of 16: sixteen CTAs of two tiles each).
 // The code is kept short on purpose (loops not unrolled, one place for each wait, copy and product): the warps' roles are
 // run through once or twice per call, and an SM's instruction cache holds 32 KB.
-template <int HD, int NR, bool XCH>
-__global__ void __launch_bounds__(NTHREADS, KeysShape<HD, NR>::CTAS)
-attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, const KeysArgs args)
+template <int HD, int NR, bool XCH, bool APART>
+__device__ __forceinline__ void attend_keys(const AttnParams &p, const KeysMaps &tm, const KeysArgs &args)
 {
     using C = KeysShape<HD, NR>;
     constexpr int PANELS = C::PANELS, QPANEL = NR * 128;
@@ -202,7 +274,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             fence_proxy_async();
             if (XCH) mbar_expect_tx(bar(C::BAR_X), (uint32_t)(my_tasks * S * MSG));
-            prefetch_map(&tm.kb); prefetch_map(&tm.vb);
+            if (!APART) { prefetch_map(&tm.kb); prefetch_map(&tm.vb); }
         }
         __syncwarp();
         bar_issue_arrive();
@@ -228,7 +300,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         P = P < 0 ? 0 : len_hi;
     }
     // the unit's halves: n_pre of 64 prefix keys, then the block's keys, shared out evenly
-    const int n_pre = (P + HALF - 1) / HALF, n_all = n_pre + 1;
+    const int n_pre = (P + HALF - 1) / HALF, n_all = n_pre + !APART;
     const int share = XCH ? (int)__umulhi((unsigned)n_all, args.inv_s32) : n_all, rest = n_all - share * S;
     auto first_half = [&](int k) { return XCH ? k * share + (int)((uint32_t)(k * rest) * args.inv_s >> 16) : k * share; };  // k * n_all / S
     const int a0 = first_half(rank), a1 = first_half(rank + 1);
@@ -253,7 +325,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         const uint32_t d = sbase + C::OFF_RING + slot * C::KV_BYTES + (a & 1) * (HALF * 128), fb = bar(C::BAR_FULL + slot);
 #pragma unroll
         for (int s = 0; s < PANELS; ++s) {
-            if (a < n_mine || p.blk_in_cache)                 // (rows behind the keys hold anything: masked, cleared in V)
+            if (APART || a < n_mine || p.blk_in_cache)        // (rows behind the keys hold anything: masked, cleared in V)
                 tma_load_2d(d + s * PANEL, v ? &tm.v : &tm.k, s * 64, row_base + (a < n_mine ? (a0 + a) * HALF : P), fb, policy);
             else                                              // rows >= K are out of bounds and arrive as zeros
                 tma_load_4d(d + s * PANEL, v ? &tm.vb : &tm.kb, s * 64, h, 0, b, fb);
@@ -266,6 +338,12 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         const long long unit_row = (((long long)b * p.K + i0) * p.Hq + h * p.G) * HD;
         const uint4 *q = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.q) + unit_row);
         __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(p.out) + unit_row;
+        // the block's own keys and values, where they are kept apart from the tiles
+        const long long blk0 = APART && !p.blk_in_cache ? ((long long)b * p.K * p.Hkv + h) * HD : ((long long)row_base + P) * HD;
+        const __nv_bfloat16 *bk = static_cast<const __nv_bfloat16 *>(APART && !p.blk_in_cache ? p.k_blk : p.k_cache) + blk0;
+        const __nv_bfloat16 *bv = static_cast<const __nv_bfloat16 *>(APART && !p.blk_in_cache ? p.v_blk : p.v_cache) + blk0;
+        const long long blk_stride = p.blk_in_cache ? HD : (long long)p.Hkv * HD;
+        if (APART && tid < 4 * p.K) prefetch_l2((tid & 1 ? bv : bk) + (tid >> 2) * blk_stride + (tid >> 1 & 1) * 64);
         {
             // where this thread's chunks (16 bytes each) come from; rows past M are zero
             constexpr int QCH = HD / 8, QN = (NR * QCH + ST - 1) / ST;
@@ -309,7 +387,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         for (int t = wg, u = 0; t < n_tiles; t += 2, ++u) {
             const int a = 2 * t + (kt >> 6), j = kt & 63;     // this thread's half and key in it
             // rows below lo do not see the key (all, if the key does not exist)
-            const int lo = j >= half_keys(a) ? NR : (a >= n_mine && p.causal ? (j - i0) * p.G : 0);
+            const int lo = j >= half_keys(a) ? NR : (!APART && a >= n_mine && p.causal ? (j - i0) * p.G : 0);
             const bool masks = __any_sync(0xffffffffu, lo > 0);
             if (u > 0) mbar_wait_warp_call(bar(C::BAR_PV + wg), (u - 1) & 1, abort_flag);   // P buffer and O^T at rest
             mbar_wait_warp_call(bar(C::BAR_S + wg), u & 1, abort_flag);
@@ -527,13 +605,27 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll
                 for (int k = 0; k < 4; ++k) at[k] = 4 * g + k < M ? row_off(4 * g + k) + col : -1;
             };
-            places(warp);
-            // (the wait outlasts every other one: a CTA of the cluster that gave one up sends all the same)
-            const bool got = __all_sync(0xffffffffu, mbar_wait_long(bar(C::BAR_X), 0));
-            if (!got && lane == 0 && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
-            float *wt = reinterpret_cast<float *>(smem + C::OFF_XW) + warp * (MAX_CLUSTER * 4);
+            float *wt = reinterpret_cast<float *>(smem + C::OFF_XW) + warp * ((MAX_CLUSTER + 1) * 4);
 #pragma unroll 1
-            for (int n = warp; n < my_tasks && got; n += SW) {
+            for (int n = warp; n < my_tasks; n += SW) {
+                places(n);
+                BlockPart bp;
+                if constexpr (APART) {
+                    const int g = (n * S + rank) / (HD / 32), row = min(4 * g + (lane >> 2 & 3), M - 1);
+                    bp = block_part(reinterpret_cast<const __nv_bfloat16 *>(q) + row_off(row), bk, bv + (n * S + rank) % (HD / 32) * 32,
+                                    blk_stride, p.K, p.causal ? i0 + (int)((uint32_t)row * args.inv_g >> 16) + 1 : p.K, p.scale_log2, lane);
+                    if (lane < 16) {
+                        float *o = reinterpret_cast<float *>(smem + C::OFF_XB) + warp * 128 + (lane >> 2) * 32 + (lane & 3) * 2;
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) *reinterpret_cast<float2 *>(o + t * 8) = make_float2(bp.o[t][0], bp.o[t][1]);
+                    }
+                }
+                if (n == warp) {
+                    // (the wait outlasts every other one: a CTA of the cluster that gave one up sends all the same)
+                    const bool got = __all_sync(0xffffffffu, mbar_wait_long(bar(C::BAR_X), 0));
+                    if (!got && lane == 0 && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
+                    if (!got) break;
+                }
                 const unsigned char *msg = smem + n * S * MSG;
                 // weights: lane = (row, CTA and CTA + 8)
                 const int r = lane >> 3, j0 = lane & 7, j1 = j0 + 8;
@@ -542,6 +634,11 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 if (j0 < S) { m0 = ml[j0 * (MSG / 4)]; l0 = ml[j0 * (MSG / 4) + 4]; }
                 if (j1 < S) { m1 = ml[j1 * (MSG / 4)]; l1 = ml[j1 * (MSG / 4) + 4]; }
                 float m = fmaxf(l0 > 0.f ? m0 : -INFINITY, l1 > 0.f ? m1 : -INFINITY);
+                float mb = 0.f, lb = 0.f;                     // of this lane's row from the block's own keys
+                if constexpr (APART) {
+                    mb = __shfl_sync(0xffffffffu, bp.m, 4 * r); lb = __shfl_sync(0xffffffffu, bp.l, 4 * r);
+                    m = fmaxf(m, lb > 0.f ? mb : -INFINITY);
+                }
 #pragma unroll
                 for (int off = 4; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
                 // (a sum that is not a number has no order: its row is void with it)
@@ -549,11 +646,19 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
                 float L = fmaf(w0, l0, w1 * l1);
 #pragma unroll
                 for (int off = 4; off; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+                const float wb = lb > 0.f ? ex2(mb - m) : lb;
+                if constexpr (APART) L = fmaf(wb, lb, L);
                 const float inv = L == 0.f ? 0.f : __frcp_rn(L);
                 wt[j0 * 4 + r] = w0 * inv;
                 wt[j1 * 4 + r] = w1 * inv;
+                if (APART && j0 == 0) wt[MAX_CLUSTER * 4 + r] = wb * inv;
                 __syncwarp();
                 float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                if constexpr (APART) {
+                    const float4 w = *reinterpret_cast<const float4 *>(wt + MAX_CLUSTER * 4);
+                    const float *o = reinterpret_cast<const float *>(smem + C::OFF_XB) + warp * 128 + lane;
+                    acc = make_float4(w.x * o[0], w.y * o[32], w.z * o[64], w.w * o[96]);
+                }
 #pragma unroll 4
                 for (int j = 0; j < S; ++j) {
                     const float4 v = *reinterpret_cast<const float4 *>(msg + j * MSG + lane * 16);
@@ -565,7 +670,6 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     if (at[k] >= 0) out[at[k]] = __float2bfloat16_rn(y[k]);
-                if (n + SW < my_tasks) places(n + SW);
                 __syncwarp();
             }
         }
@@ -641,7 +745,7 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
         constexpr uint32_t IDESC_PV = keys_idesc(NR, 1, 1);   // A = V tile, B = P, both MN-major
         const uint32_t tmem = *tmem_slot;
         bool ok = __all_sync(0xffffffffu, !*abort_flag);
-        if (quiescent && nh > n_mine) {
+        if (!APART && quiescent && nh > n_mine) {
             // the block's own half of the last tile, where the producer's first round has left it out
             griddep_wait();
             if (ok && elect_one()) {
@@ -741,8 +845,26 @@ attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, cons
     }
 }
 
+template <int HD, int NR, bool XCH>
+__global__ void __launch_bounds__(NTHREADS, KeysShape<HD, NR>::CTAS)
+attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, const KeysArgs args)
+{
+    attend_keys<HD, NR, XCH, false>(p, tm, args);
+}
+template <int HD, int NR>
+__global__ void __launch_bounds__(NTHREADS, KeysShape<HD, NR>::CTAS)
+apart_attend_keys_kernel(const AttnParams p, const __grid_constant__ KeysMaps tm, const KeysArgs args)
+{
+    attend_keys<HD, NR, true, true>(p, tm, args);
+}
+template <int HD, int NR, bool XCH, bool APART> constexpr auto keys_kernel()
+{
+    if constexpr (APART) return apart_attend_keys_kernel<HD, NR>;
+    else return attend_keys_kernel<HD, NR, XCH>;
+}
+
 // function attributes belong to a device: set them once on each device that launches
-template <int HD, int NR, bool XCH> cudaError_t configure(int *dev)
+template <int HD, int NR, bool XCH, bool APART> cudaError_t configure(int *dev)
 {
     constexpr int kMaxDevices = 64;
     static std::mutex mu;
@@ -752,7 +874,7 @@ template <int HD, int NR, bool XCH> cudaError_t configure(int *dev)
     if (*dev < 0 || *dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!configured[*dev]) {
-        auto kern = attend_keys_kernel<HD, NR, XCH>;
+        auto kern = keys_kernel<HD, NR, XCH, APART>();
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, KeysShape<HD, NR>::SMEM_BYTES);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess)
@@ -785,7 +907,8 @@ template <int HD, int NR, bool XCH> cudaError_t configure(int *dev)
 // Against sweeps of 1 to 92 units, 64 to 8000 keys and all sizes, the choice is 0.5 to 0.6 % above the best size in the mean at
 // 4, 32 and 64 rows and both head sizes, where the count of residents by half-sized clusters and the line at five ninths took 3.8 to 4.9 %.
 // Where it misses most: 16 or 17 units of 24 to 26 halves, which get 13 CTAs and are 5 to 12 % faster with 8.
-template <int HD, int NR> int choose_splits(int units, int halves)
+struct Pick { int S, cost; };
+template <int HD, int NR> Pick choose_splits(int units, int halves)
 {
     constexpr bool FULL = HD == 128 && NR == 64;
     constexpr int TILE2 = HD == 128 ? 9 : 6, TILE3 = HD == 128 ? 16 : NR == 128 ? 15 : 10;
@@ -805,18 +928,21 @@ template <int HD, int NR> int choose_splits(int units, int halves)
         best = S;
         best_cost = cost;
     }
-    return best;
+    return {best, best_cost};
 }
 
-template <int HD, int NR, bool XCH = true>
+template <int HD, int NR, bool XCH = true, bool APART = false>
 cudaError_t launch_shape(const AttnParams &p, const KeysMaps &tm, int flags, cudaStream_t st)
 {
-    if constexpr (XCH)
+    if constexpr (XCH && !APART) {
         if (p.n_splits == 1) return launch_shape<HD, NR, false>(p, tm, flags, st);
+        if constexpr (HD == 128 && NR == 64)
+            if (p.apart) return launch_shape<HD, NR, true, true>(p, tm, flags, st);
+    }
     using C = KeysShape<HD, NR>;
-    auto kern = attend_keys_kernel<HD, NR, XCH>;
+    auto kern = keys_kernel<HD, NR, XCH, APART>();
     int dev = 0;
-    cudaError_t e = configure<HD, NR, XCH>(&dev);
+    cudaError_t e = configure<HD, NR, XCH, APART>(&dev);
     if (e != cudaSuccess) return e;
     const int S = p.n_splits, units = p.B * p.Hkv, kb = keys_kb_rows(HD, p.G, p.K), tiles = (p.K + kb - 1) / kb;
     cudaLaunchConfig_t cfg = {};
@@ -883,22 +1009,36 @@ int keys_kb_rows(int d, int G, int K)
     return (K + tiles - 1) / tiles;
 }
 
-int keys_splits(int d, int G, int K, int units, int max_len)
+// `apart`: the block's own keys are left out of the tiles.  That takes a merging warp 1.4 us for each of its tasks, a third of it while
+// it would wait; worth it where those keys alone are a tile more for the longest CTA and no warp has two tasks (64 rows, 4096 keys: 8
+// units in sixteen CTAs 10.5 us a call, 9.7 so, 4 units 8.2 and 7.4).
+int keys_splits(int d, int G, int K, int units, int max_len, bool *apart)
 {
+    constexpr int APART_COST = 11;
     // the layers of a pass ask the same question: the last answer of this thread is kept
-    struct Key { int dev, d, nr, units, halves, S; };
-    static thread_local Key last = {-1, 0, 0, 0, 0, 0};
-    Key k = {-1, d, keys_rows(d, G, K), units, (max_len + HALF - 1) / HALF + 1, 0};   // (prefix and block in halves of their own)
+    struct Key { int dev, d, nr, units, halves, S; bool apart; };
+    static thread_local Key last = {-1, 0, 0, 0, 0, 0, false};
+    Key k = {-1, d, keys_rows(d, G, K), units, (max_len + HALF - 1) / HALF + 1, 0, false};   // (prefix and block in halves of their own)
     if (cudaGetDevice(&k.dev) != cudaSuccess) { (void)cudaGetLastError(); k.dev = -2; }
-    if (k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.units == last.units && k.halves == last.halves) return last.S;
-    switch (k.nr) {
-    case 16: k.S = d == 64 ? choose_splits<64, 16>(units, k.halves) : choose_splits<128, 16>(units, k.halves); break;
-    case 32: k.S = d == 64 ? choose_splits<64, 32>(units, k.halves) : choose_splits<128, 32>(units, k.halves); break;
-    case 64: k.S = d == 64 ? choose_splits<64, 64>(units, k.halves) : choose_splits<128, 64>(units, k.halves); break;
-    default: k.S = choose_splits<64, 128>(units, k.halves);
+    if (!(k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.units == last.units && k.halves == last.halves)) {
+        switch (k.nr) {
+        case 16: k.S = (d == 64 ? choose_splits<64, 16>(units, k.halves) : choose_splits<128, 16>(units, k.halves)).S; break;
+        case 32: k.S = (d == 64 ? choose_splits<64, 32>(units, k.halves) : choose_splits<128, 32>(units, k.halves)).S; break;
+        case 64:
+            if (d == 64) {
+                k.S = choose_splits<64, 64>(units, k.halves).S;
+            } else {
+                const Pick with = choose_splits<128, 64>(units, k.halves), without = choose_splits<128, 64>(units, k.halves - 1);
+                k.apart = without.S >= 8 && without.cost + APART_COST < with.cost;      // (64 tasks)
+                k.S = k.apart ? without.S : with.S;
+            }
+            break;
+        default: k.S = choose_splits<64, 128>(units, k.halves).S;
+        }
+        last = k;
     }
-    last = k;
-    return k.S;
+    *apart = last.apart;
+    return last.S;
 }
 
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st)

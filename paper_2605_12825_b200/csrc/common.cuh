@@ -45,6 +45,7 @@ struct AttnParams {
     long long len_cap;  // largest admissible prefix length: capacity - block width
     float scale_log2;   // softmax scale times log2(e)
     int early;          // host side: launch as a programmatic dependent
+    int apart;          // host side, keys kernel: the block's own keys apart from the tiles
 };
 
 // split s of a unit covers prefix positions [s*chunk, min((s+1)*chunk, P)); the split
@@ -131,7 +132,8 @@ size_t tc_stream_workspace_bytes(int B, int Hkv, int n_ctas);
 cudaError_t launch_attend_tc_stream(const AttnParams &p, int n_ctas, void *ws_body, int flags, cudaStream_t st);
 int keys_rows(int d, int G, int K);      // MMA columns of a query tile on the keys kernel (0: not its shape)
 int keys_kb_rows(int d, int G, int K);   // block positions of such a query tile
-int keys_splits(int d, int G, int K, int units, int max_len);   // CTAs per (unit, query tile) on the current device
+// CTAs per (unit, query tile) on the current device; whether the block's own keys are to be kept apart from the tiles
+int keys_splits(int d, int G, int K, int units, int max_len, bool *apart);
 int tc_kb_rows(int G, int K);            // block positions per query tile of 128 rows
 cudaError_t launch_attend_keys(const AttnParams &p, int flags, cudaStream_t st);        // n_splits = cluster size
 cudaError_t launch_combine(const AttnParams &p, int dtype, cudaStream_t st);
