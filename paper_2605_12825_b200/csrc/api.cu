@@ -261,39 +261,38 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 }
 
 // 33 to 64 query rows at head_dim 128 can run on either tcgen05 kernel: with the keys on the MMA's rows
-// (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).
+// (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).  (Us a call, keys against wide, 64 rows.)
+//  - Prefixes of one tile of 64 keys at most: the wide kernel, which needs no merge for them (8 units of 64 keys 5.2 and 4.4).
 //  - Where the caller promises a quiescent cache, the keys kernel has its first three tiles in shared memory by the time the
-//    query rows come, and is the rule up to 64 units (us a call, keys against wide, 64 rows: 8 units of 1000 keys 5.3 and
-//    6.8, of 4000 8.6 and 10.0; 16 of 2000 8.7 and 9.9; 32 of 1000 9.0 and 10.0, of 3500 14.3 and 14.9; 40 of 4000 18.8 and 22.2; 48
-//    of 3000 17.4 and 18.6; 64 of 2000 16.8 and 16.7; level at 8 of 300, 5.7 and 5.6).  From 24 units on only with bounds of
-//    1024 keys and more: below, the wide kernel is level where the lengths reach the bound (32 of 300 6.5 and 6.3) and the
-//    faster one where they do not (40 of 71 to 435 under a bound of 690, two layers of a decoder 65 and 60).
-//  - With more units the SMs are full in any case, and the wide kernel's takes less per key (128 units of 500, 1000 and 2000 keys
-//    13.5 and 11.8, 18.3 and 16.8, 28.0 and 26.3; 320 of 1000 51.5 and 46.5), unless its clusters are not all resident at
-//    once (256 of 2000, cut in two, 46.3 and 53.6; 160 of 1024 23.5 and 28.4, where 160 of 768, not cut, take 19.3 and 17.9).
-//  - Without the promise every load waits for the preceding kernel.  Up to 9 units, whose clusters of 16 the wide kernel merges
-//    slowly, the keys kernel is still the faster one while sixteen CTAs have two tiles each or fewer (8 units of 600 keys 6.6 and 8.0, of
-//    2000 7.8 and 9.7, of 3500 10.0 and 10.9; 2 of 1000 6.2 and 7.6; but of 300 6.6 and 6.4, of 4096 11.5 and 11.3).  For more units the
-//    two are within ten per cent of one another either way (32 of 2000 13.0 and 12.7; 64 of 2000 18.3 and 17.7).  There the wide kernel is the rule, short prefixes included, where its plan, whose clusters are powers of two, suits
-//    the number of units: not where its clusters are not all resident (34 to 37 units cut in 8: 37 of 1700 keys 14.5 and
-//    20.3), nor where clusters of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix
-//    is long (12 units of 8000 keys 15.9 and 18.4, 44 of 6000 29.0 and 30.8; at 2500 keys the wide one still won).
-//    Rows that do not fill warps of 32 cost the wide kernel a second way through its softmax, so that the line
-//    lies lower there (48 rows, 10 units of 3500 keys 9.8 and 11.8, 42 of 2500 16.1 and 17.3).
-//    Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys are a draw, and the equal rounding with
-//    width-1 steps decides for the keys kernel: a width-1 step (M <= 32) runs on it too, and cut into as many CTAs the two
-//    agree to the last bit, where the two kernels agree up to the rounding of their sums.  A program that wants the same
-//    bits from both widths throughout promises a quiescent cache or sets ORTHRUS_TC_SMALL_ROWS=1.
+//    query rows come, and is the rule while three CTAs a unit have an SM each (8 units of 500, 1000, 2000, 4000 and 8000 keys 5.2 and
+//    5.7, 5.3 and 6.0, 6.3 and 7.8, 8.6 and 9.9, 13.4 and 13.6; 16 of 2000 8.2 and 9.1; 32 of 3500 14.0 and 14.3; 40 of 4000 18.7 and 21.7;
+//    48 of 2000 14.6 and 14.6).  With more units the SMs are full in any case, and the wide kernel takes less per key (56 of 1000
+//    12.9 and 11.1, 64 of 2000 17.5 and 16.1).  A few tiles a unit do not pay for its merge where the clusters of 8 do not all find SMs
+//    of their own (9 to 23 units of up to 384 keys: 12 of 300 5.9 and 5.4; but 8 level), unless the rows do not fill warps of 32, which
+//    costs the wide kernel a second way through its softmax (12 of 300 keys, 48 rows, level).  From 24 units on only with bounds of
+//    1024 keys and more: below, the two are level where the lengths reach the bound, and the wide one is the faster where they do not.
+//  - Without the promise every load waits for the preceding kernel.  Up to 9 units the keys kernel is the faster one from 512 keys on while
+//    sixteen CTAs have two tiles each or fewer (8 units of 700 keys 6.5 and 6.8, of 2000 7.9 and 8.5, of 3500 10.0 and 10.4; of 300 6.2
+//    and 5.8, of 4096 11.3 and 10.7).  Else the wide kernel is the rule where its plan, whose clusters are mostly powers of two, suits
+//    the number of units: not where its clusters are not all resident (36 units of 1500 keys cut in 8 10.2 and 14.9), nor where clusters
+//    of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix is long (12 units of
+//    8000 keys 16.4 and 18.6, 44 of 6000 27.3 and 32.2); rows that do not fill warps of 32 draw that line lower.
+//    Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys go to the keys kernel, on which a width-1 step
+//    (M <= 32) runs too: it rounds the same probabilities and sums the same rounded ones (32 units of 2000 13.0 and 12.0).
+// So the promise decides which kernel serves some calls, and with it their rounding: see the flag in orthrus.h.
 static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
 {
     if (!tc_usable(L)) return false;
-    const int units = L->batch * L->n_kv_heads, M = L->n_q_heads / L->n_kv_heads * L->block;
-    if ((L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units <= 64 && (units < 24 || max_len_of(L) >= 1024)) return false;
-    if (units <= 9 && max_len_of(L) > 512 && max_len_of(L) + L->block <= 4032) return false;
+    const int units = L->batch * L->n_kv_heads, M = L->n_q_heads / L->n_kv_heads * L->block, max_len = max_len_of(L);
+    if (max_len <= tc_tile_positions()) return true;
+    if ((L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && 3 * units <= num_sms()) {
+        if (25 * units <= 4 * num_sms()) return M == 64 && max_len <= 384 && 17 * units > num_sms();      // to 23 units, from 9 on
+        if (max_len >= 1024) return false;
+    }
+    if (units <= 9 && max_len > 512 && max_len + L->block <= 4032) return false;
     const int S = make_plan(L, true, kn).n_splits;
     if (S > 1 && units > clusters_resident(S, 2)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
-    const int max_len = max_len_of(L);
     if (S == 8 && !roomy) return max_len <= 1536 || max_len > 3072;
     return !((S == 4 || S == 8) && roomy && max_len > (M == 64 ? 4096 : 2048));
 }
@@ -308,8 +307,8 @@ static int keys_tiles(const orthrus_layer_t *L)
 // to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
 // rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
 // 65 to 128 rows at head_dim 128 are two tiles there, which read the same keys: the faster way where latency counts, that is, with
-// the promise of a quiescent cache, up to 16 tiles and 8192 keys (keys against wide: 2 units of 77 rows, 3000 keys 5.9 and
-// 8.6 us, 4 of 128, 2000 keys 6.1 and 9.0, 8 of 128, 500, 2000 and 8000 keys 5.9 and 8.0, 8.7 and 9.1, 16.4 and 16.4).
+// the promise of a quiescent cache, up to 16 tiles and 8192 keys (keys against wide, 128 rows: 4 units of 700, 2000 and 8000 keys 5.4
+// and 6.7 us, 6.3 and 8.4, 13.2 and 13.0; 8 units 6.3 and 6.9, 8.8 and 8.9, 15.6 and 15.5).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
 // from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).
@@ -322,7 +321,7 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     const int M = L->n_q_heads / L->n_kv_heads * L->block, units = L->batch * L->n_kv_heads;
     if (L->head_dim == 128 && M > 64)
         return kn.small_rows < 0 && (L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units * keys_tiles(L) <= 16 &&
-               max_len_of(L) <= 8192;
+               max_len_of(L) > tc_tile_positions() && max_len_of(L) <= 8192;
     if (kn.small_rows > 0) return true;
     if (rows > 64) return max_len_of(L) > 320;
     return rows < 64 || L->head_dim == 64 || !wide_better(L, kn);

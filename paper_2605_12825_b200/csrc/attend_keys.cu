@@ -893,7 +893,7 @@ template <int HD, int NR, bool XCH, bool APART> cudaError_t configure(int *dev)
 //    each: 7.2 us at 2 CTAs, 6.2 at 3, 5.7 at 4 to 6).  At 64 rows that is worth CTAs without a key of their own (one unit of 100
 //    keys 6.0 us at 3, 5.0 at 8).
 //  - From 32 rows on there is much to tell, and CTAs that share an SM share the way to the others: once the clusters of a call do not all
-//    find SMs of their own, it takes 1 to 1.5 us more at 64 rows, 0.5 at 32.  A cluster stays within a GPC, so that this depends on the size of the
+//    find SMs of their own, it takes 1 to 1.5 us more at 33 to 64 rows, 0.5 at 32.  A cluster stays within a GPC, so that this depends on the size of the
 //    cluster (a B200 has SMs for 45, 33, 26, 22, 15, 15, 15, 11 and 7 clusters of 3 to 11 CTAs and for 7 of 12 to 16; us a call, 300 keys:
 //    clusters of 3, 36 units 6.7 and 48 8.4; of 4, 28 6.3 and 36 8.0; of 5, 24 6.5 and 28 7.6; of 6, 20 6.6 and 24 8.1; of 7, 14
 //    6.1 and 16 7.4).  A line at five ninths of the SMs, which stood here before, kept 28 units of 200 keys at 2 CTAs: 7.3 us, 6.3 at 4.
@@ -908,20 +908,21 @@ template <int HD, int NR, bool XCH, bool APART> cudaError_t configure(int *dev)
 // 4, 32 and 64 rows and both head sizes, where the count of residents by half-sized clusters and the line at five ninths took 3.8 to 4.9 %.
 // Where it misses most: 16 or 17 units of 24 to 26 halves, which get 13 CTAs and are 5 to 12 % faster with 8.
 struct Pick { int S, cost; };
-template <int HD, int NR> Pick choose_splits(int units, int halves)
+template <int HD, int NR> Pick choose_splits(int units, int halves, int rows)
 {
     constexpr bool FULL = HD == 128 && NR == 64;
     constexpr int TILE2 = HD == 128 ? 9 : 6, TILE3 = HD == 128 ? 16 : NR == 128 ? 15 : 10;
-    constexpr int TASKS = NR / 4 * (HD / 32), ALONE = NR >= 64 ? 10 : 6, MERGE = FULL ? 10 : 7;
-    constexpr int SHARED = NR == 64 ? (HD == 128 ? 15 : 8) : NR == 32 ? 5 : 0;    // CTAs of a call share SMs
+    constexpr int ALONE = NR >= 64 ? 10 : 6, MERGE = FULL ? 10 : 7;
+    const int tasks = FULL ? (rows + 3) / 4 * (HD / 32) : NR / 4 * (HD / 32);
+    const int shared = FULL ? (rows > 48 ? 15 : 11) : NR == 64 ? 8 : NR == 32 ? 5 : 0;        // CTAs of a call share SMs
     constexpr int PER_SM = KeysShape<HD, NR>::CTAS;
     const int sms = num_sms();
     int best = 1, best_cost = 1 << 30;
     for (int S = 1; S <= MAX_CLUSTER && S <= (FULL ? max(halves, 8) : halves); ++S) {
         const int tiles = ((halves + S - 1) / S + 1) / 2, ctas = units * S;
         int cost = (tiles > 1 ? TILE2 : 0) + (tiles > 2 ? min(tiles - 2, 1 << 20) * TILE3 : 0);
-        cost += S == 1 ? ALONE : MERGE + 4 * ((TASKS + 8 * S - 1) / (8 * S));
-        if (SHARED && S > (NR == 32 ? 2 : 1) && units > clusters_resident(S, 1)) cost += SHARED;
+        cost += S == 1 ? ALONE : MERGE + 4 * ((tasks + 8 * S - 1) / (8 * S));
+        if (shared && S > (NR == 32 ? 2 : 1) && units > clusters_resident(S, 1)) cost += shared;
         if (S > 1 && ctas > sms) cost += FULL ? 3 + 4 * (ctas - sms) / sms : 5 + min(5 * (ctas - sms) / sms, 10);
         if (S <= 8 && (tiles > 1 || 2 * ctas <= sms) ? cost > best_cost : cost >= best_cost) continue;
         if (S > 1 && (units > clusters_resident(S, PER_SM) || (S > 2 && 16 * ctas > 15 * PER_SM * sms))) continue;
@@ -1009,31 +1010,32 @@ int keys_kb_rows(int d, int G, int K)
     return (K + tiles - 1) / tiles;
 }
 
-// `apart`: the block's own keys are left out of the tiles.  That takes a merging warp 1.4 us for each of its tasks, a third of it while
-// it would wait; worth it where those keys alone are a tile more for the longest CTA and no warp has two tasks (64 rows, 4096 keys: 8
-// units in sixteen CTAs 10.5 us a call, 9.7 so, 4 units 8.2 and 7.4).
+// `apart`: the block's own keys are left out of the tiles.  That takes a merging warp 1.4 us for each of its tasks and sixteen keys, a
+// third of it while it would wait; worth it where those keys alone are a tile more for the longest CTA, no warp has two tasks and
+// every CTA an SM (64 rows, 4096 keys: 8 units in sixteen CTAs 10.5 us a call, 9.7 so, 4 units 8.2 and 7.4; but 32 units of 2000 keys in eight
+// 11.8 and 13.0, blocks of 32 with 4 units of 128 rows 10.0 and 10.7).
 int keys_splits(int d, int G, int K, int units, int max_len, bool *apart)
 {
-    constexpr int APART_COST = 11;
     // the layers of a pass ask the same question: the last answer of this thread is kept
-    struct Key { int dev, d, nr, units, halves, S; bool apart; };
-    static thread_local Key last = {-1, 0, 0, 0, 0, 0, false};
-    Key k = {-1, d, keys_rows(d, G, K), units, (max_len + HALF - 1) / HALF + 1, 0, false};   // (prefix and block in halves of their own)
+    struct Key { int dev, d, nr, rows, units, halves, S; bool few, apart; };
+    static thread_local Key last = {-1, 0, 0, 0, 0, 0, 0, false, false};
+    Key k = {-1, d, keys_rows(d, G, K), keys_kb_rows(d, G, K) * G, units, (max_len + HALF - 1) / HALF + 1, 0, K <= 16, false};   // (prefix and block in halves of their own)
     if (cudaGetDevice(&k.dev) != cudaSuccess) { (void)cudaGetLastError(); k.dev = -2; }
-    if (!(k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.units == last.units && k.halves == last.halves)) {
+    if (!(k.dev == last.dev && k.d == last.d && k.nr == last.nr && k.rows == last.rows && k.units == last.units && k.halves == last.halves &&
+          k.few == last.few)) {
         switch (k.nr) {
-        case 16: k.S = (d == 64 ? choose_splits<64, 16>(units, k.halves) : choose_splits<128, 16>(units, k.halves)).S; break;
-        case 32: k.S = (d == 64 ? choose_splits<64, 32>(units, k.halves) : choose_splits<128, 32>(units, k.halves)).S; break;
+        case 16: k.S = (d == 64 ? choose_splits<64, 16>(units, k.halves, k.rows) : choose_splits<128, 16>(units, k.halves, k.rows)).S; break;
+        case 32: k.S = (d == 64 ? choose_splits<64, 32>(units, k.halves, k.rows) : choose_splits<128, 32>(units, k.halves, k.rows)).S; break;
         case 64:
             if (d == 64) {
-                k.S = choose_splits<64, 64>(units, k.halves).S;
+                k.S = choose_splits<64, 64>(units, k.halves, k.rows).S;
             } else {
-                const Pick with = choose_splits<128, 64>(units, k.halves), without = choose_splits<128, 64>(units, k.halves - 1);
-                k.apart = without.S >= 8 && without.cost + APART_COST < with.cost;      // (64 tasks)
+                const Pick with = choose_splits<128, 64>(units, k.halves, k.rows), without = choose_splits<128, 64>(units, k.halves - 1, k.rows);
+                k.apart = k.few && without.S >= 8 && without.S * units <= num_sms() && without.cost + 11 < with.cost;      // (64 tasks)
                 k.S = k.apart ? without.S : with.S;
             }
             break;
-        default: k.S = choose_splits<64, 128>(units, k.halves).S;
+        default: k.S = choose_splits<64, 128>(units, k.halves, k.rows).S;
         }
         last = k;
     }

@@ -57,3 +57,20 @@ def test_clusters_at_the_lines(units, bound, splits, monkeypatch):
 def test_clusters_of_sixteen_of_the_wide_kernel(units, rows, bound, in_cache, splits, monkeypatch):
     flags = binding().LAYER_BLOCK_IN_CACHE if in_cache else 0
     assert planned(units, rows, bound, monkeypatch, flags, kernel="attend_tc_kernel") == (splits, 1)
+
+
+# with the promise of a quiescent cache: units, rows, bound, kernel
+@pytest.mark.parametrize("units,rows,bound,kernel", [
+    (8, 64, 64, "attend_tc_kernel"), (8, 64, 65, "attend_keys_kernel"), (8, 36, 64, "attend_tc_kernel"), (2, 128, 64, "attend_tc_kernel"),
+    (2, 128, 65, "attend_keys_kernel"), (9, 64, 384, "attend_tc_kernel"), (9, 64, 385, "attend_keys_kernel"), (9, 60, 300, "attend_keys_kernel"),
+    (23, 64, 1000, "attend_keys_kernel"), (24, 64, 1000, "attend_tc_kernel"), (49, 64, 1024, "attend_keys_kernel"), (50, 64, 1024, "attend_tc_kernel")])
+def test_lines_with_the_promise(units, rows, bound, kernel):
+    b = binding()
+    K = rows // 4
+    cache = torch.empty(units, 1, bound + K, 128, dtype=torch.bfloat16, device="cuda")
+    ln = torch.zeros(units, dtype=torch.int32, device="cuda")
+    q, kb = (torch.empty(units, K, h, 128, dtype=torch.bfloat16, device="cuda") for h in (4, 1))
+    layer = b.make_layer(cache, cache, ln, 4, K, bound, 0.0, b.LAYER_CACHE_QUIESCENT)
+    ws = b.new_workspace(b.orthrus_attend_workspace_bytes(layer))
+    (name, _), = captured_launches(lambda: b.orthrus_ar_verify_attend(layer, q, kb, kb, q, ws))
+    assert kernel in name

@@ -1,5 +1,5 @@
 """The keys kernel with the block's own keys apart from the tiles, which it takes where those keys alone would be a tile more for the
-longest CTA (64 rows, bounds just above sixteen CTAs of two tiles less one half): against the oracle over blocks of one to 64
+longest CTA (64 rows, bounds just above sixteen CTAs of two tiles less one half): against the oracle over blocks of one to sixteen
 positions, both views, the block as a tensor and in the cache, empty and short prefixes under the same bound, NaN behind the
 keys, peaked scores; the line of the rule; the same numbers behind a preceding call."""
 import pytest
@@ -18,8 +18,8 @@ def name_of(call):
     return name
 
 
-# 33 to 64 rows in one query tile, 66 and 128 in two: (Hq, Hkv, K); blocks of 17 to 64 take several groups of sixteen keys
-@pytest.mark.parametrize("shape", [(8, 2, 9), (8, 2, 16), (7, 1, 9), (2, 1, 17), (2, 1, 32), (1, 1, 33), (1, 1, 64), (8, 2, 32), (6, 2, 22)])
+# 33 to 64 rows in one query tile, 68 to 128 in two: (Hq, Hkv, K)
+@pytest.mark.parametrize("shape", [(8, 2, 9), (8, 2, 16), (7, 1, 9), (9, 1, 4), (16, 1, 4), (35, 1, 1), (6, 1, 12), (8, 1, 16)])
 @pytest.mark.parametrize("view", [oracle.VIEW_DIFFUSION, oracle.VIEW_AR])
 @pytest.mark.parametrize("peak", [1.0, 40.0])
 @pytest.mark.parametrize("in_cache", [False, True])
@@ -57,7 +57,7 @@ def test_apart_from_the_tiles(shape, view, peak, in_cache):
 
 
 @pytest.mark.parametrize("units,bound,apart", [(8, 4032, False), (8, 4033, True), (8, 4096, True), (8, 4097, False), (9, 4096, True),
-                                               (8, 2000, False), (8, 6000, False)])
+                                               (8, 2000, False), (8, 6000, False), (32, 2000, False)])
 def test_where_they_are_kept_apart(units, bound, apart):
     b = binding()
     if torch.cuda.get_device_properties(0).multi_processor_count != 148:
