@@ -221,9 +221,9 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
         }
         // Sixteen only where every cluster finds SMs of its own (up to 7 units on a B200; a cluster stays within a GPC): on shared ones
         // the CTAs of a cluster share the way to the others, which the merge fills.  Else the largest size that does and has a
-        // merge of its own (128 rows, 8 units of 500, 2000, 4000 and 16000 keys 7.9, 11.7, 13.1 and 25.7 us at 16, 6.7, 8.9, 11.1 and 25.3
-        // at 10; 6 units of 8000 13.1 at 16, 15.8 at 10), until streaming the keys is nearly all there is (24000 keys 34.6 and 34.9; 64
-        // rows, 2000 and 4000 keys 8.4 and 9.9 at 16, 7.8 and 10.0 at 10).  Behind a rotary write, whose CTAs are in between, 128 rows
+        // merge of its own (128 rows, 8 units of 2000, 4000, 8000 and 16000 keys 11.6, 12.9, 16.9 and 25.7 us at 16, 8.9, 11.1, 15.4 and
+        // 25.3 at 10; 6 units of 8000 13.1 at 16, 15.8 at 10), until streaming the keys is nearly all there is (24000 keys 34.5 and 34.9; 64
+        // rows, 2000 and 4000 keys 8.3 and 9.9 at 16, 7.8 and 10.1 at 10).  Behind a rotary write, whose CTAs are in between, 128 rows
         // and clusters of 10 do not go together (4000, 8000 and 16000 keys 14.1, 20.0 and 32.0 at 8, 16.5, 22.8 and 35.3 at 10, 15.6, 19.1
         // and 27.5 at 16).
         const int rows = G * L->block;
@@ -262,23 +262,24 @@ static Plan make_plan(const orthrus_layer_t *L, bool tc, const Knobs &kn)
 
 // 33 to 64 query rows at head_dim 128 can run on either tcgen05 kernel: with the keys on the MMA's rows
 // (attend_keys.cu) or with the query rows there, padded to 128 (attend_tc.cu, the wide kernel).  (Us a call, keys against wide, 64 rows.)
-//  - Prefixes of one tile of 64 keys at most: the wide kernel, which needs no merge for them (8 units of 64 keys 5.2 and 4.4).
+//  - Prefixes of one tile of 64 keys at most: the wide kernel, which needs no merge for them (8 units of 64 keys 5.3 and 4.4).
 //  - Where the caller promises a quiescent cache, the keys kernel has its first three tiles in shared memory by the time the
-//    query rows come, and is the rule while three CTAs a unit have an SM each (8 units of 500, 1000, 2000, 4000 and 8000 keys 5.2 and
-//    5.7, 5.3 and 6.0, 6.3 and 7.8, 8.6 and 9.9, 13.4 and 13.6; 16 of 2000 8.2 and 9.1; 32 of 3500 14.0 and 14.3; 40 of 4000 18.7 and 21.7;
-//    48 of 2000 14.6 and 14.6).  With more units the SMs are full in any case, and the wide kernel takes less per key (56 of 1000
-//    12.9 and 11.1, 64 of 2000 17.5 and 16.1).  A few tiles a unit do not pay for its merge where the clusters of 8 do not all find SMs
-//    of their own (9 to 23 units of up to 384 keys: 12 of 300 5.9 and 5.4; but 8 level), unless the rows do not fill warps of 32, which
-//    costs the wide kernel a second way through its softmax (12 of 300 keys, 48 rows, level).  From 24 units on only with bounds of
-//    1024 keys and more: below, the two are level where the lengths reach the bound, and the wide one is the faster where they do not.
+//    query rows come, and is the rule while three CTAs a unit have an SM each (8 units of 500, 1000, 2000, 4000 and 8000 keys 5.4 and
+//    6.2, 5.5 and 6.6, 6.3 and 7.7, 8.7 and 9.9, 13.5 and 13.5; 16 of 2000 8.8 and 9.6; 40 of 4000 18.7 and 21.2; 48 of 2000 14.2 and 14.2;
+//    but 28 to 33, whom the wide kernel's clusters of 8 suit, 32 of 2000 11.8 and 11.0, kept for the reason at the end).  With more
+//    units the SMs are full in any case, and the wide kernel takes less per key (56 of 1000 11.6 and 10.0, 64 of 2000 16.4 and 15.1).  A
+//    few tiles a unit do not pay for its merge from 9 units on (12 of 300 keys 5.8 and 5.4; 8 level), unless the rows do not fill warps
+//    of 32, which costs the wide kernel a second way through its softmax (12 of 300 keys, 48 rows, 5.3 and 5.4).  From 24 units on
+//    only with bounds of 1024 keys and more: below, the two are level where the lengths reach the bound, and the wide one is the faster
+//    where they do not.
 //  - Without the promise every load waits for the preceding kernel.  Up to 9 units the keys kernel is the faster one from 512 keys on while
-//    sixteen CTAs have two tiles each or fewer (8 units of 700 keys 6.5 and 6.8, of 2000 7.9 and 8.5, of 3500 10.0 and 10.4; of 300 6.2
-//    and 5.8, of 4096 11.3 and 10.7).  Else the wide kernel is the rule where its plan, whose clusters are mostly powers of two, suits
-//    the number of units: not where its clusters are not all resident (36 units of 1500 keys cut in 8 10.2 and 14.9), nor where clusters
+//    sixteen CTAs have two tiles each or fewer (8 units of 700 keys 6.4 and 6.7, of 2000 8.0 and 8.5, of 3500 10.3 and 10.4; of 300 6.2
+//    and 5.8, of 4096 11.8 and 10.8).  Else the wide kernel is the rule where its plan, whose clusters are mostly powers of two, suits
+//    the number of units: not where its clusters are not all resident (36 units of 1500 keys cut in 8 11.8 and 16.9), nor where clusters
 //    of 4 or 8 leave more than two fifths of the places empty (10 to 22 and 38 to 44 units) and the prefix is long (12 units of
-//    8000 keys 16.4 and 18.6, 44 of 6000 27.3 and 32.2); rows that do not fill warps of 32 draw that line lower.
+//    8000 keys 15.4 and 17.7, 44 of 6000 26.5 and 30.8); rows that do not fill warps of 32 draw that line lower.
 //    Where clusters of 8 fill the grid (23 to 33 units), bounds of 1537 to 3072 keys go to the keys kernel, on which a width-1 step
-//    (M <= 32) runs too: it rounds the same probabilities and sums the same rounded ones (32 units of 2000 13.0 and 12.0).
+//    (M <= 32) runs too: it rounds the same probabilities and sums the same rounded ones (32 units of 2000 13.0 and 11.9).
 // So the promise decides which kernel serves some calls, and with it their rounding: see the flag in orthrus.h.
 static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
 {
@@ -289,7 +290,8 @@ static bool wide_better(const orthrus_layer_t *L, const Knobs &kn)
         if (25 * units <= 4 * num_sms()) return M == 64 && max_len <= 384 && 17 * units > num_sms();      // to 23 units, from 9 on
         if (max_len >= 1024) return false;
     }
-    if (units <= 9 && max_len > 512 && max_len + L->block <= 4032) return false;
+    constexpr int kTwoTiles = 16 * 2 * 128 - 64;              // two tiles for each of sixteen CTAs, but for the block's half
+    if (16 * units <= num_sms() && max_len > 512 && max_len + L->block <= kTwoTiles) return false;
     const int S = make_plan(L, true, kn).n_splits;
     if (S > 1 && units > clusters_resident(S, 2)) return false;   // (the two kernels' CTAs fit an SM alike)
     const bool roomy = 5 * units * S < 3 * tc_ctas_per_sm(1) * num_sms();
@@ -307,8 +309,8 @@ static int keys_tiles(const orthrus_layer_t *L)
 // to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
 // rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
 // 65 to 128 rows at head_dim 128 are two tiles there, which read the same keys: the faster way where latency counts, that is, with
-// the promise of a quiescent cache, up to 16 tiles and 8192 keys (keys against wide, 128 rows: 4 units of 700, 2000 and 8000 keys 5.4
-// and 6.7 us, 6.3 and 8.4, 13.2 and 13.0; 8 units 6.3 and 6.9, 8.8 and 8.9, 15.6 and 15.5).
+// the promise of a quiescent cache, while nine CTAs a tile have SMs (up to 16 tiles), and up to 8192 keys (keys against wide, 128 rows: 4 units of 700, 2000 and 8000 keys 5.4
+// and 7.2 us, 6.3 and 8.7, 13.1 and 13.0; 8 units 6.3 and 7.2, 8.9 and 8.8, 15.5 and 15.4; of 64 keys 5.3 and 5.2).
 // Wide units at head_dim 64 with short prefixes stay on mma.sync: a CTA of 128 rows has an SM to itself
 // and takes about 9 us before its first key (128 units of 128 rows, bound 150, 9.3 against 12.1 us;
 // from 400 on it is the better one: 29 against 16 us, bound 2000 60 against 38 us).
@@ -320,7 +322,7 @@ static bool keys_usable(const orthrus_layer_t *L, const Knobs &kn)
     if (!rows || cache >= 0x7fffffffull || L->batch > 65535 || (long long)L->n_kv_heads * keys_tiles(L) > 65535 || !tc_driver_ok()) return false;
     const int M = L->n_q_heads / L->n_kv_heads * L->block, units = L->batch * L->n_kv_heads;
     if (L->head_dim == 128 && M > 64)
-        return kn.small_rows < 0 && (L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && units * keys_tiles(L) <= 16 &&
+        return kn.small_rows < 0 && (L->flags & ORTHRUS_LAYER_CACHE_QUIESCENT) && 9 * units * keys_tiles(L) <= num_sms() &&
                max_len_of(L) > tc_tile_positions() && max_len_of(L) <= 8192;
     if (kn.small_rows > 0) return true;
     if (rows > 64) return max_len_of(L) > 320;

@@ -70,7 +70,6 @@ constexpr int PANEL = KT * 128;            // bytes of [128 keys][64 columns]
 constexpr int MAX_CLUSTER = 16;
 constexpr uint32_t P_HIGH = 0x5380, P_LOW = 0x2180;   // 2^40 and 2^-60 as bf16: what an unshifted probability may be
 constexpr int MSG = 512 + 32;              // a message of the merge: 32 columns of four rows, their references, their sums
-constexpr int AHEAD = 1;                   // ring items asked into L2 beyond those the slots hold
 
 struct KeysMaps { CUtensorMap k, v, kb, vb; };
 struct KeysArgs {
@@ -891,16 +890,17 @@ template <int HD, int NR, bool XCH, bool APART> cudaError_t configure(int *dev)
 //    of 4 rows, 500 keys, 1, 2, 3 and 5 tiles a CTA 3.5, 4.4, 5.9 and 8.6 us; d = 64, 32 rows, 2 units of 500 keys 3.5, 4.2, 5.1, 7.0.
 //  - The merge: a warp takes some 0.4 us for a task, and the CTAs share the tasks (64 rows, 8 units of 300 keys, one tile
 //    each: 7.2 us at 2 CTAs, 6.2 at 3, 5.7 at 4 to 6).  At 64 rows that is worth CTAs without a key of their own (one unit of 100
-//    keys 6.0 us at 3, 5.0 at 8).
+//    keys 6.2 us at 3, 5.1 at 8).
 //  - From 32 rows on there is much to tell, and CTAs that share an SM share the way to the others: once the clusters of a call do not all
 //    find SMs of their own, it takes 1 to 1.5 us more at 33 to 64 rows, 0.5 at 32.  A cluster stays within a GPC, so that this depends on the size of the
 //    cluster (a B200 has SMs for 45, 33, 26, 22, 15, 15, 15, 11 and 7 clusters of 3 to 11 CTAs and for 7 of 12 to 16; us a call, 300 keys:
 //    clusters of 3, 36 units 6.7 and 48 8.4; of 4, 28 6.3 and 36 8.0; of 5, 24 6.5 and 28 7.6; of 6, 20 6.6 and 24 8.1; of 7, 14
-//    6.1 and 16 7.4).  A line at five ninths of the SMs, which stood here before, kept 28 units of 200 keys at 2 CTAs: 7.3 us, 6.3 at 4.
+//    6.3 and 16 7.6).  A line at five ninths of the SMs, which stood here before, kept 28 units of 200 keys at 2 CTAs: 7.3 us, 6.3 at 4.
 //  - Once they do not fit beside one another at all, the next call starts late (32 units of 1000 keys, 4 rows 5.8 us at 5 CTAs, 6.3
 //    at 8), the more so where clusters fill the GPU to the last place (56 units of 32 rows, 3000 keys 17.1 us at 4, 19.9 at 5).
 // Of sizes that cost the same the largest up to 8 (lengths are often below the bound the plan is
-// made for, and then the larger size has fewer tiles), else the smallest, and so where a CTA has one tile in any case
+// made for, and then the larger size has fewer tiles) and beyond where a CTA has three tiles or more (the last may be half: 8 units of 64
+// rows, 4096 keys 10.7 us at 11, 10.0 at 16); the smallest where a CTA has one tile in any case
 // and half the SMs are taken (16 units of 64 rows, 300 keys 5.8 us at 4, 6.3 at 6; but 8 of 4 rows 3.6 at 3, 3.4 at 6).  A second wave of clusters costs more than any
 // split gains (32 units of 64 rows, 1000 keys 9.1 us at 8, 12.8 at 9; 22 of 4000 keys 13.7 at 10, 20.7 at 11; 72 units of 32 rows,
 // 1000 keys 10.4 at 3, 17.4 at 4).
@@ -924,7 +924,8 @@ template <int HD, int NR> Pick choose_splits(int units, int halves, int rows)
         cost += S == 1 ? ALONE : MERGE + 4 * ((tasks + 8 * S - 1) / (8 * S));
         if (shared && S > (NR == 32 ? 2 : 1) && units > clusters_resident(S, 1)) cost += shared;
         if (S > 1 && ctas > sms) cost += FULL ? 3 + 4 * (ctas - sms) / sms : 5 + min(5 * (ctas - sms) / sms, 10);
-        if (S <= 8 && (tiles > 1 || 2 * ctas <= sms) ? cost > best_cost : cost >= best_cost) continue;
+        const bool larger = S <= 8 ? tiles > 1 || 2 * ctas <= sms : HD == 128 && tiles > 2;     // of two that cost the same
+        if (larger ? cost > best_cost : cost >= best_cost) continue;
         if (S > 1 && (units > clusters_resident(S, PER_SM) || (S > 2 && 16 * ctas > 15 * PER_SM * sms))) continue;
         best = S;
         best_cost = cost;

@@ -36,7 +36,7 @@
 // costs some 25 cycles, a chain of address arithmetic for each message as much again.  So there is an instance for each size of
 // cluster that plans come to, whose merge is straight-line code for that size (merge_fixed); other sizes, and the two-tile CTA, go through
 // loops (merge).  Us a call, with one merge for all sizes in loops and now: 8 units of 64 rows and 300 keys 6.4 and 5.3, of 1000
-// 7.4 and 6.6, of 4096 11.0 and 10.2; one unit of 2000 keys 8.5 and 7.0; 128 rows, 8 units of 500 keys 7.3 and 6.7.
+// 7.4 and 6.6, of 4096 11.0 and 10.0; one unit of 2000 keys 8.5 and 7.0; 128 rows, 8 units of 500 keys 7.3 and 6.7.
 // Before that the merge went through two cluster barriers with a release, and at clusters of 16 through L2: 5.8, 7.0, 10.2, 6.6 and 7.6.
 // (16 is where L2 was the better way still: one unit of 64 rows 6.6 against 7.0, 8 of 128 rows and 4096 keys 12.7 against 13.2; api.cu
 // has fewer of them.)
@@ -54,7 +54,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
-#include <type_traits>
 #include <unordered_map>
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -207,8 +206,8 @@ __device__ inline void merge(uint32_t tm_row, unsigned char *smem, uint32_t buf,
 
 // The same for the sizes that plans come to, straight through: no loop, no branch, no address that depends on one.  The
 // merge is run through once per call, and what it takes is its chains of instructions and not its bytes (a taken branch alone some 25
-// cycles): per call, merge() and this, 64 rows: a unit of 200 keys in a cluster of 2, 6.8 and 6.0 us, 8 units of 300 keys in 4, 6.4 and
-// 5.3, of 1000 in 8, 7.4 and 6.6, of 4096 in 16, 11.0 and 10.2; 128 rows, 8 units of 500 keys in 8, 7.3 and 6.7.
+// cycles): per call, merge() and this, 64 rows: a unit of 200 keys in a cluster of 2, 6.8 and 5.8 us, 8 units of 300 keys in 4, 6.4 and
+// 5.3, of 1000 in 8, 7.4 and 6.6, of 4096 in 16, 11.0 and 10.0; 128 rows, 8 units of 500 keys in 8, 7.3 and 6.7.
 template <int SP>
 __device__ inline void merge_fixed(uint32_t tm_row, unsigned char *smem, uint32_t buf, uint32_t x_bar, int rank, int r, bool valid, bool have_o,
                                    float m, float l, __nv_bfloat16 *row, int32_t *status)

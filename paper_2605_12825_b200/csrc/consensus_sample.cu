@@ -142,17 +142,14 @@ template <typename T> __device__ __noinline__ VecOf<T> load_part(const T *row, i
     for (int e = 0; e < Elem<T>::N; ++e) r.x[e] = i0 + e >= 0 && i0 + e < V ? Elem<T>::load(row + i0 + e) : -INFINITY;
     return r;
 }
-template <typename T, bool CALL> __device__ inline void load_vec(const T *row, const RowShape &s, int v, float (&x)[Elem<T>::N]) {
+template <typename T> __device__ inline void load_vec(const T *row, const RowShape &s, int v, float (&x)[Elem<T>::N]) {
     const int i0 = v * Elem<T>::N - s.a;
     if (whole<T>(s, v)) {
         Elem<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(row + i0)), x);
-    } else if (CALL) {
+    } else {
         const VecOf<T> r = load_part<T>(row, i0, s.V);
 #pragma unroll
         for (int e = 0; e < Elem<T>::N; ++e) x[e] = r.x[e];
-    } else {
-#pragma unroll
-        for (int e = 0; e < Elem<T>::N; ++e) x[e] = i0 + e >= 0 && i0 + e < s.V ? Elem<T>::load(row + i0 + e) : -INFINITY;
     }
 }
 
@@ -268,8 +265,8 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const T *la, con
             }
             else for (int e = v0 + lane; e < v1; e += 32) {
                 float f[1][N];
-                load_vec<T, true>(ra, sh, e, f[0]); absorb<1, N>(a, f, c);
-                load_vec<T, true>(rd, sh, e, f[0]); absorb<1, N>(d, f, c);
+                load_vec<T>(ra, sh, e, f[0]); absorb<1, N>(a, f, c);
+                load_vec<T>(rd, sh, e, f[0]); absorb<1, N>(d, f, c);
             }
             a = warp_fold(a);
             d = warp_fold(d);
@@ -395,7 +392,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
             if (v < w1) {
                 float x[N], y[N];
                 if (whole<T>(sh, v)) { Elem<T>::unpack(cx, x); Elem<T>::unpack(cy, y); }
-                else { load_vec<T, true>(ra, sh, v, x); load_vec<T, true>(rd, sh, v, y); }
+                else { load_vec<T>(ra, sh, v, x); load_vec<T>(rd, sh, v, y); }
                 double m[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
                 for (int e = 0; e < N; ++e) m[e & 3] += mass_of(x[e], y[e], c, st, use_p);
@@ -472,7 +469,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2) sample_finish_kernel(const 
             const int v = q0 + r * 32 + lane;
             float x[N], y[N];
             double mine[N], sum = 0.0;
-            if (v < q1) { load_vec<T, true>(ra, sh, v, x); load_vec<T, true>(rd, sh, v, y); }
+            if (v < q1) { load_vec<T>(ra, sh, v, x); load_vec<T>(rd, sh, v, y); }
 #pragma unroll
             for (int e = 0; e < N; ++e) {
                 mine[e] = v < q1 ? mass_of(x[e], y[e], c, st, use_p) : 0.0;

@@ -120,8 +120,7 @@ __device__ inline void griddep_launch() { asm volatile("griddepcontrol.launch_de
 __device__ inline void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-// (without the release, which waits for the thread's stores: 330 cycles against 18)
+// (without a release, which waits for the thread's stores: 330 cycles against 18)
 __device__ inline void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ inline uint32_t cluster_rank() {
