@@ -32,6 +32,11 @@
  *       draft, committed, ar_argmax  [B][K] int32;  n_commit, next_anchor, cache_len [B] int32
  *     Query head hq reads KV head hq / (Hq / Hkv).
  *   - dtype ORTHRUS_BF16: bf16 inputs/outputs, fp32 softmax and accumulation.
+ *     Range of the attention calls on tensor cores: a row's probabilities carry a
+ *     common factor that puts the largest anywhere between 2^-60 and 2^40, and their
+ *     products with V are summed in fp32.  Over up to 2^16 keys nothing overflows or is
+ *     lost while the magnitudes of V are zero or between 2^-50 and 2^70; a row that sees
+ *     a score of +inf or NaN is NaN, keys with a score of -inf do not count.
  *     dtype ORTHRUS_FP32: fp32 everywhere (a slow test mode).
  */
 #ifndef ORTHRUS_H_
@@ -97,7 +102,12 @@ typedef struct {
  * serialisation: they may start while the preceding kernel is still running and wait
  * for it on the device before touching anything it may have produced.  With this
  * flag they request the first prefix K/V tiles before that wait.  Without it nothing
- * is read early and any caller is safe.
+ * is read early and any caller is safe.  The flag also has a say in which of two kernels
+ * serves calls of 33 to 128 query rows (block * n_q_heads / n_kv_heads) at head_dim 128.
+ * Both round the same probabilities to bf16; one sums the rounded ones for the softmax
+ * denominator, the other the unrounded ones, so that with and without the flag a result
+ * may differ by up to 2^-9 of itself and by the order of fp32 sums.  Neither is the more
+ * exact one; a caller that compares bits keeps the flag as it is.
  *
  * ORTHRUS_LAYER_NO_EARLY_LAUNCH: launch with ordinary stream order only.  (Calls without a
  * layer are always launched early; ORTHRUS_NO_EARLY_LAUNCH=1 in the environment, read at

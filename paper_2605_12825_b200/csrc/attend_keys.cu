@@ -37,7 +37,10 @@
 // relative precision whatever the reference, so that the maximum itself is not needed.  Otherwise (a vote of the warpgroup) the
 // references are raised to the rows' maxima (redux.sync over the warp, shared memory over the four warps) and what
 // earlier tiles have added up is rescaled.  The result is the exact softmax because
-// numerator and denominator use the same reference.  References are integers: another reference
+// numerator and denominator use the same reference.  A tile that moves them takes its exponentials twice: 8 units of 64 rows, 4000 keys, with
+// all scores about +60 or -60 10.4 us a call instead of 8.6 (9.9 in a kernel that took every tile's maxima), 128 rows 13.4 instead of
+// 11.2 (12.2), 4 rows 6.5 instead of 6.2; scores of standard deviation 3 cost nothing.  (The first key's scores as
+// references before the maxima gained 0.1 us of it where all scores are alike and lost 1 where they are not.)  References are integers: another reference
 // scales a probability by a power of two, so that its rounding to bf16, and with it the result of this kernel up to
 // the order of fp32 sums, does not depend on how the keys were cut.  Probabilities are written as
 // bf16 rows [key][row], which is the MN-major B operand of the second product; their sums are taken

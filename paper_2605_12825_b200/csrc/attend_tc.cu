@@ -24,7 +24,9 @@
 // The output accumulator O stays in TMEM for the whole CTA.  A row's reference starts at 0 and is left alone as long as no
 // probability exceeds 2^40 and, in the first tile that shows the row a key, the largest is not below 2^-60: floating-point
 // numbers keep their relative precision whatever the reference, so that no tile pays for its row maxima.  Otherwise the
-// owner threads set the reference to the tile's maximum, or raise it, and rescale their O rows in TMEM.  The result is the
+// owner threads set the reference to the tile's maximum, or raise it, and rescale their O rows in TMEM, and the tile takes its
+// exponentials twice (8 units of 128 rows, 4000 keys, without the promise below, all scores about +60 or -60: 12.3 us a call instead of
+// 11.6, 32 of 1000 keys 13.9 instead of 13.0; 13.1 and 14.2 in a kernel that took every tile's maxima).  The result is the
 // exact softmax because the same shift is used for the numerator and the denominator.
 //
 // Merge of the S partial results of a unit, inside the kernel (there is no second launch), through distributed shared

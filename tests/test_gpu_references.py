@@ -157,3 +157,24 @@ def test_range_of_values(shape, splits, sign, scale, monkeypatch):
         t[v] *= 2.0 ** scale
     got = run(t, shape, 1024, splits, monkeypatch)
     assert torch.equal(got.float() * 2.0 ** -scale, plain.float())
+
+
+@pytest.mark.parametrize("shape,lens", [((8, 2, 16), [1000, 800]), ((8, 2, 16), [4096, 70]), ((14, 2, 11), [1000, 513]), ((8, 2, 32), [2000, 64])])
+def test_the_promise_changes_rounding_at_most(shape, lens):
+    """With the promise of a quiescent cache these shapes run on the keys kernel, without it on either: the same probabilities, sums of
+    them before or after rounding (2^-9 at most between them), each output rounded to bf16 (2^-9 each)."""
+    b = binding()
+    Hq, Hkv, K = shape
+    t = inputs(("", Hq, Hkv, 128, K), lens, max(lens), None)
+    g = {k: v.cuda() for k, v in t.items()}
+    outs = []
+    for flags in (0, b.LAYER_CACHE_QUIESCENT):
+        layer = b.make_layer(g["k_cache"], g["v_cache"], g["cache_len"], Hq, K, max(lens), 0.0, flags)
+        ws = b.new_workspace(b.orthrus_attend_workspace_bytes(layer))
+        out = torch.empty_like(g["q_ar"])
+        b.orthrus_ar_verify_attend(layer, g["q_ar"], g["k_ar_blk"], g["v_ar_blk"], out, ws)
+        assert b.orthrus_read_status(ws) == 0
+        outs.append(out.double().cpu())
+    x, y = outs
+    # (fp32 sums of up to 4096 products in another order: 4096 * 2^-24 of the sum of their magnitudes at most, which is below max|V| = 3)
+    assert ((x - y).abs() <= 3 * 2.0 ** -9 * torch.maximum(x.abs(), y.abs()) + 3 * 4096 * 2.0 ** -24).all()
