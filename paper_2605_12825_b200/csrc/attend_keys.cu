@@ -902,9 +902,9 @@ template <int HD, int NR, bool XCH, bool APART> cudaError_t configure(int *dev)
 //  - Once they do not fit beside one another at all, the next call starts late (32 units of 1000 keys, 4 rows 5.8 us at 5 CTAs, 6.3
 //    at 8), the more so where clusters fill the GPU to the last place (56 units of 32 rows, 3000 keys 17.1 us at 4, 19.9 at 5).
 // Of sizes that cost the same the largest up to 8 (lengths are often below the bound the plan is
-// made for, and then the larger size has fewer tiles) and beyond where a CTA has three tiles or more (the last may be half: 8 units of 64
-// rows, 4096 keys 10.7 us at 11, 10.0 at 16); the smallest where a CTA has one tile in any case
-// and half the SMs are taken (16 units of 64 rows, 300 keys 5.8 us at 4, 6.3 at 6; but 8 of 4 rows 3.6 at 3, 3.4 at 6).  A second wave of clusters costs more than any
+// made for, and then the larger size has fewer tiles) and beyond where a CTA has three tiles or more, of which the last is only half
+// with the larger size (8 units of 64 rows, 4096 keys 10.5 us at 11, 9.8 at 16; but 15 of 4000 keys, eight halves a CTA either way, 11.3 at 8, 11.7 at 9);
+// the smallest where a CTA has one tile in any case and half the SMs are taken (16 units of 64 rows, 300 keys 5.8 us at 4, 6.3 at 6; but 8 of 4 rows 3.6 at 3, 3.4 at 6).  A second wave of clusters costs more than any
 // split gains (32 units of 64 rows, 1000 keys 9.1 us at 8, 12.8 at 9; 22 of 4000 keys 13.7 at 10, 20.7 at 11; 72 units of 32 rows,
 // 1000 keys 10.4 at 3, 17.4 at 4).
 // Against sweeps of 1 to 92 units, 64 to 8000 keys and all sizes, the choice is 0.5 to 0.6 % above the best size in the mean at
@@ -922,12 +922,13 @@ template <int HD, int NR> Pick choose_splits(int units, int halves, int rows)
     const int sms = num_sms();
     int best = 1, best_cost = 1 << 30;
     for (int S = 1; S <= MAX_CLUSTER && S <= (FULL ? max(halves, 8) : halves); ++S) {
-        const int tiles = ((halves + S - 1) / S + 1) / 2, ctas = units * S;
+        const int chunk = (halves + S - 1) / S, tiles = (chunk + 1) / 2, ctas = units * S;
         int cost = (tiles > 1 ? TILE2 : 0) + (tiles > 2 ? min(tiles - 2, 1 << 20) * TILE3 : 0);
         cost += S == 1 ? ALONE : MERGE + 4 * ((tasks + 8 * S - 1) / (8 * S));
         if (shared && S > (NR == 32 ? 2 : 1) && units > clusters_resident(S, 1)) cost += shared;
         if (S > 1 && ctas > sms) cost += FULL ? 3 + 4 * (ctas - sms) / sms : 5 + min(5 * (ctas - sms) / sms, 10);
-        const bool larger = S <= 8 ? tiles > 1 || 2 * ctas <= sms : HD == 128 && tiles > 2;     // of two that cost the same
+        // of two that cost the same
+        const bool larger = S <= 8 ? tiles > 1 || 2 * ctas <= sms : HD == 128 && tiles > 2 && chunk < (halves + best - 1) / best;
         if (larger ? cost > best_cost : cost >= best_cost) continue;
         if (S > 1 && (units > clusters_resident(S, PER_SM) || (S > 2 && 16 * ctas > 15 * PER_SM * sms))) continue;
         best = S;
