@@ -57,6 +57,7 @@
 // Every mbarrier wait is bounded: on expiry the CTA raises ORTHRUS_DEV_WAIT_TIMEOUT, its warps go
 // on through their barriers with void results, the MMAs and copies in flight are waited for, and it ends.
 #include <cuda.h>
+#include <float.h>
 #include <atomic>
 #include <mutex>
 #include "common.cuh"
@@ -460,7 +461,8 @@ __device__ __forceinline__ void attend_keys(const AttnParams &p, const KeysMaps 
                     const float m = ceilf(fmaxf(fmaxf(red[kt], red[NR + kt]), fmaxf(red[2 * NR + kt], red[3 * NR + kt])) * sc);
                     const float m_old = -ref[kt], m_new = u > 0 ? fmaxf(m, m_old) : m;
                     red[kt] = u > 0 ? ex2(m_old - m_new) : 1.f;           // the factor of what row kt has summed up so far
-                    ref[kt] = m_new == -INFINITY ? 0.f : -m_new;
+                    // (a row that has met scores of -inf only: a reference so low that the first other score is out of proportion)
+                    ref[kt] = m_new == -INFINITY ? FLT_MAX : -m_new;
                 }
                 bar_group(wg);
                 if (u > 0) {

@@ -455,7 +455,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
         const uint32_t lane_base = *tmem_slot + ((uint32_t)(wq * 32) << 16);
         const uint32_t TM_O = C::tm_o(ti);
         float m_run = 0.f, l_run = 0.f;
-        bool fresh = true;                  // the row has seen no key yet
+        bool fresh = true;                  // the row has seen no key yet, or only such with scores of -inf
         bool have_o = false;
         int a_row = 0, k0_row = 0;          // packed form: this row's anchor, first key of its block
         if constexpr (PACK) {
@@ -577,8 +577,8 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
                     }
                 }
                 if (!ok) break;
-                fresh = fresh && !(lim > lo);
                 l_run += (acc0.x + acc0.y) + (acc1.x + acc1.y);
+                fresh = fresh && !(l_run > 0.f);               // (nothing but scores of -inf tells of no reference)
                 // P over the scores, 2 bf16 per 32-bit column
                 tmem_st32(lane_base + TM_S, pk);
                 tmem_st_wait();

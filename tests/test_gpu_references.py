@@ -135,6 +135,24 @@ def test_scores_that_are_not_finite(shape, splits, value, at, monkeypatch):
 
 
 @pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("splits", [None, 1, 2, 4])
+@pytest.mark.parametrize("void", [64, 128, 256, 390])
+def test_tiles_of_minus_infinity_ahead_of_low_scores(shape, splits, void, monkeypatch):
+    """The first `void` keys have scores of -inf for every row, the others about -90: the first tiles tell nothing of where a
+    row's scores are, and the reference moves in the first one that does."""
+    t = inputs(shape, [400, 513], 1024, None)
+    a = math.sqrt(90.0 * math.sqrt(shape[3]))
+    t["q_ar"][..., 0] = a
+    for k in ("k_cache", "k_ar_blk"):
+        t[k][..., 0] = -a
+    t["k_cache"][:, :, :void, 0] = -math.inf
+    for b, p in enumerate([400, 513]):
+        t["k_cache"][b, :, p:] = float("nan")
+    got = run(t, shape, 1024, splits, monkeypatch)
+    assert_close(got, oracle_attend(oracle.VIEW_AR, t), torch.bfloat16, f"{shape} void={void} splits={splits}")
+
+
+@pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("splits", [1, 2, 8])
 @pytest.mark.parametrize("sign,scale", [(1, 70), (-1, -48)])
 def test_range_of_values(shape, splits, sign, scale, monkeypatch):
