@@ -339,6 +339,7 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
     // The producer is to ask for its first tiles as early as can be: it sets up the barriers of the ring and waits for nobody.
     if (warp == C::PRODUCER_WARP) {
         if (lane == 0) {
+            *abort_flag = aligned ? 0 : 1;                    // (here, as this warp reads it without having waited for another)
             int n_tiles_q = 0;                                // query tiles with rows = MMA warps at work
             for (int ti = 0; ti < NT; ++ti) n_tiles_q += tile_rows(ti) > 0;
 #pragma unroll 1
@@ -353,7 +354,6 @@ attend_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps tm, const in
         bar_start_arrive(NTHREADS);
     } else if (warp == C::MMA_WARP) {
         if (lane == 0) {
-            *abort_flag = aligned ? 0 : 1;
             mbar_init(bar(BAR_QFULL), 1);
             for (int x = 0; x < NT; ++x) {
                 const int rows = tile_rows(x), n_act = max(1, (rows + 31) >> 5);      // softmax warps with rows
