@@ -307,7 +307,8 @@ static int keys_tiles(const orthrus_layer_t *L)
 
 // Units of at most 32 query rows (4 rows, 8 units of 4000 keys 5.7 against 9.7 us on the wide kernel, 32 rows 6.9), of 33
 // to 64 by the rule above, and of any number at head_dim 64 run with the keys on the MMA's
-// rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits (measurement knobs).
+// rows.  ORTHRUS_TC_SMALL_ROWS=0 keeps them on the other kernels, =1 puts there whatever fits but 65 to 128 rows at
+// head_dim 128, which then stay on the wide kernel (measurement knobs).
 // 65 to 128 rows at head_dim 128 are two tiles there, which read the same keys: the faster way where latency counts, that is, with
 // the promise of a quiescent cache, while nine CTAs a tile have SMs (up to 16 tiles), and up to 8192 keys (keys against wide, 128 rows: 4 units of 700, 2000 and 8000 keys 5.4
 // and 7.2 us, 6.3 and 8.7, 13.1 and 13.0; 8 units 6.3 and 7.2, 8.9 and 8.8, 15.5 and 15.4; of 64 keys 5.3 and 5.2).

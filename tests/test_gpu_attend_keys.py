@@ -67,7 +67,7 @@ def test_block_in_the_cache(view, shape):
 
 @pytest.mark.parametrize("shape", [(16, 4, 64, 8), (32, 8, 128, 1), (16, 4, 128, 13)])
 def test_many_units_of_unequal_length(shape):
-    """More clusters than fit at once: handed out longest prefix first; peaked scores move the running maximum."""
+    """More clusters than fit at once: handed out longest prefix first; scores of a few units to either side."""
     lens = [int(x) for x in torch.randint(0, 3000, (40,), generator=torch.Generator().manual_seed(3))]
     wl, t = inputs(shape, lens, 3000)
     t["q_ar"] *= 8

@@ -1,7 +1,7 @@
 """The keys kernel with its first tiles asked for ahead of the preceding kernel, several calls one behind the other: CTAs of
 one to many tiles (two of them fold into three slots at head_dim 128; from three on the slots of the ring are used again), the
 block's own keys alone in a tile and beside prefix keys, scores that make the references move in the first
-tile and in later ones."""
+tile of each softmax warpgroup (later ones: test_gpu_references.py)."""
 import pytest
 import torch
 

@@ -1,6 +1,6 @@
 """The tcgen05 kernels' softmax references, which start at zero and move only when a tile's probabilities are out of proportion
 with them: all scores far above or far below zero, one key far above the rest in the first tile (as attention sinks are), in the
-middle or at the end, references that rise tile by tile, at the cluster sizes the library uses most and at uneven ones; the packed
+middle or at the end, references that rise tile by tile, or of some rows in one tile and of others in another, at the cluster sizes the library uses most and at uneven ones; the packed
 multi-block form, whose rows see their first key at different tiles; visible scores that are not finite; the range of values
 that the header states."""
 import math
@@ -73,6 +73,30 @@ def test_references_that_move(shape, score, splits, monkeypatch):
         t = inputs(shape, lens, 1024, score)
         got = run(t, shape, 1024, splits, monkeypatch)
         assert_close(got, oracle_attend(oracle.VIEW_AR, t), torch.bfloat16, f"{shape} {score} {lens} splits={splits}")
+
+
+# references of some rows: further widths of the keys kernel's second operand (32 and 48 rows)
+@pytest.mark.parametrize("shape", SHAPES + [("keys", 8, 2, 128, 8), ("keys", 8, 2, 64, 8), ("keys", 8, 2, 64, 12)])
+@pytest.mark.parametrize("splits", [1, 2])
+@pytest.mark.parametrize("first", [0.0, -60.0])
+def test_references_of_some_rows(shape, splits, first, monkeypatch):
+    """Every third row meets scores of +60 from key 256 on and of +120 from key 512 on, every other third of +60 from key 640 to
+    767 only: with one CTA a unit those are the second and third 128-key tile of one softmax warpgroup of the keys kernel and the
+    third of the other.  `first`: the scores of all rows over the first 256 keys, each warpgroup's first tile."""
+    t = inputs(shape, [1000, 700], 1024, None)
+    _, Hq, Hkv, d, K = shape
+    a = math.sqrt(60.0 * math.sqrt(d))
+    row = torch.arange(K)[:, None] * (Hq // Hkv) + torch.arange(Hq)[None, :] % (Hq // Hkv)       # a row's place in its query tile
+    t["q_ar"][..., 0], t["q_ar"][..., 1], t["q_ar"][..., 2] = a * (row % 3 == 1), a * (row % 3 == 2), a
+    for k in ("k_cache", "k_ar_blk"):
+        t[k][..., :3] = 0
+    k = t["k_cache"]
+    k[:, :, :256, 2] = a * first / 60.0
+    k[:, :, 256:512, 0], k[:, :, 512:, 0], k[:, :, 640:768, 1] = a, 2 * a, a
+    for b, p in enumerate([1000, 700]):
+        k[b, :, p:] = float("nan")
+    got = run(t, shape, 1024, splits, monkeypatch)
+    assert_close(got, oracle_attend(oracle.VIEW_AR, t), torch.bfloat16, f"{shape} splits={splits} first={first}")
 
 
 # the packed form: blocks per sequence, width, heads (several blocks in a query tile of 128 rows)

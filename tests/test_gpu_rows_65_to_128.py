@@ -23,7 +23,7 @@ def inputs(shape, lens, hint):
     return t
 
 
-def run(t, shape, hint, flags, view=oracle.VIEW_AR):
+def run(t, shape, hint, flags, view=oracle.VIEW_AR, grids=None):
     b = binding()
     Hq, Hkv, K = shape
     x = "ar" if view == oracle.VIEW_AR else "diff"
@@ -33,7 +33,7 @@ def run(t, shape, hint, flags, view=oracle.VIEW_AR):
     out = torch.full_like(g["q_" + x], float("nan"))
     f = b.orthrus_ar_verify_attend if view == oracle.VIEW_AR else b.orthrus_diffusion_block_attend
     blk = [None, None] if flags & b.LAYER_BLOCK_IN_CACHE else [g[f"k_{x}_blk"], g[f"v_{x}_blk"]]
-    (name, _), = captured_launches(lambda: f(layer, g["q_" + x], *blk, out, ws))
+    (name, _), = captured_launches(lambda: f(layer, g["q_" + x], *blk, out, ws), grids)
     f(layer, g["q_" + x], *blk, out, ws)
     assert b.orthrus_read_status(ws) == 0
     return out.cpu(), "keys" if "attend_keys_kernel" in name else "wide" if "attend_tc_kernel" in name else name
@@ -106,12 +106,18 @@ def test_uneven_clusters_of_the_wide_kernel(splits, peak, monkeypatch):
     assert_close(got, oracle_attend(oracle.VIEW_AR, t), torch.bfloat16, f"splits={splits} peak={peak}")
 
 
-@pytest.mark.parametrize("shape", [(16, 4, 24), (16, 4, 4)])
-@pytest.mark.parametrize("B", [33, 70, 128])
-def test_batches_in_the_order_of_their_length(shape, B):
-    """More clusters than fit at once on either kernel, equal lengths among them."""
+@pytest.mark.parametrize("K", [24, 4])
+@pytest.mark.parametrize("B,Hkv", [(33, 16), (70, 8), (97, 8), (128, 4)])
+@pytest.mark.parametrize("lens", ["some equal", "all equal"])
+def test_batches_in_the_order_of_their_length(K, B, Hkv, lens):
+    """More clusters than fit at once on either kernel (two CTAs to an SM), so that they are handed out by length: entries that are there
+    for some of a lane's four registers, all lengths alike, the largest an exact power of two."""
     g = torch.Generator().manual_seed(B)
-    lens = [int(x) for x in torch.randint(0, 12, (B,), generator=g) * 60]
-    t = inputs(shape, lens, 700)
-    got, _ = run(t, shape, 700, 0)
+    lens = [256] + [int(x) for x in torch.randint(0, 12, (B - 1,), generator=g) * 20] if lens == "some equal" else [256] * B
+    shape = (4 * Hkv, Hkv, K)
+    t = inputs(shape, lens, 256)
+    grids = []
+    got, _ = run(t, shape, 256, 0, grids=grids)
+    x, y, z = grids[0]
+    assert x * y * z > 2 * torch.cuda.get_device_properties(0).multi_processor_count
     assert_close(got, oracle_attend(oracle.VIEW_AR, t), torch.bfloat16, f"{shape} {B}")
