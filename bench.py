@@ -63,9 +63,9 @@ def measured_tensor_peak():
 # DRAM bytes (read + write) per launch from the ncu captures summarised under profiles/, each
 # with the first 16 hex digits of the SHA-256 of the kernel sources the capture was taken
 # from: once those files change the figure is stale and None is reported.
-NCU_TRAFFIC = {"cfg2_8b_b1": (17064576, "b761ffb8afe492c6"), "cfg3_ragged": (512661248, "b761ffb8afe492c6"),
-               "cfg4_long": (542857088, "b761ffb8afe492c6")}
-NCU_TRAFFIC_SOURCES = ("attend_tc.cu", "tc_ptx.cuh")
+_KEYS_SOURCES, _WIDE_SOURCES = ("attend_keys.cu", "tc_ptx.cuh"), ("attend_tc.cu", "tc_ptx.cuh")
+NCU_TRAFFIC = {"cfg2_8b_b1": (17037184, "9280a89184272723", _KEYS_SOURCES), "cfg3_ragged": (512398832, "210a8939e1d68383", _WIDE_SOURCES),
+               "cfg4_long": (541228416, "210a8939e1d68383", _WIDE_SOURCES)}
 NCU_TRAFFIC_LM_HEAD = {("cfg2_8b_b1", 4096): (1247972200, "a99646786b164572"),
                        ("cfg3_ragged", 4096): (1066815368, "a99646786b164572")}
 NCU_TRAFFIC_LM_HEAD_SOURCES = ("lm_head_argmax.cu", "tc_ptx.cuh")
@@ -87,7 +87,7 @@ def recorded_traffic(workload: str):
     rec = NCU_TRAFFIC.get(workload)
     if rec is None:
         return None
-    return rec[0] if _source_digest(NCU_TRAFFIC_SOURCES) == rec[1] else None
+    return rec[0] if _source_digest(rec[2]) == rec[1] else None
 
 
 def recorded_lm_head_traffic(workload: str, hidden_dim: int):
