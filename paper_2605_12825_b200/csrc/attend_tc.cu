@@ -216,7 +216,9 @@ __device__ inline void merge_fixed(uint32_t tm_row, unsigned char *smem, uint32_
 {
     constexpr bool EVEN = 16 % SP == 0;                       // every CTA has as many groups; else one more here, one fewer there
     constexpr int NG = (16 + SP - 1) / SP, W = 8 * NG, SRC = NG * 4096;       // groups and columns of a CTA at most, bytes of a source
-    constexpr int AT_ONCE = W == 8 ? 5 : W == 16 ? 3 : W == 32 ? 2 : 1;      // destinations whose columns are read together
+    // destinations whose columns are read together (at eight CTAs five and two: three at a time were level on short prefixes and 1 % of
+    // a call slower on long ones, 32 units of 128 rows, 32768 keys)
+    constexpr int AT_ONCE = W == 8 || W == 16 ? 5 : W == 32 ? 2 : 1;
     const uint32_t mine = smem_u32(smem) + buf;
     auto next = [&](int k) { return (SP & (SP - 1)) == 0 ? (rank + k) & (SP - 1) : rank + k - (rank + k >= SP ? SP : 0); };
     auto full = [&](int q) { return EVEN || first_group(q + 1, SP) - first_group(q, SP) == NG; };
