@@ -64,7 +64,7 @@ def measured_tensor_peak():
 # with the first 16 hex digits of the SHA-256 of the kernel sources the capture was taken
 # from: once those files change the figure is stale and None is reported.
 _KEYS_SOURCES, _WIDE_SOURCES = ("attend_keys.cu", "tc_ptx.cuh"), ("attend_tc.cu", "tc_ptx.cuh")
-NCU_TRAFFIC = {"cfg2_8b_b1": (17037184, "9280a89184272723", _KEYS_SOURCES), "cfg3_ragged": (511526628, "8adae529f28260d5", _WIDE_SOURCES),
+NCU_TRAFFIC = {"cfg2_8b_b1": (17039616, "fe45f048937d9bb3", _KEYS_SOURCES), "cfg3_ragged": (511526628, "8adae529f28260d5", _WIDE_SOURCES),
                "cfg4_long": (540911616, "8adae529f28260d5", _WIDE_SOURCES)}
 NCU_TRAFFIC_LM_HEAD = {("cfg2_8b_b1", 4096): (1246778368, "d326b2f1da0240ec"),
                        ("cfg3_ragged", 4096): (1065347968, "d326b2f1da0240ec")}

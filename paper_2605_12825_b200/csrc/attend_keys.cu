@@ -610,11 +610,19 @@ __device__ __forceinline__ void attend_keys(const AttnParams &p, const KeysMaps 
                 for (int k = 0; k < 4; ++k) at[k] = 4 * g + k < M ? row_off(4 * g + k) + col : -1;
             };
             float *wt = reinterpret_cast<float *>(smem + C::OFF_XW) + warp * ((MAX_CLUSTER + 1) * 4);
+            bool got = true;
+            auto wait_for_messages = [&]() {
+                // (the wait outlasts every other one: a CTA of the cluster that gave one up sends all the same)
+                got = __all_sync(0xffffffffu, mbar_wait_long(bar(C::BAR_X), 0));
+                if (!got && lane == 0 && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
+            };
+            // (the places of a task are worked out ahead of the wait, or behind the stores of the one before)
+            if constexpr (!APART) { places(warp); wait_for_messages(); }
 #pragma unroll 1
-            for (int n = warp; n < my_tasks; n += SW) {
-                places(n);
+            for (int n = warp; n < my_tasks && got; n += SW) {
                 BlockPart bp;
                 if constexpr (APART) {
+                    places(n);
                     const int g = (n * S + rank) / (HD / 32), row = min(4 * g + (lane >> 2 & 3), M - 1);
                     bp = block_part(reinterpret_cast<const __nv_bfloat16 *>(q) + row_off(row), bk, bv + (n * S + rank) % (HD / 32) * 32,
                                     blk_stride, p.K, p.causal ? i0 + (int)((uint32_t)row * args.inv_g >> 16) + 1 : p.K, p.scale_log2, lane);
@@ -624,10 +632,8 @@ __device__ __forceinline__ void attend_keys(const AttnParams &p, const KeysMaps 
                         for (int t = 0; t < 4; ++t) *reinterpret_cast<float2 *>(o + t * 8) = make_float2(bp.o[t][0], bp.o[t][1]);
                     }
                 }
-                if (n == warp) {
-                    // (the wait outlasts every other one: a CTA of the cluster that gave one up sends all the same)
-                    const bool got = __all_sync(0xffffffffu, mbar_wait_long(bar(C::BAR_X), 0));
-                    if (!got && lane == 0 && p.status) atomicOr(p.status, ORTHRUS_DEV_WAIT_TIMEOUT);
+                if (APART && n == warp) {
+                    wait_for_messages();
                     if (!got) break;
                 }
                 const unsigned char *msg = smem + n * S * MSG;
@@ -674,6 +680,7 @@ __device__ __forceinline__ void attend_keys(const AttnParams &p, const KeysMaps 
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     if (at[k] >= 0) out[at[k]] = __float2bfloat16_rn(y[k]);
+                if (!APART && n + SW < my_tasks) places(n + SW);
                 __syncwarp();
             }
         }
